@@ -139,6 +139,7 @@ size_t layout(cmcg_handle* H, const Geom& g, const cmcg_options& o, char* base) 
         H->sc = c.take<double>(SC_COUNT);
         return c.off + 256;
     }
+    H->wface = o.precision == CMCG_FP64 ? c.take<double>(np) : nullptr;
     H->ya = c.take<double>(np);
     H->yb = c.take<double>(np);
     H->tmp = c.take<double>(np);
@@ -349,7 +350,9 @@ bool use_pairs(const cmcg_handle* H, bool src) {
     return H->opt.tile[3] == 2 && std::is_same<T, float>::value && !src && step2_supported(H->g, H->order);
 }
 
-// One leapfrog step cur -> prev (in place).  FP32 3D 7-point steps without a source go through
+// One leapfrog step cur -> prev (in place).  FP64 handles step with the integer stencil sum.  The
+// FP64 periods of a mixed-precision handle (its outer gradients) keep the plain FP64 step: a
+// change of their last bits would send the FP32 inner solve along other roundings.  FP32 3D 7-point steps without a source go through
 // the bulk-copy kernel when tile[3] == 4 (tile[1] = band rows, tile[0] = planes per CTA).
 template <typename T>
 void step_one(cmcg_handle* H, const T* cur, T* prev, const T* kap, const T* S, double cs, double sn, int flags,
@@ -366,6 +369,13 @@ void step_one(cmcg_handle* H, const T* cur, T* prev, const T* kap, const T* S, d
         int ty = 0, zb = 0;
         if (step_bulk_plan(H->g, H->opt.tile[1], H->opt.tile[0], &ty, &zb)) {
             launch_step_bulk(H->g, (const float*)cur, (float*)prev, (const float*)kap, flags, ty, zb, H->sc, H->st);
+            return;
+        }
+    }
+    if constexpr (std::is_same<T, double>::value) {
+        if (H->wface) {
+            launch_step_soft(H->g, H->order, cur, prev, kap, H->wface, S, cs, sn, flags, H->src_faces,
+                             cur == (const double*)H->ya, H->st);
             return;
         }
     }
@@ -1246,7 +1256,7 @@ using namespace cmcg::detail;
 namespace cmcg {
 
 // Carve of the scratch a stand-alone FP64 period needs: coefficients, source, the two wave
-// buffers, masked copies of the initial data, reduction slots.
+// buffers, the masked copy of the initial displacement, the face weights, reduction slots.
 static size_t scratch_layout(cmcg_handle* H, const Geom& g, char* base) {
     Carver c{base};
     const size_t np = (size_t)g.np;
@@ -1258,7 +1268,7 @@ static size_t scratch_layout(cmcg_handle* H, const Geom& g, char* base) {
     H->ya = c.take<double>(np);
     H->yb = c.take<double>(np);
     H->z0 = c.take<double>(np);
-    H->z1 = c.take<double>(np);
+    H->wface = c.take<double>(np);
     long long nb = std::max<long long>(kMaxBlocksReduce, plane_blocks(g, kZcEnds));
     H->partials = c.take<double>((size_t)8 * nb);
     H->tickets = c.take<unsigned>(kNumTickets);
@@ -1311,12 +1321,13 @@ int wave_period_in_scratch(const cmcg_grid* grid, const double* c, double omega,
     if (H.dt * H.dt * cmax * cmax * rho >= 4.0) return CMCG_ERR_CFL;
     cudaMemsetAsync(H.sc, 0, sizeof(double) * SC_COUNT, st);
     launch_setup_coeffs(H.g, c, bc->dirichlet_mask, dir, H.dt, H.kap64, nullptr, H.mass, H.mask, H.red(), st);
+    launch_face_weights(H.g, H.kap64, H.wface, st);
     const bool src = f || g;
     const int zce = H.g.dim == 3 ? kZcEnds : 1;
     if (src) launch_make_source(H.g, f, g, H.kap64, H.S, zce, false, st);
+    H.src_faces = !f;
     launch_mask_copy(H.g, u0, H.kap64, H.z0, st);
-    launch_mask_copy(H.g, v0, H.kap64, H.z1, st);
-    forward_period<double>(&H, H.z0, H.z1, src, 1, uT, vT);
+    forward_period<double>(&H, H.z0, v0, src, 1, uT, vT);  // the start kernel selects v0's Dirichlet entries
     if (cudaStreamSynchronize(st) != cudaSuccess) return CMCG_ERR_CUDA;
     return cuda_status();
 }
@@ -1436,6 +1447,7 @@ int cmcg_create(const cmcg_grid* grid, const double* c, double omega, const cmcg
     if (!H->has_dir)
         for (int l = 0; l < H->nlev; ++l) H->lv[l].mask = nullptr;
     launch_reciprocal(H->g.np, H->mass, H->minv, H->st);
+    if (H->wface) launch_face_weights(H->g, H->kap64, H->wface, H->st);
     if (H->mass32) {
         launch_to_float(H->g.np, H->mass, H->mass32, H->st);
         launch_to_float(H->g.np, H->minv, H->minv32, H->st);
@@ -1495,6 +1507,7 @@ int cmcg_wave_period(cmcg_handle* h, const double* u0, const double* v0, const d
     if (h->first_order) return CMCG_ERR_UNSUPPORTED;
     const bool src = f || g;
     if (src) launch_make_source(h->g, f, g, h->kap64, h->S, h->g.dim == 3 ? kZcEnds : 1, false, h->st);
+    h->src_faces = !f;
     if (src) source_updated(h);
     launch_mask_copy(h->g, u0, h->kap64, h->z0, h->st);
     launch_mask_copy(h->g, v0, h->kap64, h->z1, h->st);
@@ -1535,7 +1548,7 @@ int cmcg_bulk_wait_selftest(int spin_limit, void* stream) {
 int cmcg_check_status(long long* count, long long* site, long long* index) {
     if (cudaDeviceSynchronize() != cudaSuccess) return CMCG_ERR_CUDA;
     long long total = 0, first_site = -1, first_index = 0;
-    for (auto read : {check_read_wave, check_read_riesz, check_read_pair}) {
+    for (auto read : {check_read_wave, check_read_riesz, check_read_pair, check_read_soft}) {
         long long w[3];
         read(w);
         if (w[0] > 0 && first_site < 0) {
@@ -1581,6 +1594,7 @@ int cmcg_solve(cmcg_handle* h, const double* f, const double* g, double tol, dou
         launch_make_source(h->g, f, g, h->kap64, h->S, h->g.dim == 3 ? kZcEnds : 1, false, h->st);
     else
         launch_fill(h->S, 2 * h->g.np, 0.0, h->st);
+    h->src_faces = !f;
     source_updated(h);
     cmcg_stats local{};
     cmcg_stats* st = stats ? stats : &local;
@@ -1615,6 +1629,7 @@ int cmcg_solve_host(cmcg_handle* h, const double* f_host, const double* g_host, 
         cudaMemcpyAsync(h->stage, g_host, bytes, cudaMemcpyHostToDevice, h->st);
         launch_make_source(h->g, nullptr, h->stage, h->kap64, h->S, zce, true, h->st);
     }
+    h->src_faces = !f_host;
     source_updated(h);
     if (cuda_status() != CMCG_OK) return CMCG_ERR_CUDA;
     cmcg_stats local{};

@@ -29,6 +29,7 @@ void note_launch(long long k);
 void check_read_wave(long long* out);
 void check_read_riesz(long long* out);
 void check_read_pair(long long* out);
+void check_read_soft(long long* out);
 long long launch_count();
 
 // ---- wave.cu --------------------------------------------------------------------------
@@ -106,6 +107,16 @@ void launch_scale_complex(long long n, double* u, double s, cudaStream_t st);
 void launch_make_source(const Geom& g, const double* f, const double* gb, const double* kap64, double* S, int zc,
                         bool accumulate, cudaStream_t st);
 long long plane_blocks(const Geom& g, int zc);
+
+// ---- step_soft.cu -----------------------------------------------------------------------
+// FP64 leapfrog step with the stencil sum in integer arithmetic (any dimension, order and step
+// flags).  wface: 1 / (1 + beta) on the absorbing faces' nodes (launch_face_weights).  src_faces:
+// S is nonzero on absorbing faces only.  reverse: blocks in descending order (alternating from
+// step to step, a step starts on the planes that the previous one left in the L2 cache).
+void launch_face_weights(const Geom& g, const double* kap, double* w, cudaStream_t st);
+void launch_step_soft(const Geom& g, int order, const double* cur, double* prev, const double* kap,
+                      const double* wface, const double* S, double cs, double sn, int flags, bool src_faces,
+                      bool reverse, cudaStream_t st);
 
 // ---- step_bulk.cu -----------------------------------------------------------------------
 // FP32 3D 7-point leapfrog step with TMA bulk-copy staging (homogeneous; flags 0, PREV_SCALED,

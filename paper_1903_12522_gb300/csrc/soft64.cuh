@@ -1,0 +1,71 @@
+// FP64 stencil sums on the integer pipes.
+//
+// GB300 issues FP64 arithmetic at 2 lanes per SM and cycle: one warp instruction holds the pipe
+// for 16 cycles, as long as 64 issue slots of the SM.  A leapfrog update is mostly the
+// neighbour sum, so the sum runs on integers instead: the stencil's values are aligned to the
+// largest exponent among them as 64-bit fixed point with six guard bits, added exactly, and the
+// sum goes back to FP64 once.  The rounding error of the sum is then at most the truncation of
+// the aligned values, 2^-6 units in the last place of the largest one each, plus one conversion,
+// where the chain of FP64 additions rounds every partial sum (up to 6 |y|) to 2^-53 of itself.
+//
+// The largest exponent field must lie in [kExpLo, kExpLo + kExpSpan) (magnitudes from 2^-895
+// to 2^1017): infinities, NaN, overflowing sums and fields that are zero or tiny throughout take
+// the plain FP64 sum instead, which is what every value took before.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include "common.cuh"
+
+namespace cmcg {
+namespace soft64 {
+
+constexpr unsigned kExpLo = 128u << 20;
+constexpr unsigned kExpSpan = 1912u << 20;
+
+// A finite double as a signed fixed-point mantissa (53 bits and six guard bits) and the exponent
+// field of its high word.  A zero or subnormal counts as 2^-1023 (1 + ...): aligned to an
+// exponent field of kExpLo or more it is shifted out.
+struct Term {
+    long long m;
+    unsigned e;
+};
+
+__device__ __forceinline__ Term term(double y) {
+    const unsigned hi = (unsigned)__double2hiint(y), lo = (unsigned)__double2loint(y);
+    Term t;
+    t.e = hi & 0x7ff00000u;
+    const unsigned mh = (hi & 0xfffffu) | 0x100000u;
+    const unsigned long long m = ((unsigned long long)__funnelshift_l(lo, mh, 6) << 32) | (lo << 6);
+    const long long s = (long long)((int)hi >> 31);
+    t.m = ((long long)m ^ s) - s;
+    return t;
+}
+
+// The term in units of 2^(E - 1081), E << 20 = emax (a shift of 63 or more leaves the sign).
+__device__ __forceinline__ long long align(const Term& t, unsigned emax) {
+    long long r;
+    asm("shr.s64 %0, %1, %2;" : "=l"(r) : "l"(t.m), "r"((emax - t.e) >> 20));
+    return r;
+}
+
+// Is the fixed-point sum safe for terms with this largest exponent field?
+__device__ __forceinline__ bool in_range(unsigned emax) { return emax - kExpLo < kExpSpan; }
+
+// x 2^(E - 1081) as a double, truncated to 53 bits; *ok turns false when |x| < 2^32 (the sum
+// cancelled to nearly nothing, or is zero), which the caller leaves to the FP64 sum.
+__device__ __forceinline__ double to_double(long long x, unsigned emax, bool* ok) {
+    const long long s = x >> 63;
+    const unsigned long long a = (unsigned long long)((x ^ s) - s);
+    const unsigned ah = (unsigned)(a >> 32), al = (unsigned)a;
+    *ok = ah != 0u;
+    const int lz = __clz((int)ah);  // 0 .. 31 where ok
+    const unsigned nh = __funnelshift_l(al, ah, lz), nl = al << (lz & 31);
+    const unsigned hi = (nh >> 11) + emax + ((unsigned)(4 - lz) << 20);
+    return __hiloint2double((int)(hi | ((unsigned)(s >> 32) & 0x80000000u)), (int)__funnelshift_r(nl, nh, 11));
+}
+
+__device__ __forceinline__ unsigned max3(unsigned a, unsigned b, unsigned c) { return max(max(a, b), c); }
+
+}  // namespace soft64
+}  // namespace cmcg

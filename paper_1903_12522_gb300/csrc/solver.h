@@ -35,6 +35,8 @@ struct cmcg_handle {
     float* S32 = nullptr;  // FP32 copy of S, the source of FP32 leapfrog steps (FP32 / mixed)
     float *mass32 = nullptr, *minv32 = nullptr;  // FP32 copies of M and M^-1 (FP32 / mixed)
     unsigned char* scol = nullptr;  // 3D: columns with source inside the grid (launch_source_columns)
+    double* wface = nullptr;  // FP64: 1 / (1 + beta) on absorbing faces (launch_face_weights)
+    bool src_faces = false;   // S is nonzero on absorbing faces only (a boundary datum, no interior source)
     unsigned char* mask = nullptr;
     const double* warm = nullptr;  // cmcg_solve_warm: the start field U (complex, interleaved) of this solve
     // wave buffers (sized for double; FP32 stepping uses the first half) + FP64 temp
