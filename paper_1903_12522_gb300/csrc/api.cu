@@ -235,6 +235,18 @@ void l2_kappa_end(cmcg_handle* H) {
     H->l2_kappa = false;
 }
 
+void set_source(cmcg_handle* H, const double* f, const double* g) {
+    const Geom& G = H->g;
+    H->src_faces = !f;
+    if (H->scol) cudaMemsetAsync(H->scol, 0, (size_t)G.sx * G.sy, H->st);
+    if (f || g) {
+        launch_make_source(G, f, g, H->kap64, H->S, H->S32, H->scol, G.dim == 3 ? kZcEnds : 1, false, H->st);
+    } else {
+        cudaMemsetAsync(H->S, 0, sizeof(double) * 2 * G.np, H->st);
+        if (H->S32) cudaMemsetAsync(H->S32, 0, sizeof(float) * 2 * G.np, H->st);
+    }
+}
+
 void source_updated(cmcg_handle* H) {
     if (H->S32) launch_to_float(2 * H->g.np, H->S, H->S32, H->st);
     if (H->scol) launch_source_columns(H->g, H->S, H->scol, H->st);
@@ -323,8 +335,15 @@ PeriodBuffers fwd_begin(cmcg_handle* H, const double* w0, const double* w1, bool
         if (!w0f_ready) launch_to_float(g.np, w0, w0f, H->st);
         b.w0t = w0f;
     }
-    launch_start<T>(g, H->order, (const T*)b.w0t, w1, (T*)b.prev, (T*)b.cur, kap, src ? H->S : nullptr, H->dt,
-                    zce, H->st, v32);
+    if constexpr (std::is_same<T, double>::value) {
+        if (H->wface) {
+            launch_start_soft(g, H->order, w0, w1, (double*)b.prev, (double*)b.cur, kap, H->wface,
+                              src ? H->S : nullptr, H->src_faces, H->dt, zce, H->st);
+            return b;
+        }
+    }
+    launch_start<T>(g, H->order, (const T*)b.w0t, w1, (T*)b.prev, (T*)b.cur, kap, src ? H->S : nullptr,
+                    H->src_faces, H->dt, zce, H->st, v32);
     return b;
 }
 
@@ -445,8 +464,17 @@ void fwd_end(cmcg_handle* H, const PeriodBuffers& b, const double* w1, bool src,
     const T* kap = std::is_same<T, float>::value ? (const T*)H->kap32 : (const T*)H->kap64;
     const double thN = H->omega * H->N * H->dt;
     const int m = fp32_handoff<T>(mode) ? (H->vec32_active ? 3 : 2) : mode;
+    if constexpr (std::is_same<T, double>::value) {
+        if (H->wface) {
+            launch_end_soft(g, H->order, m, (const double*)b.cur, (const double*)b.prev, (const double*)b.w0t, w1, kap,
+                            H->mass, H->wface, src ? H->S : nullptr, H->src_faces, cos(thN), sin(thN), out0, out1,
+                            H->red(), H->dt, zce, H->st);
+            H->periods += 1;
+            return;
+        }
+    }
     launch_end<T>(g, H->order, m, (const T*)b.cur, (const T*)b.prev, (const T*)b.w0t, w1, kap, step_mass<T>(H),
-                  src ? H->S : nullptr, cos(thN), sin(thN), out0, out1, H->red(), H->dt, zce, H->st);
+                  src ? H->S : nullptr, H->src_faces, cos(thN), sin(thN), out0, out1, H->red(), H->dt, zce, H->st);
     H->periods += 1;
 }
 
@@ -477,6 +505,14 @@ PeriodBuffers adj_begin(cmcg_handle* H, const double* a, const double* bb, int m
         }
     }
     T* t = (T*)H->tmp;
+    if constexpr (std::is_same<T, double>::value) {
+        if (H->wface) {
+            launch_adj_prep_soft(g, bb, H->minv, H->wface, t, zce, H->st);
+            launch_adj_start_soft(g, H->order, a, t, H->minv, kap, H->wface, (double*)b.cur, (double*)b.prev, H->dt, zce,
+                                  H->st);
+            return b;
+        }
+    }
     launch_adj_prep<T>(g, bb, step_mass<T>(H), kap, t, zce, H->st);
     launch_adj_start<T>(g, H->order, a, t, step_mass<T>(H), kap, (T*)b.cur, (T*)b.prev, H->dt, zce, H->st);
     return b;
@@ -519,6 +555,14 @@ void adj_end(cmcg_handle* H, const PeriodBuffers& b, const double* a, const doub
     const int zce = g.dim == 3 ? kZcEnds : 1;
     const T* kap = std::is_same<T, float>::value ? (const T*)H->kap32 : (const T*)H->kap64;
     const int m = fp32_handoff<T>(mode) ? (H->vec32_active ? 3 : 2) : mode;
+    if constexpr (std::is_same<T, double>::value) {
+        if (H->wface) {
+            launch_adj_final_soft(g, H->order, m, (const double*)b.cur, (const double*)b.prev, H->mass, kap, H->wface,
+                                  H->minv, a, bb, d0, d1, o0, o1, gt1, H->red(), H->dt, zce, H->st);
+            H->periods += 1;
+            return;
+        }
+    }
     launch_adj_final<T>(g, H->order, m, (const T*)b.cur, (const T*)b.prev, step_mass<T>(H), kap, H->minv, a, bb, d0, d1, o0,
                         o1, gt1, H->red(), H->dt, zce, H->st);
     H->periods += 1;
@@ -576,10 +620,18 @@ void runup(cmcg_handle* H, int periods, double* w0, double* w1) {
         std::swap(cur, prev);
     }
     const double tN = total * H->dt;
-    launch_end<T>(g, H->order, 1, cur, prev, (const T*)nullptr, nullptr, kap, step_mass<T>(H), H->S,
+    H->periods += periods;
+    if constexpr (std::is_same<T, double>::value) {
+        if (H->wface) {
+            launch_end_soft(g, H->order, 1, cur, prev, nullptr, nullptr, kap, H->mass, H->wface, H->S, H->src_faces,
+                            ramp(tN, ttr) * cos(H->omega * tN), ramp(tN, ttr) * sin(H->omega * tN), w0, w1, H->red(),
+                            H->dt, zce, H->st);
+            return;
+        }
+    }
+    launch_end<T>(g, H->order, 1, cur, prev, (const T*)nullptr, nullptr, kap, step_mass<T>(H), H->S, H->src_faces,
                   ramp(tN, ttr) * cos(H->omega * tN), ramp(tN, ttr) * sin(H->omega * tN), w0, w1, H->red(), H->dt,
                   zce, H->st);
-    H->periods += periods;
 }
 
 // The FP32 run-up split around a step loop that runs elsewhere (the engine's batched
@@ -597,7 +649,7 @@ void runup_finish_f32(cmcg_handle* H, int periods, double* w0, double* w1) {
     const float* cur = (const float*)(odd ? H->ya : H->yb);
     const float* prev = (const float*)(odd ? H->yb : H->ya);
     const double ttr = periods * H->T, tN = total * H->dt;
-    launch_end<float>(g, H->order, 1, cur, prev, (const float*)nullptr, nullptr, H->kap32, step_mass<float>(H), H->S,
+    launch_end<float>(g, H->order, 1, cur, prev, (const float*)nullptr, nullptr, H->kap32, step_mass<float>(H), H->S, H->src_faces,
                       ramp(tN, ttr) * cos(H->omega * tN), ramp(tN, ttr) * sin(H->omega * tN), w0, w1, H->red(),
                       H->dt, g.dim == 3 ? kZcEnds : 1, H->st);
     H->periods += periods;
@@ -1324,9 +1376,9 @@ int wave_period_in_scratch(const cmcg_grid* grid, const double* c, double omega,
     launch_face_weights(H.g, H.kap64, H.wface, st);
     const bool src = f || g;
     const int zce = H.g.dim == 3 ? kZcEnds : 1;
-    if (src) launch_make_source(H.g, f, g, H.kap64, H.S, zce, false, st);
+    if (src) launch_make_source(H.g, f, g, H.kap64, H.S, nullptr, nullptr, zce, false, st);
     H.src_faces = !f;
-    launch_mask_copy(H.g, u0, H.kap64, H.z0, st);
+    launch_mask_copy<double>(H.g, u0, H.has_dir ? H.mask : nullptr, H.z0, st);
     forward_period<double>(&H, H.z0, v0, src, 1, uT, vT);  // the start kernel selects v0's Dirichlet entries
     if (cudaStreamSynchronize(st) != cudaSuccess) return CMCG_ERR_CUDA;
     return cuda_status();
@@ -1506,15 +1558,20 @@ int cmcg_wave_period(cmcg_handle* h, const double* u0, const double* v0, const d
     if (!h || !u0 || !v0 || !uT || !vT) return CMCG_ERR_INVALID_ARG;
     if (h->first_order) return CMCG_ERR_UNSUPPORTED;
     const bool src = f || g;
-    if (src) launch_make_source(h->g, f, g, h->kap64, h->S, h->g.dim == 3 ? kZcEnds : 1, false, h->st);
-    h->src_faces = !f;
-    if (src) source_updated(h);
-    launch_mask_copy(h->g, u0, h->kap64, h->z0, h->st);
-    launch_mask_copy(h->g, v0, h->kap64, h->z1, h->st);
-    if (h->opt.precision == CMCG_FP32)
-        forward_period<float>(h, h->z0, h->z1, src, 1, uT, vT);
-    else
-        forward_period<double>(h, h->z0, h->z1, src, 1, uT, vT);
+    if (src) set_source(h, f, g);
+    // the stencils need u0 with zeros on the Dirichlet nodes (v0's entries there are selected away
+    // by the start kernel); FP32 periods read it as the float copy of the temp buffer
+    if (h->opt.precision == CMCG_FP32) {
+        launch_mask_copy<float>(h->g, u0, h->has_dir ? h->mask : nullptr, (float*)h->tmp, h->st);
+        forward_period<float>(h, u0, v0, src, 1, uT, vT, true);
+    } else {
+        const double* w0 = u0;
+        if (h->has_dir) {
+            launch_mask_copy<double>(h->g, u0, h->mask, h->z0, h->st);
+            w0 = h->z0;
+        }
+        forward_period<double>(h, w0, v0, src, 1, uT, vT);
+    }
     if (cudaStreamSynchronize(h->st) != cudaSuccess) return CMCG_ERR_CUDA;
     return cuda_status();
 }
@@ -1522,12 +1579,11 @@ int cmcg_wave_period(cmcg_handle* h, const double* u0, const double* v0, const d
 int cmcg_adjoint_period(cmcg_handle* h, const double* a, const double* b, double* q0, double* q1) {
     if (!h || !a || !b || !q0 || !q1) return CMCG_ERR_INVALID_ARG;
     if (h->first_order) return CMCG_ERR_UNSUPPORTED;
-    launch_mask_copy(h->g, a, h->kap64, h->z0, h->st);
-    launch_mask_copy(h->g, b, h->kap64, h->z1, h->st);
+    // the adjoint's start kernels select the Dirichlet entries of a and b away
     if (h->opt.precision == CMCG_FP32)
-        adjoint_period<float>(h, h->z0, h->z1, 1, nullptr, nullptr, q0, q1, nullptr);
+        adjoint_period<float>(h, a, b, 1, nullptr, nullptr, q0, q1, nullptr);
     else
-        adjoint_period<double>(h, h->z0, h->z1, 1, nullptr, nullptr, q0, q1, nullptr);
+        adjoint_period<double>(h, a, b, 1, nullptr, nullptr, q0, q1, nullptr);
     if (cudaStreamSynchronize(h->st) != cudaSuccess) return CMCG_ERR_CUDA;
     return cuda_status();
 }
@@ -1572,8 +1628,7 @@ int cmcg_fo_period(cmcg_handle* h, const double* s0, const double* f, const doub
     if (!h || !s0 || !sT) return CMCG_ERR_INVALID_ARG;
     if (!h->first_order) return CMCG_ERR_UNSUPPORTED;
     const bool src = f || g;
-    if (src) launch_make_source(h->g, f, g, h->kap64, h->S, h->g.dim == 3 ? kZcEnds : 1, false, h->st);
-    if (src) source_updated(h);
+    if (src) set_source(h, f, g);
     if (fo_period(h, s0, src, sT) != CMCG_OK) return CMCG_ERR_CUDA;
     if (cudaStreamSynchronize(h->st) != cudaSuccess) return CMCG_ERR_CUDA;
     return cuda_status();
@@ -1590,12 +1645,7 @@ int cmcg_fo_adjoint_period(cmcg_handle* h, const double* y, double* out) {
 int cmcg_solve(cmcg_handle* h, const double* f, const double* g, double tol, double* u, cmcg_stats* stats) {
     if (!h || !u || !(tol > 0)) return CMCG_ERR_INVALID_ARG;
     const auto t0 = std::chrono::steady_clock::now();
-    if (f || g)
-        launch_make_source(h->g, f, g, h->kap64, h->S, h->g.dim == 3 ? kZcEnds : 1, false, h->st);
-    else
-        launch_fill(h->S, 2 * h->g.np, 0.0, h->st);
-    h->src_faces = !f;
-    source_updated(h);
+    set_source(h, f, g);
     cmcg_stats local{};
     cmcg_stats* st = stats ? stats : &local;
     const int rc = solve_prepared(h, tol, u, st, stats != nullptr);
@@ -1623,11 +1673,11 @@ int cmcg_solve_host(cmcg_handle* h, const double* f_host, const double* g_host, 
     launch_fill(h->S, 2 * n, 0.0, h->st);
     if (f_host) {
         cudaMemcpyAsync(h->stage, f_host, bytes, cudaMemcpyHostToDevice, h->st);
-        launch_make_source(h->g, h->stage, nullptr, h->kap64, h->S, zce, true, h->st);
+        launch_make_source(h->g, h->stage, nullptr, h->kap64, h->S, nullptr, nullptr, zce, true, h->st);
     }
     if (g_host) {
         cudaMemcpyAsync(h->stage, g_host, bytes, cudaMemcpyHostToDevice, h->st);
-        launch_make_source(h->g, nullptr, h->stage, h->kap64, h->S, zce, true, h->st);
+        launch_make_source(h->g, nullptr, h->stage, h->kap64, h->S, nullptr, nullptr, zce, true, h->st);
     }
     h->src_faces = !f_host;
     source_updated(h);

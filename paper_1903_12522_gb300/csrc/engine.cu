@@ -470,11 +470,7 @@ int cmcg_engine_submit(cmcg_engine* e, cmcg_handle* h, const double* f, const do
     sl.runup = h->opt.precision == CMCG_MIXED ? runup_count(h) : 0;
     h->riesz_iters = 0;
     h->periods = 0;
-    if (f || g)
-        launch_make_source(h->g, f, g, h->kap64, h->S, h->g.dim == 3 ? kZcEnds : 1, false, h->st);
-    else
-        launch_fill(h->S, 2 * h->g.np, 0.0, h->st);
-    source_updated(h);
+    set_source(h, f, g);
     if (h->opt.precision == CMCG_MIXED) {
         launch_fill(h->wo0, h->g.np, 0.0, h->st);
         launch_fill(h->wo1, h->g.np, 0.0, h->st);

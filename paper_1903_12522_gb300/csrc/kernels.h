@@ -42,17 +42,18 @@ void launch_step(const Geom& g, int order, const T* cur, T* prev, const T* kap, 
 // scol of S (3D): one byte per (x, y) column
 void launch_source_columns(const Geom& g, const double* S, unsigned char* scol, cudaStream_t st);
 template <typename T>
+// src_faces (with S): S is nonzero on absorbing faces only, and is read there only.
 // w1_float (T = float): w1 points to floats (the FP32 CG vectors of a mixed-precision inner solve)
 void launch_start(const Geom& g, int order, const T* w0t, const double* w1, T* y0, T* y1, const T* kap,
-                  const double* S, double dt, int zc, cudaStream_t st, bool w1_float = false);
+                  const double* S, bool src_faces, double dt, int zc, cudaStream_t st, bool w1_float = false);
 // mode 0: z = E (Pi(w) - w) and J; mode 1: (y(T), y_t(T)); mode 2 (T = float only): mode 0
 // with z0 and t = D^-1 z1 written as floats into out0 and out1 (the FP32 hand-off to the
 // adjoint period: launch_adj_start with a = z0 and t, then launch_adj_final mode 2); mode 3
 // (T = float only): mode 2 with w1 pointing to floats (FP32 CG vectors).
 template <typename T>
 void launch_end(const Geom& g, int order, int mode, const T* yN, const T* yNm1, const T* w0t, const double* w1,
-                const T* kap, const T* mass, const double* S, double cs, double sn, double* out0, double* out1,
-                Red red, double dt, int zc, cudaStream_t st);
+                const T* kap, const T* mass, const double* S, bool src_faces, double cs, double sn, double* out0,
+                double* out1, Red red, double dt, int zc, cudaStream_t st);
 template <typename T>
 void launch_adj_prep(const Geom& g, const double* b, const T* mass, const T* kap, T* t, int zc,
                      cudaStream_t st);
@@ -104,8 +105,10 @@ void launch_step_filter(const Geom& g, int order, const double* cur, double* pre
                         const double* S, double cs, double sn, double* acc, double fc, double fs, double cv, int zc,
                         cudaStream_t st);
 void launch_scale_complex(long long n, double* u, double s, cudaStream_t st);
-void launch_make_source(const Geom& g, const double* f, const double* gb, const double* kap64, double* S, int zc,
-                        bool accumulate, cudaStream_t st);
+// The source array S from f and g (either nullable), with its FP32 copy S32 and the source columns
+// scol (both nullable; scol must be zeroed before); accumulate: S += instead, without the copies.
+void launch_make_source(const Geom& g, const double* f, const double* gb, const double* kap64, double* S, float* S32,
+                        unsigned char* scol, int zc, bool accumulate, cudaStream_t st);
 long long plane_blocks(const Geom& g, int zc);
 
 // ---- step_soft.cu -----------------------------------------------------------------------
@@ -117,6 +120,25 @@ void launch_face_weights(const Geom& g, const double* kap, double* w, cudaStream
 void launch_step_soft(const Geom& g, int order, const double* cur, double* prev, const double* kap,
                       const double* wface, const double* S, double cs, double sn, int flags, bool src_faces,
                       bool reverse, cudaStream_t st);
+
+// The endpoint kernels with the same stencil sum: arguments and modes (0 and 1) as launch_start,
+// launch_end, launch_adj_prep, launch_adj_start and launch_adj_final; minv = 1 / M.
+void launch_start_soft(const Geom& g, int order, const double* w0, const double* w1, double* y0, double* y1,
+                       const double* kap, const double* wface, const double* S, bool src_faces, double dt, int zc,
+                       cudaStream_t st);
+void launch_end_soft(const Geom& g, int order, int mode, const double* yN, const double* yNm1, const double* w0,
+                     const double* w1, const double* kap, const double* mass, const double* wface, const double* S,
+                     bool src_faces, double cs, double sn, double* out0, double* out1, Red red, double dt, int zc,
+                     cudaStream_t st);
+void launch_adj_prep_soft(const Geom& g, const double* b, const double* minv, const double* wface, double* t, int zc,
+                          cudaStream_t st);
+void launch_adj_start_soft(const Geom& g, int order, const double* a, const double* t, const double* minv,
+                           const double* kap, const double* wface, double* cur, double* prev, double dt, int zc,
+                           cudaStream_t st);
+void launch_adj_final_soft(const Geom& g, int order, int mode, const double* s, const double* u1, const double* mass,
+                           const double* kap, const double* wface, const double* minv, const double* z0,
+                           const double* z1, const double* d0, const double* d1, double* o0, double* o1, double* gt1,
+                           Red red, double dt, int zc, cudaStream_t st);
 
 // ---- step_bulk.cu -----------------------------------------------------------------------
 // FP32 3D 7-point leapfrog step with TMA bulk-copy staging (homogeneous; flags 0, PREV_SCALED,
@@ -145,7 +167,9 @@ void launch_step_bulk(const Geom& g, const float* cur, float* prev, const float*
 void launch_setup_coeffs(const Geom& g, const double* c, const unsigned char* user_mask, unsigned face_dir,
                          double dt, double* kap64, float* kap32, double* mass, unsigned char* mask, Red red,
                          cudaStream_t st);
-void launch_mask_copy(const Geom& g, const double* in, const double* kap64, double* out, cudaStream_t st);
+// out = in, 0 on Dirichlet nodes (mask bytes; null: none); T = float converts.
+template <typename T>
+void launch_mask_copy(const Geom& g, const double* in, const unsigned char* mask, T* out, cudaStream_t st);
 void launch_fill(double* p, long long n, double v, cudaStream_t st);
 // (w0, w1) = (Re u, wh Im u) on active nodes, 0 on Dirichlet nodes (kap64 = 0); u interleaved.
 void launch_warm_start(long long n, const double* u, const double* kap64, double wh, double* w0, double* w1,

@@ -5,6 +5,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "soft64.cuh"
 
 namespace cmcg {
 
@@ -86,11 +87,17 @@ __global__ void __launch_bounds__(kT) k_setup(const double* __restrict__ c, cons
     }
 }
 
-__global__ void k_mask_copy(const double* __restrict__ in, const double* __restrict__ kap64, double* __restrict__ out,
+// Reads the mask byte rather than kappa: 1 byte per node instead of 8, and no FP64 comparison.
+template <typename T>
+__global__ void k_mask_copy(const double* __restrict__ in, const unsigned char* __restrict__ mask, T* __restrict__ out,
                             long long n) {
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += stride)
-        out[j] = kap64[j] == 0.0 ? 0.0 : in[j];
+    for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += stride) {
+        const double x = in[j];
+        const bool dir = mask && mask[j];
+        if constexpr (sizeof(T) == 4) out[j] = dir ? 0.0f : soft64::to_f32(x);
+        else out[j] = dir ? 0.0 : x;
+    }
 }
 
 __global__ void k_fill(double* p, long long n, double v) {
@@ -481,10 +488,13 @@ void launch_setup_coeffs(const Geom& g, const double* c, const unsigned char* us
     k_setup<<<vec_blocks(g.np), kT, 0, st>>>(c, user_mask, face_dir, dt, kap64, kap32, mass, mask, red, g);
 }
 
-void launch_mask_copy(const Geom& g, const double* in, const double* kap64, double* out, cudaStream_t st) {
+template <typename T>
+void launch_mask_copy(const Geom& g, const double* in, const unsigned char* mask, T* out, cudaStream_t st) {
     note_launch(1);
-    k_mask_copy<<<vec_blocks(g.np), kT, 0, st>>>(in, kap64, out, g.np);
+    k_mask_copy<T><<<vec_blocks(g.np), kT, 0, st>>>(in, mask, out, g.np);
 }
+template void launch_mask_copy<float>(const Geom&, const double*, const unsigned char*, float*, cudaStream_t);
+template void launch_mask_copy<double>(const Geom&, const double*, const unsigned char*, double*, cudaStream_t);
 
 void launch_fill(double* p, long long n, double v, cudaStream_t st) {
     note_launch(1);

@@ -13,6 +13,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "soft64.cuh"
 
 namespace cmcg {
 
@@ -595,7 +596,8 @@ __global__ void __launch_bounds__(kT) k_applyK(Geom g, const unsigned char* __re
 
 __global__ void k_to_float(long long n, const double* __restrict__ in, float* __restrict__ out) {
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += stride) out[j] = (float)in[j];
+    for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < n; j += stride)
+        out[j] = soft64::to_f32(in[j]);
 }
 
 __global__ void __launch_bounds__(kT) k_reduce_sum(long long n, const double* __restrict__ x, Red red, int slot) {

@@ -65,6 +65,37 @@ __device__ __forceinline__ double to_double(long long x, unsigned emax, bool* ok
     return __hiloint2double((int)(hi | ((unsigned)(s >> 32) & 0x80000000u)), (int)__funnelshift_r(nl, nh, 11));
 }
 
+// Conversions between FP32 and FP64 by bit operations: the hardware's run on the FP64 pipe too.
+// Normal values in both formats; zeros, subnormals, infinities, NaN and what rounds past the
+// largest float take the hardware conversion, out of line.  Same results, bit for bit.
+static __device__ __noinline__ float to_f32_hw(double x) { return (float)x; }
+static __device__ __noinline__ double to_f64_hw(float x) { return (double)x; }
+
+__device__ __forceinline__ float to_f32(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    const unsigned a = hi & 0x7fffffffu;
+    if (a - 0x38100000u < 0x0fd00000u) {  // 2^-126 <= |x| < 2^127
+        const unsigned u = ((a - 0x38000000u) << 3) | (lo >> 29);
+        const unsigned inc = (lo << 3) + (u & 1u) > 0x80000000u ? 1u : 0u;  // round to nearest even
+        return __uint_as_float((u + inc) | (hi & 0x80000000u));
+    }
+    if ((a | lo) == 0u) return __uint_as_float(hi);
+    return to_f32_hw(x);
+}
+
+__device__ __forceinline__ double to_f64(float x) {
+    const unsigned u = __float_as_uint(x), a = u & 0x7fffffffu;
+    if (a - 0x00800000u < 0x7f000000u)
+        return __hiloint2double((int)(((a >> 3) + 0x38000000u) | (u & 0x80000000u)), (int)(u << 29));
+    if (a == 0u) return __hiloint2double((int)u, 0);
+    return to_f64_hw(x);
+}
+
+// x == 0 without a comparison on the FP64 pipe.
+__device__ __forceinline__ bool is_zero(double x) {
+    return ((unsigned)__double2loint(x) | ((unsigned)__double2hiint(x) & 0x7fffffffu)) == 0u;
+}
+
 __device__ __forceinline__ unsigned max3(unsigned a, unsigned b, unsigned c) { return max(max(a, b), c); }
 
 }  // namespace soft64

@@ -101,7 +101,9 @@ struct PeriodBuffers {
 };
 
 int cuda_status();
-// After every change of S: refresh its FP32 copy (FP32 and mixed-precision handles).
+// S from f and g (either may be null) with its FP32 copy and source columns.
+void set_source(cmcg_handle* H, const double* f, const double* g);
+// After S was accumulated in pieces: its FP32 copy (FP32 and mixed precision) and source columns.
 void source_updated(cmcg_handle* H);
 // The lumped mass M in precision T (what the period kernels of that precision read).
 template <typename T>

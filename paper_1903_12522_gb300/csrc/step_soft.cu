@@ -1,7 +1,9 @@
-// FP64 leapfrog steps with the stencil sum in integer arithmetic (soft64.cuh).
+// FP64 leapfrog steps and period endpoints with the stencil sum in integer arithmetic
+// (soft64.cuh), for handles in FP64.
 #include <math.h>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 #include "kernels.h"
@@ -15,18 +17,31 @@ using soft64::Term;
 
 constexpr int kST = 256;
 
-// The negated unscaled Laplacian at a node in plain FP64, for the values the fixed-point sum
-// does not take.  Out of line: inlined, its additions would be predicated into every update.
-template <int ORDER>
-__device__ __noinline__ double neg_lap_plain(const double* __restrict__ cur, const Geom& g, int j, int ix, int iy,
-                                             int iz) {
-    auto f = [cur](long long i) { return cur[i]; };
-    return -lap_t<ORDER, double>(g, f, (long long)j, ix, iy, iz);
+struct Values {
+    const double* __restrict__ p;
+    __device__ __forceinline__ double operator()(int i) const { return p[i]; }
+};
+
+struct Difference {  // a - b, formed in FP64 before the stencil sums it
+    const double* __restrict__ a;
+    const double* __restrict__ b;
+    __device__ __forceinline__ double operator()(int i) const { return a[i] - b[i]; }
+};
+
+// The rare cases stay out of line: inlined, their FP64 instructions would be predicated into
+// every update, and a predicated-off FP64 instruction costs as much as an executed one.
+
+// The negated unscaled Laplacian of f at a node in plain FP64, for the values the fixed-point
+// sum does not take.
+template <int ORDER, typename F>
+__device__ __noinline__ double neg_lap_plain(F f, const Geom& g, int j, int ix, int iy, int iz) {
+    auto at = [f](long long i) { return f((int)i); };
+    return -lap_t<ORDER, double>(g, at, (long long)j, ix, iy, iz);
 }
 
 // The update on an absorbing face, w = 1 / (1 + beta): out = w rhs - (1 - beta) w yp with
 // (1 - beta) w = 2 w - 1, and the adjoint's first and last variants (the previous term already
-// scaled; no division).  Out of line for the same reason.
+// scaled; no division).
 template <int FLAGS>
 __device__ __noinline__ double face_update(double rhs, double yp, double w) {
     if (FLAGS & kStepNoDiv) {
@@ -37,63 +52,90 @@ __device__ __noinline__ double face_update(double rhs, double yp, double w) {
     return fma(rhs, w, -(fma(2.0, w, -1.0) * yp));
 }
 
+// (1 - beta) x and x / (1 + beta) on an absorbing face.
+__device__ __noinline__ double face_minus(double x, double w) { return (2.0 - 1.0 / w) * x; }
+__device__ __noinline__ double face_over(double x, double w) { return x * w; }
+
 __device__ __noinline__ double add_source(double d, const double* __restrict__ S, int j, double cs, double sn) {
     const double2 s = reinterpret_cast<const double2*>(S)[j];
     return d + fma(s.x, cs, s.y * sn);
 }
 
-// One leapfrog step, one thread per (x, y) column of zc planes (2D: one node).
-//
-// Bound: issue slots of the integer pipes and latency (FP64 work left per update: 2 y - y_prev
-// and the fused multiply-add with kappa, against nine operations and, on the faces, a square
-// root and a division).  The z-neighbours' terms stay in registers.
-template <int DIM, int ORDER, int FLAGS, bool SRC_FACES>
-__global__ void __launch_bounds__(kST, ORDER == 2 ? 4 : 3)
-    k_step_soft(const double* __restrict__ cur, double* __restrict__ prev_out, const double* __restrict__ kap,
-                const double* __restrict__ wface, const double* __restrict__ S, double cs, double sn, Geom g, int zc,
-                int reverse) {
-    const int plane = g.sx * g.sy;
-    const int bx = reverse ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
-    const int by = reverse ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
-    const int p = bx * kST + (int)threadIdx.x;
-    if (p >= plane) return;
-    const int iy = (int)((unsigned)p / (unsigned)g.sx), ix = p - iy * g.sx;
-    const int z0 = DIM == 3 ? by * zc : 0, z1 = DIM == 3 ? min(z0 + zc, g.sz) : 1;
-    if (!column_in_range(g, ix, iy, z0, z1, ORDER / 2, kSiteColumn)) return;
-    const int sZ = plane;
-    const int oxm = (int)off_m1(ix, 1), oxp = (int)off_p1(ix, g.nx, 1);
-    const int oym = (int)off_m1(iy, g.sx), oyp = (int)off_p1(iy, g.ny, g.sx);
-    bool fxy = (ix == 0 && (g.abc & 1u)) || (ix == g.nx && (g.abc & 2u)) || (iy == 0 && (g.abc & 4u)) ||
-               (iy == g.ny && (g.abc & 8u));
-    int ox2m = 0, ox2p = 0, oy2m = 0, oy2p = 0;
-    if (ORDER == 4) {
-        ox2m = (int)off_m2(ix, 1), ox2p = (int)off_p2(ix, g.nx, 1);
-        oy2m = (int)off_m2(iy, g.sx), oy2p = (int)off_p2(iy, g.ny, g.sx);
+// One thread's column of a launch: its (x, y), its planes, its faces.
+template <int DIM>
+struct Column {
+    int ix, iy, z0, z1, j;  // j: node of plane z0
+    bool valid, fxy;        // fxy: on an absorbing x or y face
+    unsigned abc;
+    int nz;
+    __device__ __forceinline__ Column(const Geom& g, int zc, int radius, bool reverse) {
+        const int plane = g.sx * g.sy;
+        const int bx = reverse ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
+        const int by = reverse ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
+        const int p = bx * kST + (int)threadIdx.x;
+        valid = p < plane;
+        const int pp = valid ? p : 0;
+        iy = (int)((unsigned)pp / (unsigned)g.sx);
+        ix = pp - iy * g.sx;
+        z0 = DIM == 3 ? by * zc : 0;
+        z1 = DIM == 3 ? min(z0 + zc, g.sz) : 1;
+        j = pp + plane * z0;
+        abc = g.abc;
+        nz = g.nz;
+        fxy = (ix == 0 && (abc & 1u)) || (ix == g.nx && (abc & 2u)) || (iy == 0 && (abc & 4u)) ||
+              (iy == g.ny && (abc & 8u));
+        if (valid && !column_in_range(g, ix, iy, z0, z1, radius, kSiteColumn)) valid = false;
     }
-    int j = p + sZ * z0;
-    double yc = cur[j];
-    Term c = soft64::term(yc), zm{}, zp{}, zm2{}, zp2{};
-    double yz = 0.0;  // ORDER 4: the raw value of plane iz + 1
-    if (DIM == 3) {
-        zm = soft64::term(cur[j + (z0 > 0 ? -sZ : sZ)]);
+    // is the node of plane iz on an absorbing face?
+    __device__ __forceinline__ bool face(int iz) const {
+        return fxy || (DIM == 3 && ((iz == 0 && (abc & 16u)) || (iz == nz && (abc & 32u))));
+    }
+};
+
+// -Lt(f) along a column, the z-neighbours' terms carried in registers.  For the 4th order the
+// integer sum is 3/4 of it, a1 - a2 / 16 - (15/8) DIM y, whose weights are shifts.
+template <int DIM, int ORDER, typename F>
+struct SoftLap {
+    F f;
+    const Geom& g;
+    int ix, iy, sZ, oxm, oxp, oym, oyp, ox2m, ox2p, oy2m, oy2p;
+    double yc, yz;  // f at the current plane, and (4th order) at the next one
+    Term c, zm, zp, zm2;
+    __device__ __forceinline__ SoftLap(F f_, const Geom& g_, int ix_, int iy_)
+        : f(f_), g(g_), ix(ix_), iy(iy_), sZ(g_.sx * g_.sy), yc(0.0), yz(0.0), c{}, zm{}, zp{}, zm2{} {
+        oxm = (int)off_m1(ix, 1), oxp = (int)off_p1(ix, g.nx, 1);
+        oym = (int)off_m1(iy, g.sx), oyp = (int)off_p1(iy, g.ny, g.sx);
+        ox2m = ox2p = oy2m = oy2p = 0;
         if (ORDER == 4) {
-            zm2 = soft64::term(cur[j + (int)off_m2(z0, sZ)]);
-            yz = cur[j + (z0 < g.nz ? sZ : -sZ)];
-            zp = soft64::term(yz);
+            ox2m = (int)off_m2(ix, 1), ox2p = (int)off_p2(ix, g.nx, 1);
+            oy2m = (int)off_m2(iy, g.sx), oy2p = (int)off_p2(iy, g.ny, g.sx);
         }
     }
-    for (int iz = z0; iz < z1; ++iz) {
-        double znew = 0.0;
-        if (DIM == 3) znew = cur[j + (ORDER == 2 ? (iz < g.nz ? sZ : -sZ) : (int)off_p2(iz, g.nz, sZ))];
-        const double x0 = cur[j + oxm], x1 = cur[j + oxp], y0 = cur[j + oym], y1 = cur[j + oyp];
+    __device__ __forceinline__ void start(int j, int iz) {
+        yc = f(j);
+        c = soft64::term(yc);
+        if (DIM == 3) {
+            zm = soft64::term(f(j + (iz > 0 ? -sZ : sZ)));
+            if (ORDER == 4) {
+                zm2 = soft64::term(f(j + (int)off_m2(iz, sZ)));
+                yz = f(j + (iz < g.nz ? sZ : -sZ));
+                zp = soft64::term(yz);
+            }
+        }
+    }
+    // -Lt(f) at plane iz (node j), then on to plane iz + 1; y receives f there.
+    __device__ __forceinline__ double next(int j, int iz, double* y) {
+        double zn = 0.0;
+        if (DIM == 3) zn = f(j + (ORDER == 2 ? (iz < g.nz ? sZ : -sZ) : (int)off_p2(iz, g.nz, sZ)));
+        const double x0 = f(j + oxm), x1 = f(j + oxp), y0 = f(j + oym), y1 = f(j + oyp);
         double u0 = 0.0, u1 = 0.0, v0 = 0.0, v1 = 0.0;
-        if (ORDER == 4) u0 = cur[j + ox2m], u1 = cur[j + ox2p], v0 = cur[j + oy2m], v1 = cur[j + oy2p];
-        const double k = kap[j], yp = prev_out[j];
+        if (ORDER == 4) u0 = f(j + ox2m), u1 = f(j + ox2p), v0 = f(j + oy2m), v1 = f(j + oy2p);
         const Term a0 = soft64::term(x0), a1 = soft64::term(x1), b0 = soft64::term(y0), b1 = soft64::term(y1);
         unsigned e = soft64::max3(soft64::max3(c.e, a0.e, a1.e), b0.e, b1.e);
+        Term zp2{};
         if (DIM == 3) {
-            if (ORDER == 2) zp = soft64::term(znew);
-            else zp2 = soft64::term(znew);
+            if (ORDER == 2) zp = soft64::term(zn);
+            else zp2 = soft64::term(zn);
             e = soft64::max3(e, zm.e, zp.e);
         }
         Term c0{}, c1{}, d0{}, d1{};
@@ -102,58 +144,240 @@ __global__ void __launch_bounds__(kST, ORDER == 2 ? 4 : 3)
             e = soft64::max3(soft64::max3(e, c0.e, c1.e), d0.e, d1.e);
             if (DIM == 3) e = soft64::max3(e, zm2.e, zp2.e);
         }
-        // L = -Lt(y)
-        bool ok = soft64::in_range(e);
         const long long C = soft64::align(c, e);
         long long s1 = (soft64::align(a0, e) + soft64::align(a1, e)) + (soft64::align(b0, e) + soft64::align(b1, e));
         if (DIM == 3) s1 += soft64::align(zm, e) + soft64::align(zp, e);
         double L;
-        bool big;
+        bool ok;
         if (ORDER == 2) {
-            L = soft64::to_double(s1 - (DIM == 3 ? 4 * C + 2 * C : 4 * C), e, &big);
+            L = soft64::to_double(s1 - (DIM == 3 ? 4 * C + 2 * C : 4 * C), e, &ok);
         } else {
-            // 3/4 of the 4th-order sum: a1 - a2 / 16 - (DIM 15/8) y, so that its weights are shifts
             long long s2 = (soft64::align(c0, e) + soft64::align(c1, e)) + (soft64::align(d0, e) + soft64::align(d1, e));
             if (DIM == 3) s2 += soft64::align(zm2, e) + soft64::align(zp2, e);
             const long long q = DIM == 3 ? 6 * C - (3 * C >> 3) : 4 * C - (C >> 2);
-            L = soft64::to_double(s1 - (s2 >> 4) - q, e, &big);
+            L = (4.0 / 3.0) * soft64::to_double(s1 - (s2 >> 4) - q, e, &ok);
         }
-        ok = ok && big;
-        double kk = k;
-        if (ORDER == 4) kk = k * (4.0 / 3.0);
-        if (!ok) {
-            L = neg_lap_plain<ORDER>(cur, g, j, ix, iy, iz);
-            kk = k;
-        }
-        const bool fz = DIM == 3 && ((iz == 0 && (g.abc & 16u)) || (iz == g.nz && (g.abc & 32u)));
-        double out;
-        if (fxy || fz) {
-            double rhs = fma(kk, L, 2.0 * yc);
-            if (FLAGS & kStepSrc) rhs = add_source(rhs, S, j, cs, sn);
-            out = face_update<FLAGS>(rhs, yp, wface[j]);
-        } else {
-            out = fma(kk, L, fma(2.0, yc, -yp));
-            if ((FLAGS & kStepSrc) && !SRC_FACES) out = add_source(out, S, j, cs, sn);
-        }
-        prev_out[j] = out;
+        if (!(ok && soft64::in_range(e))) L = neg_lap_plain<ORDER, F>(f, g, j, ix, iy, iz);
+        *y = yc;
         if (DIM == 3) {
             if (ORDER == 2) {
                 zm = c;
                 c = zp;
-                yc = znew;
+                yc = zn;
             } else {
                 zm2 = zm;
                 zm = c;
                 c = zp;
                 zp = zp2;
                 yc = yz;
-                yz = znew;
+                yz = zn;
             }
         }
-        j += sZ;
+        return L;
+    }
+};
+
+// One leapfrog step, one thread per (x, y) column of zc planes (2D: one node).
+//
+// Bound: issue slots of the integer pipes and latency (FP64 work left per update: 2 y - y_prev
+// and the fused multiply-add with kappa, against nine operations and, on the faces, a square
+// root and a division).
+template <int DIM, int ORDER, int FLAGS, bool SRC_FACES>
+__global__ void __launch_bounds__(kST, ORDER == 2 ? 4 : 3)
+    k_step_soft(const double* __restrict__ cur, double* __restrict__ prev_out, const double* __restrict__ kap,
+                const double* __restrict__ wface, const double* __restrict__ S, double cs, double sn, Geom g, int zc,
+                int reverse) {
+    const Column<DIM> m(g, zc, ORDER / 2, reverse != 0);
+    if (!m.valid) return;
+    SoftLap<DIM, ORDER, Values> lap(Values{cur}, g, m.ix, m.iy);
+    int j = m.j;
+    lap.start(j, m.z0);
+    for (int iz = m.z0; iz < m.z1; ++iz) {
+        const double k = kap[j], yp = prev_out[j];
+        double yc;
+        const double L = lap.next(j, iz, &yc);
+        double out;
+        if (m.face(iz)) {
+            double rhs = fma(k, L, 2.0 * yc);
+            if (FLAGS & kStepSrc) rhs = add_source(rhs, S, j, cs, sn);
+            out = face_update<FLAGS>(rhs, yp, wface[j]);
+        } else {
+            out = fma(k, L, fma(2.0, yc, -yp));
+            if ((FLAGS & kStepSrc) && !SRC_FACES) out = add_source(out, S, j, cs, sn);
+        }
+        prev_out[j] = out;
+        j += lap.sZ;
     }
 }
 
+// The period's endpoint kernels in FP64 (the formulas are those of k_start, k_end, k_adj_* in
+// wave.cu) with the same stencil sum, the face factors and 1 / dt, 1 / M precomputed: the plain
+// kernels spend 30 to 50 FP64 operations per node, most of them in divisions.
+template <int DIM, int ORDER, bool SRC>
+__global__ void __launch_bounds__(kST, 3)
+    k_start_soft(const double* __restrict__ w0, const double* __restrict__ w1, double* __restrict__ y0,
+                 double* __restrict__ y1, const double* __restrict__ kap, const double* __restrict__ wface,
+                 const double* __restrict__ S, Geom g, double dt, int zc, int src_faces) {
+    const Column<DIM> m(g, zc, ORDER / 2, false);
+    if (!m.valid) return;
+    SoftLap<DIM, ORDER, Values> lap(Values{w0}, g, m.ix, m.iy);
+    int j = m.j;
+    lap.start(j, m.z0);
+    for (int iz = m.z0; iz < m.z1; ++iz) {
+        const double k = kap[j];
+        double vj = w1[j], yc;
+        const double L = lap.next(j, iz, &yc);
+        const bool face = m.face(iz);
+        if (face) vj = face_minus(vj, wface[j]);
+        double v = fma(0.5 * k, L, fma(dt, vj, yc));
+        if (SRC && (face || !src_faces)) v = add_source(v, S, j, 0.5, 0.0);
+        const bool dir = soft64::is_zero(k);  // Dirichlet
+        y0[j] = dir ? 0.0 : yc;
+        y1[j] = dir ? 0.0 : v;
+        j += lap.sZ;
+    }
+}
+
+// MODE 0: z = E (Pi(w) - w) and J; MODE 1: (y(T), y_t(T)).  hs, hc: half the source factors.
+template <int DIM, int ORDER, bool SRC, int MODE>
+__global__ void __launch_bounds__(kST, MODE == 0 ? 2 : 3)
+    k_end_soft(const double* __restrict__ yN, const double* __restrict__ yNm1, const double* __restrict__ w0,
+               const double* __restrict__ w1, const double* __restrict__ kap, const double* __restrict__ mass,
+               const double* __restrict__ wface, const double* __restrict__ S, double hc, double hs,
+               double* __restrict__ out0, double* __restrict__ out1, Red red, Geom g, double inv_dt, double ck, int zc,
+               int src_faces) {
+    const Column<DIM> m(g, zc, ORDER / 2, false);
+    double acc[1] = {0.0};
+    if (m.valid) {
+        SoftLap<DIM, ORDER, Values> lap(Values{yN}, g, m.ix, m.iy);
+        SoftLap<DIM, ORDER, Difference> lape(Difference{yN, w0}, g, m.ix, m.iy);
+        int j = m.j;
+        lap.start(j, m.z0);
+        if (MODE == 0) lape.start(j, m.z0);
+        for (int iz = m.z0; iz < m.z1; ++iz) {
+            const double k = kap[j], ym = yNm1[j];
+            double yn;
+            const double L = lap.next(j, iz, &yn);
+            const bool face = m.face(iz), dir = soft64::is_zero(k);
+            double t = fma(0.5 * k, L, yn - ym);
+            if (SRC && (face || !src_faces)) t = add_source(t, S, j, hc, hs);
+            double vN = t * inv_dt;
+            if (face) vN = face_over(vN, wface[j]);
+            if (MODE == 1) {
+                out0[j] = dir ? 0.0 : yn;
+                out1[j] = dir ? 0.0 : vN;
+            } else {
+                double e0;
+                const double Le = lape.next(j, iz, &e0);
+                const double e1 = vN - w1[j];
+                int ends = (m.ix == 0 || m.ix == g.nx) + (m.iy == 0 || m.iy == g.ny);
+                if (DIM == 3) ends += (iz == 0 || iz == g.nz);
+                const double z0 = -(ck * Le) * __hiloint2double((1023 - ends) << 20, 0);
+                const double z1 = mass[j] * e1;
+                out0[j] = dir ? 0.0 : z0;
+                out1[j] = dir ? 0.0 : z1;
+                if (!dir) acc[0] += fma(e0, z0, e1 * z1);
+            }
+            j += lap.sZ;
+        }
+    }
+    if (MODE == 0) {
+        acc[0] *= 0.5;
+        if (grid_sum<1>(acc, red.partials, red.ticket) && threadIdx.x == 0) red.sc[SC_J] = acc[0];
+    }
+}
+
+// t = D^-1 b = b / (M (1 + beta)).
+template <int DIM>
+__global__ void __launch_bounds__(kST) k_adj_prep_soft(const double* __restrict__ b, const double* __restrict__ minv,
+                                                       const double* __restrict__ wface, double* __restrict__ t, Geom g,
+                                                       int zc) {
+    const Column<DIM> m(g, zc, 1, false);
+    if (!m.valid) return;
+    int j = m.j;
+    for (int iz = m.z0; iz < m.z1; ++iz, j += g.sx * g.sy) {
+        const double mi = minv[j];
+        double v = b[j] * mi;
+        if (m.face(iz)) v = face_over(v, wface[j]);
+        t[j] = soft64::is_zero(mi) ? 0.0 : v;  // Dirichlet: 1/M is stored as 0
+    }
+}
+
+template <int DIM, int ORDER>
+__global__ void __launch_bounds__(kST, 3)
+    k_adj_start_soft(const double* __restrict__ a, const double* __restrict__ t, const double* __restrict__ minv,
+                     const double* __restrict__ kap, const double* __restrict__ wface, double* __restrict__ cur,
+                     double* __restrict__ prev, Geom g, double inv_dt, int zc) {
+    const Column<DIM> m(g, zc, ORDER / 2, false);
+    if (!m.valid) return;
+    SoftLap<DIM, ORDER, Values> lap(Values{t}, g, m.ix, m.iy);
+    int j = m.j;
+    lap.start(j, m.z0);
+    for (int iz = m.z0; iz < m.z1; ++iz) {
+        const double k = kap[j], aj = a[j], mi = minv[j];
+        double tj;
+        const double L = lap.next(j, iz, &tj);
+        double u = fma(aj, mi, inv_dt * fma(0.5 * k, L, tj));
+        if (m.face(iz)) u = face_over(u, wface[j]);
+        const bool dir = soft64::is_zero(k);
+        cur[j] = dir ? 0.0 : u;
+        prev[j] = dir ? 0.0 : tj * inv_dt;
+        j += lap.sZ;
+    }
+}
+
+// MODE 0: ghat = q - z, g~1 = ghat1 / M (gt1 nullable), (ghat . d, sum ghat0); MODE 1: q.
+// cq = dt^2 / 2 h^d / h^2.
+template <int DIM, int ORDER, int MODE>
+__global__ void __launch_bounds__(kST, 3)
+    k_adj_final_soft(const double* __restrict__ s, const double* __restrict__ u1, const double* __restrict__ mass,
+                     const double* __restrict__ kap, const double* __restrict__ wface, const double* __restrict__ minv,
+                     const double* __restrict__ z0, const double* __restrict__ z1, const double* __restrict__ d0,
+                     const double* __restrict__ d1, double* __restrict__ o0, double* __restrict__ o1,
+                     double* __restrict__ gt1, Red red, Geom g, double dt, double cq, int zc) {
+    const Column<DIM> m(g, zc, ORDER / 2, false);
+    double acc[2] = {0.0, 0.0};
+    if (m.valid) {
+        SoftLap<DIM, ORDER, Values> lap(Values{s}, g, m.ix, m.iy);
+        int j = m.j;
+        lap.start(j, m.z0);
+        for (int iz = m.z0; iz < m.z1; ++iz) {
+            const double k = kap[j], M = mass[j];
+            double u = u1[j], sj;
+            const double L = lap.next(j, iz, &sj);
+            double sb = sj;
+            if (m.face(iz)) {
+                const double w = wface[j];
+                u = face_minus(u, w);
+                sb = face_minus(sj, w);
+            }
+            int ends = (m.ix == 0 || m.ix == g.nx) + (m.iy == 0 || m.iy == g.ny);
+            if (DIM == 3) ends += (iz == 0 || iz == g.nz);
+            const double c = cq * __hiloint2double((1023 - ends) << 20, 0);
+            const double q0 = fma(c, L, M * (sj - u));
+            const double q1 = (dt * M) * sb;
+            const bool dir = soft64::is_zero(k);
+            if (MODE == 1) {
+                o0[j] = dir ? 0.0 : q0;
+                o1[j] = dir ? 0.0 : q1;
+            } else {
+                const double g0 = q0 - z0[j], g1 = q1 - z1[j];
+                o0[j] = dir ? 0.0 : g0;
+                o1[j] = dir ? 0.0 : g1;
+                if (gt1) gt1[j] = dir ? 0.0 : g1 * minv[j];
+                if (!dir) {
+                    acc[0] += fma(g0, d0[j], g1 * d1[j]);
+                    acc[1] += g0;
+                }
+            }
+            j += lap.sZ;
+        }
+    }
+    if (MODE == 0 && grid_sum<2>(acc, red.partials, red.ticket) && threadIdx.x == 0) {
+        red.sc[SC_GD] = acc[0];
+        red.sc[SC_GSUM] = acc[1];
+    }
+}
 
 // w = 1 / (1 + beta) on the nodes of absorbing faces (other entries are not read).
 __global__ void __launch_bounds__(kST) k_face_weights(Geom g, const double* __restrict__ kap, double* __restrict__ w) {
@@ -229,6 +453,85 @@ void launch_step_soft(const Geom& g, int order, const double* cur, double* prev,
         if (order == 2) soft_flags<2, 2>(g, cur, prev, kap, wface, S, cs, sn, flags, src_faces, reverse, st);
         else soft_flags<2, 4>(g, cur, prev, kap, wface, S, cs, sn, flags, src_faces, reverse, st);
     }
+}
+
+// The endpoint kernels: `run` is called with the dimension and order as compile-time constants.
+template <typename F>
+static void by_stencil(const Geom& g, int order, F run) {
+    using std::integral_constant;
+    note_launch(1);
+    if (g.dim == 3) {
+        if (order == 2) run(integral_constant<int, 3>(), integral_constant<int, 2>());
+        else run(integral_constant<int, 3>(), integral_constant<int, 4>());
+    } else {
+        if (order == 2) run(integral_constant<int, 2>(), integral_constant<int, 2>());
+        else run(integral_constant<int, 2>(), integral_constant<int, 4>());
+    }
+}
+
+static dim3 column_grid(const Geom& g, int zc) {
+    return dim3((unsigned)(((long long)g.sx * g.sy + kST - 1) / kST), (unsigned)((g.sz + zc - 1) / zc));
+}
+
+static double h_pow(const Geom& g) { return (g.dim == 3 ? g.h * g.h * g.h : g.h * g.h) / (g.h * g.h); }
+
+void launch_start_soft(const Geom& g, int order, const double* w0, const double* w1, double* y0, double* y1,
+                       const double* kap, const double* wface, const double* S, bool src_faces, double dt, int zc,
+                       cudaStream_t st) {
+    by_stencil(g, order, [&](auto D, auto O) {
+        const dim3 grid = column_grid(g, zc);
+        if (S)
+            k_start_soft<D(), O(), true><<<grid, kST, 0, st>>>(w0, w1, y0, y1, kap, wface, S, g, dt, zc, src_faces);
+        else
+            k_start_soft<D(), O(), false><<<grid, kST, 0, st>>>(w0, w1, y0, y1, kap, wface, S, g, dt, zc, 0);
+    });
+}
+
+void launch_end_soft(const Geom& g, int order, int mode, const double* yN, const double* yNm1, const double* w0,
+                     const double* w1, const double* kap, const double* mass, const double* wface, const double* S,
+                     bool src_faces, double cs, double sn, double* out0, double* out1, Red red, double dt, int zc,
+                     cudaStream_t st) {
+    by_stencil(g, order, [&](auto D, auto O) {
+        const dim3 grid = column_grid(g, zc);
+        const double ck = h_pow(g), id = 1.0 / dt, hc = 0.5 * cs, hs = 0.5 * sn;
+        const int sf = src_faces ? 1 : 0;
+        auto go = [&](auto kernel) {
+            kernel<<<grid, kST, 0, st>>>(yN, yNm1, w0, w1, kap, mass, wface, S, hc, hs, out0, out1, red, g, id, ck, zc,
+                                         sf);
+        };
+        if (mode == 0) S ? go(k_end_soft<D(), O(), true, 0>) : go(k_end_soft<D(), O(), false, 0>);
+        else S ? go(k_end_soft<D(), O(), true, 1>) : go(k_end_soft<D(), O(), false, 1>);
+    });
+}
+
+void launch_adj_prep_soft(const Geom& g, const double* b, const double* minv, const double* wface, double* t, int zc,
+                          cudaStream_t st) {
+    note_launch(1);
+    if (g.dim == 3) k_adj_prep_soft<3><<<column_grid(g, zc), kST, 0, st>>>(b, minv, wface, t, g, zc);
+    else k_adj_prep_soft<2><<<column_grid(g, zc), kST, 0, st>>>(b, minv, wface, t, g, zc);
+}
+
+void launch_adj_start_soft(const Geom& g, int order, const double* a, const double* t, const double* minv,
+                           const double* kap, const double* wface, double* cur, double* prev, double dt, int zc,
+                           cudaStream_t st) {
+    by_stencil(g, order, [&](auto D, auto O) {
+        k_adj_start_soft<D(), O()>
+            <<<column_grid(g, zc), kST, 0, st>>>(a, t, minv, kap, wface, cur, prev, g, 1.0 / dt, zc);
+    });
+}
+
+void launch_adj_final_soft(const Geom& g, int order, int mode, const double* s, const double* u1, const double* mass,
+                           const double* kap, const double* wface, const double* minv, const double* z0,
+                           const double* z1, const double* d0, const double* d1, double* o0, double* o1, double* gt1,
+                           Red red, double dt, int zc, cudaStream_t st) {
+    by_stencil(g, order, [&](auto D, auto O) {
+        const double cq = 0.5 * dt * dt * h_pow(g);
+        auto go = [&](auto kernel) {
+            kernel<<<column_grid(g, zc), kST, 0, st>>>(s, u1, mass, kap, wface, minv, z0, z1, d0, d1, o0, o1, gt1, red, g,
+                                                       dt, cq, zc);
+        };
+        mode == 0 ? go(k_adj_final_soft<D(), O(), 0>) : go(k_adj_final_soft<D(), O(), 1>);
+    });
 }
 
 CMCG_CHECK_TU(soft)

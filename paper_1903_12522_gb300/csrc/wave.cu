@@ -22,6 +22,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "soft64.cuh"
 
 namespace cmcg {
 
@@ -56,11 +57,17 @@ struct Ld {
     __device__ __forceinline__ T operator()(long long i) const { return p[i]; }
 };
 
+// FP64 <-> stepping precision without the FP64 pipe (soft64.cuh; same bits as the casts).
+template <typename T, typename V>
+__device__ __forceinline__ T as_step(V v) {
+    if constexpr (std::is_same<T, float>::value && std::is_same<V, double>::value) return soft64::to_f32(v);
+    else return (T)v;
+}
 template <typename T>
-struct LdD {  // loads T, returns double
-    const T* __restrict__ p;
-    __device__ __forceinline__ double operator()(long long i) const { return (double)p[i]; }
-};
+__device__ __forceinline__ double as_f64(T v) {
+    if constexpr (std::is_same<T, float>::value) return soft64::to_f64(v);
+    else return v;
+}
 
 template <typename T>
 struct DiffT {  // a[i] - b[i] in T
@@ -637,12 +644,13 @@ __device__ __forceinline__ R weight_t(const Geom& g, int ix, int iy, int iz) {
     return w;
 }
 
-// Period start: y0 = w0, y1 = w0 + dt (1 - beta) w1 + (S_re - kappa Lt w0) / 2.
+// Period start: y0 = w0, y1 = w0 + dt (1 - beta) w1 + (S_re - kappa Lt w0) / 2.  src_faces: S is
+// read on absorbing faces only (elsewhere it is zero).
 template <typename T, int ORDER, bool SRC, typename V = double>
 __global__ void __launch_bounds__(kThreads) k_start(const T* __restrict__ w0t, const V* __restrict__ w1,
                                                     T* __restrict__ y0, T* __restrict__ y1,
                                                     const T* __restrict__ kap, const double* __restrict__ S,
-                                                    Geom g, double dt, int zc) {
+                                                    Geom g, double dt, int zc, int src_faces) {
     const PlaneMap m = plane_map(g, zc, ORDER / 2);
     if (!m.valid || m.z0 >= m.z1) return;
     Ld<T> f{w0t};
@@ -659,8 +667,8 @@ __global__ void __launch_bounds__(kThreads) k_start(const T* __restrict__ w0t, c
         const int nbf = num_abc(g, m.ix, m.iy, iz);
         const T beta = nbf ? (T)nbf * sqrt(k) : T(0);
         const T w0j = w0t[j];
-        T v = w0j + dtT * (T(1) - beta) * (T)w1[j] - T(0.5) * k * L;
-        if (SRC) v += (T)(0.5 * S[2 * j]);
+        T v = w0j + dtT * (T(1) - beta) * as_step<T>(w1[j]) - T(0.5) * k * L;
+        if (SRC && (nbf || !src_faces)) v += as_step<T>(0.5 * S[2 * j]);
         const bool dir = k == T(0);
         y0[j] = dir ? T(0) : w0j;
         y1[j] = dir ? T(0) : v;
@@ -684,7 +692,7 @@ __global__ void __launch_bounds__(kThreads, kEndMinBlocks<T>) k_end(const T* __r
                                                   const T* __restrict__ kap, const T* __restrict__ mass,
                                                   const double* __restrict__ S, double cs, double sn,
                                                   double* __restrict__ out0, double* __restrict__ out1,
-                                                  Red red, Geom g, double dt, int zc) {
+                                                  Red red, Geom g, double dt, int zc, int src_faces) {
     const PlaneMap m = plane_map(g, zc, ORDER / 2);
     double acc[1] = {0.0};
     KahanF accf;  // FP32 periods: the thread's part of J without FP64 arithmetic
@@ -701,15 +709,15 @@ __global__ void __launch_bounds__(kThreads, kEndMinBlocks<T>) k_end(const T* __r
             const int nbf = num_abc(g, m.ix, m.iy, iz);
         const T beta = nbf ? (T)nbf * sqrt(k) : T(0);
             T src = T(0);
-            if (SRC) src = (T)(S[2 * j] * cs + S[2 * j + 1] * sn);
+            if (SRC && (nbf || !src_faces)) src = as_step<T>(S[2 * j] * cs + S[2 * j + 1] * sn);
             const T yn = yN[j];
             const T vN = ((yn - yNm1[j]) / dtT + (src - k * L) / (T(2) * dtT)) / (T(1) + beta);
             if (MODE == 1) {
-                out0[j] = dir ? 0.0 : (double)yn;
-                out1[j] = dir ? 0.0 : (double)vN;
+                out0[j] = as_f64(dir ? T(0) : yn);
+                out1[j] = as_f64(dir ? T(0) : vN);
             } else {
                 const T e0 = yn - w0t[j];
-                const T e1 = vN - (T)w1[j];
+                const T e1 = vN - as_step<T>(w1[j]);
                 const T W = weight_t<T>(g, m.ix, m.iy, iz);
                 const T z0 = W * ih2 * lap_t<ORDER, T>(g, fe, j, m.ix, m.iy, iz);
                 const T z1 = (T)mass[j] * e1;
@@ -717,8 +725,8 @@ __global__ void __launch_bounds__(kThreads, kEndMinBlocks<T>) k_end(const T* __r
                     ((float*)out0)[j] = dir ? 0.f : (float)z0;
                     ((float*)out1)[j] = dir ? 0.f : (float)(e1 / (T(1) + beta));
                 } else {
-                    out0[j] = dir ? 0.0 : (double)z0;
-                    out1[j] = dir ? 0.0 : (double)z1;
+                    out0[j] = as_f64(dir ? T(0) : z0);
+                    out1[j] = as_f64(dir ? T(0) : z1);
                 }
                 if (std::is_same<T, float>::value)
                     accf.add(dir ? 0.0f : (float)(e0 * z0 + e1 * z1));
@@ -744,7 +752,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_prep(const double* __restrict_
         const T k = kap[j];  // Dirichlet (kappa = 0) only selects the store (see k_start)
         const int nbf = num_abc(g, m.ix, m.iy, iz);
         const T beta = nbf ? (T)nbf * sqrt(k) : T(0);
-        const T v = (T)b[j] / ((T)mass[j] * (T(1) + beta));  // 0/0 on Dirichlet nodes: not stored
+        const T v = as_step<T>(b[j]) / ((T)mass[j] * (T(1) + beta));  // 0/0 on Dirichlet nodes: not stored
         t[j] = k == T(0) ? T(0) : v;
     }
 }
@@ -767,7 +775,7 @@ __global__ void __launch_bounds__(kThreads) k_adj_start(const A* __restrict__ a,
         const int nbf = num_abc(g, m.ix, m.iy, iz);
         const T beta = nbf ? (T)nbf * sqrt(k) : T(0);
         const T tj = t[j];
-        const T u = ((T)a[j] / (T)mass[j] + tj / dtT - k * L / (T(2) * dtT)) / (T(1) + beta);  // 0/0 at Dirichlet
+        const T u = (as_step<T>(a[j]) / (T)mass[j] + tj / dtT - k * L / (T(2) * dtT)) / (T(1) + beta);  // 0/0 at Dirichlet
         const bool dir = k == T(0);
         cur[j] = dir ? T(0) : u;
         prev[j] = dir ? T(0) : tj / dtT;
@@ -811,8 +819,13 @@ __global__ void __launch_bounds__(kThreads, kEndMinBlocks<T>) k_adj_final(const 
             const T q0 = M * (sj - (T(1) - beta) * u1[j]) - T(0.5) * dtT * dtT * W * ih2 * L;
             const T q1 = dtT * M * (T(1) - beta) * sj;
             if (MODE == 1) {
-                o0[j] = dir ? V(0) : (V)q0;
-                o1[j] = dir ? V(0) : (V)q1;
+                if constexpr (std::is_same<V, double>::value) {
+                    o0[j] = as_f64(dir ? T(0) : q0);
+                    o1[j] = as_f64(dir ? T(0) : q1);
+                } else {
+                    o0[j] = dir ? V(0) : (V)q0;
+                    o1[j] = dir ? V(0) : (V)q1;
+                }
             } else if (std::is_same<T, float>::value) {
                 // FP32 periods: z came from FP32 values, so the differences and products stay in
                 // FP32 (FP64 only holds the stored vectors)
@@ -821,15 +834,20 @@ __global__ void __launch_bounds__(kThreads, kEndMinBlocks<T>) k_adj_final(const 
                     zz0 = ((const float*)z0)[j];
                     zz1 = (float)M * ((float)(T(1) + beta) * ((const float*)z1)[j]);
                 } else {
-                    zz0 = (float)z0[j];
-                    zz1 = (float)z1[j];
+                    zz0 = soft64::to_f32(z0[j]);
+                    zz1 = soft64::to_f32(z1[j]);
                 }
                 const float g0 = (float)q0 - zz0;
                 const float g1 = (float)q1 - zz1;
-                const float pd = g0 * (float)d0[j] + g1 * (float)d1[j];
-                o0[j] = dir ? V(0) : (V)g0;
-                o1[j] = dir ? V(0) : (V)g1;
-                if (gt1) gt1[j] = dir ? 0.0 : (double)(g1 * (float)minv[j]);
+                const float pd = g0 * as_step<float>(d0[j]) + g1 * as_step<float>(d1[j]);
+                if constexpr (std::is_same<V, double>::value) {
+                    o0[j] = soft64::to_f64(dir ? 0.0f : g0);
+                    o1[j] = soft64::to_f64(dir ? 0.0f : g1);
+                } else {
+                    o0[j] = dir ? V(0) : (V)g0;
+                    o1[j] = dir ? V(0) : (V)g1;
+                }
+                if (gt1) gt1[j] = soft64::to_f64(dir ? 0.0f : g1 * soft64::to_f32(minv[j]));
                 accf0.add(dir ? 0.0f : pd);
                 accf1.add(dir ? 0.0f : g0);
             } else {
@@ -857,35 +875,51 @@ __global__ void __launch_bounds__(kThreads, kEndMinBlocks<T>) k_adj_final(const 
     }
 }
 
-// S = dt^2 M^-1 (W f + A g) = kappa h^2 (f + (2 nb / h) g), zero on Dirichlet nodes
-// (or added to S when accumulating).
+// S = dt^2 M^-1 (W f + A g) = kappa h^2 (f + (2 nb / h) g), zero on Dirichlet nodes (or added
+// to S when accumulating), its FP32 copy S32 (nullable) and the source columns scol (nullable,
+// zeroed by the caller): scol[x + sx y] = 1 if S != 0 at some node (x, y, z) with 0 < z < nz.
+// One pass over f, kappa and the outputs: g and, without f, kappa are read on the absorbing
+// faces only, where A is not zero.  a1..a3 = 2 nb / h for nb = 1..3 faces (a division per node
+// costs more FP64 time than the rest of the node).
+template <bool ACC>
 __global__ void __launch_bounds__(kThreads) k_make_source(const double* __restrict__ f, const double* __restrict__ gb,
                                                           const double* __restrict__ kap64, double* __restrict__ S,
-                                                          Geom g, int zc, int accumulate) {
+                                                          float* __restrict__ S32, unsigned char* __restrict__ scol,
+                                                          Geom g, int zc, double a1, double a2, double a3) {
     const PlaneMap m = plane_map(g, zc);
     if (!m.valid) return;
-    for (int iz = m.z0; iz < m.z1; ++iz) {
-        const long long j = node(g, m.ix, m.iy, iz);
-        const double k = kap64[j];
-        const double sc = k * g.h * g.h;
-        double re = 0.0, im = 0.0;
-        if (f) {
-            re += f[2 * j];
-            im += f[2 * j + 1];
+    const long long sZ = (long long)g.sx * g.sy;
+    long long j = node(g, m.ix, m.iy, m.z0);
+    bool any = false;
+    for (int iz = m.z0; iz < m.z1; ++iz, j += sZ) {
+        const int nb = gb ? num_abc(g, m.ix, m.iy, iz) : 0;
+        double sr = 0.0, si = 0.0;
+        if (f || nb) {
+            const double k = kap64[j];
+            const double sc = k * g.h * g.h;
+            double re = 0.0, im = 0.0;
+            if (f) {
+                re += f[2 * j];
+                im += f[2 * j + 1];
+            }
+            if (nb) {
+                const double a = nb == 1 ? a1 : (nb == 2 ? a2 : a3);
+                re += a * gb[2 * j];
+                im += a * gb[2 * j + 1];
+            }
+            sr = sc * re;
+            si = sc * im;
+            if (ACC) {
+                S[2 * j] += sr;
+                S[2 * j + 1] += si;
+            }
         }
-        if (gb) {
-            const double a = 2.0 * num_abc(g, m.ix, m.iy, iz) / g.h;
-            re += a * gb[2 * j];
-            im += a * gb[2 * j + 1];
-        }
-        if (accumulate) {
-            S[2 * j] += sc * re;
-            S[2 * j + 1] += sc * im;
-        } else {
-            S[2 * j] = sc * re;
-            S[2 * j + 1] = sc * im;
-        }
+        if (ACC) continue;
+        reinterpret_cast<double2*>(S)[j] = make_double2(sr, si);
+        if (S32) reinterpret_cast<float2*>(S32)[j] = make_float2(soft64::to_f32(sr), soft64::to_f32(si));
+        any |= iz > 0 && iz < g.nz && !(soft64::is_zero(sr) && soft64::is_zero(si));
     }
+    if (scol && any) scol[m.ix + (long long)g.sx * m.iy] = 1;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1190,40 +1224,42 @@ void launch_source_columns(const Geom& g, const double* S, unsigned char* scol, 
 
 template <typename T>
 void launch_start(const Geom& g, int order, const T* w0t, const double* w1, T* y0, T* y1, const T* kap,
-                  const double* S, double dt, int zc, cudaStream_t st, bool w1_float) {
+                  const double* S, bool src_faces, double dt, int zc, cudaStream_t st, bool w1_float) {
+    const int sf = src_faces ? 1 : 0;
     note_launch(1);
     const dim3 grid = plane_grid(g, zc);
     if constexpr (std::is_same<T, float>::value) {
         if (w1_float) {  // FP32 CG vectors: w1 holds floats
             const float* w1f = (const float*)w1;
             if (order == 2) {
-                if (S) k_start<T, 2, true, float><<<grid, kThreads, 0, st>>>(w0t, w1f, y0, y1, kap, S, g, dt, zc);
-                else k_start<T, 2, false, float><<<grid, kThreads, 0, st>>>(w0t, w1f, y0, y1, kap, S, g, dt, zc);
+                if (S) k_start<T, 2, true, float><<<grid, kThreads, 0, st>>>(w0t, w1f, y0, y1, kap, S, g, dt, zc, sf);
+                else k_start<T, 2, false, float><<<grid, kThreads, 0, st>>>(w0t, w1f, y0, y1, kap, S, g, dt, zc, sf);
             } else {
-                if (S) k_start<T, 4, true, float><<<grid, kThreads, 0, st>>>(w0t, w1f, y0, y1, kap, S, g, dt, zc);
-                else k_start<T, 4, false, float><<<grid, kThreads, 0, st>>>(w0t, w1f, y0, y1, kap, S, g, dt, zc);
+                if (S) k_start<T, 4, true, float><<<grid, kThreads, 0, st>>>(w0t, w1f, y0, y1, kap, S, g, dt, zc, sf);
+                else k_start<T, 4, false, float><<<grid, kThreads, 0, st>>>(w0t, w1f, y0, y1, kap, S, g, dt, zc, sf);
             }
             return;
         }
     }
     if (order == 2) {
-        if (S) k_start<T, 2, true><<<grid, kThreads, 0, st>>>(w0t, w1, y0, y1, kap, S, g, dt, zc);
-        else k_start<T, 2, false><<<grid, kThreads, 0, st>>>(w0t, w1, y0, y1, kap, S, g, dt, zc);
+        if (S) k_start<T, 2, true><<<grid, kThreads, 0, st>>>(w0t, w1, y0, y1, kap, S, g, dt, zc, sf);
+        else k_start<T, 2, false><<<grid, kThreads, 0, st>>>(w0t, w1, y0, y1, kap, S, g, dt, zc, sf);
     } else {
-        if (S) k_start<T, 4, true><<<grid, kThreads, 0, st>>>(w0t, w1, y0, y1, kap, S, g, dt, zc);
-        else k_start<T, 4, false><<<grid, kThreads, 0, st>>>(w0t, w1, y0, y1, kap, S, g, dt, zc);
+        if (S) k_start<T, 4, true><<<grid, kThreads, 0, st>>>(w0t, w1, y0, y1, kap, S, g, dt, zc, sf);
+        else k_start<T, 4, false><<<grid, kThreads, 0, st>>>(w0t, w1, y0, y1, kap, S, g, dt, zc, sf);
     }
 }
 
 template <typename T>
 void launch_end(const Geom& g, int order, int mode, const T* yN, const T* yNm1, const T* w0t, const double* w1,
-                const T* kap, const T* mass, const double* S, double cs, double sn, double* out0, double* out1,
-                Red red, double dt, int zc, cudaStream_t st) {
+                const T* kap, const T* mass, const double* S, bool src_faces, double cs, double sn, double* out0,
+                double* out1, Red red, double dt, int zc, cudaStream_t st) {
+    const int sf = src_faces ? 1 : 0;
     note_launch(1);
     const dim3 grid = plane_grid(g, zc);
 #define CMCG_END(O, SRC, MODE)                                                                                \
     k_end<T, O, SRC, MODE><<<grid, kThreads, 0, st>>>(yN, yNm1, w0t, w1, kap, mass, S, cs, sn, out0, out1, red, \
-                                                      g, dt, zc)
+                                                      g, dt, zc, sf)
     const bool src = S != nullptr;
     if constexpr (std::is_same<T, float>::value) {
         if (mode == 2) {
@@ -1235,7 +1271,7 @@ void launch_end(const Geom& g, int order, int mode, const T* yN, const T* yNm1, 
             const float* w1f = (const float*)w1;
 #define CMCG_END3(O, SRC)                                                                                      \
     k_end<T, O, SRC, 2, float><<<grid, kThreads, 0, st>>>(yN, yNm1, w0t, w1f, kap, mass, S, cs, sn, out0, out1, \
-                                                          red, g, dt, zc)
+                                                          red, g, dt, zc, sf)
             if (order == 2) { if (src) CMCG_END3(2, true); else CMCG_END3(2, false); }
             else { if (src) CMCG_END3(4, true); else CMCG_END3(4, false); }
 #undef CMCG_END3
@@ -1302,10 +1338,14 @@ void launch_adj_final(const Geom& g, int order, int mode, const T* s, const T* u
 #undef CMCG_FIN
 }
 
-void launch_make_source(const Geom& g, const double* f, const double* gb, const double* kap64, double* S, int zc,
-                        bool accumulate, cudaStream_t st) {
+void launch_make_source(const Geom& g, const double* f, const double* gb, const double* kap64, double* S, float* S32,
+                        unsigned char* scol, int zc, bool accumulate, cudaStream_t st) {
     note_launch(1);
-    k_make_source<<<plane_grid(g, zc), kThreads, 0, st>>>(f, gb, kap64, S, g, zc, accumulate ? 1 : 0);
+    const double a1 = 2.0 * 1 / g.h, a2 = 2.0 * 2 / g.h, a3 = 2.0 * 3 / g.h;
+    if (accumulate)
+        k_make_source<true><<<plane_grid(g, zc), kThreads, 0, st>>>(f, gb, kap64, S, nullptr, nullptr, g, zc, a1, a2, a3);
+    else
+        k_make_source<false><<<plane_grid(g, zc), kThreads, 0, st>>>(f, gb, kap64, S, S32, scol, g, zc, a1, a2, a3);
 }
 
 long long plane_blocks(const Geom& g, int zc) {
@@ -1317,9 +1357,9 @@ long long plane_blocks(const Geom& g, int zc) {
     template void launch_step<T>(const Geom&, int, const T*, T*, const T*, const T*, double, double, int,        \
                                  int, cudaStream_t, const unsigned char*);                                     \
     template void launch_start<T>(const Geom&, int, const T*, const double*, T*, T*, const T*, const double*,   \
-                                  double, int, cudaStream_t, bool);                                            \
+                                  bool, double, int, cudaStream_t, bool);                                      \
     template void launch_end<T>(const Geom&, int, int, const T*, const T*, const T*, const double*, const T*,   \
-                                const T*, const double*, double, double, double*, double*, Red, double,         \
+                                const T*, const double*, bool, double, double, double*, double*, Red, double,   \
                                 int, cudaStream_t);                                                            \
     template void launch_adj_prep<T>(const Geom&, const double*, const T*, const T*, T*, int, cudaStream_t);    \
     template void launch_adj_start<T, double>(const Geom&, int, const double*, const T*, const T*, const T*,    \
