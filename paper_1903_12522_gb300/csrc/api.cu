@@ -150,6 +150,10 @@ size_t layout(cmcg_handle* H, const Geom& g, const cmcg_options& o, char* base) 
         H->wo0 = c.take<double>(np);
         H->wo1 = c.take<double>(np);
     }
+    if (band_plan(g, H->order, o.precision == CMCG_FP64 ? 8 : 4, kBandStop, &H->band)) {
+        H->band_words = c.take<unsigned long long>(H->band.words);
+        H->band_count = c.take<unsigned>(kBandStop + 1);
+    }
     H->pr = c.take<double>(np);
     H->pp = c.take<double>(np);
     H->pAp = c.take<double>(np);
@@ -269,9 +273,24 @@ void collect_timing(cmcg_handle* H) {
     H->ev_used = 0;
 }
 
+// The exchange words and step counts of the 2D band kernel at their start.
+void band_reset(cmcg_handle* H) {
+    cudaMemsetAsync(H->band_words, 0, sizeof(unsigned long long) * H->band.words, H->st);
+    cudaMemsetAsync(H->band_count, 0, sizeof(unsigned) * (kBandStop + 1), H->st);
+}
+
+// After a synchronisation: did a band kernel's wait run out?
+int band_status(cmcg_handle* H) {
+    if (!H->band_count || H->hsc[SC_COUNT] == 0.0) return CMCG_OK;
+    H->hsc[SC_COUNT] = 0.0;
+    band_reset(H);
+    return CMCG_ERR_DEVICE_TIMEOUT;
+}
+
 int sync_read(cmcg_handle* H) {
     cudaMemcpyAsync(H->hsc, H->sc, sizeof(double) * SC_COUNT, cudaMemcpyDeviceToHost, H->st);
     if (cudaStreamSynchronize(H->st) != cudaSuccess) return CMCG_ERR_CUDA;
+    if (const int rc = band_status(H)) return rc;
     if (H->timing) collect_timing(H);
     return cuda_status();
 }
@@ -401,10 +420,45 @@ void step_one(cmcg_handle* H, const T* cur, T* prev, const T* kap, const T* S, d
     launch_step<T>(H->g, H->order, cur, prev, kap, S, cs, sn, flags, zc, H->st, H->scol);
 }
 
+// `count` steps from b in one launch (or a few: kBandSteps steps each) where the grid fits the
+// chip: 2D grids, FP32 steps and the FP64 steps of FP64 handles.  factors(n, &cs, &sn): source
+// factors of the n-th step (n = 0, 1, ...), with src.  Returns false, with nothing launched, if
+// the loop has to run step by step.
+template <typename T, typename F>
+bool band_steps(cmcg_handle* H, PeriodBuffers& b, long long count, bool src, bool adjoint, F factors) {
+    constexpr bool f32 = std::is_same<T, float>::value;
+    if (H->band_off || !f32 != (H->opt.precision == CMCG_FP64) || count < 1 || !band_fits(H->band, src && !H->src_faces))
+        return false;
+    const T* kap = f32 ? (const T*)H->kap32 : (const T*)H->kap64;
+    const T* S = src ? step_source<T>(H) : nullptr;
+    double cs[kBandSteps], sn[kBandSteps];
+    const int tp = timing_begin(H, f32, (int)((count + kBandSteps - 1) / kBandSteps));
+    for (long long n0 = 0; n0 < count; n0 += kBandSteps) {
+        const int m = (int)std::min<long long>(kBandSteps, count - n0);
+        for (int s = 0; src && s < m; ++s) factors(n0 + s, &cs[s], &sn[s]);
+        const cudaError_t e = launch_step_band<T>(H->g, H->order, H->band, (T*)b.cur, (T*)b.prev, kap, S, H->src_faces,
+                                                  H->wface, H->band_words, H->band_count, H->hsc + SC_COUNT, m, cs, sn,
+                                                  step_zc(H) == kZcFlat ? 1 : 0, adjoint && n0 == 0, adjoint && n0 + m == count, H->st);
+        if (e != cudaSuccess) {
+            if (n0 == 0) {  // no cooperative launch to be had (shared device limits): step by step
+                cudaGetLastError();
+                H->band.bands = 0;
+                timing_end(H, tp);
+                return false;
+            }
+            break;  // the error stays pending for cuda_status()
+        }
+        if (m & 1) std::swap(b.cur, b.prev);
+    }
+    timing_end(H, tp);
+    return true;
+}
+
 // `count` homogeneous steps from b (in pairs where possible, else one by one).
 template <typename T>
 void plain_steps(cmcg_handle* H, PeriodBuffers& b, int count) {
     const Geom& g = H->g;
+    if (band_steps<T>(H, b, count, false, false, [](long long, double*, double*) {})) return;
     const int zc = step_zc(H);
     const T* kap = std::is_same<T, float>::value ? (const T*)H->kap32 : (const T*)H->kap64;
     if (use_pairs<T>(H, false) && count >= 2) {
@@ -446,6 +500,12 @@ void fwd_steps(cmcg_handle* H, PeriodBuffers& b, bool src) {
         return;
     }
     const T* S = step_source<T>(H);
+    if (band_steps<T>(H, b, H->N - 1, true, false, [H](long long n, double* cs, double* sn) {
+            const double th = H->omega * (double)(n + 1) * H->dt;
+            *cs = cos(th);
+            *sn = sin(th);
+        }))
+        return;
     const int tp = timing_begin(H, std::is_same<T, float>::value, H->N - 1);
     for (int n = 1; n < H->N; ++n) {
         const double th = H->omega * n * H->dt;
@@ -535,6 +595,7 @@ void adj_steps(cmcg_handle* H, PeriodBuffers& b) {
         step_one<T>(H, (const T*)b.cur, (T*)b.prev, kap, nullptr, 0.0, 0.0, adj_step_flags(k, H->N), zc);
         std::swap(b.cur, b.prev);
     };
+    if (band_steps<T>(H, b, n, false, true, [](long long, double*, double*) {})) return;
     if (use_pairs<T>(H, false)) {
         single(0);
         if (n >= 3) plain_steps<T>(H, b, n - 2);
@@ -612,7 +673,15 @@ void runup(cmcg_handle* H, int periods, double* w0, double* w1) {
     cudaMemsetAsync(prev, 0, sizeof(T) * g.np, H->st);
     const long long total = (long long)periods * H->N;
     const double ttr = periods * H->T;
-    for (long long n = 1; n < total; ++n) {
+    PeriodBuffers b{cur, prev, nullptr};
+    const bool band = band_steps<T>(H, b, total - 1, true, false, [H, ttr](long long n, double* cs, double* sn) {
+        const double t = (double)(n + 1) * H->dt, th = ramp(t, ttr);
+        *cs = th * cos(H->omega * t);
+        *sn = th * sin(H->omega * t);
+    });
+    cur = (T*)b.cur;
+    prev = (T*)b.prev;
+    for (long long n = 1; n < total && !band; ++n) {
         const double t = n * H->dt;
         const double th = ramp(t, ttr);
         step_one<T>(H, cur, prev, kap, step_source<T>(H), th * cos(H->omega * t), th * sin(H->omega * t), kStepSrc,
@@ -1395,6 +1464,7 @@ size_t cmcg_workspace_size(const cmcg_grid* grid, const cmcg_options* opts) {
     if (opts) o = *opts;
     if (o.precision < CMCG_FP64 || o.precision > CMCG_MIXED) return 0;
     cmcg_handle tmp;
+    tmp.order = grid->order;
     Geom g = make_geom(grid, 0);
     return layout(&tmp, g, o, nullptr);
 }
@@ -1444,9 +1514,22 @@ int cmcg_create(const cmcg_grid* grid, const double* c, double omega, const cmcg
     }
     H->volume = 1.0;
     for (int a = 0; a < grid->dim; ++a) H->volume *= grid->n[a] * grid->h;
-    if (cudaMallocHost((void**)&H->hsc, sizeof(double) * SC_COUNT) != cudaSuccess) {
+    if (cudaMallocHost((void**)&H->hsc, sizeof(double) * (SC_COUNT + 1)) != cudaSuccess) {
         delete H;
         return CMCG_ERR_CUDA;
+    }
+    H->hsc[SC_COUNT] = 0.0;
+    if (H->band_count) {
+        int dev = 0, sms = 0, coop = 0;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        const size_t words = H->band.words;
+        if (!coop || !band_plan(H->g, H->order, o.precision == CMCG_FP64 ? 8 : 4, std::min(sms, kBandStop), &H->band) ||
+            H->band.words > words)
+            H->band.bands = 0;
+        else
+            band_reset(H);
     }
     H->timing = (o.flags & CMCG_FLAG_TIMING) != 0;
     H->vec32 = o.precision == CMCG_MIXED && (o.flags & CMCG_FLAG_INEXACT_RIESZ) && !(o.flags & CMCG_FLAG_FIRST_ORDER);
@@ -1573,6 +1656,7 @@ int cmcg_wave_period(cmcg_handle* h, const double* u0, const double* v0, const d
         forward_period<double>(h, w0, v0, src, 1, uT, vT);
     }
     if (cudaStreamSynchronize(h->st) != cudaSuccess) return CMCG_ERR_CUDA;
+    if (const int rc = band_status(h)) return rc;
     return cuda_status();
 }
 
@@ -1585,6 +1669,7 @@ int cmcg_adjoint_period(cmcg_handle* h, const double* a, const double* b, double
     else
         adjoint_period<double>(h, a, b, 1, nullptr, nullptr, q0, q1, nullptr);
     if (cudaStreamSynchronize(h->st) != cudaSuccess) return CMCG_ERR_CUDA;
+    if (const int rc = band_status(h)) return rc;
     return cuda_status();
 }
 
@@ -1604,7 +1689,7 @@ int cmcg_bulk_wait_selftest(int spin_limit, void* stream) {
 int cmcg_check_status(long long* count, long long* site, long long* index) {
     if (cudaDeviceSynchronize() != cudaSuccess) return CMCG_ERR_CUDA;
     long long total = 0, first_site = -1, first_index = 0;
-    for (auto read : {check_read_wave, check_read_riesz, check_read_pair, check_read_soft}) {
+    for (auto read : {check_read_wave, check_read_riesz, check_read_pair, check_read_soft, check_read_band}) {
         long long w[3];
         read(w);
         if (w[0] > 0 && first_site < 0) {

@@ -172,7 +172,9 @@ template <typename F>
 void on_side(cmcg_engine* e, cmcg_handle* h, int k, F f) {
     cudaStream_t own = h->st;
     h->st = e->side[k % cmcg_engine::kSide];
+    h->band_off = true;  // no cooperative launches side by side
     f(h);
+    h->band_off = false;
     h->st = own;
 }
 

@@ -30,6 +30,7 @@ void check_read_wave(long long* out);
 void check_read_riesz(long long* out);
 void check_read_pair(long long* out);
 void check_read_soft(long long* out);
+void check_read_band(long long* out);
 long long launch_count();
 
 // ---- wave.cu --------------------------------------------------------------------------
@@ -139,6 +140,32 @@ void launch_adj_final_soft(const Geom& g, int order, int mode, const double* s, 
                            const double* kap, const double* wface, const double* minv, const double* z0,
                            const double* z1, const double* d0, const double* d1, double* o0, double* o1, double* gt1,
                            Red red, double dt, int zc, cudaStream_t st);
+
+// ---- step_band.cu -----------------------------------------------------------------------
+// 2D step loops in one cooperative launch, the grid held on chip in bands of rows, one per SM.
+constexpr int kBandSteps = 200;  // most steps of one launch (their source factors are arguments)
+constexpr int kBandStop = 152;   // index of the stop word behind the per-band step counts
+struct BandPlan {
+    int bands = 0, rows = 0, extra = 0;  // bands (0: the grid does not suit the kernel) and their rows
+    int npt = 0;                         // nodes, or float4 chunks, per thread
+    int face_slots = 0;                  // face nodes (or chunks) whose factors a band holds
+    int cluster = 0;                     // bands in one cluster (0: exchange through global memory)
+    size_t smem[2] = {0, 0};                      // without / with a source away from the faces
+    size_t words = 0;                             // exchange words (8 bytes each)
+};
+// elem_size: 4 (FP32 steps) or 8 (FP64 steps with the integer stencil sum).
+bool band_plan(const Geom& g, int order, int elem_size, int sms, BandPlan* p);
+bool band_fits(const BandPlan& p, bool volume_source);
+// nsteps <= kBandSteps steps from (cur = y^n, prev = y^{n-1}); cur and prev have swapped roles
+// afterwards if nsteps is odd.  S (nullable) with the factors cs, sn of each step; src_faces as
+// for launch_step_soft; adj_first / adj_last: the first / last step is the adjoint's.  words
+// (p.words of them, zero at first), count (kBandStop + 1, zero at first) and err (host memory)
+// as described in step_band.cu.
+template <typename T>
+cudaError_t launch_step_band(const Geom& g, int order, const BandPlan& p, T* cur, T* prev, const T* kap, const T* S,
+                             bool src_faces, const double* wface, unsigned long long* words, unsigned* count,
+                             double* err, int nsteps, const double* cs, const double* sn, int src_form,
+                             bool adj_first, bool adj_last, cudaStream_t st);
 
 // ---- step_bulk.cu -----------------------------------------------------------------------
 // FP32 3D 7-point leapfrog step with TMA bulk-copy staging (homogeneous; flags 0, PREV_SCALED,

@@ -52,6 +52,12 @@ struct cmcg_handle {
     int blk_level = -1;       // first level run inside one thread block (-1: none)
     BlockLevels blk{};
     int riesz_guess = 0;      // PCG iterations of the previous Riesz solve
+    // 2D step loops in one launch (step_band.cu); band_off: step by step instead (the engine, whose
+    // per-slot kernels run side by side)
+    BandPlan band{};
+    unsigned long long* band_words = nullptr;
+    unsigned* band_count = nullptr;
+    bool band_off = false;
     // first-order formulation (CMCG_FLAG_FIRST_ORDER): CG vectors on the state (p, v) of
     // (dim + 1) N_p doubles, and the two stepping buffers (sized for double)
     double *fo_s = nullptr, *fo_r = nullptr, *fo_d = nullptr, *fo_e = nullptr, *fo_g = nullptr, *fo_x = nullptr;
@@ -63,7 +69,7 @@ struct cmcg_handle {
     double* partials = nullptr;
     unsigned* tickets = nullptr;
     double* sc = nullptr;
-    double* hsc = nullptr;  // pinned host mirror of sc
+    double* hsc = nullptr;  // pinned host mirror of sc; [SC_COUNT]: error word written by k_band
     // FP32 CG vectors: a mixed-precision handle with the V-cycle Riesz map keeps the vectors of
     // its inner (FP32-period) flexible CG -- w, rhat, d, ghat, z -- as floats in the first half
     // of their buffers; vec32_active is set while such an inner iteration is being enqueued
