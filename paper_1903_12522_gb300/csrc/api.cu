@@ -438,7 +438,7 @@ bool band_steps(cmcg_handle* H, PeriodBuffers& b, long long count, bool src, boo
         for (int s = 0; src && s < m; ++s) factors(n0 + s, &cs[s], &sn[s]);
         const cudaError_t e = launch_step_band<T>(H->g, H->order, H->band, (T*)b.cur, (T*)b.prev, kap, S, H->src_faces,
                                                   H->wface, H->band_words, H->band_count, H->hsc + SC_COUNT, m, cs, sn,
-                                                  step_zc(H) == kZcFlat ? 1 : 0, adjoint && n0 == 0, adjoint && n0 + m == count, H->st);
+                                                  adjoint && n0 == 0, adjoint && n0 + m == count, H->st);
         if (e != cudaSuccess) {
             if (n0 == 0) {  // no cooperative launch to be had (shared device limits): step by step
                 cudaGetLastError();
@@ -735,9 +735,9 @@ int coarse_sweeps(const Geom& g) {
 void vcycle(cmcg_handle* H, int l) {
     MGLevel& L = H->lv[l];
     const float om = jacobi_omega(L.g);
-    if (l == H->blk_level) {
-        const BlockLevels& B = H->blk;
-        launch_mg_block_vcycle(B, L.b, L.x, om, 2, coarse_sweeps(B.g[B.n - 1]), H->st);
+    if (l == H->coarse_level) {
+        const CoarseLevels& B = H->coarse;
+        launch_mg_coarse(B, L.b, L.x, om, coarse_sweeps(B.g[B.n - 1]), H->st);
         return;
     }
     if (l == H->nlev - 1) {  // coarsest level too large for one block: Jacobi sweeps
@@ -748,21 +748,14 @@ void vcycle(cmcg_handle* H, int l) {
         }
         return;
     }
-    const int nu = 2;
-    launch_mg_jacobi(L, nullptr, L.x, L.b, om, true, H->st);
-    for (int s = 1; s < nu; ++s) {
-        launch_mg_jacobi(L, L.x, L.x2, L.b, om, false, H->st);
-        std::swap(L.x, L.x2);
-    }
+    launch_mg_first(L, L.x, L.b, om, H->st);  // two sweeps
     MGLevel& C = H->lv[l + 1];
     launch_mg_residual(L, L.x, L.b, L.r, H->st);
     launch_mg_restrict(L, L.r, C, C.b, H->st);
     vcycle(H, l + 1);
     launch_mg_prolong_add(C, C.x, L, L.x, H->st);
-    for (int s = 0; s < nu; ++s) {
-        launch_mg_jacobi(L, L.x, L.x2, L.b, om, false, H->st);
-        std::swap(L.x, L.x2);
-    }
+    launch_mg_jacobi(L, L.x, L.x2, L.b, om, false, H->st);
+    launch_mg_jacobi(L, L.x2, L.x, L.b, om, false, H->st);
 }
 
 void precondition(cmcg_handle* H, const double* r) {
@@ -779,22 +772,40 @@ int riesz_solve(cmcg_handle* H, const double* rhs, double* x, int* iters_out) {
     const double tol = H->opt.riesz_tol;
     Red red = H->red();
     launch_pcg_project(g, rhs, H->pr, H->mask, H->volume, red, project, H->st);
-    launch_fill(x, n, 0.0, H->st);
-    precondition(H, H->pr);
-    launch_pcg_dots_after_precond(n, H->pr, H->lv[0].x, nullptr, H->pzd, red, H->st);
-    launch_pcg_p_update(n, H->pp, H->pzd, red, true, H->st);
+    // FP64 handles take the vector passes made for the FP64 pipe; the exact map of an FP32 or mixed
+    // solve keeps its rounding (its FP32 periods would follow any change of it)
+    const bool fast = H->wface != nullptr;
+    const int zce = g.dim == 3 ? kZcEnds : 1;
+    float* const zf = H->lv[0].b;
+    auto direction = [&](bool first) {  // z = B r, then p
+        if (fast) {
+            if (first) launch_to_float(n, H->pr, zf, H->st);  // later: written with r
+            vcycle(H, 0);
+            launch_pcg_dots(n, H->pr, H->lv[0].x, first ? nullptr : H->pAp, red, H->st);
+            launch_pcg_p(n, H->pp, H->lv[0].x, red, first, H->st);
+            return;
+        }
+        precondition(H, H->pr);
+        launch_pcg_dots_after_precond(n, H->pr, H->lv[0].x, first ? nullptr : H->pAp, H->pzd, red, H->st);
+        launch_pcg_p_update(n, H->pp, H->pzd, red, first, H->st);
+    };
+    if (!fast) launch_fill(x, n, 0.0, H->st);
+    direction(true);
     int it = 0;
     bool converged = false;
     double bb = -1.0;
     // the previous solve's iteration count, less a margin, runs without host checks
     const int blind = std::max(0, std::min(H->riesz_guess - 2, H->opt.riesz_max_iter - 1));
     for (it = 1; it <= H->opt.riesz_max_iter; ++it) {
-        launch_applyK(g, H->order, H->mask, H->pp, H->pAp, H->pp, red, SC_P_PAP, H->st);
-        launch_pcg_xr_update(n, x, H->pr, H->pp, H->pAp, red, H->st);
+        if (fast) {
+            launch_pcg_applyK(g, H->order, H->mask, H->pp, H->pAp, red, zce, H->st);
+            launch_pcg_xr(n, x, H->pr, H->pp, H->pAp, zf, red, it == 1, H->st);
+        } else {
+            launch_applyK(g, H->order, H->mask, H->pp, H->pAp, H->pp, red, SC_P_PAP, H->st);
+            launch_pcg_xr_update(n, x, H->pr, H->pp, H->pAp, red, H->st);
+        }
         if (it <= blind) {
-            precondition(H, H->pr);
-            launch_pcg_dots_after_precond(n, H->pr, H->lv[0].x, H->pAp, H->pzd, red, H->st);
-            launch_pcg_p_update(n, H->pp, H->pzd, red, false, H->st);
+            direction(false);
             continue;
         }
         int rc = sync_read(H);
@@ -806,9 +817,7 @@ int riesz_solve(cmcg_handle* H, const double* rhs, double* x, int* iters_out) {
             converged = true;
             break;
         }
-        precondition(H, H->pr);
-        launch_pcg_dots_after_precond(n, H->pr, H->lv[0].x, H->pAp, H->pzd, red, H->st);
-        launch_pcg_p_update(n, H->pp, H->pzd, red, false, H->st);
+        direction(false);
     }
     if (project) launch_mean_remove(g, x, H->volume, red, H->st);
     if (converged) H->riesz_guess = it;
@@ -1587,19 +1596,8 @@ int cmcg_create(const cmcg_grid* grid, const double* c, double omega, const cmcg
         launch_to_float(H->g.np, H->mass, H->mass32, H->st);
         launch_to_float(H->g.np, H->minv, H->minv32, H->st);
     }
-    H->blk_level = -1;
-    for (int l = 0; l < H->nlev; ++l)
-        if (H->lv[l].g.np <= mg_block_max_nodes()) {
-            H->blk_level = l;
-            break;
-        }
-    if (H->blk_level >= 0) {
-        H->blk.n = std::min(H->nlev - H->blk_level, kBlockLevelsMax);
-        for (int i = 0; i < H->blk.n; ++i) {
-            H->blk.g[i] = H->lv[H->blk_level + i].g;
-            H->blk.mask[i] = H->lv[H->blk_level + i].mask;
-        }
-    }
+    for (int l = 0; l < H->nlev && H->coarse_level < 0; ++l)
+        if (mg_coarse_plan(H->lv, H->nlev, l, &H->coarse)) H->coarse_level = l;
     if (sync_read(H) != CMCG_OK) return fail(CMCG_ERR_CUDA);
     if (o.flags & CMCG_FLAG_L2_KAPPA) l2_kappa_begin(H);
     *out = H;

@@ -164,8 +164,18 @@ bool band_fits(const BandPlan& p, bool volume_source);
 template <typename T>
 cudaError_t launch_step_band(const Geom& g, int order, const BandPlan& p, T* cur, T* prev, const T* kap, const T* S,
                              bool src_faces, const double* wface, unsigned long long* words, unsigned* count,
-                             double* err, int nsteps, const double* cs, const double* sn, int src_form,
-                             bool adj_first, bool adj_last, cudaStream_t st);
+                             double* err, int nsteps, const double* cs, const double* sn, bool adj_first,
+                             bool adj_last, cudaStream_t st);
+
+// The FP64 vector passes of the Riesz PCG for FP64 handles: as launch_applyK and launch_pcg_*, with
+// the integer stencil sum, the scalars formed once per kernel, z read as the V-cycle's floats, and
+// the V-cycle's next right-hand side bf = float(r) written by the residual update.
+void launch_pcg_applyK(const Geom& g, int order, const unsigned char* mask, const double* p, double* Ap, Red red, int zc,
+                       cudaStream_t st);  // SC_P_PAP, SC_P_ALPHA
+void launch_pcg_xr(long long n, double* x, double* r, const double* p, const double* Ap, float* bf, Red red, bool first,
+                   cudaStream_t st);  // SC_P_RR; first: x starts at zero
+void launch_pcg_dots(long long n, const double* r, const float* z, const double* Ap, Red red, cudaStream_t st);
+void launch_pcg_p(long long n, double* p, const float* z, Red red, bool first, cudaStream_t st);
 
 // ---- step_bulk.cu -----------------------------------------------------------------------
 // FP32 3D 7-point leapfrog step with TMA bulk-copy staging (homogeneous; flags 0, PREV_SCALED,
@@ -248,22 +258,36 @@ struct MGLevel {
 void launch_mg_coarsen_mask(const MGLevel& fine, const MGLevel& coarse, cudaStream_t st);
 void launch_mg_jacobi(const MGLevel& L, const float* xin, float* xout, const float* b, float omega, bool zero_init,
                       cudaStream_t st);
+// The first two sweeps, from x = 0.
+void launch_mg_first(const MGLevel& L, float* xout, const float* b, float omega, cudaStream_t st);
 void launch_mg_residual(const MGLevel& L, const float* x, const float* b, float* r, cudaStream_t st);
 void launch_mg_restrict(const MGLevel& fine, const float* rf, const MGLevel& coarse, float* bc, cudaStream_t st);
 void launch_mg_prolong_add(const MGLevel& coarse, const float* xc, const MGLevel& fine, float* xf, cudaStream_t st);
-// Coarse end of the V-cycle in one thread block (levels up to kBlockLevelsMax, total nodes
-// within the shared-memory budget).
-constexpr int kBlockLevelsMax = 8;
-constexpr int kBlockMaxNodes = 6000;  // nodes of the first in-block level
-struct BlockLevels {
-    int n;
-    Geom g[kBlockLevelsMax];
-    const unsigned char* mask[kBlockLevelsMax];
+// Coarse end of the V-cycle in one cluster launch (riesz.cu): levels 0 .. nc-1 spread over ctas
+// CTAs, the rest in the first one.
+constexpr int kCoarseMax = 10;
+constexpr long long kSpreadMaxNodes = 40000;
+constexpr long long kSpreadMinNodes = 2000;
+constexpr long long kCoarsestMaxNodes = 6000;  // larger: the coarsest level gets a few grid-wide sweeps instead
+struct CoarseLevel {
+    int np, lo, cnt;  // nodes, and the CTA's run of them
+    int chunk, sx, sy, sxy, nx, ny, nz, dim;
+    int fused;                 // see lap_rn
+    float cK, cB, inv2d;       // MGConst
+    unsigned x, r, b;          // offsets in shared memory: iterate, residual / second buffer, right-hand side
+    unsigned mask;             // Dirichlet bytes (0: none)
+    unsigned long long m_chunk, m_sx, m_sy;  // factors of the divisions by chunk, sx, sy
 };
-void launch_mg_block_vcycle(const BlockLevels& lv, const float* b, float* x, float omega, int nu, int coarse_sweeps,
-                            cudaStream_t st);
-size_t mg_block_smem_bytes(const BlockLevels& lv);
-int mg_block_max_nodes();
+struct CoarseLevels {
+    int n = 0, nc = 0, ctas = 1;
+    Geom g[kCoarseMax] = {};
+    const unsigned char* mask[kCoarseMax] = {};
+    CoarseLevel level[kCoarseMax] = {};
+};
+// The levels first .. nlev-1; false if they do not fit.
+bool mg_coarse_plan(const MGLevel* levels, int nlev, int first, CoarseLevels* lv);
+cudaError_t launch_mg_coarse(const CoarseLevels& lv, const float* b, float* x, float omega, int coarse_sweeps,
+                             cudaStream_t st);
 // FP64 PCG pieces on the fine level
 void launch_applyK(const Geom& g, int order, const unsigned char* mask, const double* x, double* y,
                    const double* dotwith, Red red, int slot, cudaStream_t st);

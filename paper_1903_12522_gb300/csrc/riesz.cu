@@ -7,7 +7,7 @@
 //     from the nearest fine node;
 //   - damped Jacobi smoothing, residual restriction by the transpose of (bi/tri)linear
 //     interpolation, prolongation by that interpolation;
-//   - the levels below kBlockMaxNodes nodes run as one V-cycle inside one thread block in
+//   - the levels below kSpreadMaxNodes nodes run as one V-cycle inside one thread-block cluster in
 //     shared memory; its coarsest level is solved by Jacobi sweeps.
 #include <math.h>
 
@@ -84,19 +84,30 @@ __device__ __forceinline__ MGConst mg_const(const Geom& g) {
 }
 
 // One damped Jacobi update at node j (xin == nullptr: from x = 0).
-__device__ __forceinline__ float jacobi_node(const Geom& g, const MGConst& c, const float* xin, float bj, float omega,
-                                             long long j, int ix, int iy, int iz) {
-    const float inv_s = (float)(1 << axis_ends(g, ix, iy, iz));
-    if (!xin) return omega * c.cB * inv_s * bj;
-    Ld<float> f{xin};
-    const float L = lap_t<2, float>(g, f, j, ix, iy, iz);
-    return xin[j] + omega * (c.cB * inv_s * bj - c.inv2d * L);
+__device__ __forceinline__ float jacobi_zero(const MGConst& c, float bj, float omega, int ends) {
+    const float inv_s = (float)(1 << ends);
+    return omega * c.cB * inv_s * bj;
 }
 
-__device__ __forceinline__ float residual_node(const Geom& g, const MGConst& c, const float* x, float bj, long long j,
-                                               int ix, int iy, int iz) {
+// f: the values of x by node index (global memory, or a cluster's shared memory).
+template <typename F>
+__device__ __forceinline__ float jacobi_from(const Geom& g, const MGConst& c, F f, float bj, float omega, long long j,
+                                             int ix, int iy, int iz) {
+    const float inv_s = (float)(1 << axis_ends(g, ix, iy, iz));
+    const float L = lap_t<2, float>(g, f, j, ix, iy, iz);
+    return f(j) + omega * (c.cB * inv_s * bj - c.inv2d * L);
+}
+
+__device__ __forceinline__ float jacobi_node(const Geom& g, const MGConst& c, const float* xin, float bj, float omega,
+                                             long long j, int ix, int iy, int iz) {
+    if (!xin) return jacobi_zero(c, bj, omega, axis_ends(g, ix, iy, iz));
+    return jacobi_from(g, c, Ld<float>{xin}, bj, omega, j, ix, iy, iz);
+}
+
+template <typename F>
+__device__ __forceinline__ float residual_node(const Geom& g, const MGConst& c, F f, float bj, long long j, int ix, int iy,
+                                               int iz) {
     const float s = 1.f / (float)(1 << axis_ends(g, ix, iy, iz));
-    Ld<float> f{x};
     return bj - c.cK * s * lap_t<2, float>(g, f, j, ix, iy, iz);
 }
 
@@ -142,7 +153,8 @@ __device__ __forceinline__ bool nested(const Geom& gf, const Geom& gc) {
 }
 
 // nested 2:1 case: weights 1 at 2J and 1/2 at 2J +- 1 per axis
-__device__ __forceinline__ float restrict_nested(const Geom& gf, const float* rf, int jx, int jy, int jz) {
+template <typename F>
+__device__ __forceinline__ float restrict_nested(const Geom& gf, F rf, int jx, int jy, int jz) {
     const int cx = 2 * jx, cy = 2 * jy, cz = 2 * jz;
     float acc = 0.f;
     const int zlo = gf.dim == 3 ? -1 : 0, zhi = gf.dim == 3 ? 1 : 0;
@@ -154,18 +166,18 @@ __device__ __forceinline__ float restrict_nested(const Geom& gf, const float* rf
             const int fy = cy + dy;
             if (fy < 0 || fy > gf.ny) continue;
             const float wy = dy == 0 ? 1.f : 0.5f;
-            const float* row = rf + node(gf, 0, fy, fz);
-            float racc = row[cx];
-            if (cx > 0) racc += 0.5f * row[cx - 1];
-            if (cx < gf.nx) racc += 0.5f * row[cx + 1];
+            const long long row = node(gf, 0, fy, fz);
+            float racc = rf(row + cx);
+            if (cx > 0) racc += 0.5f * rf(row + cx - 1);
+            if (cx < gf.nx) racc += 0.5f * rf(row + cx + 1);
             acc += wy * wz * racc;
         }
     }
     return acc;
 }
 
-__device__ __forceinline__ float restrict_node(const Geom& gf, const Geom& gc, const float* rf, int jx, int jy,
-                                               int jz) {
+template <typename F>
+__device__ __forceinline__ float restrict_node(const Geom& gf, const Geom& gc, F rf, int jx, int jy, int jz) {
     if (nested(gf, gc)) return restrict_nested(gf, rf, jx, jy, jz);
     int xlo, xhi, ylo, yhi, zlo = 0, zhi = 0;
     fine_range(jx, gf.nx, gc.nx, xlo, xhi);
@@ -181,7 +193,7 @@ __device__ __forceinline__ float restrict_node(const Geom& gf, const Geom& gc, c
             for (int fx = xlo; fx <= xhi; ++fx) {
                 const float wx = interp_weight(fx, jx, gf.nx, gc.nx);
                 if (wx == 0.f) continue;
-                acc += wx * wy * wz * rf[node(gf, fx, fy, fz)];
+                acc += wx * wy * wz * rf(node(gf, fx, fy, fz));
             }
         }
     }
@@ -198,25 +210,22 @@ __device__ __forceinline__ Interp1 interp1_fast(int i, int nf, int nc) {
     return interp1(i, nf, nc);
 }
 
-__device__ __forceinline__ float prolong_node(const Geom& gc, const float* xc, const Geom& gf, int ix, int iy, int iz) {
+template <typename F>
+__device__ __forceinline__ float prolong_node(const Geom& gc, F xc, const Geom& gf, int ix, int iy, int iz) {
     const Interp1 px = interp1_fast(ix, gf.nx, gc.nx), py = interp1_fast(iy, gf.ny, gc.ny);
     const int x1 = px.t > 0.f ? px.j0 + 1 : px.j0, y1 = py.t > 0.f ? py.j0 + 1 : py.j0;
     const float ax = 1.f - px.t, ay = 1.f - py.t;
-    float v = ay * (ax * xc[node(gc, px.j0, py.j0, 0)] + px.t * xc[node(gc, x1, py.j0, 0)]) +
-              py.t * (ax * xc[node(gc, px.j0, y1, 0)] + px.t * xc[node(gc, x1, y1, 0)]);
-    if (gf.dim == 3) {
-        const Interp1 pz = interp1_fast(iz, gf.nz, gc.nz);
-        const int z1 = pz.t > 0.f ? pz.j0 + 1 : pz.j0;
-        const long long offz0 = (long long)pz.j0 * gc.sx * gc.sy, offz1 = (long long)z1 * gc.sx * gc.sy;
-        const float* c0 = xc + offz0;
-        const float* c1 = xc + offz1;
-        const float v0 = ay * (ax * c0[node(gc, px.j0, py.j0, 0)] + px.t * c0[node(gc, x1, py.j0, 0)]) +
-                         py.t * (ax * c0[node(gc, px.j0, y1, 0)] + px.t * c0[node(gc, x1, y1, 0)]);
-        const float v1 = ay * (ax * c1[node(gc, px.j0, py.j0, 0)] + px.t * c1[node(gc, x1, py.j0, 0)]) +
-                         py.t * (ax * c1[node(gc, px.j0, y1, 0)] + px.t * c1[node(gc, x1, y1, 0)]);
-        v = (1.f - pz.t) * v0 + pz.t * v1;
-    }
-    return v;
+    if (gf.dim != 3)
+        return ay * (ax * xc(node(gc, px.j0, py.j0, 0)) + px.t * xc(node(gc, x1, py.j0, 0))) +
+               py.t * (ax * xc(node(gc, px.j0, y1, 0)) + px.t * xc(node(gc, x1, y1, 0)));
+    const Interp1 pz = interp1_fast(iz, gf.nz, gc.nz);
+    const int z1 = pz.t > 0.f ? pz.j0 + 1 : pz.j0;
+    const long long offz0 = (long long)pz.j0 * gc.sx * gc.sy, offz1 = (long long)z1 * gc.sx * gc.sy;
+    const float v0 = ay * (ax * xc(offz0 + node(gc, px.j0, py.j0, 0)) + px.t * xc(offz0 + node(gc, x1, py.j0, 0))) +
+                     py.t * (ax * xc(offz0 + node(gc, px.j0, y1, 0)) + px.t * xc(offz0 + node(gc, x1, y1, 0)));
+    const float v1 = ay * (ax * xc(offz1 + node(gc, px.j0, py.j0, 0)) + px.t * xc(offz1 + node(gc, x1, py.j0, 0))) +
+                     py.t * (ax * xc(offz1 + node(gc, px.j0, y1, 0)) + px.t * xc(offz1 + node(gc, x1, y1, 0)));
+    return (1.f - pz.t) * v0 + pz.t * v1;
 }
 
 struct PlaneIt {
@@ -263,7 +272,7 @@ __global__ void __launch_bounds__(kT) k_residual(Geom g, const unsigned char* __
     for (int iz = m.z0; iz < m.z1; ++iz) {
         const long long j = node(g, m.ix, m.iy, iz);
         const bool dir = mask && mask[j];  // selected at the end (see k_jacobi)
-        const float v = residual_node(g, c, x, b[j], j, m.ix, m.iy, iz);
+        const float v = residual_node(g, c, Ld<float>{x}, b[j], j, m.ix, m.iy, iz);
         r[j] = dir ? 0.f : v;
     }
 }
@@ -338,6 +347,81 @@ __global__ void __launch_bounds__(kT) k_mg3_z2(Geom g, const unsigned char* __re
         const float sx0 = x[j + o.oxm] + x[j + o.oxp], sy0 = x[j + o.oym] + x[j + o.oyp];
         update(xc, xm, xp, sx0, sy0, j, iz, b[j], mask && mask[j]);
     }
+}
+
+// The first two sweeps of a cycle, x = J(J(0)), in one pass over b: the first sweep from zero is
+// omega b / diag K at each node, formed for a node's neighbours from their b (zero on Dirichlet
+// nodes) instead of being stored and read back.  Bits as k_jacobi then k_mg3_z2.  At 129^3 the
+// two took 7.1 + 10.5 us.
+__global__ void __launch_bounds__(kT) k_mg3_first(Geom g, const unsigned char* __restrict__ mask,
+                                                  const float* __restrict__ b, float* __restrict__ out, float omega,
+                                                  int zc) {
+    const PlaneIt m = plane_it(g, zc);
+    if (!m.valid || m.z0 >= m.z1) return;
+    const MGConst c = mg_const(g);
+    const Col3 o = col3(g, m.ix, m.iy);
+    const long long sZ = o.sZ;
+    const float wcb = omega * c.cB;
+    // powers of two: a node on e grid ends has 2^e times the factor
+    auto ends = [](int i, int n) { return i == 0 || i == n ? 2.f : 1.f; };
+    const float fx = ends(m.ix, g.nx), fy = ends(m.iy, g.ny);
+    const float wc = wcb * (fx * fy);
+    const float wxm = wcb * (ends(m.ix > 0 ? m.ix - 1 : 1, g.nx) * fy), wxp = wcb * (ends(m.ix < g.nx ? m.ix + 1 : g.nx - 1, g.nx) * fy);
+    const float wym = wcb * (fx * ends(m.iy > 0 ? m.iy - 1 : 1, g.ny)), wyp = wcb * (fx * ends(m.iy < g.ny ? m.iy + 1 : g.ny - 1, g.ny));
+    const float wj = c.cB * (fx * fy);
+    auto update = [&](float bc, float bm, float bp, float b0, float b1v, float b2v, float b3v, long long jj, int iz,
+                      bool dir) {
+        const float fz = ends(iz, g.nz);
+        const float xc = wc * fz * bc;
+        float acc = __fadd_rn(wxm * fz * b0, wxp * fz * b1v);
+        acc = __fadd_rn(acc, __fadd_rn(wym * fz * b2v, wyp * fz * b3v));
+        acc = __fadd_rn(acc, __fadd_rn(wc * ends(iz > 0 ? iz - 1 : 1, g.nz) * bm, wc * ends(iz < g.nz ? iz + 1 : g.nz - 1, g.nz) * bp));
+        const float L = __fmaf_rn(6.f, xc, -acc);
+        const float v = __fmaf_rn(omega, __fmaf_rn(wj * fz, bc, -__fmul_rn(c.inv2d, L)), xc);
+        out[jj] = dir ? 0.f : v;
+    };
+    long long j = node(g, m.ix, m.iy, m.z0);
+    float bm = b[j + (m.z0 > 0 ? -sZ : sZ)];
+    float bc = b[j];
+    int iz = m.z0;
+    for (; iz + 1 < m.z1; iz += 2) {
+        const long long j1 = j + sZ;
+        const float b1 = b[j1];
+        const float b2 = b[j1 + (iz + 1 < g.nz ? sZ : -sZ)];
+        const float a0 = b[j + o.oxm], a1 = b[j + o.oxp], a2 = b[j + o.oym], a3 = b[j + o.oyp];
+        const float c0 = b[j1 + o.oxm], c1 = b[j1 + o.oxp], c2 = b[j1 + o.oym], c3 = b[j1 + o.oyp];
+        const bool d0 = mask && mask[j], d1 = mask && mask[j1];
+        update(bc, bm, b1, a0, a1, a2, a3, j, iz, d0);
+        update(b1, bc, b2, c0, c1, c2, c3, j1, iz + 1, d1);
+        bm = b1;
+        bc = b2;
+        j += 2 * sZ;
+    }
+    if (iz < m.z1) {
+        const float bp = b[j + (iz < g.nz ? sZ : -sZ)];
+        update(bc, bm, bp, b[j + o.oxm], b[j + o.oxp], b[j + o.oym], b[j + o.oyp], j, iz, mask && mask[j]);
+    }
+}
+
+__global__ void __launch_bounds__(kT) k_mg2_first(Geom g, const unsigned char* __restrict__ mask,
+                                                  const float* __restrict__ b, float* __restrict__ out, float omega) {
+    const PlaneIt m = plane_it(g, 1);
+    if (!m.valid) return;
+    const MGConst c = mg_const(g);
+    const float wcb = omega * c.cB;
+    auto ends = [](int i, int n) { return i == 0 || i == n ? 2.f : 1.f; };
+    const int xm = m.ix > 0 ? m.ix - 1 : 1, xp = m.ix < g.nx ? m.ix + 1 : g.nx - 1;
+    const int ym = m.iy > 0 ? m.iy - 1 : 1, yp = m.iy < g.ny ? m.iy + 1 : g.ny - 1;
+    const float fx = ends(m.ix, g.nx), fy = ends(m.iy, g.ny);
+    const long long j = m.ix + (long long)g.sx * m.iy, row = j - m.ix;
+    const float bc = b[j];
+    const float xc = wcb * (fx * fy) * bc;
+    float acc = __fadd_rn(wcb * (ends(xm, g.nx) * fy) * b[row + xm], wcb * (ends(xp, g.nx) * fy) * b[row + xp]);
+    acc = __fadd_rn(acc, __fadd_rn(wcb * (fx * ends(ym, g.ny)) * b[m.ix + (long long)g.sx * ym],
+                                   wcb * (fx * ends(yp, g.ny)) * b[m.ix + (long long)g.sx * yp]));
+    const float L = __fmaf_rn(4.f, xc, -acc);
+    const float v = __fmaf_rn(omega, __fmaf_rn(c.cB * (fx * fy), bc, -__fmul_rn(c.inv2d, L)), xc);
+    out[j] = mask && mask[j] ? 0.f : v;
 }
 
 // 3D prolongation x_f += P x_c along a thread's fine z-column.  Every fine plane blends the
@@ -449,7 +533,7 @@ __global__ void __launch_bounds__(kT) k_restrict(Geom gf, const float* __restric
     for (int iz = m.z0; iz < m.z1; ++iz) {
         const long long J = node(gc, m.ix, m.iy, iz);
         const bool dir = maskc && maskc[J];  // selected at the end (see k_jacobi)
-        const float v = restrict_node(gf, gc, rf, m.ix, m.iy, iz);
+        const float v = restrict_node(gf, gc, Ld<float>{rf}, m.ix, m.iy, iz);
         bc[J] = dir ? 0.f : v;
     }
 }
@@ -463,7 +547,7 @@ __global__ void __launch_bounds__(kT) k_prolong_add(Geom gc, const float* __rest
     for (int iz = m.z0; iz < m.z1; ++iz) {
         const long long i = node(gf, m.ix, m.iy, iz);
         const bool dir = maskf && maskf[i];  // tested at the store (see k_jacobi)
-        const float v = prolong_node(gc, xc, gf, m.ix, m.iy, iz);
+        const float v = prolong_node(gc, Ld<float>{xc}, gf, m.ix, m.iy, iz);
         const float x0 = xf[i];
         if (!dir) xf[i] = x0 + v;
     }
@@ -481,91 +565,405 @@ __global__ void k_coarsen_mask(Geom gf, const unsigned char* __restrict__ mf, Ge
     mc[J] = mf[node(gf, fx, fy, fz)];
 }
 
-// The coarse end of the V-cycle inside one thread block: levels 0..n-1 of BlockLevels live
-// in shared memory (x, x2, b, r per level); b of the first level comes from global memory and
-// its x goes back.  Same smoother, restriction and prolongation as the grid-wide kernels.
-__device__ void blk_jacobi(const Geom& g, const unsigned char* mask, const float* xin, float* xout, const float* b,
-                           float omega) {
-    const MGConst c = mg_const(g);
-    for (int j = threadIdx.x; j < (int)g.np; j += blockDim.x) {
-        if (mask && mask[j]) {
-            xout[j] = 0.f;
-            continue;
-        }
-        int ix, iy, iz;
-        coords(g, j, ix, iy, iz);
-        xout[j] = jacobi_node(g, c, xin, b[j], omega, j, ix, iy, iz);
-    }
-    __syncthreads();
+// The coarse end of the V-cycle in one launch of one thread-block cluster (up to 16 CTAs of 1024
+// threads): levels 0 .. n-1 of CoarseLevels live in the CTAs' shared memory; b of the first level
+// comes from global memory and its x goes back.  Same smoother (two sweeps before and two after),
+// restriction and prolongation as the grid-wide kernels, bit for bit.
+//
+// Bound: latency.  A launch per operation costs 5 to 8 us on these levels, whatever their size; a
+// cluster barrier and one round of shared-memory reads cost a fraction of that.  Levels 0 .. nc-1
+// are spread over the cluster in equal runs of the flat node index; a neighbour in another CTA's
+// run is read through distributed shared memory, all of a node's reads being issued before the
+// first is used (read one by one behind a branch, they made an operation four times as long).
+// Levels nc .. n-1, too small for that, run in CTA 0 with CTA barriers; the coarsest one's many
+// Jacobi sweeps keep one node per thread in registers, and only the warps that hold nodes meet.
+// The host works out a level's descriptor, and each operation takes it by value: indexed kernel
+// parameters and per-level divisions cost more than the arithmetic.
+//
+// Division of the flat index by a fixed number d: (i m) >> 40 with m = floor(2^40 / d) + 1,
+// exact for i d < 2^40.
+struct CoarseNode {
+    int i, ix, iy, iz, ends;
+    bool dir;
+};
+
+__device__ __forceinline__ unsigned shared_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ float lds(unsigned a) {
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void sts(unsigned a, float v) { asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory"); }
+
+// Element i of a level's array at shared address a: SPREAD, in whichever CTA it is (no branch, so
+// that the reads of a node's neighbours overlap); else in this CTA.
+template <bool SPREAD>
+__device__ __forceinline__ float at(const CoarseLevel& l, unsigned a, int i) {
+    if (!SPREAD) return lds(a + 4u * (unsigned)i);
+    const unsigned k = (unsigned)(i - l.lo);
+    const unsigned owner = (unsigned)(((unsigned)i * l.m_chunk) >> 40);
+    unsigned p;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(a + 4u * ((unsigned)i - owner * (unsigned)l.chunk)), "r"(owner));
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.lt.u32 q, %1, %2;\n\t@q ld.shared.f32 %0, [%3];\n\t"
+                 "@!q ld.shared::cluster.f32 %0, [%4];\n\t}"
+                 : "=f"(v)
+                 : "r"(k), "r"((unsigned)l.cnt), "r"(a + 4u * k), "r"(p)
+                 : "memory");
+    return v;
 }
 
-__global__ void __launch_bounds__(1024) k_block_vcycle(BlockLevels lv, const float* __restrict__ bglob,
-                                                       float* __restrict__ xglob, float omega, int nu,
-                                                       int coarse_sweeps) {
-    extern __shared__ float sm[];
-    float *x[kBlockLevelsMax], *x2[kBlockLevelsMax], *b[kBlockLevelsMax], *r[kBlockLevelsMax];
-    {
-        float* p = sm;
-        for (int l = 0; l < lv.n; ++l) {
-            const int np = (int)lv.g[l].np;
-            x[l] = p;
-            x2[l] = p + np;
-            b[l] = p + 2 * np;
-            r[l] = p + 3 * np;
-            p += 4 * np;
+// Element i of an array that CTA 0 holds whole.
+__device__ __forceinline__ float at_first(unsigned a, int i) {
+    unsigned p;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(a + 4u * (unsigned)i), "r"(0));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+__device__ __forceinline__ CoarseNode coarse_node(const CoarseLevel& l, int k, bool mask = true) {
+    CoarseNode n;
+    n.i = l.lo + k;
+    const unsigned t = (unsigned)(((unsigned)n.i * l.m_sx) >> 40);
+    n.ix = n.i - (int)t * l.sx;
+    n.iz = (int)((t * l.m_sy) >> 40);
+    n.iy = (int)t - n.iz * l.sy;
+    n.ends = (n.ix == 0 || n.ix == l.nx) + (n.iy == 0 || n.iy == l.ny);
+    if (l.dim == 3) n.ends += (n.iz == 0 || n.iz == l.nz);
+    n.dir = false;
+    if (mask && l.mask) {
+        unsigned m;
+        asm volatile("ld.shared.u8 %0, [%1];" : "=r"(m) : "r"(l.mask + (unsigned)k) : "memory");
+        n.dir = m != 0u;
+    }
+    return n;
+}
+
+// The roundings of the smoother and the interpolation, written out (a fused multiply-add, or a
+// product rounded before the sum), so that a level gives the same bits in whichever kernel and CTA
+// it runs.  fused: 2 d x - (neighbour sum) as one fused multiply-add, as in the grid-wide 3D
+// kernels; levels of up to kCoarsestMaxNodes nodes round the product first.
+__device__ __forceinline__ float relax_rn(float xc, float L, float bj, float omega, int ends, float cB, float inv2d) {
+    const float w = __fmul_rn(cB, (float)(1 << ends));
+    return __fmaf_rn(omega, __fmaf_rn(w, bj, -__fmul_rn(inv2d, L)), xc);
+}
+__device__ __forceinline__ float lap_rn(float xc, float acc, int dim, bool fused) {
+    const float d = dim == 3 ? 6.f : 4.f;
+    return fused ? __fmaf_rn(d, xc, -acc) : __fsub_rn(__fmul_rn(d, xc), acc);
+}
+__device__ __forceinline__ float blend_rn(float wa, float a, float wb, float b) {
+    return __fmaf_rn(wa, a, __fmul_rn(wb, b));
+}
+
+// The neighbour sum's six values at node n of the array at `a`; FIRST: of the first sweep's result
+// from zero, omega b / diag K, formed from the right-hand side at `a` (zero on Dirichlet nodes).
+template <bool SPREAD, bool FIRST>
+__device__ __forceinline__ float neighbour_sum(const CoarseLevel& l, unsigned a, const CoarseNode& n, float wcb) {
+    const int xm = n.ix > 0 ? n.ix - 1 : 1, xp = n.ix < l.nx ? n.ix + 1 : l.nx - 1;
+    const int ym = n.iy > 0 ? n.iy - 1 : 1, yp = n.iy < l.ny ? n.iy + 1 : l.ny - 1;
+    float v0 = at<SPREAD>(l, a, n.i + (xm - n.ix)), v1 = at<SPREAD>(l, a, n.i + (xp - n.ix));
+    float v2 = at<SPREAD>(l, a, n.i + (ym - n.iy) * l.sx), v3 = at<SPREAD>(l, a, n.i + (yp - n.iy) * l.sx);
+    float v4 = 0.f, v5 = 0.f;
+    int zm = 0, zp = 0;
+    if (l.dim == 3) {
+        zm = n.iz > 0 ? n.iz - 1 : 1, zp = n.iz < l.nz ? n.iz + 1 : l.nz - 1;
+        v4 = at<SPREAD>(l, a, n.i + (zm - n.iz) * l.sxy);
+        v5 = at<SPREAD>(l, a, n.i + (zp - n.iz) * l.sxy);
+    }
+    if (FIRST) {
+        const int ex = n.ends - (n.ix == 0 || n.ix == l.nx), ey = n.ends - (n.iy == 0 || n.iy == l.ny);
+        auto scale = [&](int e, int c, int m) { return wcb * (float)(1 << (e + (c == 0 || c == m))); };
+        v0 *= scale(ex, xm, l.nx), v1 *= scale(ex, xp, l.nx);
+        v2 *= scale(ey, ym, l.ny), v3 *= scale(ey, yp, l.ny);
+        if (l.dim == 3) {
+            const int ez = n.ends - (n.iz == 0 || n.iz == l.nz);
+            v4 *= scale(ez, zm, l.nz), v5 *= scale(ez, zp, l.nz);
         }
     }
-    for (int j = threadIdx.x; j < (int)lv.g[0].np; j += blockDim.x) b[0][j] = bglob[j];
+    float acc = __fadd_rn(v0, v1);
+    acc = __fadd_rn(acc, __fadd_rn(v2, v3));
+    if (l.dim == 3) acc = __fadd_rn(acc, __fadd_rn(v4, v5));
+    return acc;
+}
+
+// out = two sweeps from zero (FIRST) or one sweep from in.
+template <bool SPREAD, bool FIRST>
+__device__ __forceinline__ void coarse_sweep(const CoarseLevel l, unsigned in, unsigned out, float omega) {
+    const float wcb = omega * l.cB;
+    for (int k = (int)threadIdx.x; k < l.cnt; k += (int)blockDim.x) {
+        const CoarseNode n = coarse_node(l, k);
+        const float bj = lds(l.b + 4u * k);
+        const float xc = FIRST ? wcb * (float)(1 << n.ends) * bj : lds(in + 4u * k);
+        const float acc = neighbour_sum<SPREAD, FIRST>(l, FIRST ? l.b : in, n, wcb);
+        const float v = relax_rn(xc, lap_rn(xc, acc, l.dim, l.fused != 0), bj, omega, n.ends, l.cB, l.inv2d);
+        sts(out + 4u * k, n.dir ? 0.f : v);
+    }
+}
+
+template <bool SPREAD>
+__device__ __forceinline__ void coarse_residual(const CoarseLevel l) {
+    for (int k = (int)threadIdx.x; k < l.cnt; k += (int)blockDim.x) {
+        const CoarseNode n = coarse_node(l, k);
+        const float bj = lds(l.b + 4u * k), xc = lds(l.x + 4u * k);
+        const float s = 1.f / (float)(1 << n.ends);
+        const float L = lap_rn(xc, neighbour_sum<SPREAD, false>(l, l.x, n, 0.f), l.dim, l.fused != 0);
+        const float v = __fmaf_rn(-__fmul_rn(l.cK, s), L, bj);
+        sts(l.r + 4u * k, n.dir ? 0.f : v);
+    }
+}
+
+// restrict_nested with every read issued before the sum (rows and columns outside the grid are read
+// at a clamped place and left out): the same terms in the same order.
+template <int DIM, typename F>
+__device__ __forceinline__ float restrict_nested_ahead(const CoarseLevel& f, F rf, int jx, int jy, int jz) {
+    constexpr int NZ = DIM == 3 ? 3 : 1;
+    const int cx = 2 * jx, cy = 2 * jy, cz = DIM == 3 ? 2 * jz : 0;
+    const bool xm = cx > 0, xp = cx < f.nx;
+    float a[NZ][3], l[NZ][3], q[NZ][3];
+    bool ok[NZ][3];
+#pragma unroll
+    for (int z = 0; z < NZ; ++z)
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            const int fz = DIM == 3 ? cz + z - 1 : 0, fy = cy + y - 1;
+            ok[z][y] = fy >= 0 && fy <= f.ny && fz >= 0 && fz <= f.nz;
+            const int row = (ok[z][y] ? fy : cy) * f.sx + (ok[z][y] ? fz : cz) * f.sxy;
+            a[z][y] = rf(row + cx);
+            l[z][y] = rf(row + (xm ? cx - 1 : cx));
+            q[z][y] = rf(row + (xp ? cx + 1 : cx));
+        }
+    float acc = 0.f;
+#pragma unroll
+    for (int z = 0; z < NZ; ++z)
+#pragma unroll
+        for (int y = 0; y < 3; ++y) {
+            float r = a[z][y];
+            if (xm) r += 0.5f * l[z][y];
+            if (xp) r += 0.5f * q[z][y];
+            const float w = (y == 1 ? 1.f : 0.5f) * (DIM == 2 || z == 1 ? 1.f : 0.5f);
+            if (ok[z][y]) acc += w * r;
+        }
+    return acc;
+}
+
+// b of the coarse level = restriction of the fine level's residual.  TO_FIRST: CTA 0 holds the
+// coarse level; every CTA works out a share of it (CTA 0 alone would read all of the residual
+// through its one port) and stores it there.
+template <bool SPREAD, bool TO_FIRST>
+__device__ __forceinline__ void coarse_restrict(const Geom& gf, const Geom& gc, const CoarseLevel f, const CoarseLevel c) {
+    auto rf = [&](long long i) { return at<SPREAD>(f, f.r, (int)i); };
+    const int share = TO_FIRST ? (c.np + (int)gridDim.x - 1) / (int)gridDim.x : 0;
+    const int lo = TO_FIRST ? (int)blockIdx.x * share : 0, end = TO_FIRST ? min(lo + share, c.np) : c.cnt;
+    const bool two = nested(gf, gc);
+    for (int k = lo + (int)threadIdx.x; k < end; k += (int)blockDim.x) {
+        CoarseNode n = coarse_node(c, k, !TO_FIRST);
+        const float v = !two         ? restrict_node(gf, gc, rf, n.ix, n.iy, n.iz)
+                        : f.dim == 3 ? restrict_nested_ahead<3>(f, rf, n.ix, n.iy, n.iz)
+                                     : restrict_nested_ahead<2>(f, rf, n.ix, n.iy, n.iz);
+        if (TO_FIRST) {  // its Dirichlet bytes are in CTA 0 too
+            unsigned p;
+            if (c.mask) {
+                unsigned m;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(c.mask + (unsigned)k), "r"(0));
+                asm volatile("ld.shared::cluster.u8 %0, [%1];" : "=r"(m) : "r"(p) : "memory");
+                n.dir = m != 0u;
+            }
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(c.b + 4u * (unsigned)k), "r"(0));
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(p), "f"(n.dir ? 0.f : v) : "memory");
+        } else {
+            sts(c.b + 4u * k, n.dir ? 0.f : v);
+        }
+    }
+}
+
+// x of the fine level += prolongation of the coarse level's x; FIRST: CTA 0 holds that, and each CTA
+// fetches a copy first (interpolating from CTA 0, all CTAs would queue at its one port).
+template <bool SPREAD, bool FIRST>
+__device__ __forceinline__ void coarse_prolong(const Geom& gf, const Geom& gc, const CoarseLevel f, const CoarseLevel c) {
+    if (FIRST) {
+        if (blockIdx.x != 0)
+            for (int k = (int)threadIdx.x; k < c.np; k += (int)blockDim.x) sts(c.x + 4u * k, at_first(c.x, k));
+        __syncthreads();
+    }
+    auto xc = [&](int i) { return at<SPREAD && !FIRST>(c, c.x, i); };
+    for (int k = (int)threadIdx.x; k < f.cnt; k += (int)blockDim.x) {
+        const CoarseNode n = coarse_node(f, k);
+        const Interp1 px = interp1_fast(n.ix, gf.nx, gc.nx), py = interp1_fast(n.iy, gf.ny, gc.ny);
+        const int x1 = px.t > 0.f ? px.j0 + 1 : px.j0, y1 = py.t > 0.f ? py.j0 + 1 : py.j0;
+        const float ax = 1.f - px.t, ay = 1.f - py.t;
+        const int o00 = px.j0 + c.sx * py.j0, o10 = x1 + c.sx * py.j0, o01 = px.j0 + c.sx * y1, o11 = x1 + c.sx * y1;
+        Interp1 pz;
+        pz.j0 = 0;
+        pz.t = 0.f;
+        if (f.dim == 3) pz = interp1_fast(n.iz, gf.nz, gc.nz);
+        const int z0 = pz.j0 * c.sxy, z1 = pz.t > 0.f ? z0 + c.sxy : z0;
+        const float a0 = xc(z0 + o00), a1 = xc(z0 + o10), a2 = xc(z0 + o01), a3 = xc(z0 + o11);
+        float b0 = a0, b1 = a1, b2 = a2, b3 = a3;
+        if (f.dim == 3) b0 = xc(z1 + o00), b1 = xc(z1 + o10), b2 = xc(z1 + o01), b3 = xc(z1 + o11);
+        float v = blend_rn(ay, blend_rn(ax, a0, px.t, a1), py.t, blend_rn(ax, a2, px.t, a3));
+        if (f.dim == 3) {
+            const float w = blend_rn(ay, blend_rn(ax, b0, px.t, b1), py.t, blend_rn(ax, b2, px.t, b3));
+            v = blend_rn(1.f - pz.t, v, pz.t, w);
+        }
+        if (!n.dir) sts(f.x + 4u * k, lds(f.x + 4u * k) + v);
+    }
+}
+
+// The coarsest level's sweeps: one node per thread of the warps that hold nodes (up to 1024 nodes).
+__device__ __forceinline__ void coarsest_sweeps(const CoarseLevel l, float omega, int sweeps) {
+    const int threads = (l.np + 31) & ~31;
+    if ((int)threadIdx.x >= threads) return;
+    const bool here = (int)threadIdx.x < l.np;
+    const CoarseNode n = coarse_node(l, here ? (int)threadIdx.x : 0);
+    const unsigned x = l.x + 4u * (unsigned)n.i, flip = l.r - l.x;
+    const int d3 = l.dim == 3;
+    const unsigned a0 = x + 4u * (unsigned)(n.ix > 0 ? -1 : 1), a1 = x + 4u * (unsigned)(n.ix < l.nx ? 1 : -1);
+    const unsigned a2 = x + 4u * (unsigned)(n.iy > 0 ? -l.sx : l.sx), a3 = x + 4u * (unsigned)(n.iy < l.ny ? l.sx : -l.sx);
+    const unsigned a4 = x + 4u * (unsigned)(d3 ? (n.iz > 0 ? -l.sxy : l.sxy) : 0);
+    const unsigned a5 = x + 4u * (unsigned)(d3 ? (n.iz < l.nz ? l.sxy : -l.sxy) : 0);
+    const float bj = lds(l.b + 4u * (unsigned)n.i);
+    const float w = __fmul_rn(l.cB, (float)(1 << n.ends)), inv2d = l.inv2d, dd = d3 ? 6.f : 4.f;
+    float xj = n.dir ? 0.f : omega * l.cB * (float)(1 << n.ends) * bj;
+    if (here) sts(x, xj);
+    if (threads == 32) {  // one warp: the neighbours' values by shuffle
+        const unsigned all = 0xffffffffu;
+        const int n0 = (int)(a0 - l.x) >> 2, n1 = (int)(a1 - l.x) >> 2, n2 = (int)(a2 - l.x) >> 2, n3 = (int)(a3 - l.x) >> 2;
+        const int n4 = (int)(a4 - l.x) >> 2, n5 = (int)(a5 - l.x) >> 2;
+        for (int s = 1; s < sweeps; ++s) {
+            const float v0 = __shfl_sync(all, xj, n0), v1 = __shfl_sync(all, xj, n1);
+            const float v2 = __shfl_sync(all, xj, n2), v3 = __shfl_sync(all, xj, n3);
+            float acc = v0 + v1;
+            acc += v2 + v3;
+            if (d3) acc += __shfl_sync(all, xj, n4) + __shfl_sync(all, xj, n5);
+            const float L = __fsub_rn(__fmul_rn(dd, xj), acc);
+            const float v = __fmaf_rn(omega, __fmaf_rn(w, bj, -__fmul_rn(inv2d, L)), xj);
+            xj = n.dir ? 0.f : v;
+        }
+        if (here) sts(x, xj);
+        return;
+    }
+    unsigned o = 0;
+    for (int s = 1; s < sweeps; ++s) {
+        asm volatile("bar.sync 1, %0;" ::"r"(threads) : "memory");
+        float acc = lds(a0 + o) + lds(a1 + o);
+        acc += lds(a2 + o) + lds(a3 + o);
+        if (d3) acc += lds(a4 + o) + lds(a5 + o);
+        const float L = __fsub_rn(__fmul_rn(dd, xj), acc);
+        const float v = __fmaf_rn(omega, __fmaf_rn(w, bj, -__fmul_rn(inv2d, L)), xj);
+        xj = n.dir ? 0.f : v;
+        o = flip - o;
+        if (here) sts(x + o, xj);
+    }
+    if (o != 0 && here) sts(x, xj);  // the result in x
+}
+
+__global__ void __launch_bounds__(1024) k_coarse_vcycle(const __grid_constant__ CoarseLevels lv,
+                                                        const float* __restrict__ bglob, float* __restrict__ xglob,
+                                                        float omega, int coarse_sweeps) {
+    extern __shared__ __align__(16) float sm[];
+    __shared__ CoarseLevel lev[kCoarseMax];
+    const int rank = (int)blockIdx.x, tid = (int)threadIdx.x, nt = (int)blockDim.x;
+    const int nl = lv.n, nc = lv.nc;
+    if (tid < nl) {
+        CoarseLevel l = lv.level[tid];
+        const unsigned base = shared_addr(sm);
+        if (tid < nc) {
+            l.lo = min(rank * l.chunk, l.np);
+            l.cnt = min(l.chunk, l.np - l.lo);
+        }
+        l.x += base, l.r += base, l.b += base;
+        if (l.mask) l.mask += base;
+        lev[tid] = l;
+    }
     __syncthreads();
-    // descend
-    for (int l = 0; l + 1 < lv.n; ++l) {
-        const Geom& g = lv.g[l];
-        blk_jacobi(g, lv.mask[l], nullptr, x[l], b[l], omega);
-        for (int s = 1; s < nu; ++s) {
-            blk_jacobi(g, lv.mask[l], x[l], x2[l], b[l], omega);
-            float* t = x[l]; x[l] = x2[l]; x2[l] = t;
-        }
-        const MGConst c = mg_const(g);
-        for (int j = threadIdx.x; j < (int)g.np; j += blockDim.x) {
-            int ix, iy, iz;
-            coords(g, j, ix, iy, iz);
-            r[l][j] = (lv.mask[l] && lv.mask[l][j]) ? 0.f : residual_node(g, c, x[l], b[l][j], j, ix, iy, iz);
-        }
-        __syncthreads();
-        const Geom& gc = lv.g[l + 1];
-        for (int J = threadIdx.x; J < (int)gc.np; J += blockDim.x) {
-            int jx, jy, jz;
-            coords(gc, J, jx, jy, jz);
-            b[l + 1][J] = (lv.mask[l + 1] && lv.mask[l + 1][J]) ? 0.f : restrict_node(g, gc, r[l], jx, jy, jz);
-        }
-        __syncthreads();
-    }
-    // coarsest
-    {
-        const int l = lv.n - 1;
-        blk_jacobi(lv.g[l], lv.mask[l], nullptr, x[l], b[l], omega);
-        for (int s = 1; s < coarse_sweeps; ++s) {
-            blk_jacobi(lv.g[l], lv.mask[l], x[l], x2[l], b[l], omega);
-            float* t = x[l]; x[l] = x2[l]; x2[l] = t;
+    // masks, and the first level's right-hand side
+    for (int q = 0; q < nl; ++q) {
+        if (q >= nc && rank != 0) break;
+        const CoarseLevel& l = lev[q];
+        for (int k = tid; k < l.cnt; k += nt) {
+            if (l.mask) asm volatile("st.shared.u8 [%0], %1;" ::"r"(l.mask + (unsigned)k), "r"((unsigned)lv.mask[q][l.lo + k]) : "memory");
+            if (q == 0) sts(l.b + 4u * k, bglob[l.lo + k]);
         }
     }
-    // ascend
-    for (int l = lv.n - 2; l >= 0; --l) {
-        const Geom& g = lv.g[l];
-        const Geom& gc = lv.g[l + 1];
-        for (int j = threadIdx.x; j < (int)g.np; j += blockDim.x) {
-            if (lv.mask[l] && lv.mask[l][j]) continue;
-            int ix, iy, iz;
-            coords(g, j, ix, iy, iz);
-            x[l][j] += prolong_node(gc, x[l + 1], g, ix, iy, iz);
+    if (nc > 0) cluster_sync();
+    else __syncthreads();
+    // down through the spread levels
+    for (int q = 0; q < nc; ++q) {
+        const CoarseLevel& l = lev[q];
+        coarse_sweep<true, true>(l, 0u, l.x, omega);
+        cluster_sync();
+        coarse_residual<true>(l);
+        cluster_sync();
+        if (q + 1 < nc) coarse_restrict<true, false>(lv.g[q], lv.g[q + 1], l, lev[q + 1]);
+        else coarse_restrict<true, true>(lv.g[q], lv.g[q + 1], l, lev[q + 1]);
+        cluster_sync();
+    }
+    // the small levels, in CTA 0
+    if (rank == 0) {
+        for (int q = nc; q + 1 < nl; ++q) {
+            const CoarseLevel& l = lev[q];
+            coarse_sweep<false, true>(l, 0u, l.x, omega);
+            __syncthreads();
+            coarse_residual<false>(l);
+            __syncthreads();
+            coarse_restrict<false, false>(lv.g[q], lv.g[q + 1], l, lev[q + 1]);
+            __syncthreads();
         }
-        __syncthreads();
-        for (int s = 0; s < nu; ++s) {
-            blk_jacobi(g, lv.mask[l], x[l], x2[l], b[l], omega);
-            float* t = x[l]; x[l] = x2[l]; x2[l] = t;
+        {
+            const CoarseLevel& l = lev[nl - 1];
+            if (l.np <= nt) {
+                coarsest_sweeps(l, omega, coarse_sweeps);
+                __syncthreads();
+            } else {
+                coarse_sweep<false, true>(l, 0u, l.x, omega);  // two sweeps
+                __syncthreads();
+                unsigned in = l.x, out = l.r;
+                for (int s = 2; s < coarse_sweeps; ++s) {
+                    coarse_sweep<false, false>(l, in, out, omega);
+                    __syncthreads();
+                    const unsigned t = in;
+                    in = out;
+                    out = t;
+                }
+                if (in != l.x) {
+                    for (int k = tid; k < l.np; k += nt) sts(l.x + 4u * k, lds(in + 4u * k));
+                    __syncthreads();
+                }
+            }
+        }
+        for (int q = nl - 2; q >= nc; --q) {
+            const CoarseLevel& l = lev[q];
+            coarse_prolong<false, false>(lv.g[q], lv.g[q + 1], l, lev[q + 1]);
+            __syncthreads();
+            coarse_sweep<false, false>(l, l.x, l.r, omega);
+            __syncthreads();
+            coarse_sweep<false, false>(l, l.r, l.x, omega);
+            __syncthreads();
         }
     }
-    for (int j = threadIdx.x; j < (int)lv.g[0].np; j += blockDim.x) xglob[j] = x[0][j];
+    if (nc > 0) cluster_sync();
+    // up through the spread levels
+    for (int q = nc - 1; q >= 0; --q) {
+        const CoarseLevel& l = lev[q];
+        if (q + 1 < nc) coarse_prolong<true, false>(lv.g[q], lv.g[q + 1], l, lev[q + 1]);
+        else coarse_prolong<true, true>(lv.g[q], lv.g[q + 1], l, lev[q + 1]);
+        cluster_sync();
+        coarse_sweep<true, false>(l, l.x, l.r, omega);
+        cluster_sync();
+        coarse_sweep<true, false>(l, l.r, l.x, omega);
+        cluster_sync();
+    }
+    if (nc > 0 || rank == 0) {
+        const CoarseLevel& l = lev[0];
+        if (nc == 0) __syncthreads();
+        for (int k = tid; k < l.cnt; k += nt) xglob[l.lo + k] = lds(l.x + 4u * k);
+    }
 }
 
 // ---- FP64 PCG pieces ----------------------------------------------------------------------
@@ -704,19 +1102,36 @@ void launch_mg_coarsen_mask(const MGLevel& fine, const MGLevel& coarse, cudaStre
     k_coarsen_mask<<<node_blocks(coarse.g.np), kT, 0, st>>>(fine.g, fine.mask, coarse.g, coarse.mask);
 }
 
+// z-planes per thread of the 3D level kernels: eight, or fewer where eight leave less than one wave
+// of blocks (65^3: a sweep takes 4.3 us with two planes, 6.0 with eight; 129^3: 12.2 and 10.5).
+static int mg_zc(const Geom& g) {
+    if (g.dim != 3) return 1;
+    const long long bxy = ((long long)g.sx * g.sy + kT - 1) / kT;
+    int zc = 8;
+    while (zc > 2 && bxy * ((g.sz + zc - 1) / zc) < 152 * 6) zc >>= 1;
+    return zc;
+}
+
 void launch_mg_jacobi(const MGLevel& L, const float* xin, float* xout, const float* b, float omega, bool zero_init,
                       cudaStream_t st) {
     note_launch(1);
-    const int zc = L.g.dim == 3 ? 8 : 1;
+    const int zc = mg_zc(L.g);
     if (L.g.dim == 3 && !zero_init)
         k_mg3_z2<0><<<mg_grid(L.g, zc), kT, 0, st>>>(L.g, L.mask, xin, b, xout, omega, zc);
     else
         k_jacobi<<<mg_grid(L.g, zc), kT, 0, st>>>(L.g, L.mask, zero_init ? nullptr : xin, xout, b, omega, zc);
 }
 
+void launch_mg_first(const MGLevel& L, float* xout, const float* b, float omega, cudaStream_t st) {
+    note_launch(1);
+    const int zc = mg_zc(L.g);
+    if (L.g.dim == 3) k_mg3_first<<<mg_grid(L.g, zc), kT, 0, st>>>(L.g, L.mask, b, xout, omega, zc);
+    else k_mg2_first<<<mg_grid(L.g, 1), kT, 0, st>>>(L.g, L.mask, b, xout, omega);
+}
+
 void launch_mg_residual(const MGLevel& L, const float* x, const float* b, float* r, cudaStream_t st) {
     note_launch(1);
-    const int zc = L.g.dim == 3 ? 8 : 1;
+    const int zc = mg_zc(L.g);
     if (L.g.dim == 3)
         k_mg3_z2<1><<<mg_grid(L.g, zc), kT, 0, st>>>(L.g, L.mask, x, b, r, 0.f, zc);
     else
@@ -736,27 +1151,85 @@ void launch_mg_restrict(const MGLevel& fine, const float* rf, const MGLevel& coa
 
 void launch_mg_prolong_add(const MGLevel& coarse, const float* xc, const MGLevel& fine, float* xf, cudaStream_t st) {
     note_launch(1);
-    const int zc = fine.g.dim == 3 ? 8 : 1;
+    const int zc = mg_zc(fine.g);
     if (fine.g.dim == 3)
         k_prolong_add3<<<mg_grid(fine.g, zc), kT, 0, st>>>(coarse.g, xc, fine.g, fine.mask, xf, zc);
     else
         k_prolong_add<<<mg_grid(fine.g, zc), kT, 0, st>>>(coarse.g, xc, fine.g, fine.mask, xf, zc);
 }
 
-int mg_block_max_nodes() { return kBlockMaxNodes; }
-
-size_t mg_block_smem_bytes(const BlockLevels& lv) {
+// Which levels, from the first that fits, run in the cluster: spread ones of up to kSpreadMaxNodes
+// nodes (2.4 per thread: an operation on 33^3 nodes takes 3 us there, as a launch 6; on 49^3 8 us
+// against 5) while they have more than kSpreadMinNodes (below, one CTA is faster than the
+// cluster's barriers).
+size_t mg_coarse_smem(const CoarseLevels& lv) {
     size_t n = 0;
-    for (int l = 0; l < lv.n; ++l) n += 4 * (size_t)lv.g[l].np;
-    return n * sizeof(float);
+    for (int l = 0; l < lv.n; ++l) {
+        const size_t np = (size_t)lv.g[l].np;
+        n += 13 * (l < lv.nc ? (np + lv.ctas - 1) / lv.ctas : np);
+    }
+    return n + 16;
 }
 
-void launch_mg_block_vcycle(const BlockLevels& lv, const float* b, float* x, float omega, int nu, int coarse_sweeps,
-                            cudaStream_t st) {
+bool mg_coarse_plan(const MGLevel* levels, int nlev, int first, CoarseLevels* lv) {
+    *lv = CoarseLevels();
+    lv->n = nlev - first;
+    if (lv->n > kCoarseMax || levels[first].g.np > kSpreadMaxNodes || levels[nlev - 1].g.np > kCoarsestMaxNodes)
+        return false;
+    for (int i = 0; i < lv->n; ++i) {
+        lv->g[i] = levels[first + i].g;
+        lv->mask[i] = levels[first + i].mask;
+        if (lv->g[i].np > kSpreadMinNodes && i + 1 < lv->n) lv->nc = i + 1;
+    }
+    lv->ctas = lv->nc > 0 ? 16 : 1;
+    auto magic = [](long long d) { return (1ull << 40) / (unsigned long long)d + 1ull; };
+    unsigned floats = 0, bytes = 0;
+    for (int i = 0; i < lv->n; ++i) {
+        const Geom& g = lv->g[i];
+        CoarseLevel& l = lv->level[i];
+        l.np = l.cnt = (int)g.np;
+        l.lo = 0;
+        l.chunk = (int)((g.np + lv->ctas - 1) / lv->ctas);
+        l.sx = g.sx, l.sy = g.sy, l.sxy = g.sx * g.sy;
+        l.nx = g.nx, l.ny = g.ny, l.nz = g.nz, l.dim = g.dim;
+        l.m_chunk = magic(l.chunk), l.m_sx = magic(g.sx), l.m_sy = magic(g.sy);
+        const unsigned n = (unsigned)(i < lv->nc ? l.chunk : l.np);
+        l.x = 4 * floats, l.r = l.x + 4 * n, l.b = l.r + 4 * n;
+        floats += 3 * n;
+        l.fused = g.np > kCoarsestMaxNodes;
+        const float h = (float)g.h, hd = g.dim == 3 ? h * h * h : h * h;  // as mg_const
+        l.cK = hd / (h * h);
+        l.inv2d = 1.f / (float)(2 * g.dim);
+        l.cB = (h * h) / (hd * (float)(2 * g.dim));
+    }
+    for (int i = 0; i < lv->n; ++i) {
+        if (lv->mask[i]) lv->level[i].mask = 4 * floats + bytes;
+        bytes += (unsigned)(i < lv->nc ? lv->level[i].chunk : lv->level[i].np);
+    }
+    return mg_coarse_smem(*lv) <= (size_t)220 * 1024;
+}
+
+cudaError_t launch_mg_coarse(const CoarseLevels& lv, const float* b, float* x, float omega, int coarse_sweeps,
+                             cudaStream_t st) {
+    const size_t smem = mg_coarse_smem(lv);
+    cudaError_t e = cudaFuncSetAttribute(k_coarse_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess && lv.ctas > 8)
+        e = cudaFuncSetAttribute(k_coarse_vcycle, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)lv.ctas);
+    cfg.blockDim = dim3(1024);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)lv.ctas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
     note_launch(1);
-    const size_t smem = mg_block_smem_bytes(lv);
-    cudaFuncSetAttribute(k_block_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    k_block_vcycle<<<1, 1024, smem, st>>>(lv, b, x, omega, nu, coarse_sweeps);
+    return cudaLaunchKernelEx(&cfg, k_coarse_vcycle, lv, b, x, omega, coarse_sweeps);
 }
 
 void launch_applyK(const Geom& g, int order, const unsigned char* mask, const double* x, double* y,

@@ -49,8 +49,8 @@ struct cmcg_handle {
     double *pr, *pp, *pAp, *pzd;
     MGLevel lv[kMaxLevels];
     int nlev = 0;
-    int blk_level = -1;       // first level run inside one thread block (-1: none)
-    BlockLevels blk{};
+    int coarse_level = -1;    // first level of the V-cycle's coarse end in one launch (-1: none)
+    CoarseLevels coarse{};
     int riesz_guess = 0;      // PCG iterations of the previous Riesz solve
     // 2D step loops in one launch (step_band.cu); band_off: step by step instead (the engine, whose
     // per-slot kernels run side by side)

@@ -56,7 +56,6 @@ struct BandArgs {
     int rows, extra;      // bands 0 .. extra - 1 own rows + 1 grid rows, the others rows
     int nsteps;
     int face_slots;       // shared-memory slots of face factors
-    int src_form;         // FP32: which of the source's two products is the fused one
     int adj_first, adj_last;  // step 0 is the adjoint's first, step nsteps - 1 its last
     T cs[kBandSteps], sn[kBandSteps];
 };
@@ -219,11 +218,11 @@ __device__ __noinline__ double face_out(double rhs, double yq, const FaceNode<do
     if (flags & kStepPrevScaled) return (rhs - yq) * w;
     return fma(rhs, w, -(fma(2.0, w, -1.0) * yq));
 }
-// the source term as k_step (form 0) or k_step_v4 (form 1) rounds it
-__device__ __forceinline__ float source_term(float sr, float si, float cs, float sn, int form) {
-    return form ? __fmaf_rn(si, sn, __fmul_rn(sr, cs)) : __fmaf_rn(sr, cs, __fmul_rn(si, sn));
+// the source term as the step kernels round it
+__device__ __forceinline__ float source_term(float sr, float si, float cs, float sn) {
+    return __fmaf_rn(sr, cs, __fmul_rn(si, sn));
 }
-__device__ __forceinline__ double source_term(double sr, double si, double cs, double sn, int) {
+__device__ __forceinline__ double source_term(double sr, double si, double cs, double sn) {
     return fma(sr, cs, si * sn);
 }
 
@@ -277,17 +276,17 @@ __device__ __forceinline__ float rhs_of(const float* in, int P, float k) {
 // One node's update; face: its factors on an absorbing face, else null.
 template <int R, bool VOLUME>
 __device__ __forceinline__ float update(const float* in, int P, float k, float yq, const FaceNode<float>* face, bool src,
-                                        int flags, float sr, float si, float cs, float sn, int form) {
+                                        int flags, float sr, float si, float cs, float sn) {
     float rhs = rhs_of<R>(in, P, k);
-    if (VOLUME) rhs += source_term(sr, si, cs, sn, form);
+    if (VOLUME) rhs += source_term(sr, si, cs, sn);
     if (!face) return rhs - yq;
     const FaceNode<float> f = *face;
-    if (!VOLUME && src) rhs += source_term(f.sr, f.si, cs, sn, form);
+    if (!VOLUME && src) rhs += source_term(f.sr, f.si, cs, sn);
     return face_out(rhs, yq, f, flags);
 }
 template <int R, bool VOLUME>
 __device__ __forceinline__ double update(const double* in, int P, double k, double yq, const FaceNode<double>* face,
-                                         bool src, int flags, double sr, double si, double cs, double sn, int form) {
+                                         bool src, int flags, double sr, double si, double cs, double sn) {
     const double L = band_lap<R>(in, P), c = in[0];
     if (!face) {
         double out = fma(2.0, c, -yq);
@@ -295,8 +294,8 @@ __device__ __forceinline__ double update(const double* in, int P, double k, doub
         return fma(k, L, out);
     }
     double rhs = fma(k, L, 2.0 * c);
-    if (VOLUME) rhs += source_term(sr, si, cs, sn, form);
-    else if (src) rhs += source_term(face->sr, face->si, cs, sn, form);
+    if (VOLUME) rhs += source_term(sr, si, cs, sn);
+    else if (src) rhs += source_term(face->sr, face->si, cs, sn);
     return face_out(rhs, yq, *face, flags);
 }
 
@@ -407,8 +406,7 @@ __global__ void __launch_bounds__(kBandThreads<T>, 1) k_band(const __grid_consta
                     si = ssrc[2 * i + 1];
                 }
                 const FaceNode<T>* face = f >> 3 ? faces + ((f >> 3) - 1) : nullptr;
-                const T v = update<R, SRC == 2>(in + o, P, kap[q], prev[q], face, SRC == 1, flags, sr, si, cs, sn,
-                                                a.src_form);
+                const T v = update<R, SRC == 2>(in + o, P, kap[q], prev[q], face, SRC == 1, flags, sr, si, cs, sn);
                 prev[q] = c;
                 out[o] = v;
                 if (f & 7) {
@@ -518,8 +516,7 @@ struct FaceChunk {  // FaceNode<float> of four nodes; 1, 1, 1 for those that are
 
 template <int SRC>
 __device__ __forceinline__ float4 update4(const float* in, int P, float4 k4, float4 p4, bool first, int xe,
-                                          const FaceChunk* face, int flags, float4 s01, float4 s23, float cs, float sn,
-                                          int form) {
+                                          const FaceChunk* face, int flags, float4 s01, float4 s23, float cs, float sn) {
     const float4 c = *reinterpret_cast<const float4*>(in);
     const float4 m = *reinterpret_cast<const float4*>(in - P), p = *reinterpret_cast<const float4*>(in + P);
     float xl = in[-1], xr = in[4];
@@ -540,7 +537,7 @@ __device__ __forceinline__ float4 update4(const float* in, int P, float4 k4, flo
     if (SRC == 2) {
         const float sr[4] = {s01.x, s01.z, s23.x, s23.z}, si[4] = {s01.y, s01.w, s23.y, s23.w};
 #pragma unroll
-        for (int e = 0; e < 4; ++e) rhs[e] += source_term(sr[e], si[e], cs, sn, form);
+        for (int e = 0; e < 4; ++e) rhs[e] += source_term(sr[e], si[e], cs, sn);
     }
     if (!face) {
 #pragma unroll
@@ -553,7 +550,7 @@ __device__ __forceinline__ float4 update4(const float* in, int P, float4 k4, flo
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
             float h = rhs[e];
-            if (SRC == 1) h += source_term(sr[e], si[e], cs, sn, form);
+            if (SRC == 1) h += source_term(sr[e], si[e], cs, sn);
             const FaceNode<float> fn{c1[e], d[e], r[e], 0.f, 0.f};
             o[e] = face_out(h, pp[e], fn, flags);
         }
@@ -680,8 +677,7 @@ __global__ void __launch_bounds__(kBandThreads<float>, 1) k_band4(const __grid_c
                 }
                 const float4 c = *reinterpret_cast<const float4*>(in + o);
                 const float4 v = update4<SRC>(in + o, P, kap[q], prev[q], (f & 2u) != 0u, xe,
-                                              f >> 10 ? faces + ((f >> 10) - 1) : nullptr, flags, s01, s23, cs, sn,
-                                              a.src_form);
+                                              f >> 10 ? faces + ((f >> 10) - 1) : nullptr, flags, s01, s23, cs, sn);
                 prev[q] = c;
                 *reinterpret_cast<float4*>(out + o) = v;
                 if (f & 0x3c0u) {
@@ -843,10 +839,9 @@ bool band_fits(const BandPlan& p, bool volume_source) {
 template <typename T>
 cudaError_t launch_step_band(const Geom& g, int order, const BandPlan& p, T* cur, T* prev, const T* kap, const T* S,
                              bool src_faces, const double* wface, unsigned long long* words, unsigned* count,
-                             double* err, int nsteps, const double* cs, const double* sn, int src_form,
-                             bool adj_first, bool adj_last, cudaStream_t st) {
+                             double* err, int nsteps, const double* cs, const double* sn, bool adj_first,
+                             bool adj_last, cudaStream_t st) {
     BandArgs<T> a;
-    a.src_form = src_form;
     a.face_slots = p.face_slots;
     a.buf0 = cur;
     a.buf1 = prev;
@@ -881,10 +876,10 @@ cudaError_t launch_step_band(const Geom& g, int order, const BandPlan& p, T* cur
 }
 template cudaError_t launch_step_band<float>(const Geom&, int, const BandPlan&, float*, float*, const float*,
                                              const float*, bool, const double*, unsigned long long*, unsigned*,
-                                             double*, int, const double*, const double*, int, bool, bool, cudaStream_t);
+                                             double*, int, const double*, const double*, bool, bool, cudaStream_t);
 template cudaError_t launch_step_band<double>(const Geom&, int, const BandPlan&, double*, double*, const double*,
                                               const double*, bool, const double*, unsigned long long*, unsigned*,
-                                              double*, int, const double*, const double*, int, bool, bool, cudaStream_t);
+                                              double*, int, const double*, const double*, bool, bool, cudaStream_t);
 
 CMCG_CHECK_TU(band)
 

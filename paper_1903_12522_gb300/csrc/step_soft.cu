@@ -379,6 +379,187 @@ __global__ void __launch_bounds__(kST, 3)
     }
 }
 
+// ---- the Riesz PCG's FP64 vector passes ----------------------------------------------------
+// Bound: the FP64 pipe and latency.  Each pass keeps the operations it cannot do without (Ap 3, x
+// and r 3, dots 2, p 1 per node), reads two nodes per access, and sums its block's partials in one
+// warp: reduced in every warp by shuffles, five more FP64 instructions per warp would be a third of
+// the pass.
+constexpr int kPcgBlocks = 152 * 8;
+
+// grid_sum (common.cuh) with fewer FP64 instructions: the block's values meet in shared memory and
+// one warp adds them up.
+template <int NV>
+__device__ __forceinline__ bool pcg_sum(double (&v)[NV], double* partials, unsigned* ticket) {
+    __shared__ double part[NV][kST];
+    __shared__ bool last;
+    const int tid = (int)threadIdx.x;
+    const unsigned nb = gridDim.x * gridDim.y, bid = blockIdx.x + gridDim.x * blockIdx.y;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) part[k][tid] = v[k];
+    __syncthreads();
+    auto warp_total = [&](double (&t)[NV]) {  // of part, in lane 0 of the first warp
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            double x = 0.0;
+#pragma unroll
+            for (int q = 0; q < kST / 32; ++q) x += part[k][tid + 32 * q];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+            t[k] = x;
+        }
+    };
+    if (tid < 32) {
+        double t[NV];
+        warp_total(t);
+        if (tid == 0) {
+#pragma unroll
+            for (int k = 0; k < NV; ++k) partials[(size_t)k * nb + bid] = t[k];
+            __threadfence();
+            last = atomicAdd(ticket, 1u) == nb - 1;
+        }
+    }
+    __syncthreads();
+    if (!last) return false;
+    __threadfence();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) {
+        double x = 0.0;
+        for (unsigned q = tid; q < nb; q += kST) x += __ldcg(&partials[(size_t)k * nb + q]);
+        part[k][tid] = x;
+    }
+    __syncthreads();
+    if (tid < 32) {
+        warp_total(v);
+        if (tid == 0) *ticket = 0u;
+    }
+    return tid == 0;
+}
+
+// f(j, two): the nodes 2 q and 2 q + 1 (two) or the last node alone, q over the grid.
+template <typename F>
+__device__ __forceinline__ void for_pairs(long long n, F f) {
+    const long long pairs = n >> 1, stride = (long long)gridDim.x * kST;
+    const long long t = (long long)blockIdx.x * kST + threadIdx.x;
+#pragma unroll 2
+    for (long long q = t; q < pairs; q += stride) f(2 * q, true);
+    if ((n & 1) && t == 0) f(n - 1, false);
+}
+
+// Ap = K p and p . Ap; alpha = (r . z) / (p . Ap).
+template <int DIM, int ORDER>
+__global__ void __launch_bounds__(kST, 3)
+    k_pcg_applyK(const double* __restrict__ p, double* __restrict__ Ap, const unsigned char* __restrict__ mask, Red red,
+                 Geom g, double ck, int zc) {
+    const Column<DIM> m(g, zc, ORDER / 2, false);
+    double acc[1] = {0.0};
+    if (m.valid) {
+        SoftLap<DIM, ORDER, Values> lap(Values{p}, g, m.ix, m.iy);
+        int j = m.j;
+        lap.start(j, m.z0);
+        for (int iz = m.z0; iz < m.z1; ++iz) {
+            const bool dir = mask && mask[j];
+            double pj;
+            const double L = lap.next(j, iz, &pj);
+            int ends = (m.ix == 0 || m.ix == g.nx) + (m.iy == 0 || m.iy == g.ny);
+            if (DIM == 3) ends += (iz == 0 || iz == g.nz);
+            // the weight's power of two goes into the constant's exponent
+            const double c = __hiloint2double(__double2hiint(ck) - (ends << 20), __double2loint(ck));
+            const double v = dir ? 0.0 : c * L;
+            Ap[j] = v;
+            acc[0] = fma(pj, v, acc[0]);
+            j += lap.sZ;
+        }
+    }
+    if (pcg_sum<1>(acc, red.partials, red.ticket)) {
+        red.sc[SC_P_PAP] = acc[0];
+        red.sc[SC_P_ALPHA] = acc[0] != 0.0 ? red.sc[SC_P_RZ] / acc[0] : 0.0;  // p = 0 only for a zero residual
+    }
+}
+
+// XV: x is 16-byte aligned (it is the caller's; the other arrays are the workspace's).
+template <bool XV>
+__global__ void __launch_bounds__(kST, 4) k_pcg_xr(long long n, double* __restrict__ x, double* __restrict__ r,
+                                                   const double* __restrict__ p, const double* __restrict__ Ap,
+                                                   float* __restrict__ bf, Red red, int first) {
+    const double alpha = red.sc[SC_P_ALPHA];
+    double acc[1] = {0.0};
+    for_pairs(n, [&](long long j, bool two) {
+        if (two) {
+            const double2 pv = *reinterpret_cast<const double2*>(p + j), av = *reinterpret_cast<const double2*>(Ap + j);
+            double2 rv = *reinterpret_cast<const double2*>(r + j);
+            double2 xv = make_double2(0.0, 0.0);
+            if (!first) {
+                if (XV) xv = *reinterpret_cast<const double2*>(x + j);
+                else xv = make_double2(x[j], x[j + 1]);
+            }
+            xv.x = fma(alpha, pv.x, xv.x), xv.y = fma(alpha, pv.y, xv.y);
+            rv.x = fma(-alpha, av.x, rv.x), rv.y = fma(-alpha, av.y, rv.y);
+            if (XV) {
+                *reinterpret_cast<double2*>(x + j) = xv;
+            } else {
+                x[j] = xv.x;
+                x[j + 1] = xv.y;
+            }
+            *reinterpret_cast<double2*>(r + j) = rv;
+            *reinterpret_cast<float2*>(bf + j) = make_float2(soft64::to_f32(rv.x), soft64::to_f32(rv.y));
+            acc[0] = fma(rv.x, rv.x, fma(rv.y, rv.y, acc[0]));
+        } else {
+            x[j] = fma(alpha, p[j], first ? 0.0 : x[j]);
+            const double v = fma(-alpha, Ap[j], r[j]);
+            r[j] = v;
+            bf[j] = soft64::to_f32(v);
+            acc[0] = fma(v, v, acc[0]);
+        }
+    });
+    if (pcg_sum<1>(acc, red.partials, red.ticket)) red.sc[SC_P_RR] = acc[0];
+}
+
+// r . z and z . Ap; flexible (Polak-Ribiere) beta = -alpha (z . Ap) / (r . z)_old.
+__global__ void __launch_bounds__(kST, 4) k_pcg_dots(long long n, const double* __restrict__ r, const float* __restrict__ z,
+                                                     const double* __restrict__ Ap, Red red) {
+    double acc[2] = {0.0, 0.0};
+    for_pairs(n, [&](long long j, bool two) {
+        if (two) {
+            const double2 rv = *reinterpret_cast<const double2*>(r + j);
+            const float2 zv = *reinterpret_cast<const float2*>(z + j);
+            const double z0 = soft64::to_f64(zv.x), z1 = soft64::to_f64(zv.y);
+            acc[0] = fma(rv.x, z0, fma(rv.y, z1, acc[0]));
+            if (Ap) {
+                const double2 av = *reinterpret_cast<const double2*>(Ap + j);
+                acc[1] = fma(av.x, z0, fma(av.y, z1, acc[1]));
+            }
+        } else {
+            const double zz = soft64::to_f64(z[j]);
+            acc[0] = fma(r[j], zz, acc[0]);
+            if (Ap) acc[1] = fma(zz, Ap[j], acc[1]);
+        }
+    });
+    if (pcg_sum<2>(acc, red.partials, red.ticket)) {
+        const double rz_old = red.sc[SC_P_RZ];
+        red.sc[SC_P_BETA] = (!Ap || rz_old == 0.0) ? 0.0 : -red.sc[SC_P_ALPHA] * acc[1] / rz_old;
+        red.sc[SC_P_RZ] = acc[0];
+    }
+}
+
+__global__ void __launch_bounds__(kST, 4) k_pcg_p(long long n, double* __restrict__ p, const float* __restrict__ z,
+                                                  const double* __restrict__ sc, int first) {
+    const double beta = first ? 0.0 : sc[SC_P_BETA];
+    for_pairs(n, [&](long long j, bool two) {
+        if (two) {
+            const float2 zv = *reinterpret_cast<const float2*>(z + j);
+            double2 v = make_double2(soft64::to_f64(zv.x), soft64::to_f64(zv.y));
+            if (!first) {
+                const double2 o = *reinterpret_cast<const double2*>(p + j);
+                v.x = fma(beta, o.x, v.x), v.y = fma(beta, o.y, v.y);
+            }
+            *reinterpret_cast<double2*>(p + j) = v;
+        } else {
+            const double zz = soft64::to_f64(z[j]);
+            p[j] = first ? zz : fma(beta, p[j], zz);
+        }
+    });
+}
+
 // w = 1 / (1 + beta) on the nodes of absorbing faces (other entries are not read).
 __global__ void __launch_bounds__(kST) k_face_weights(Geom g, const double* __restrict__ kap, double* __restrict__ w) {
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -532,6 +713,35 @@ void launch_adj_final_soft(const Geom& g, int order, int mode, const double* s, 
         };
         mode == 0 ? go(k_adj_final_soft<D(), O(), 0>) : go(k_adj_final_soft<D(), O(), 1>);
     });
+}
+
+static unsigned pcg_blocks(long long n) {
+    return (unsigned)std::max<long long>(1, std::min<long long>((n / 2 + kST - 1) / kST, kPcgBlocks / 2));
+}
+
+void launch_pcg_applyK(const Geom& g, int order, const unsigned char* mask, const double* p, double* Ap, Red red, int zc,
+                       cudaStream_t st) {
+    by_stencil(g, order, [&](auto D, auto O) {
+        // K = W (-Lap): -Lt comes from the kernel, so the constant is negative
+        k_pcg_applyK<D(), O()><<<column_grid(g, zc), kST, 0, st>>>(p, Ap, mask, red, g, -h_pow(g), zc);
+    });
+}
+
+void launch_pcg_xr(long long n, double* x, double* r, const double* p, const double* Ap, float* bf, Red red, bool first,
+                   cudaStream_t st) {
+    note_launch(1);
+    if (((uintptr_t)x & 15u) == 0) k_pcg_xr<true><<<pcg_blocks(n), kST, 0, st>>>(n, x, r, p, Ap, bf, red, first);
+    else k_pcg_xr<false><<<pcg_blocks(n), kST, 0, st>>>(n, x, r, p, Ap, bf, red, first);
+}
+
+void launch_pcg_dots(long long n, const double* r, const float* z, const double* Ap, Red red, cudaStream_t st) {
+    note_launch(1);
+    k_pcg_dots<<<pcg_blocks(n), kST, 0, st>>>(n, r, z, Ap, red);
+}
+
+void launch_pcg_p(long long n, double* p, const float* z, Red red, bool first, cudaStream_t st) {
+    note_launch(1);
+    k_pcg_p<<<pcg_blocks(n), kST, 0, st>>>(n, p, z, red.sc, first);
 }
 
 CMCG_CHECK_TU(soft)
