@@ -119,7 +119,7 @@ def method_config(args):
 
 def tile_config(solver):
     t = list(solver.opts.tile)
-    scheme = {2: "two steps per launch", 3: "one step per launch, two z-planes per thread",
+    scheme = {0: "one step per launch, rows padded to float4s", 2: "two steps per launch", 3: "one step per launch, two z-planes per thread",
               4: "one step per launch, operands staged by TMA bulk copies into a shared-memory ring"}
     return {"tile": t, "step_scheme": scheme.get(t[3], "one step per launch")}
 
@@ -566,12 +566,15 @@ def run_ours(args):
         per_launch, bpl, upl = s32 / n32, STEP_BYTES_FP32, 1
         name, prof, src = ("k_step3d7_z2<float>: FP32 leapfrog step, 3D 7-point, two z-planes per thread",
                            "step3d7z2_fp32_sphere.json", "k_step3d7_z2(")
+    elif n32 > 0 and s.opts.tile[3] == 0:
+        per_launch, bpl, upl = s32 / n32, STEP_BYTES_FP32, 1
+        name, prof, src = "k_step_row<2>: FP32 leapfrog step, 3D 7-point, rows padded to float4s", None, None
     elif n32 > 0:
         per_launch, bpl, upl = s32 / n32, STEP_BYTES_FP32, 1
         name, prof, src = "k_step3d7<float>: FP32 leapfrog step, 3D 7-point", "step3d7_fp32_sphere.json", "k_step3d7("
     else:
         per_launch, bpl, upl = s64 / max(n64, 1), STEP_BYTES_FP64, 1
-        name, prof, src = "k_step3d7<double>: FP64 leapfrog step, 3D 7-point", None, "k_step3d7("
+        name, prof, src = "k_step_soft<3, 2>: FP64 leapfrog step, 3D 7-point, integer stencil sum", None, None
     peak, peak_src = hbm_peak()
     achieved = bpl * w.num_nodes / per_launch / 1e9
     traffic = kernel_traffic(prof, kernel_src_hash(src)) if prof else None

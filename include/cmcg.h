@@ -157,8 +157,9 @@ typedef struct {
                                at a given tol does not depend on the run-up.                  */
     int tile[4];            /* launch shape of the leapfrog kernels, 0 = default.  [3] selects
                                the step scheme of 3D 7-point steps (the others keep one step per
-                               launch): 0 = the default, scheme 3 on 3D 7-point grids and
-                               scheme 5 on 2D 5-point grids (the fastest measured); 1 = one
+                               launch): 0 = the default (the fastest measured): FP32 3D steps on
+                               rows padded to whole float4s (scheme 3 where the grid is too narrow
+                               or too large for it), scheme 5 on 2D 5-point grids; 1 = one
                                step per launch, [0] z-planes per thread
                                (16); 2 = two FP32 steps per launch (temporal blocking), [0]
                                planes staged ahead (1..3, 0 = 2), [1] z-planes per block
@@ -173,7 +174,9 @@ typedef struct {
                                asynchronous copies several planes ahead, [0] z-planes per
                                CTA, [1] rows per band, [2] planes in flight (2 or 3; 0 =
                                automatic).  Chosen per grid class by the autotuner
-                               (paper_1903_12522_gb300/autotune.py). */
+                               (paper_1903_12522_gb300/autotune.py).  2D grids that fit on chip run
+                               a period's whole step loop in one launch, whatever the scheme; FP64
+                               handles have one FP64 step kernel. */
 } cmcg_options;
 
 typedef struct {

@@ -150,6 +150,12 @@ size_t layout(cmcg_handle* H, const Geom& g, const cmcg_options& o, char* base) 
         H->wo0 = c.take<double>(np);
         H->wo1 = c.take<double>(np);
     }
+    if (o.precision != CMCG_FP64 && row_fits(g)) {
+        const size_t pp = (size_t)row_pitch(g) * g.sy * g.sz;
+        H->row_a = c.take<float>(pp);
+        H->row_b = c.take<float>(pp);
+        H->row_kap = c.take<float>(pp);
+    }
     if (band_plan(g, H->order, o.precision == CMCG_FP64 ? 8 : 4, kBandStop, &H->band)) {
         H->band_words = c.take<unsigned long long>(H->band.words);
         H->band_count = c.take<unsigned>(kBandStop + 1);
@@ -196,7 +202,9 @@ void l2_kappa_begin(cmcg_handle* H) {
         cudaGetLastError();
         return;
     }
-    const size_t bytes = sizeof(float) * (size_t)H->g.np;
+    // the copy that the step kernels read
+    const float* kap = H->row_kap && H->opt.tile[3] == 0 ? H->row_kap : H->kap32;
+    const size_t bytes = sizeof(float) * (kap == H->kap32 ? (size_t)H->g.np : (size_t)row_pitch(H->g) * H->g.sy * H->g.sz);
     if (max_persist <= 0 || bytes > (size_t)max_persist) return;
     std::lock_guard<std::mutex> lock(g_l2_mu);
     size_t cur = 0;
@@ -210,7 +218,7 @@ void l2_kappa_begin(cmcg_handle* H) {
         return;
     }
     cudaStreamAttrValue attr = {};
-    attr.accessPolicyWindow.base_ptr = (void*)H->kap32;
+    attr.accessPolicyWindow.base_ptr = (void*)kap;
     attr.accessPolicyWindow.num_bytes = bytes;
     attr.accessPolicyWindow.hitRatio = 1.0f;
     attr.accessPolicyWindow.hitProp = cudaAccessPropertyPersisting;
@@ -454,11 +462,53 @@ bool band_steps(cmcg_handle* H, PeriodBuffers& b, long long count, bool src, boo
     return true;
 }
 
+// `count` FP32 3D steps from b on padded rows: the default scheme's one-step kernels.  factors as for
+// band_steps.  Returns false, with nothing launched, where they do not apply.
+template <typename T, typename F>
+bool row_steps(cmcg_handle* H, PeriodBuffers& b, long long count, bool src, bool adjoint, F factors) {
+    if (!std::is_same<T, float>::value || !H->row_kap || H->opt.tile[3] != 0 || count < 2) return false;
+    RowStep a{};
+    a.g = H->g;
+    a.px = row_pitch(H->g);
+    a.kap = H->row_kap;
+    a.S = src ? H->S32 : nullptr;
+    a.src_faces = H->src_faces;
+    a.scol = H->scol;
+    float *cur = H->row_a, *prev = H->row_b;
+    const int tp = timing_begin(H, true, (int)std::min<long long>(count, INT32_MAX));
+    for (long long n = 0; n < count; ++n) {
+        a.flags = src ? kStepSrc : 0;
+        if (adjoint && n == 0) a.flags |= kStepPrevScaled;
+        if (adjoint && n == count - 1) a.flags |= kStepNoDiv;
+        if (src) factors(n, &a.cs, &a.sn);
+        a.reverse = (int)(n & 1);
+        if (n == 0) {
+            a.flat = 1;
+            a.cur = (const float*)b.cur;
+            a.prev = (const float*)b.prev;
+            a.out = cur;
+            a.copy = prev;
+        } else {
+            a.flat = n == count - 1 ? 2 : 0;
+            a.cur = cur;
+            a.prev = prev;
+            a.out = a.flat ? (float*)b.prev : prev;
+            a.copy = (float*)b.cur;
+            std::swap(cur, prev);
+        }
+        launch_step_row(a, H->order, H->st);
+    }
+    std::swap(b.cur, b.prev);  // the last step wrote y^{n+1} over the flat y^{n-1}, y^n over y^n
+    timing_end(H, tp);
+    return true;
+}
+
 // `count` homogeneous steps from b (in pairs where possible, else one by one).
 template <typename T>
 void plain_steps(cmcg_handle* H, PeriodBuffers& b, int count) {
     const Geom& g = H->g;
-    if (band_steps<T>(H, b, count, false, false, [](long long, double*, double*) {})) return;
+    auto none = [](long long, double*, double*) {};
+    if (band_steps<T>(H, b, count, false, false, none) || row_steps<T>(H, b, count, false, false, none)) return;
     const int zc = step_zc(H);
     const T* kap = std::is_same<T, float>::value ? (const T*)H->kap32 : (const T*)H->kap64;
     if (use_pairs<T>(H, false) && count >= 2) {
@@ -500,12 +550,12 @@ void fwd_steps(cmcg_handle* H, PeriodBuffers& b, bool src) {
         return;
     }
     const T* S = step_source<T>(H);
-    if (band_steps<T>(H, b, H->N - 1, true, false, [H](long long n, double* cs, double* sn) {
-            const double th = H->omega * (double)(n + 1) * H->dt;
-            *cs = cos(th);
-            *sn = sin(th);
-        }))
-        return;
+    auto factors = [H](long long n, double* cs, double* sn) {
+        const double th = H->omega * (double)(n + 1) * H->dt;
+        *cs = cos(th);
+        *sn = sin(th);
+    };
+    if (band_steps<T>(H, b, H->N - 1, true, false, factors) || row_steps<T>(H, b, H->N - 1, true, false, factors)) return;
     const int tp = timing_begin(H, std::is_same<T, float>::value, H->N - 1);
     for (int n = 1; n < H->N; ++n) {
         const double th = H->omega * n * H->dt;
@@ -595,7 +645,8 @@ void adj_steps(cmcg_handle* H, PeriodBuffers& b) {
         step_one<T>(H, (const T*)b.cur, (T*)b.prev, kap, nullptr, 0.0, 0.0, adj_step_flags(k, H->N), zc);
         std::swap(b.cur, b.prev);
     };
-    if (band_steps<T>(H, b, n, false, true, [](long long, double*, double*) {})) return;
+    auto none = [](long long, double*, double*) {};
+    if (band_steps<T>(H, b, n, false, true, none) || row_steps<T>(H, b, n, false, true, none)) return;
     if (use_pairs<T>(H, false)) {
         single(0);
         if (n >= 3) plain_steps<T>(H, b, n - 2);
@@ -674,14 +725,16 @@ void runup(cmcg_handle* H, int periods, double* w0, double* w1) {
     const long long total = (long long)periods * H->N;
     const double ttr = periods * H->T;
     PeriodBuffers b{cur, prev, nullptr};
-    const bool band = band_steps<T>(H, b, total - 1, true, false, [H, ttr](long long n, double* cs, double* sn) {
+    auto factors = [H, ttr](long long n, double* cs, double* sn) {
         const double t = (double)(n + 1) * H->dt, th = ramp(t, ttr);
         *cs = th * cos(H->omega * t);
         *sn = th * sin(H->omega * t);
-    });
+    };
+    const bool done = band_steps<T>(H, b, total - 1, true, false, factors) ||
+                      row_steps<T>(H, b, total - 1, true, false, factors);
     cur = (T*)b.cur;
     prev = (T*)b.prev;
-    for (long long n = 1; n < total && !band; ++n) {
+    for (long long n = 1; n < total && !done; ++n) {
         const double t = n * H->dt;
         const double th = ramp(t, ttr);
         step_one<T>(H, cur, prev, kap, step_source<T>(H), th * cos(H->omega * t), th * sin(H->omega * t), kStepSrc,
@@ -1592,6 +1645,7 @@ int cmcg_create(const cmcg_grid* grid, const double* c, double omega, const cmcg
         for (int l = 0; l < H->nlev; ++l) H->lv[l].mask = nullptr;
     launch_reciprocal(H->g.np, H->mass, H->minv, H->st);
     if (H->wface) launch_face_weights(H->g, H->kap64, H->wface, H->st);
+    if (H->row_kap) launch_row_pad(H->g, H->kap32, H->row_kap, H->st);
     if (H->mass32) {
         launch_to_float(H->g.np, H->mass, H->mass32, H->st);
         launch_to_float(H->g.np, H->minv, H->minv32, H->st);

@@ -177,6 +177,26 @@ void launch_pcg_xr(long long n, double* x, double* r, const double* p, const dou
 void launch_pcg_dots(long long n, const double* r, const float* z, const double* Ap, Red red, cudaStream_t st);
 void launch_pcg_p(long long n, double* p, const float* z, Red red, bool first, cudaStream_t st);
 
+// ---- step_row.cu ------------------------------------------------------------------------
+// FP32 3D steps on rows padded to whole float4s (pitch row_pitch).  flat: 0 cur, prev, out padded
+// (out == prev); 1 cur, prev flat, out and copy (y^n) padded; 2 cur, prev padded, out and copy
+// flat.  flags: one of 0, kStepSrc, kStepPrevScaled, kStepNoDiv.  kap is padded, S flat.
+struct RowStep {
+    Geom g;
+    int px, flat, flags;
+    const float *cur, *prev;
+    float *out, *copy;
+    const float *kap, *S;
+    double cs, sn;
+    bool src_faces;
+    int reverse;
+    const unsigned char* scol;
+};
+int row_pitch(const Geom& g);
+bool row_fits(const Geom& g);
+void launch_row_pad(const Geom& g, const float* flat, float* padded, cudaStream_t st);
+void launch_step_row(const RowStep& a, int order, cudaStream_t st);
+
 // ---- step_bulk.cu -----------------------------------------------------------------------
 // FP32 3D 7-point leapfrog step with TMA bulk-copy staging (homogeneous; flags 0, PREV_SCALED,
 // NO_DIV).  step_bulk_plan picks the band height ty and the planes per CTA zc (requests <= 0 mean

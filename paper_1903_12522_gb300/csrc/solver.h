@@ -52,6 +52,8 @@ struct cmcg_handle {
     int coarse_level = -1;    // first level of the V-cycle's coarse end in one launch (-1: none)
     CoarseLevels coarse{};
     int riesz_guess = 0;      // PCG iterations of the previous Riesz solve
+    // FP32 3D step loops on padded rows (step_row.cu): the two wave fields and kappa
+    float *row_a = nullptr, *row_b = nullptr, *row_kap = nullptr;
     // 2D step loops in one launch (step_band.cu); band_off: step by step instead (the engine, whose
     // per-slot kernels run side by side)
     BandPlan band{};
