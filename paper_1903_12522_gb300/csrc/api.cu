@@ -156,8 +156,11 @@ size_t layout(cmcg_handle* H, const Geom& g, const cmcg_options& o, char* base) 
         H->row_b = c.take<float>(pp);
         H->row_kap = c.take<float>(pp);
     }
-    if (band_plan(g, H->order, o.precision == CMCG_FP64 ? 8 : 4, kBandStop, &H->band)) {
-        H->band_words = c.take<unsigned long long>(H->band.words);
+    // at most as many bands or blocks as a GB300 has SMs (fewer SMs: a plan of fewer words, at create)
+    if (band_plan(g, H->order, o.precision == CMCG_FP64 ? 8 : 4, kBandStop, &H->band) ||
+        (o.precision != CMCG_FP64 && H->order == 2 && block_plan(g, kBandStop, &H->block))) {
+        H->exchange_words = H->band.words + H->block.words;
+        H->band_words = c.take<unsigned long long>(H->exchange_words);
         H->band_count = c.take<unsigned>(kBandStop + 1);
     }
     H->pr = c.take<double>(np);
@@ -281,9 +284,9 @@ void collect_timing(cmcg_handle* H) {
     H->ev_used = 0;
 }
 
-// The exchange words and step counts of the 2D band kernel at their start.
+// The exchange words and step counts of the one-launch loops at their start.
 void band_reset(cmcg_handle* H) {
-    cudaMemsetAsync(H->band_words, 0, sizeof(unsigned long long) * H->band.words, H->st);
+    cudaMemsetAsync(H->band_words, 0, sizeof(unsigned long long) * H->exchange_words, H->st);
     cudaMemsetAsync(H->band_count, 0, sizeof(unsigned) * (kBandStop + 1), H->st);
 }
 
@@ -429,14 +432,15 @@ void step_one(cmcg_handle* H, const T* cur, T* prev, const T* kap, const T* S, d
 }
 
 // `count` steps from b in one launch (or a few: kBandSteps steps each) where the grid fits the
-// chip: 2D grids, FP32 steps and the FP64 steps of FP64 handles.  factors(n, &cs, &sn): source
-// factors of the n-th step (n = 0, 1, ...), with src.  Returns false, with nothing launched, if
-// the loop has to run step by step.
+// chip: 2D grids (FP32 steps and the FP64 steps of FP64 handles), and FP32 3D 7-point grids in the
+// default scheme.  factors(n, &cs, &sn): source factors of the n-th step (n = 0, 1, ...), with
+// src.  Returns false, with nothing launched, if the loop has to run step by step.
 template <typename T, typename F>
 bool band_steps(cmcg_handle* H, PeriodBuffers& b, long long count, bool src, bool adjoint, F factors) {
     constexpr bool f32 = std::is_same<T, float>::value;
-    if (H->band_off || !f32 != (H->opt.precision == CMCG_FP64) || count < 1 || !band_fits(H->band, src && !H->src_faces))
-        return false;
+    if (H->band_off || !f32 != (H->opt.precision == CMCG_FP64) || count < 1) return false;
+    const bool block = f32 && H->g.dim == 3 && H->opt.tile[3] == 0 && H->block.ny_blocks > 0;
+    if (!block && !band_fits(H->band, src && !H->src_faces)) return false;
     const T* kap = f32 ? (const T*)H->kap32 : (const T*)H->kap64;
     const T* S = src ? step_source<T>(H) : nullptr;
     double cs[kBandSteps], sn[kBandSteps];
@@ -444,13 +448,18 @@ bool band_steps(cmcg_handle* H, PeriodBuffers& b, long long count, bool src, boo
     for (long long n0 = 0; n0 < count; n0 += kBandSteps) {
         const int m = (int)std::min<long long>(kBandSteps, count - n0);
         for (int s = 0; src && s < m; ++s) factors(n0 + s, &cs[s], &sn[s]);
-        const cudaError_t e = launch_step_band<T>(H->g, H->order, H->band, (T*)b.cur, (T*)b.prev, kap, S, H->src_faces,
-                                                  H->wface, H->band_words, H->band_count, H->hsc + SC_COUNT, m, cs, sn,
-                                                  adjoint && n0 == 0, adjoint && n0 + m == count, H->st);
+        const bool a0 = adjoint && n0 == 0, a1 = adjoint && n0 + m == count;
+        const cudaError_t e =
+            block ? launch_step_block(H->g, H->block, (float*)b.cur, (float*)b.prev, H->kap32, (const float*)S, H->scol,
+                                      H->src_faces, H->band_words, H->band_count, H->hsc + SC_COUNT, m, cs, sn, a0, a1,
+                                      H->st)
+                  : launch_step_band<T>(H->g, H->order, H->band, (T*)b.cur, (T*)b.prev, kap, S, H->src_faces, H->wface,
+                                        H->band_words, H->band_count, H->hsc + SC_COUNT, m, cs, sn, a0, a1, H->st);
         if (e != cudaSuccess) {
             if (n0 == 0) {  // no cooperative launch to be had (shared device limits): step by step
                 cudaGetLastError();
                 H->band.bands = 0;
+                H->block.ny_blocks = 0;
                 timing_end(H, tp);
                 return false;
             }
@@ -1586,12 +1595,16 @@ int cmcg_create(const cmcg_grid* grid, const double* c, double omega, const cmcg
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-        const size_t words = H->band.words;
-        if (!coop || !band_plan(H->g, H->order, o.precision == CMCG_FP64 ? 8 : 4, std::min(sms, kBandStop), &H->band) ||
-            H->band.words > words)
+        const int most = std::min(sms, kBandStop);
+        if (H->band.bands > 0 && !band_plan(H->g, H->order, o.precision == CMCG_FP64 ? 8 : 4, most, &H->band))
             H->band.bands = 0;
-        else
+        if (H->block.ny_blocks > 0 && !block_plan(H->g, most, &H->block)) H->block.ny_blocks = 0;
+        if (!coop || H->band.words + H->block.words > H->exchange_words) {
+            H->band.bands = 0;
+            H->block.ny_blocks = 0;
+        } else {
             band_reset(H);
+        }
     }
     H->timing = (o.flags & CMCG_FLAG_TIMING) != 0;
     H->vec32 = o.precision == CMCG_MIXED && (o.flags & CMCG_FLAG_INEXACT_RIESZ) && !(o.flags & CMCG_FLAG_FIRST_ORDER);
@@ -1741,7 +1754,7 @@ int cmcg_bulk_wait_selftest(int spin_limit, void* stream) {
 int cmcg_check_status(long long* count, long long* site, long long* index) {
     if (cudaDeviceSynchronize() != cudaSuccess) return CMCG_ERR_CUDA;
     long long total = 0, first_site = -1, first_index = 0;
-    for (auto read : {check_read_wave, check_read_riesz, check_read_pair, check_read_soft, check_read_band}) {
+    for (auto read : {check_read_wave, check_read_riesz, check_read_pair, check_read_soft, check_read_band, check_read_block}) {
         long long w[3];
         read(w);
         if (w[0] > 0 && first_site < 0) {

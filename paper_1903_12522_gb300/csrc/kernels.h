@@ -31,6 +31,7 @@ void check_read_riesz(long long* out);
 void check_read_pair(long long* out);
 void check_read_soft(long long* out);
 void check_read_band(long long* out);
+void check_read_block(long long* out);
 long long launch_count();
 
 // ---- wave.cu --------------------------------------------------------------------------
@@ -176,6 +177,20 @@ void launch_pcg_xr(long long n, double* x, double* r, const double* p, const dou
                    cudaStream_t st);  // SC_P_RR; first: x starts at zero
 void launch_pcg_dots(long long n, const double* r, const float* z, const double* Ap, Red red, cudaStream_t st);
 void launch_pcg_p(long long n, double* p, const float* z, Red red, bool first, cudaStream_t st);
+
+// ---- step_block.cu ----------------------------------------------------------------------
+// FP32 3D 7-point step loops in one cooperative launch, the grid held on chip in blocks of x rows.
+struct BlockPlan {
+    int ny_blocks = 0, nz_blocks = 0;  // blocks along y and z (0: the grid does not suit the kernel)
+    int npc = 0, side = 0;             // float4 chunks per thread; exchange words of one side
+    size_t smem = 0, words = 0;        // shared memory per block; exchange words (8 bytes each)
+};
+bool block_plan(const Geom& g, int sms, BlockPlan* p);
+// As launch_step_band; scol as in launch_step.
+cudaError_t launch_step_block(const Geom& g, const BlockPlan& p, float* cur, float* prev, const float* kap, const float* S,
+                              const unsigned char* scol, bool src_faces, unsigned long long* words, unsigned* count,
+                              double* err, int nsteps, const double* cs, const double* sn, bool adj_first, bool adj_last,
+                              cudaStream_t st);
 
 // ---- step_row.cu ------------------------------------------------------------------------
 // FP32 3D steps on rows padded to whole float4s (pitch row_pitch).  flat: 0 cur, prev, out padded

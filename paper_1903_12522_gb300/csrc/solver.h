@@ -54,10 +54,13 @@ struct cmcg_handle {
     int riesz_guess = 0;      // PCG iterations of the previous Riesz solve
     // FP32 3D step loops on padded rows (step_row.cu): the two wave fields and kappa
     float *row_a = nullptr, *row_b = nullptr, *row_kap = nullptr;
-    // 2D step loops in one launch (step_band.cu); band_off: step by step instead (the engine, whose
-    // per-slot kernels run side by side)
+    // step loops in one launch, 2D (step_band.cu) and FP32 3D 7-point (step_block.cu): exchange_words
+    // exchange words, and the steps done per band or block; band_off: step by step instead (the
+    // engine, whose per-slot kernels run side by side)
     BandPlan band{};
+    BlockPlan block{};
     unsigned long long* band_words = nullptr;
+    size_t exchange_words = 0;
     unsigned* band_count = nullptr;
     bool band_off = false;
     // first-order formulation (CMCG_FLAG_FIRST_ORDER): CG vectors on the state (p, v) of
