@@ -122,7 +122,7 @@ size_t layout(cmcg_handle* H, const Geom& g, const cmcg_options& o, char* base) 
     H->S32 = f32_copies ? c.take<float>(2 * np + 4) : nullptr;
     H->mass32 = f32_copies ? c.take<float>(np) : nullptr;
     H->minv32 = f32_copies ? c.take<float>(np) : nullptr;
-    H->scol = g.dim == 3 && !(o.flags & CMCG_FLAG_FIRST_ORDER) ? c.take<unsigned char>((size_t)g.sx * g.sy) : nullptr;
+    H->scol = g.dim == 3 ? c.take<unsigned char>((size_t)g.sx * g.sy) : nullptr;
     if (o.flags & CMCG_FLAG_FIRST_ORDER) {
         // first-order state (p, v): CG vectors and the two stepping buffers; no Riesz map
         const size_t ns = (size_t)(g.dim + 1) * np;
@@ -131,6 +131,8 @@ size_t layout(cmcg_handle* H, const Geom& g, const cmcg_options& o, char* base) 
         H->fo_a = c.take<double>(ns);
         H->fo_b = c.take<double>(ns);
         H->first_order = true;
+        // (the FP32 stepping state's padded rows fit fo_a and fo_b, which hold as many doubles)
+        if (o.precision != CMCG_FP64 && g.dim == 3) H->row_kap = c.take<float>((size_t)row_pitch(g) * g.sy * g.sz);
         H->nlev = 0;
         H->stage = (o.flags & CMCG_FLAG_HOST_IO) ? c.take<double>(2 * np) : nullptr;
         long long nb = std::max<long long>(kMaxBlocksReduce, plane_blocks(g, kZcEnds));
@@ -206,7 +208,7 @@ void l2_kappa_begin(cmcg_handle* H) {
         return;
     }
     // the copy that the step kernels read
-    const float* kap = H->row_kap && H->opt.tile[3] == 0 ? H->row_kap : H->kap32;
+    const float* kap = H->row_kap && (H->first_order || H->opt.tile[3] == 0) ? H->row_kap : H->kap32;
     const size_t bytes = sizeof(float) * (kap == H->kap32 ? (size_t)H->g.np : (size_t)row_pitch(H->g) * H->g.sy * H->g.sz);
     if (max_persist <= 0 || bytes > (size_t)max_persist) return;
     std::lock_guard<std::mutex> lock(g_l2_mu);

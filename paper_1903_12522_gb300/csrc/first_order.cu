@@ -21,6 +21,7 @@
 
 #include <algorithm>
 
+#include "soft64.cuh"
 #include "solver.h"
 
 namespace cmcg {
@@ -60,6 +61,16 @@ struct Elem {
 
 __device__ __forceinline__ Elem elem(const Geom& g, long long e) {
     Elem r;
+    if (e >> 32 == 0 && g.np >> 32 == 0) {  // (the 64-bit divisions cost more than the rest of an element)
+        const unsigned c = (unsigned)e / (unsigned)g.np, j = (unsigned)e - c * (unsigned)g.np;
+        const unsigned t = j / (unsigned)g.sx, z = t / (unsigned)g.sy;
+        r.comp = (int)c;
+        r.j = j;
+        r.ix = (int)(j - t * (unsigned)g.sx);
+        r.iz = (int)z;
+        r.iy = (int)(t - z * (unsigned)g.sy);
+        return r;
+    }
     r.comp = (int)(e / g.np);
     r.j = e - (long long)r.comp * g.np;
     const long long t = r.j / g.sx;
@@ -69,10 +80,28 @@ __device__ __forceinline__ Elem elem(const Geom& g, long long e) {
     return r;
 }
 
+// The element's place in a stepping state whose rows have pitch px.
+__device__ __forceinline__ long long place(const Geom& g, const Elem& r, int px) {
+    return r.ix + px * (r.iy + g.sy * (r.iz + (long long)g.sz * r.comp));
+}
+
 // Energy weight of element e: W_e for a link component, M for the velocity.
 __device__ __forceinline__ double e_weight(const Geom& g, const double* mass, const Elem& r) {
     return r.comp < g.dim ? link_mass(g, r.comp, r.ix, r.iy, r.iz) : mass[r.j];
 }
+
+// The face terms of k_fo_step.  The FP64 ones are out of line: inlined, the compiler makes their
+// instructions conditional, and an FP64 instruction holds the pipe even where no lane executes it.
+__device__ __forceinline__ bool is_zero(float k) { return k == 0.f; }
+__device__ __forceinline__ bool is_zero(double k) { return soft64::is_zero(k); }
+__device__ __forceinline__ float rounded_mul(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double rounded_mul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float face_beta(float k, int nb) { return __fmul_rn((float)nb, sqrtf(k)); }
+__device__ __noinline__ double face_beta(double k, int nb) { return nb * sqrt(k); }
+__device__ __forceinline__ float face_rhs(float v, float beta, float t) { return __fmaf_rn(1.f - beta, v, -t); }
+__device__ __noinline__ double face_rhs(double v, double beta, double t) { return __fma_rn(1.0 - beta, v, -t); }
+__device__ __forceinline__ float face_over(float x, float beta) { return x / (1.f + beta); }
+__device__ __noinline__ double face_over(double x, double beta) { return x / (1.0 + beta); }
 
 // One staggered leapfrog step for a column of z-planes (3D) or one node (2D).  SRC adds the
 // source at t_{n+1/2} (cs, sn already divided by dt); ACC accumulates v^n e^{i w t_n} into acc.
@@ -83,7 +112,7 @@ template <typename T, int DIM, bool SRC, bool ACC>
 __global__ void __launch_bounds__(kFT) k_fo_step(const T* __restrict__ sin_, T* __restrict__ sout,
                                                  const T* __restrict__ kap, const double* __restrict__ S, double cs,
                                                  double sn, T tau, T sig, Geom g, int zc, double* __restrict__ acc,
-                                                 double ca, double sa) {
+                                                 double ca, double sa, const unsigned char* __restrict__ scol) {
     const long long plane = (long long)g.sx * g.sy;
     const long long pidx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const bool valid = pidx < plane;
@@ -106,6 +135,7 @@ __global__ void __launch_bounds__(kFT) k_fo_step(const T* __restrict__ sin_, T* 
     T* w = sout + (long long)DIM * np;
     const T rx = (T)inv_w(ix, g.nx), ry = (T)inv_w(iy, g.ny);
     const bool hx0 = ix > 0, hx1 = ix < g.nx, hy0 = iy > 0, hy1 = iy < g.ny;
+    const bool vol = !SRC || !scol || scol[pc];  // a source in the column inside the grid
     int nbxy = 0;
     nbxy += (ix == 0) & (int)(g.abc & 1u);
     nbxy += (ix == g.nx) & (int)((g.abc >> 1) & 1u);
@@ -140,11 +170,20 @@ __global__ void __launch_bounds__(kFT) k_fo_step(const T* __restrict__ sin_, T* 
         }
         const T k = __ldcs(kap + j);  // streamed: the fields are what the next step re-reads
         T out = T(0);
-        if (k != T(0)) {
-            const T beta = (T)nb * sqrt(k);
-            T rhs = (T(1) - beta) * vc - sig * k * div;
-            if (SRC) rhs += (T)(S[2 * j] * cs + S[2 * j + 1] * sn);
-            out = nb == 0 ? rhs : rhs / (T(1) + beta);
+        if (!is_zero(k)) {
+            // (beta only on the faces: an FP64 square root for every node is most of the FP64 step)
+            T rhs = rounded_mul(sig * k, div), beta = T(0);
+            if (nb == 0) {
+                rhs = vc - rhs;
+            } else {
+                beta = face_beta(k, nb);
+                rhs = face_rhs(vc, beta, rhs);
+            }
+            if (SRC && (vol || iz == 0 || iz == g.nz)) {
+                const double2 s = reinterpret_cast<const double2*>(S)[j];
+                if (!(soft64::is_zero(s.x) && soft64::is_zero(s.y))) rhs += (T)__fma_rn(s.x, cs, __dmul_rn(s.y, sn));
+            }
+            out = nb == 0 ? rhs : face_over(rhs, beta);
         }
         if (valid) {
             if (ACC) {
@@ -164,6 +203,163 @@ __global__ void __launch_bounds__(kFT) k_fo_step(const T* __restrict__ sin_, T* 
     }
 }
 
+// The same step in FP32 on a 3D grid.  The stepping state's rows are padded to whole float4s (pitch
+// px; the padding holds zeros), and so is kappa: a thread owns four consecutive nodes of a row and
+// marches z.  Per four nodes nine 16-byte loads and four stores; the x neighbours come by shuffles.
+// scol: the columns with sources inside the grid; elsewhere S (FP64, and its sum FP64 arithmetic) is
+// read on the lowest and highest plane only.
+//
+// Bound: L2 and latency.  At 129^3 (36 B per node, 78 MB of state and kappa, which stay in L2) 41.6 us
+// a step with one node per thread, of which 11 us are the source's FP64 arithmetic on every node and
+// the rest 4-byte accesses; now 16 us backward, 19 us with a source on the faces.  Whole backward
+// periods of 46 steps, before and after: 33^3 855 and 241 us, 97^3 1071 and 454, 129^3 1445 and 758,
+// 257^3 8493 and 4761.
+//
+// The roundings are those of k_fo_step<float>, written out: same bits.
+constexpr int kFR = 128;
+
+struct F4 {
+    float e[4];
+};
+__device__ __forceinline__ F4 get4(const float* p) {
+    const float4 t = *reinterpret_cast<const float4*>(p);
+    return F4{{t.x, t.y, t.z, t.w}};
+}
+__device__ __forceinline__ void put4(float* p, const F4& v) {
+    *reinterpret_cast<float4*>(p) = make_float4(v.e[0], v.e[1], v.e[2], v.e[3]);
+}
+// p + tau (b - a): a link's update
+__device__ __forceinline__ float link(float p, float tau, float b, float a) { return __fmaf_rn(tau, b - a, p); }
+__device__ __forceinline__ F4 link4(const F4& p, float tau, const F4& b, const F4& a) {
+    F4 r;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) r.e[e] = link(p.e[e], tau, b.e[e], a.e[e]);
+    return r;
+}
+
+template <bool SRC>
+__global__ void __launch_bounds__(kFR, 8) k_fo_row(const float* __restrict__ in, float* __restrict__ out,
+                                                   const float* __restrict__ kap, const double* __restrict__ S,
+                                                   const unsigned char* __restrict__ scol, double cs, double sn,
+                                                   float tau, float sig, Geom g, int px, int zc, int reverse) {
+    const int cx = px >> 2, plane4 = cx * g.sy;
+    const int bx = reverse ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
+    const int by = reverse ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
+    const int p = bx * kFR + (int)threadIdx.x;
+    const bool valid = p < plane4;
+    const int pc = valid ? p : plane4 - 1;  // (idle lanes take part in the shuffles)
+    const int iy = (int)((unsigned)pc / (unsigned)cx), ic = pc - iy * cx, x0 = 4 * ic;
+    const int z0 = by * zc, z1 = min(z0 + zc, g.sz);
+    const int lane = (int)threadIdx.x & 31;
+    const bool first = ic == 0;
+    const int xe = g.nx - x0;  // element of the node x = nx (0 .. 3 in a row's last chunk)
+    const int m = min(4, g.sx - x0);
+    const int sZ = px * g.sy;
+    const long long field = (long long)sZ * g.sz;
+    const float *qx = in, *qy = in + field, *qz = in + 2 * field, *v = in + 3 * field;
+    float *ox = out, *oy = out + field, *oz = out + 2 * field, *ov = out + 3 * field;
+    const bool hy0 = iy > 0, hy1 = iy < g.ny;
+    const bool needl = lane == 0 && !first, needr = lane == 31 && xe >= 4;
+    const float ry = hy0 && hy1 ? 1.f : 2.f;
+    const int nby = (!hy0 ? (int)((g.abc >> 2) & 1u) : 0) + (!hy1 ? (int)((g.abc >> 3) & 1u) : 0);
+    const int nbl = first ? (int)(g.abc & 1u) : 0, nbr = xe < 4 ? (int)((g.abc >> 1) & 1u) : 0;
+    // the chunk's columns with sources: none, one (the x faces' nodes: with the FP64 sum for one node,
+    // not for each of the four, a step with a source on the faces takes 13 instead of 17 us at 129^3),
+    // several
+    int cols = 0, col = 0;
+    if (SRC) {
+        for (int e = 0; e < m; ++e) {
+            if (scol[x0 + e + g.sx * iy]) {
+                ++cols;
+                col = e;
+            }
+        }
+    }
+    int j = 4 * pc + sZ * z0;
+    F4 c = get4(v + j), zl{};  // zl: the new value of the z-link below
+    if (z0 > 0) zl = link4(get4(qz + j - sZ), tau, c, get4(v + j - sZ));
+    for (int iz = z0; iz < z1; ++iz) {
+        const bool top = iz == g.nz;
+        const F4 up = get4(v + (top ? j : j + sZ)), zo = get4(qz + j);
+        const F4 ya = get4(v + (hy0 ? j - px : j)), yb = get4(v + (hy1 ? j + px : j));
+        const F4 yo = get4(qy + j), yl = get4(qy + (hy0 ? j - px : j));
+        const F4 xo = get4(qx + j), k = get4(kap + j);
+        float el = 0.f, er = 0.f, ep = 0.f;
+        if (needl) {
+            el = v[j - 1];
+            ep = qx[j - 1];
+        }
+        if (needr) er = v[j + 4];
+        float vl = __shfl_up_sync(0xffffffffu, c.e[3], 1), vr = __shfl_down_sync(0xffffffffu, c.e[0], 1);
+        float pl = __shfl_up_sync(0xffffffffu, xo.e[3], 1);
+        if (lane == 0) {
+            vl = el;
+            pl = ep;
+        }
+        if (lane == 31) vr = er;
+        F4 zr{}, yr{}, yd{}, xr, div;
+        if (!top) zr = link4(zo, tau, up, c);
+        if (hy1) yr = link4(yo, tau, yb, c);
+        if (hy0) yd = link4(yl, tau, c, ya);
+        const float nx[4] = {c.e[1], c.e[2], c.e[3], vr};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) xr.e[e] = e < xe ? link(xo.e[e], tau, nx[e], c.e[e]) : 0.f;
+        const float xl[4] = {first ? 0.f : link(pl, tau, c.e[0], vl), xr.e[0], xr.e[1], xr.e[2]};
+        const float rz = iz > 0 && !top ? 1.f : 2.f;
+        F4 w;
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            // (the products with 1 / w, 1 or 2, are exact)
+            const float rx = (e == 0 && first) || e == xe ? 2.f : 1.f;
+            div.e[e] = __fmaf_rn(xl[e] - xr.e[e], rx, (yd.e[e] - yr.e[e]) * ry);
+            div.e[e] = __fmaf_rn(zl.e[e] - zr.e[e], rz, div.e[e]);
+            w.e[e] = __fsub_rn(c.e[e], __fmul_rn(__fmul_rn(sig, k.e[e]), div.e[e]));
+        }
+        const int nbz = (iz == 0 ? (int)((g.abc >> 4) & 1u) : 0) + (top ? (int)((g.abc >> 5) & 1u) : 0);
+        const bool face = (nby | nbl | nbr | nbz) != 0;
+        float beta[4];
+        if (face) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int nb = nby + nbz + (e == 0 ? nbl : 0) + (e == xe ? nbr : 0);
+                beta[e] = __fmul_rn((float)nb, sqrtf(k.e[e]));
+                w.e[e] = __fmaf_rn(1.f - beta[e], c.e[e], -__fmul_rn(__fmul_rn(sig, k.e[e]), div.e[e]));
+            }
+        }
+        if (SRC && (cols || iz == 0 || top)) {
+            const double2* sp = reinterpret_cast<const double2*>(S) + x0 + (long long)g.sx * (iy + (long long)g.sy * iz);
+            if (cols == 1 && iz > 0 && !top) {
+                const double2 s = sp[col];
+                const float t = (float)__fma_rn(s.x, cs, __dmul_rn(s.y, sn));
+#pragma unroll
+                for (int e = 0; e < 4; ++e) w.e[e] += e == col ? t : 0.f;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    if (e >= m) continue;
+                    const double2 s = sp[e];
+                    if (soft64::is_zero(s.x) && soft64::is_zero(s.y)) continue;
+                    w.e[e] += (float)__fma_rn(s.x, cs, __dmul_rn(s.y, sn));
+                }
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (face && beta[e] != 0.f) w.e[e] = w.e[e] / (1.f + beta[e]);
+            if (k.e[e] == 0.f) w.e[e] = 0.f;  // Dirichlet nodes (and the padding)
+        }
+        if (valid) {
+            put4(ox + j, xr);
+            put4(oy + j, yr);
+            put4(oz + j, zr);
+            put4(ov + j, w);
+        }
+        zl = zr;
+        c = up;
+        j += sZ;
+    }
+}
+
 // FP64 state -> stepping precision; MODE 0 a copy (0 on missing links and Dirichlet nodes),
 // MODE 1 the adjoint's entry variables
 // (q, u) = (p, v / (1 + beta)) (the input already E-scaled), MODE 2 the same from an unscaled
@@ -178,7 +374,8 @@ __global__ void __launch_bounds__(kFT) k_fo_load(const double* __restrict__ src,
         const Elem r = elem(g, e);
         double x = src[e];
         if (MODE == 0) {
-            const bool keep = r.comp < g.dim ? link_mass(g, r.comp, r.ix, r.iy, r.iz) > 0.0 : kap64[r.j] != 0.0;
+            const int i = r.comp == 0 ? r.ix : (r.comp == 1 ? r.iy : r.iz), n = r.comp == 0 ? g.nx : (r.comp == 1 ? g.ny : g.nz);
+            const bool keep = r.comp < g.dim ? i < n : !soft64::is_zero(kap64[r.j]);
             dst[e] = keep ? (T)x : T(0);
             continue;
         }
@@ -207,18 +404,19 @@ __global__ void __launch_bounds__(kFT) k_fo_load(const double* __restrict__ src,
 template <typename T, int MODE>
 __global__ void __launch_bounds__(kFT) k_fo_end(const T* __restrict__ sN, const double* __restrict__ s0,
                                                 double* __restrict__ out, const double* __restrict__ mass, Geom g,
-                                                Red red) {
+                                                Red red, int px) {
     const long long n = (long long)(g.dim + 1) * g.np;
     double acc[1] = {0.0};
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += stride) {
         if (MODE == 1) {
-            out[e] = (double)sN[e];
+            out[e] = (double)sN[e];  // (px == sx here)
             continue;
         }
-        const double d = (double)sN[e] - (double)(T)s0[e];  // against the copy the period started from
+        const Elem r = elem(g, e);
+        const double d = (double)sN[place(g, r, px)] - (double)(T)s0[e];  // against the copy the period started from
         out[e] = d;
-        acc[0] += e_weight(g, mass, elem(g, e)) * d * d;
+        acc[0] += e_weight(g, mass, r) * d * d;
     }
     if (MODE == 0 && grid_sum<1>(acc, red.partials, red.ticket) && threadIdx.x == 0) red.sc[SC_J] = 0.5 * acc[0];
 }
@@ -229,13 +427,13 @@ template <typename T, int MODE>
 __global__ void __launch_bounds__(kFT) k_fo_adj_end(const T* __restrict__ s, const double* __restrict__ e_in,
                                                     const double* __restrict__ d, double* __restrict__ out,
                                                     const double* __restrict__ kap64, const double* __restrict__ mass,
-                                                    Geom g, Red red) {
+                                                    Geom g, Red red, int px) {
     const long long n = (long long)(g.dim + 1) * g.np;
     double acc[1] = {0.0};
     const long long stride = (long long)gridDim.x * blockDim.x;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += stride) {
         const Elem r = elem(g, e);
-        double x = (double)s[e];
+        double x = (double)s[place(g, r, px)];
         double wgt;
         if (r.comp < g.dim) {
             wgt = link_mass(g, r.comp, r.ix, r.iy, r.iz);
@@ -253,6 +451,120 @@ __global__ void __launch_bounds__(kFT) k_fo_adj_end(const T* __restrict__ s, con
         acc[0] += wgt * gv * d[e];
     }
     if (MODE == 0 && grid_sum<1>(acc, red.partials, red.ticket) && threadIdx.x == 0) red.sc[SC_GD] = acc[0];
+}
+
+// k_fo_load, k_fo_end<1> and k_fo_adj_end<1> for the padded FP32 state: one padded node per thread
+// and turn, all four components.  Bound: HBM (129^3: 103 MB).  On the elements of the flat state, with
+// three 64-bit divisions, FP64 conversions and, in the loads, FP64 divisions each, the FP64 pipe and
+// the index arithmetic took 89 us for MODE 0 at 129^3; now 27 us.
+struct RowNode {
+    int x, iy, iz;
+    long long j;  // in a flat field
+    bool in, live[3];  // a node (not padding), its links
+};
+__device__ __forceinline__ RowNode row_node(const Geom& g, int px, unsigned i) {
+    RowNode r;
+    const unsigned t = i / (unsigned)px, z = t / (unsigned)g.sy;
+    r.x = (int)(i - t * (unsigned)px);
+    r.iy = (int)(t - z * (unsigned)g.sy);
+    r.iz = (int)z;
+    r.j = r.x + (long long)g.sx * t;
+    r.in = r.x < g.sx;
+    r.live[0] = r.x < g.nx;
+    r.live[1] = r.iy < g.ny;
+    r.live[2] = r.iz < g.nz;
+    return r;
+}
+// link_mass of an existing link: h^3 halved for each of the other axes whose end the node is at
+__device__ __forceinline__ double row_link_mass(const Geom& g, const RowNode& r, int a, double h3) {
+    const int ends[3] = {r.x == 0 || r.x == g.nx, r.iy == 0 || r.iy == g.ny, r.iz == 0 || r.iz == g.nz};
+    const int halvings = (a != 0 ? ends[0] : 0) + (a != 1 ? ends[1] : 0) + (a != 2 ? ends[2] : 0);
+    return __hiloint2double(__double2hiint(h3) - (halvings << 20), __double2loint(h3));
+}
+__device__ __noinline__ double over_one_plus(double x, double nb, double k) { return x / (1.0 + nb * sqrt(k)); }
+__device__ __noinline__ double times_one_plus(double x, double nb, double k) { return x * (1.0 + nb * sqrt(k)); }
+__device__ __noinline__ float quotient_f32(double x, double d) { return (float)(x / d); }
+
+// (float)(x / d), the division rounded to FP64 first, with r = 1 / d: x r is within two units in the
+// last place of the quotient, so unless the 29 bits that the float drops are that close to one half,
+// both round to the same float.
+__device__ __forceinline__ float div_f32(double x, double d, double r) {
+    const double q = x * r;
+    const unsigned hi = (unsigned)__double2hiint(q) & 0x7fffffffu, lo = (unsigned)__double2loint(q) & 0x1fffffffu;
+    if (hi - 0x38100000u < 0x0fc00000u && lo - 0x0ffffffcu > 8u) return soft64::to_f32(q);
+    return quotient_f32(x, d);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(kFT) k_fo_row_load(const double* __restrict__ src, float* __restrict__ dst,
+                                                     const double* __restrict__ kap64, const double* __restrict__ mass,
+                                                     Geom g, int px) {
+    const unsigned field = (unsigned)px * (unsigned)(g.sy * g.sz), stride = gridDim.x * blockDim.x;
+    const double h3 = g.h * g.h * g.h;
+    double rw[3];  // the reciprocals of h^3, h^3 / 2, h^3 / 4
+    if (MODE == 2) {
+        rw[0] = 1.0 / h3;
+        rw[1] = 2.0 * rw[0];
+        rw[2] = 4.0 * rw[0];
+    }
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < field; i += stride) {
+        const RowNode r = row_node(g, px, i);
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            float x = 0.f;
+            if (r.in && (MODE == 1 || r.live[a])) {
+                const double y = src[r.j + a * g.np];
+                if (MODE != 2) {
+                    x = soft64::to_f32(y);
+                } else {
+                    const double we = row_link_mass(g, r, a, h3);
+                    const int halvings = (__double2hiint(h3) - __double2hiint(we)) >> 20;
+                    x = div_f32(y, we, halvings == 0 ? rw[0] : (halvings == 1 ? rw[1] : rw[2]));
+                }
+            }
+            dst[i + (size_t)a * field] = x;
+        }
+        float x = 0.f;
+        if (r.in) {
+            const double k = kap64[r.j];
+            if (!soft64::is_zero(k)) {
+                double y = src[r.j + 3 * g.np];
+                if (MODE == 2) y /= mass[r.j];
+                const int nb = MODE == 0 ? 0 : num_abc(g, r.x, r.iy, r.iz);
+                if (nb) y = over_one_plus(y, nb, k);
+                x = soft64::to_f32(y);
+            }
+        }
+        dst[i + (size_t)3 * field] = x;
+    }
+}
+
+// ADJ: out = E (q, (1 + beta) u), else the state itself
+template <bool ADJ>
+__global__ void __launch_bounds__(kFT) k_fo_row_end(const float* __restrict__ s, double* __restrict__ out,
+                                                    const double* __restrict__ kap64, const double* __restrict__ mass,
+                                                    Geom g, int px) {
+    const unsigned field = (unsigned)px * (unsigned)(g.sy * g.sz), stride = gridDim.x * blockDim.x;
+    const double h3 = g.h * g.h * g.h;
+    for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < field; i += stride) {
+        const RowNode r = row_node(g, px, i);
+        if (!r.in) continue;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            double x = soft64::to_f64(s[i + (size_t)a * field]);
+            if (ADJ) x = r.live[a] ? row_link_mass(g, r, a, h3) * x : 0.0;
+            out[r.j + a * g.np] = x;
+        }
+        double x = soft64::to_f64(s[i + (size_t)3 * field]);
+        if (ADJ) {
+            const double k = kap64[r.j];
+            const int nb = num_abc(g, r.x, r.iy, r.iz);
+            if (soft64::is_zero(k)) x = 0.0;
+            else if (nb) x = times_one_plus(x, nb, k);
+            x *= mass[r.j];
+        }
+        out[r.j + 3 * g.np] = x;
+    }
 }
 
 // (4) r = d = g; gamma = gamma0 = (g, g)_E.
@@ -370,27 +682,58 @@ __global__ void k_fo_filter_final(long long np, double* __restrict__ u, double s
 
 template <typename T, int DIM>
 void step_launch(const Geom& g, const T* a, T* b, const T* kap, const double* S, double cs, double sn, double tau,
-                 double sig, int zc, double* acc, double ca, double sa, cudaStream_t st) {
+                 double sig, int zc, double* acc, double ca, double sa, const unsigned char* scol, cudaStream_t st) {
     note_launch(1);
     const dim3 grid = fo_grid(g, DIM == 3 ? zc : 1);
-    if (S && acc)
-        k_fo_step<T, DIM, true, true><<<grid, kFT, 0, st>>>(a, b, kap, S, cs, sn, (T)tau, (T)sig, g, zc, acc, ca, sa);
-    else if (S)
-        k_fo_step<T, DIM, true, false><<<grid, kFT, 0, st>>>(a, b, kap, S, cs, sn, (T)tau, (T)sig, g, zc, acc, ca, sa);
-    else
-        k_fo_step<T, DIM, false, false><<<grid, kFT, 0, st>>>(a, b, kap, S, cs, sn, (T)tau, (T)sig, g, zc, acc, ca,
-                                                               sa);
+    auto go = [&](auto kernel) {
+        kernel<<<grid, kFT, 0, st>>>(a, b, kap, S, cs, sn, (T)tau, (T)sig, g, zc, acc, ca, sa, scol);
+    };
+    if constexpr (std::is_same<T, double>::value) {
+        if (S && acc) return go(k_fo_step<T, DIM, true, true>);
+    }
+    if (S) go(k_fo_step<T, DIM, true, false>);
+    else go(k_fo_step<T, DIM, false, false>);
+}
+
+void row_launch(const Geom& g, const float* a, float* b, const float* kap, const double* S, const unsigned char* scol,
+                double cs, double sn, double tau, double sig, int reverse, cudaStream_t st) {
+    note_launch(1);
+    const int px = row_pitch(g), plane4 = (px >> 2) * g.sy;
+    const unsigned bxy = (unsigned)((plane4 + kFR - 1) / kFR);
+    // planes per thread: one while that makes one wave of blocks at most (65^3, backward period: 338
+    // us with one, 424 with four), else two (129^3: 771, 811 with one; 201^3: 2438, 2516 with four)
+    const int zc = (long long)bxy * g.sz <= 152ll * 8 ? 1 : 2;
+    const dim3 grid(bxy, (unsigned)((g.sz + zc - 1) / zc));
+    auto go = [&](auto kernel) {
+        kernel<<<grid, kFR, 0, st>>>(a, b, kap, S, scol, cs, sn, (float)tau, (float)sig, g, px, zc, reverse);
+    };
+    if (S) go(k_fo_row<true>);
+    else go(k_fo_row<false>);
 }
 
 }  // namespace
 
 namespace detail {
 
-constexpr int kZcFO = 16;
+// z-planes per thread of k_fo_step: as many (16 at most) as leave a wave of blocks; each start of a
+// column works the z-link below out again.  With 16 planes always, an FP64 backward period of 46
+// steps took 2263 us at 33^3 (487 now) and 3908 at 97^3 (2513): too few warps for FP64 latencies.
+int fo_zc(const Geom& g) {
+    const long long plane = ((long long)g.sx * g.sy + kFT - 1) / kFT;
+    int zc = 16;
+    while (zc > 1 && plane * ((g.sz + zc - 1) / zc) < 152ll * 8) zc /= 2;
+    return zc;
+}
 
 template <typename T>
 const T* fo_kap(const cmcg_handle* H) {
     return std::is_same<T, float>::value ? (const T*)H->kap32 : (const T*)H->kap64;
+}
+
+// Row pitch of the stepping state: FP32 states on 3D grids are padded.
+template <typename T>
+int fo_pitch(const Geom& g) {
+    return std::is_same<T, float>::value && g.dim == 3 ? row_pitch(g) : g.sx;
 }
 
 template <typename T>
@@ -404,10 +747,43 @@ void fo_step(cmcg_handle* H, const T* a, T* b, bool src, int n, bool backward, d
     const double tau = (backward ? -1.0 : 1.0) * H->dt / g.h;
     const double sig = (backward ? -1.0 : 1.0) * g.h / H->dt;
     const double* S = src ? H->S : nullptr;
-    if (g.dim == 3)
-        step_launch<T, 3>(g, a, b, fo_kap<T>(H), S, cs, sn, tau, sig, kZcFO, acc, ca, sa, H->st);
-    else
-        step_launch<T, 2>(g, a, b, fo_kap<T>(H), S, cs, sn, tau, sig, 1, acc, ca, sa, H->st);
+    if (g.dim == 3) {
+        if constexpr (std::is_same<T, float>::value)
+            row_launch(g, a, b, H->row_kap, S, H->scol, cs, sn, tau, sig, a == (const float*)H->fo_b, H->st);
+        else
+            step_launch<T, 3>(g, a, b, fo_kap<T>(H), S, cs, sn, tau, sig, fo_zc(g), acc, ca, sa, H->scol, H->st);
+    } else {
+        step_launch<T, 2>(g, a, b, fo_kap<T>(H), S, cs, sn, tau, sig, 1, acc, ca, sa, nullptr, H->st);
+    }
+}
+
+// FP64 state -> stepping state (MODE of k_fo_load), and back at the end of a period.
+template <typename T, int MODE>
+void fo_load(cmcg_handle* H, const double* src, T* dst) {
+    const Geom& g = H->g;
+    note_launch(1);
+    if constexpr (std::is_same<T, float>::value) {
+        if (g.dim == 3) {
+            const int px = row_pitch(g);
+            k_fo_row_load<MODE><<<fo_vec_blocks((long long)px * g.sy * g.sz), kFT, 0, H->st>>>(src, dst, H->kap64, H->mass, g, px);
+            return;
+        }
+    }
+    k_fo_load<T, MODE><<<fo_vec_blocks((long long)(g.dim + 1) * g.np), kFT, 0, H->st>>>(src, dst, H->kap64, H->mass, g);
+}
+
+template <typename T>
+void fo_state_end(cmcg_handle* H, const T* s, double* out) {
+    const Geom& g = H->g;
+    note_launch(1);
+    if constexpr (std::is_same<T, float>::value) {
+        if (g.dim == 3) {
+            const int px = row_pitch(g);
+            k_fo_row_end<false><<<fo_vec_blocks((long long)px * g.sy * g.sz), kFT, 0, H->st>>>(s, out, H->kap64, H->mass, g, px);
+            return;
+        }
+    }
+    k_fo_end<T, 1><<<fo_vec_blocks((long long)(g.dim + 1) * g.np), kFT, 0, H->st>>>(s, out, out, H->mass, g, H->red(), g.sx);
 }
 
 // Forward period from the FP64 state s0.  mode 0: out = Pi(s0) - s0 and J; mode 1: out = Pi(s0).
@@ -418,19 +794,19 @@ void fo_forward(cmcg_handle* H, const double* s0, bool src, int mode, double* ou
     const long long n = (long long)(g.dim + 1) * g.np;
     T* a = (T*)H->fo_a;
     T* b = (T*)H->fo_b;
-    note_launch(1);
-    k_fo_load<T, 0><<<fo_vec_blocks(n), kFT, 0, H->st>>>(s0, a, H->kap64, H->mass, g);
+    fo_load<T, 0>(H, s0, a);
     const int slot = timing_begin(H, std::is_same<T, float>::value, H->N);
     for (int k = 0; k < H->N; ++k) {
         fo_step<T>(H, a, b, src, k, false, acc);
         std::swap(a, b);
     }
     timing_end(H, slot);
-    note_launch(1);
-    if (mode == 0)
-        k_fo_end<T, 0><<<fo_vec_blocks(n), kFT, 0, H->st>>>(a, s0, out, H->mass, g, H->red());
-    else
-        k_fo_end<T, 1><<<fo_vec_blocks(n), kFT, 0, H->st>>>(a, s0, out, H->mass, g, H->red());
+    if (mode == 0) {
+        note_launch(1);
+        k_fo_end<T, 0><<<fo_vec_blocks(n), kFT, 0, H->st>>>(a, s0, out, H->mass, g, H->red(), fo_pitch<T>(g));
+    } else {
+        fo_state_end<T>(H, a, out);
+    }
     H->periods += 1;
 }
 
@@ -443,11 +819,10 @@ void fo_backward(cmcg_handle* H, const double* y, const double* d, int mode, dou
     const long long n = (long long)(g.dim + 1) * g.np;
     T* a = (T*)H->fo_a;
     T* b = (T*)H->fo_b;
-    note_launch(1);
     if (mode == 0)
-        k_fo_load<T, 1><<<fo_vec_blocks(n), kFT, 0, H->st>>>(y, a, H->kap64, H->mass, g);
+        fo_load<T, 1>(H, y, a);
     else
-        k_fo_load<T, 2><<<fo_vec_blocks(n), kFT, 0, H->st>>>(y, a, H->kap64, H->mass, g);
+        fo_load<T, 2>(H, y, a);
     const int slot = timing_begin(H, std::is_same<T, float>::value, H->N);
     for (int k = 0; k < H->N; ++k) {
         fo_step<T>(H, a, b, false, k, true, nullptr);
@@ -455,11 +830,19 @@ void fo_backward(cmcg_handle* H, const double* y, const double* d, int mode, dou
     }
     timing_end(H, slot);
     note_launch(1);
-    if (mode == 0)
-        k_fo_adj_end<T, 0><<<fo_vec_blocks(n), kFT, 0, H->st>>>(a, y, d, out, H->kap64, H->mass, g, H->red());
-    else
-        k_fo_adj_end<T, 1><<<fo_vec_blocks(n), kFT, 0, H->st>>>(a, y, d, out, H->kap64, H->mass, g, H->red());
     H->periods += 1;
+    if constexpr (std::is_same<T, float>::value) {
+        if (mode == 1 && g.dim == 3) {
+            const int px = row_pitch(g);
+            k_fo_row_end<true><<<fo_vec_blocks((long long)px * g.sy * g.sz), kFT, 0, H->st>>>(a, out, H->kap64, H->mass, g, px);
+            return;
+        }
+    }
+    auto go = [&](auto kernel) {
+        kernel<<<fo_vec_blocks(n), kFT, 0, H->st>>>(a, y, d, out, H->kap64, H->mass, g, H->red(), fo_pitch<T>(g));
+    };
+    if (mode == 0) go(k_fo_adj_end<T, 0>);
+    else go(k_fo_adj_end<T, 1>);
 }
 
 // Steps 5.1-5.8 of the CMCG Algorithm on the first-order state, from r = d = g already set
@@ -525,18 +908,16 @@ int fo_cg_start(cmcg_handle* H, double* x) {
 template <typename T>
 void fo_runup(cmcg_handle* H, int periods, double* out) {
     const Geom& g = H->g;
-    const long long n = (long long)(g.dim + 1) * g.np;
     T* a = (T*)H->fo_a;
     T* b = (T*)H->fo_b;
-    cudaMemsetAsync(a, 0, sizeof(T) * n, H->st);
+    cudaMemsetAsync(a, 0, sizeof(T) * (size_t)(g.dim + 1) * fo_pitch<T>(g) * g.sy * g.sz, H->st);
     const long long total = (long long)periods * H->N;
     const double ttr = total * H->dt;
     for (long long k = 0; k < total; ++k) {
         fo_step<T>(H, a, b, true, (int)(k % H->N), false, nullptr, ramp((k + 0.5) * H->dt, ttr));
         std::swap(a, b);
     }
-    note_launch(1);
-    k_fo_end<T, 1><<<fo_vec_blocks(n), kFT, 0, H->st>>>(a, out, out, H->mass, g, H->red());
+    fo_state_end<T>(H, a, out);
     H->periods += periods;
 }
 
