@@ -165,6 +165,8 @@ size_t layout(cmcg_handle* H, const Geom& g, const cmcg_options& o, char* base) 
         H->band_words = c.take<unsigned long long>(H->exchange_words);
         H->band_count = c.take<unsigned>(kBandStop + 1);
     }
+    H->side.bands = 0;
+    if (o.precision != CMCG_FP64 && H->band.bands > 0) band_plan(g, H->order, 4, 16, &H->side);
     H->pr = c.take<double>(np);
     H->pp = c.take<double>(np);
     H->pAp = c.take<double>(np);
@@ -440,9 +442,10 @@ void step_one(cmcg_handle* H, const T* cur, T* prev, const T* kap, const T* S, d
 template <typename T, typename F>
 bool band_steps(cmcg_handle* H, PeriodBuffers& b, long long count, bool src, bool adjoint, F factors) {
     constexpr bool f32 = std::is_same<T, float>::value;
-    if (H->band_off || !f32 != (H->opt.precision == CMCG_FP64) || count < 1) return false;
-    const bool block = f32 && H->g.dim == 3 && H->opt.tile[3] == 0 && H->block.ny_blocks > 0;
-    if (!block && !band_fits(H->band, src && !H->src_faces)) return false;
+    if (!f32 != (H->opt.precision == CMCG_FP64) || count < 1) return false;
+    BandPlan& band = H->side_by_side ? H->side : H->band;
+    const bool block = f32 && H->g.dim == 3 && H->opt.tile[3] == 0 && H->block.ny_blocks > 0 && !H->side_by_side;
+    if (!block && !band_fits(band, src && !H->src_faces)) return false;
     const T* kap = f32 ? (const T*)H->kap32 : (const T*)H->kap64;
     const T* S = src ? step_source<T>(H) : nullptr;
     double cs[kBandSteps], sn[kBandSteps];
@@ -455,13 +458,13 @@ bool band_steps(cmcg_handle* H, PeriodBuffers& b, long long count, bool src, boo
             block ? launch_step_block(H->g, H->block, (float*)b.cur, (float*)b.prev, H->kap32, (const float*)S, H->scol,
                                       H->src_faces, H->band_words, H->band_count, H->hsc + SC_COUNT, m, cs, sn, a0, a1,
                                       H->st)
-                  : launch_step_band<T>(H->g, H->order, H->band, (T*)b.cur, (T*)b.prev, kap, S, H->src_faces, H->wface,
+                  : launch_step_band<T>(H->g, H->order, band, (T*)b.cur, (T*)b.prev, kap, S, H->src_faces, H->wface,
                                         H->band_words, H->band_count, H->hsc + SC_COUNT, m, cs, sn, a0, a1, H->st);
         if (e != cudaSuccess) {
             if (n0 == 0) {  // no cooperative launch to be had (shared device limits): step by step
                 cudaGetLastError();
-                H->band.bands = 0;
-                H->block.ny_blocks = 0;
+                band.bands = 0;
+                if (block) H->block.ny_blocks = 0;
                 timing_end(H, tp);
                 return false;
             }
@@ -1426,6 +1429,8 @@ int solve_prepared(cmcg_handle* h, double tol, double* u, cmcg_stats* st, bool w
 
 template PeriodBuffers fwd_begin<float>(cmcg_handle*, const double*, const double*, bool, bool);
 template PeriodBuffers fwd_begin<double>(cmcg_handle*, const double*, const double*, bool, bool);
+template void fwd_steps<float>(cmcg_handle*, PeriodBuffers&, bool);
+template void adj_steps<float>(cmcg_handle*, PeriodBuffers&);
 template void fwd_end<float>(cmcg_handle*, const PeriodBuffers&, const double*, bool, int, double*, double*);
 template void fwd_end<double>(cmcg_handle*, const PeriodBuffers&, const double*, bool, int, double*, double*);
 template PeriodBuffers adj_begin<float>(cmcg_handle*, const double*, const double*, int);

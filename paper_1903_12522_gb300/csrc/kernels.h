@@ -154,7 +154,8 @@ struct BandPlan {
     size_t smem[2] = {0, 0};                      // without / with a source away from the faces
     size_t words = 0;                             // exchange words (8 bytes each)
 };
-// elem_size: 4 (FP32 steps) or 8 (FP64 steps with the integer stencil sum).
+// elem_size: 4 (FP32 steps) or 8 (FP64 steps with the integer stencil sum); sms: most bands, 16 for
+// one cluster.
 bool band_plan(const Geom& g, int order, int elem_size, int sms, BandPlan* p);
 bool band_fits(const BandPlan& p, bool volume_source);
 // nsteps <= kBandSteps steps from (cur = y^n, prev = y^{n-1}); cur and prev have swapped roles

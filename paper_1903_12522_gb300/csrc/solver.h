@@ -55,14 +55,15 @@ struct cmcg_handle {
     // FP32 3D step loops on padded rows (step_row.cu): the two wave fields and kappa
     float *row_a = nullptr, *row_b = nullptr, *row_kap = nullptr;
     // step loops in one launch, 2D (step_band.cu) and FP32 3D 7-point (step_block.cu): exchange_words
-    // exchange words, and the steps done per band or block; band_off: step by step instead (the
-    // engine, whose per-slot kernels run side by side)
-    BandPlan band{};
+    // exchange words, and the steps done per band or block; side_by_side: in the engine, whose
+    // per-slot kernels run side by side, FP32 2D loops that fit one cluster (or CTA) only, and
+    // everything else step by step
+    BandPlan band{}, side{};
     BlockPlan block{};
     unsigned long long* band_words = nullptr;
     size_t exchange_words = 0;
     unsigned* band_count = nullptr;
-    bool band_off = false;
+    bool side_by_side = false;
     // first-order formulation (CMCG_FLAG_FIRST_ORDER): CG vectors on the state (p, v) of
     // (dim + 1) N_p doubles, and the two stepping buffers (sized for double)
     double *fo_s = nullptr, *fo_r = nullptr, *fo_d = nullptr, *fo_e = nullptr, *fo_g = nullptr, *fo_x = nullptr;
@@ -129,6 +130,7 @@ const T* step_source(const cmcg_handle* H) {
     else return H->S;
 }
 int sync_read(cmcg_handle* H);
+int band_status(cmcg_handle* H);  // after a synchronisation: CMCG_ERR_DEVICE_TIMEOUT if a one-launch loop gave up
 bool inexact(const cmcg_handle* H);
 // b_ready: the finest level's right-hand side already holds float(rhat0) (written by the
 // flexible-CG update), so the conversion pass is skipped.
@@ -147,6 +149,10 @@ constexpr bool fp32_handoff(int mode) {
 // w0f_ready (FP32): the temp buffer already holds float(w0) (written by the CG direction update).
 template <typename T>
 PeriodBuffers fwd_begin(cmcg_handle* H, const double* w0, const double* w1, bool src, bool w0f_ready = false);
+template <typename T>
+void fwd_steps(cmcg_handle* H, PeriodBuffers& b, bool src);  // b: the buffers after the steps
+template <typename T>
+void adj_steps(cmcg_handle* H, PeriodBuffers& b);
 template <typename T>
 void fwd_end(cmcg_handle* H, const PeriodBuffers& b, const double* w1, bool src, int mode, double* out0,
              double* out1);

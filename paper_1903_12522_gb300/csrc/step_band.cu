@@ -670,6 +670,8 @@ __global__ void __launch_bounds__(kBandThreads<float>, 1) k_band4(const __grid_c
         unsigned long long w[4] = {0ull, 0ull, 0ull, 0ull};
 #pragma unroll
         for (int q = 0; q < NPC; ++q) {
+            // (opaque: what follows from them is worked out each step, not kept in registers)
+            asm volatile("" : "+r"(off[q]), "+r"(fl[q]));
             const unsigned f = fl[q];
             if (f & 1u) {
                 const int o = off[q], xe = (int)(f >> 2) & 15;
@@ -762,7 +764,7 @@ cudaError_t band_go(K kernel, const BandArgs<T>& a, const BandPlan& p, size_t sm
         attr[0].val.cooperative = 1;
     }
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = p.bands > 1 ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
@@ -772,7 +774,8 @@ cudaError_t band_kernel(int order, const BandArgs<T>& a, const BandPlan& p, cuda
     if constexpr (std::is_same<T, float>::value) {
         if (order == 2) {
             if (p.npt <= 1) return band_go(k_band4<1, SRC, CL>, a, p, smem, st);
-            return band_go(k_band4<2, SRC, CL>, a, p, smem, st);
+            if (p.npt <= 2) return band_go(k_band4<2, SRC, CL>, a, p, smem, st);
+            if constexpr (CL) return band_go(k_band4<3, SRC, CL>, a, p, smem, st);
         }
         if (p.npt <= 2) return band_go(k_band<float, 2, 2, SRC, CL>, a, p, smem, st);
         return band_go(k_band<float, 2, 8, SRC, CL>, a, p, smem, st);
@@ -790,6 +793,7 @@ cudaError_t band_kernel(int order, const BandArgs<T>& a, const BandPlan& p, cuda
 
 }  // namespace
 
+// With sms = 16: a plan for kernels that run side by side, one cluster each (up to 443^2 in FP32).
 // Bands: as many as there are SMs, but at least R + 1 rows each (a band holds the rows that its
 // mirror rows repeat) and enough nodes to occupy a CTA; a grid of a few nodes per thread runs in
 // one CTA, without exchange.
@@ -818,7 +822,7 @@ bool band_plan(const Geom& g, int order, int elem_size, int sms, BandPlan* p) {
     const long long rows = (g.sy + bands - 1) / bands;
     const long long per_thread = (rows * cx + bt - 1) / bt;
     const long long buf = (rows + 2 * R) * pitch;
-    if (per_thread > (vec ? 2 : 8) || buf > 65535) return false;
+    if (per_thread > (vec ? (bands <= 16 ? 3 : 2) : 8) || buf > 65535) return false;
     const long long side_words = (vec ? 4 * cx : R * g.sx) * (elem_size / 4);
     p->cluster = bands > 1 && bands <= 16 ? (int)bands : 0;
     p->face_slots = (int)(2 * rows + (bands == 1 ? 2 : 1) * cx);
