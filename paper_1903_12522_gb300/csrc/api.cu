@@ -161,7 +161,8 @@ size_t layout(cmcg_handle* H, const Geom& g, const cmcg_options& o, char* base) 
     // at most as many bands or blocks as a GB300 has SMs (fewer SMs: a plan of fewer words, at create)
     if (band_plan(g, H->order, o.precision == CMCG_FP64 ? 8 : 4, kBandStop, &H->band) ||
         (o.precision != CMCG_FP64 && H->order == 2 && block_plan(g, kBandStop, &H->block))) {
-        H->exchange_words = H->band.words + H->block.words;
+        if (o.precision != CMCG_FP64) band_plan(g, H->order, 8, kBandStop, &H->band64);
+        H->exchange_words = std::max(H->band.words + H->block.words, H->band64.words);
         H->band_words = c.take<unsigned long long>(H->exchange_words);
         H->band_count = c.take<unsigned>(kBandStop + 1);
     }
@@ -442,8 +443,9 @@ void step_one(cmcg_handle* H, const T* cur, T* prev, const T* kap, const T* S, d
 template <typename T, typename F>
 bool band_steps(cmcg_handle* H, PeriodBuffers& b, long long count, bool src, bool adjoint, F factors) {
     constexpr bool f32 = std::is_same<T, float>::value;
-    if (!f32 != (H->opt.precision == CMCG_FP64) || count < 1) return false;
-    BandPlan& band = H->side_by_side ? H->side : H->band;
+    const bool fp64 = H->opt.precision == CMCG_FP64;
+    if ((f32 ? fp64 : H->wface == nullptr) || count < 1) return false;
+    BandPlan& band = f32 && H->side_by_side ? H->side : (!f32 && !fp64 ? H->band64 : H->band);
     const bool block = f32 && H->g.dim == 3 && H->opt.tile[3] == 0 && H->block.ny_blocks > 0 && !H->side_by_side;
     if (!block && !band_fits(band, src && !H->src_faces)) return false;
     const T* kap = f32 ? (const T*)H->kap32 : (const T*)H->kap64;
@@ -1399,7 +1401,15 @@ int solve_prepared(cmcg_handle* h, double tol, double* u, cmcg_stats* st, bool w
     const long long periods_solve = h->periods;
     // J at the returned iterate (FP64 period with the sources)
     if (want_J) {
+        // (FP32 and mixed handles: the integer stencil sums too, with the face weights in a vector
+        // that is free now.  Plain FP64 arithmetic took 2.1 ms of an 8.0 ms solve at 97^3.)
+        double* const own = h->wface;
+        if (!own) {
+            h->wface = h->gt1;
+            launch_face_weights(h->g, h->kap64, h->wface, h->st);
+        }
         forward_period<double>(h, h->w0, h->w1, true, 0, h->z0, h->z1);
+        h->wface = own;
         if (sync_read(h) != CMCG_OK) return CMCG_ERR_CUDA;
         st->J_final = h->hsc[SC_J];
     }
@@ -1606,8 +1616,9 @@ int cmcg_create(const cmcg_grid* grid, const double* c, double omega, const cmcg
         if (H->band.bands > 0 && !band_plan(H->g, H->order, o.precision == CMCG_FP64 ? 8 : 4, most, &H->band))
             H->band.bands = 0;
         if (H->block.ny_blocks > 0 && !block_plan(H->g, most, &H->block)) H->block.ny_blocks = 0;
-        if (!coop || H->band.words + H->block.words > H->exchange_words) {
-            H->band.bands = 0;
+        if (H->band64.bands > 0 && !band_plan(H->g, H->order, 8, most, &H->band64)) H->band64.bands = 0;
+        if (!coop || std::max(H->band.words + H->block.words, H->band64.words) > H->exchange_words) {
+            H->band.bands = H->band64.bands = 0;
             H->block.ny_blocks = 0;
         } else {
             band_reset(H);

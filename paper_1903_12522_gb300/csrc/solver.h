@@ -58,7 +58,8 @@ struct cmcg_handle {
     // exchange words, and the steps done per band or block; side_by_side: in the engine, whose
     // per-slot kernels run side by side, FP32 2D loops that fit one cluster (or CTA) only, and
     // everything else step by step
-    BandPlan band{}, side{};
+    // (band64: FP64 loops of FP32 and mixed handles, for J at the result)
+    BandPlan band{}, side{}, band64{};
     BlockPlan block{};
     unsigned long long* band_words = nullptr;
     size_t exchange_words = 0;

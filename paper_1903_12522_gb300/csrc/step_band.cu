@@ -17,8 +17,9 @@
 //
 // Up to 16 bands run as one thread-block cluster and write the words straight into the
 // neighbour's shared memory; more bands exchange through global memory (L2) in a cooperative
-// launch.  In global memory the step numbers run on from launch to launch (each CTA keeps its
-// count; all counts are equal between launches), so no slot has to be cleared.
+// launch.  In global memory the step numbers run on from launch to launch (each CTA has a count of
+// its own; all counts are equal between launches), so no slot has to be cleared, and loops of
+// different precision, whose bands and words lie differently, can share them.
 //
 // Bound: one trip of the exchange (DSMEM or L2) and, in bands of more than a few rows, shared-memory
 // reads.  Microseconds per step (slope over the step count; in brackets step by step): FP32 129^2
@@ -54,7 +55,7 @@ struct BandArgs {
     const T* S;           // source (complex interleaved), or null
     const double* wface;  // FP64: 1 / (1 + beta)
     unsigned long long* words;
-    unsigned* count;      // per band: steps done in all launches so far; [kMaxBands]: stop word
+    unsigned* count;      // kMaxBands times: steps done in all launches so far; [kMaxBands]: stop word
     double* err;
     Geom g;
     int rows, extra;      // bands 0 .. extra - 1 own rows + 1 grid rows, the others rows
@@ -506,7 +507,8 @@ __global__ void __launch_bounds__(kBandThreads<T>, 1) k_band(const __grid_consta
             gp[j] = prev[q];
         }
     }
-    if (!CL && tid == 0) a.count[band] = base + (unsigned)a.nsteps;
+    // (the counts past the last band too: a handle's next loop may have more bands)
+    if (!CL && band + tid * nbands < kBandStop) a.count[band + tid * nbands] = base + (unsigned)a.nsteps;
 }
 
 // The FP32 2nd-order loop, four consecutive nodes of a row (one aligned float4 of shared memory)
@@ -739,7 +741,8 @@ __global__ void __launch_bounds__(kBandThreads<float>, 1) k_band4(const __grid_c
                 gp[j + e] = pv[e];
             }
     }
-    if (!CL && tid == 0) a.count[band] = base + (unsigned)a.nsteps;
+    // (the counts past the last band too: a handle's next loop may have more bands)
+    if (!CL && band + tid * nbands < kBandStop) a.count[band + tid * nbands] = base + (unsigned)a.nsteps;
 }
 
 template <typename T, typename K>
