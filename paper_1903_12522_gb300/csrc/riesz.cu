@@ -120,11 +120,15 @@ struct Interp1 {
     float t;
 };
 
+// floor(a b / d); 32-bit division (a fraction of the 64-bit one's instructions) where the product fits
+__device__ __forceinline__ int scaled(int a, int b, int d, bool small) {
+    return small ? (int)((unsigned)a * (unsigned)b / (unsigned)d) : (int)((long long)a * b / d);
+}
+
 __device__ __forceinline__ Interp1 interp1(int i, int nf, int nc) {
-    const long long num = (long long)i * nc;
     Interp1 r;
-    r.j0 = (int)(num / nf);
-    r.t = (float)(num - (long long)r.j0 * nf) / (float)nf;
+    r.j0 = scaled(i, nc, nf, nf < 46000);
+    r.t = (float)(int)((long long)i * nc - (long long)r.j0 * nf) / (float)nf;
     if (r.j0 >= nc) {
         r.j0 = nc;
         r.t = 0.f;
@@ -140,12 +144,50 @@ __device__ __forceinline__ float interp_weight(int i, int J, int nf, int nc) {
     return 0.f;
 }
 
-__device__ __forceinline__ void fine_range(int J, int nf, int nc, int& lo, int& hi) {
-    // fine nodes whose interpolation stencil can include coarse node J
-    lo = (int)(((long long)(J - 1) * nf) / nc);
-    hi = (int)(((long long)(J + 1) * nf + nc - 1) / nc);
-    lo = lo < 0 ? 0 : lo;
-    hi = hi > nf ? nf : hi;
+// The fine nodes that contribute to coarse node J along one axis, first .. first + 3 at most (those
+// with J - 1 < xi < J + 1; xi steps by n_c / n_f >= 1/2), and their weights (0: none).
+struct AxisWeights {
+    int first;
+    float w[4];
+};
+
+__device__ __forceinline__ AxisWeights axis_weights(int J, int nf, int nc) {
+    AxisWeights r;
+    r.first = J > 0 ? scaled(J - 1, nf, nc, nf < 46000) + 1 : 0;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) r.w[e] = r.first + e <= nf ? interp_weight(r.first + e, J, nf, nc) : 0.f;
+    return r;
+}
+
+// Restriction with general weights: the sum over z, y, x in this order, one fused multiply-add per
+// contributing fine node.  All of a plane's reads are issued before the sum.  (With the weights, two
+// 64-bit divisions each, worked out in the innermost loop, a coarse plane's launch took 179 us on a
+// 102x88x94 grid; now 14.)
+template <typename F>
+__device__ __forceinline__ float restrict_weighted(const Geom& gf, F rf, const AxisWeights& X, const AxisWeights& Y,
+                                                   const AxisWeights& Z) {
+    const int last = gf.nx - X.first;  // (reads without a weight stay in the row)
+    float acc = 0.f;
+#pragma unroll 1
+    for (int z = 0; z < (gf.dim == 3 ? 4 : 1); ++z) {
+        const float wz = Z.w[0] * (z == 0 ? 1.f : 0.f) + Z.w[1] * (z == 1 ? 1.f : 0.f) + Z.w[2] * (z == 2 ? 1.f : 0.f) +
+                         Z.w[3] * (z == 3 ? 1.f : 0.f);  // Z.w[z]
+        if (wz == 0.f) continue;
+        float r[4][4];
+#pragma unroll
+        for (int y = 0; y < 4; ++y) {
+            const long long row = node(gf, X.first, Y.w[y] != 0.f ? Y.first + y : Y.first, Z.first + z);
+#pragma unroll
+            for (int x = 0; x < 4; ++x) r[y][x] = rf(row + min(x, last));
+        }
+#pragma unroll
+        for (int y = 0; y < 4; ++y)
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+                if (Y.w[y] != 0.f && X.w[x] != 0.f)
+                    acc = __fmaf_rn(__fmul_rn(__fmul_rn(X.w[x], Y.w[y]), wz), r[y][x], acc);
+    }
+    return acc;
 }
 
 __device__ __forceinline__ bool nested(const Geom& gf, const Geom& gc) {
@@ -176,28 +218,9 @@ __device__ __forceinline__ float restrict_nested(const Geom& gf, F rf, int jx, i
     return acc;
 }
 
-template <typename F>
-__device__ __forceinline__ float restrict_node(const Geom& gf, const Geom& gc, F rf, int jx, int jy, int jz) {
-    if (nested(gf, gc)) return restrict_nested(gf, rf, jx, jy, jz);
-    int xlo, xhi, ylo, yhi, zlo = 0, zhi = 0;
-    fine_range(jx, gf.nx, gc.nx, xlo, xhi);
-    fine_range(jy, gf.ny, gc.ny, ylo, yhi);
-    if (gf.dim == 3) fine_range(jz, gf.nz, gc.nz, zlo, zhi);
-    float acc = 0.f;
-    for (int fz = zlo; fz <= zhi; ++fz) {
-        const float wz = gf.dim == 3 ? interp_weight(fz, jz, gf.nz, gc.nz) : 1.f;
-        if (wz == 0.f) continue;
-        for (int fy = ylo; fy <= yhi; ++fy) {
-            const float wy = interp_weight(fy, jy, gf.ny, gc.ny);
-            if (wy == 0.f) continue;
-            for (int fx = xlo; fx <= xhi; ++fx) {
-                const float wx = interp_weight(fx, jx, gf.nx, gc.nx);
-                if (wx == 0.f) continue;
-                acc += wx * wy * wz * rf(node(gf, fx, fy, fz));
-            }
-        }
-    }
-    return acc;
+__device__ __forceinline__ AxisWeights axis_weights_z(const Geom& gf, const Geom& gc, int jz) {
+    if (gf.dim == 3) return axis_weights(jz, gf.nz, gc.nz);
+    return AxisWeights{0, {1.f, 0.f, 0.f, 0.f}};
 }
 
 __device__ __forceinline__ Interp1 interp1_fast(int i, int nf, int nc) {
@@ -524,16 +547,23 @@ __global__ void __launch_bounds__(kT) k_restrict3_nested(Geom gf, const float* _
     }
 }
 
-// b_c[J] = sum over fine nodes i with |i - 2J|_inf <= 1 of prod_a (1 or 1/2) r_f[i].
+// b_c[J] = sum over fine nodes i of the interpolation weights times r_f[i].
 __global__ void __launch_bounds__(kT) k_restrict(Geom gf, const float* __restrict__ rf, Geom gc,
                                                  const unsigned char* __restrict__ maskc, float* __restrict__ bc,
                                                  int zc) {
     const PlaneIt m = plane_it(gc, zc);
     if (!m.valid) return;
+    const bool two = nested(gf, gc);
+    AxisWeights X{}, Y{};
+    if (!two) {
+        X = axis_weights(m.ix, gf.nx, gc.nx);
+        Y = axis_weights(m.iy, gf.ny, gc.ny);
+    }
     for (int iz = m.z0; iz < m.z1; ++iz) {
         const long long J = node(gc, m.ix, m.iy, iz);
         const bool dir = maskc && maskc[J];  // selected at the end (see k_jacobi)
-        const float v = restrict_node(gf, gc, Ld<float>{rf}, m.ix, m.iy, iz);
+        const float v = two ? restrict_nested(gf, Ld<float>{rf}, m.ix, m.iy, iz)
+                            : restrict_weighted(gf, Ld<float>{rf}, X, Y, axis_weights_z(gf, gc, iz));
         bc[J] = dir ? 0.f : v;
     }
 }
@@ -572,20 +602,26 @@ __global__ void k_coarsen_mask(Geom gf, const unsigned char* __restrict__ mf, Ge
 //
 // Bound: latency.  A launch per operation costs 5 to 8 us on these levels, whatever their size; a
 // cluster barrier and one round of shared-memory reads cost a fraction of that.  Levels 0 .. nc-1
-// are spread over the cluster in equal runs of the flat node index; a neighbour in another CTA's
-// run is read through distributed shared memory, all of a node's reads being issued before the
-// first is used (read one by one behind a branch, they made an operation four times as long).
+// are spread over the cluster in equal runs of the flat node index.  A CTA holds, next to its run of
+// an iterate, copies of the `halo` entries before and after it (a row in 2D, a plane in 3D); whoever
+// works out a value near the end of a run stores it into the neighbour's copy too, so that sweeps
+// and residuals read their own shared memory only.  Restriction and prolongation, which reach
+// further, read through distributed shared memory, with all of a node's reads issued before the
+// first is used.  What an operation needs to know of a node (which faces it is on, Dirichlet) is
+// worked out once, a byte per node.
 // Levels nc .. n-1, too small for that, run in CTA 0 with CTA barriers; the coarsest one's many
 // Jacobi sweeps keep one node per thread in registers, and only the warps that hold nodes meet.
 // The host works out a level's descriptor, and each operation takes it by value: indexed kernel
 // parameters and per-level divisions cost more than the arithmetic.
+// Microseconds of a cycle from this level down: 33^3 114 as launches, 67 with every neighbour in
+// another CTA read remotely, 45 now; 129^2 43 and 35; 151x111 (ragged coarsening) 77 and 48.
 //
 // Division of the flat index by a fixed number d: (i m) >> 40 with m = floor(2^40 / d) + 1,
 // exact for i d < 2^40.
 struct CoarseNode {
-    int i, ix, iy, iz, ends;
-    bool dir;
+    int i, ix, iy, iz;
 };
+// A node's byte: bits 0-5 it is on the first / last x, y, z face, bit 6 Dirichlet.
 
 __device__ __forceinline__ unsigned shared_addr(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 
@@ -627,23 +663,52 @@ __device__ __forceinline__ void cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-__device__ __forceinline__ CoarseNode coarse_node(const CoarseLevel& l, int k, bool mask = true) {
+__device__ __forceinline__ CoarseNode coarse_node(const CoarseLevel& l, int k) {
     CoarseNode n;
     n.i = l.lo + k;
     const unsigned t = (unsigned)(((unsigned)n.i * l.m_sx) >> 40);
     n.ix = n.i - (int)t * l.sx;
     n.iz = (int)((t * l.m_sy) >> 40);
     n.iy = (int)t - n.iz * l.sy;
-    n.ends = (n.ix == 0 || n.ix == l.nx) + (n.iy == 0 || n.iy == l.ny);
-    if (l.dim == 3) n.ends += (n.iz == 0 || n.iz == l.nz);
-    n.dir = false;
-    if (mask && l.mask) {
-        unsigned m;
-        asm volatile("ld.shared.u8 %0, [%1];" : "=r"(m) : "r"(l.mask + (unsigned)k) : "memory");
-        n.dir = m != 0u;
-    }
     return n;
 }
+__device__ __forceinline__ unsigned faces_of(const CoarseLevel& l, const CoarseNode& n) {
+    unsigned d = (n.ix == 0 ? 1u : 0u) | (n.ix == l.nx ? 2u : 0u) | (n.iy == 0 ? 4u : 0u) | (n.iy == l.ny ? 8u : 0u);
+    if (l.dim == 3) d |= (n.iz == 0 ? 16u : 0u) | (n.iz == l.nz ? 32u : 0u);
+    return d;
+}
+__device__ __forceinline__ unsigned node_byte(const CoarseLevel& l, int k) {
+    unsigned d;
+    asm volatile("ld.shared.u8 %0, [%1];" : "=r"(d) : "r"(l.node + (unsigned)k) : "memory");
+    return d;
+}
+__device__ __forceinline__ int ends_of(unsigned d) { return __popc(d & 63u); }
+
+// Stores of an iterate's values: in this CTA, and SPREAD in the neighbours' copies.
+template <bool SPREAD>
+struct Put {
+    unsigned own, before, after;
+    int halo, tail;
+    __device__ __forceinline__ Put(const CoarseLevel& l, unsigned a) : own(a), before(0), after(0), halo(0), tail(INT_MAX) {
+        if (!SPREAD) return;
+        if (blockIdx.x > 0) {
+            halo = l.halo;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(before) : "r"(a), "r"(blockIdx.x - 1u));
+            before += 4u * (unsigned)l.chunk;
+        }
+        if (l.lo + l.cnt < l.np) {
+            tail = l.cnt - l.halo;
+            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(after) : "r"(a), "r"(blockIdx.x + 1u));
+            after -= 4u * (unsigned)l.cnt;
+        }
+    }
+    __device__ __forceinline__ void operator()(int k, float v) const {
+        sts(own + 4u * (unsigned)k, v);
+        if (!SPREAD) return;
+        if (k < halo) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(before + 4u * (unsigned)k), "f"(v) : "memory");
+        if (k >= tail) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(after + 4u * (unsigned)k), "f"(v) : "memory");
+    }
+};
 
 // The roundings of the smoother and the interpolation, written out (a fused multiply-add, or a
 // product rounded before the sum), so that a level gives the same bits in whichever kernel and CTA
@@ -661,30 +726,15 @@ __device__ __forceinline__ float blend_rn(float wa, float a, float wb, float b) 
     return __fmaf_rn(wa, a, __fmul_rn(wb, b));
 }
 
-// The neighbour sum's six values at node n of the array at `a`; FIRST: of the first sweep's result
-// from zero, omega b / diag K, formed from the right-hand side at `a` (zero on Dirichlet nodes).
-template <bool SPREAD, bool FIRST>
-__device__ __forceinline__ float neighbour_sum(const CoarseLevel& l, unsigned a, const CoarseNode& n, float wcb) {
-    const int xm = n.ix > 0 ? n.ix - 1 : 1, xp = n.ix < l.nx ? n.ix + 1 : l.nx - 1;
-    const int ym = n.iy > 0 ? n.iy - 1 : 1, yp = n.iy < l.ny ? n.iy + 1 : l.ny - 1;
-    float v0 = at<SPREAD>(l, a, n.i + (xm - n.ix)), v1 = at<SPREAD>(l, a, n.i + (xp - n.ix));
-    float v2 = at<SPREAD>(l, a, n.i + (ym - n.iy) * l.sx), v3 = at<SPREAD>(l, a, n.i + (yp - n.iy) * l.sx);
+// The neighbour sum at node k (byte d) of the array at `a`.
+__device__ __forceinline__ float neighbour_sum(const CoarseLevel& l, unsigned a, int k, unsigned d) {
+    const unsigned p = a + 4u * (unsigned)k, sy = 4u * (unsigned)l.sx, sz = 4u * (unsigned)l.sxy;
+    const float v0 = lds(p + (d & 1u ? 4u : -4u)), v1 = lds(p + (d & 2u ? -4u : 4u));
+    const float v2 = lds(p + (d & 4u ? sy : -sy)), v3 = lds(p + (d & 8u ? -sy : sy));
     float v4 = 0.f, v5 = 0.f;
-    int zm = 0, zp = 0;
     if (l.dim == 3) {
-        zm = n.iz > 0 ? n.iz - 1 : 1, zp = n.iz < l.nz ? n.iz + 1 : l.nz - 1;
-        v4 = at<SPREAD>(l, a, n.i + (zm - n.iz) * l.sxy);
-        v5 = at<SPREAD>(l, a, n.i + (zp - n.iz) * l.sxy);
-    }
-    if (FIRST) {
-        const int ex = n.ends - (n.ix == 0 || n.ix == l.nx), ey = n.ends - (n.iy == 0 || n.iy == l.ny);
-        auto scale = [&](int e, int c, int m) { return wcb * (float)(1 << (e + (c == 0 || c == m))); };
-        v0 *= scale(ex, xm, l.nx), v1 *= scale(ex, xp, l.nx);
-        v2 *= scale(ey, ym, l.ny), v3 *= scale(ey, yp, l.ny);
-        if (l.dim == 3) {
-            const int ez = n.ends - (n.iz == 0 || n.iz == l.nz);
-            v4 *= scale(ez, zm, l.nz), v5 *= scale(ez, zp, l.nz);
-        }
+        v4 = lds(p + (d & 16u ? sz : -sz));
+        v5 = lds(p + (d & 32u ? -sz : sz));
     }
     float acc = __fadd_rn(v0, v1);
     acc = __fadd_rn(acc, __fadd_rn(v2, v3));
@@ -692,93 +742,116 @@ __device__ __forceinline__ float neighbour_sum(const CoarseLevel& l, unsigned a,
     return acc;
 }
 
-// out = two sweeps from zero (FIRST) or one sweep from in.
-template <bool SPREAD, bool FIRST>
-__device__ __forceinline__ void coarse_sweep(const CoarseLevel l, unsigned in, unsigned out, float omega) {
-    const float wcb = omega * l.cB;
-    for (int k = (int)threadIdx.x; k < l.cnt; k += (int)blockDim.x) {
-        const CoarseNode n = coarse_node(l, k);
-        const float bj = lds(l.b + 4u * k);
-        const float xc = FIRST ? wcb * (float)(1 << n.ends) * bj : lds(in + 4u * k);
-        const float acc = neighbour_sum<SPREAD, FIRST>(l, FIRST ? l.b : in, n, wcb);
-        const float v = relax_rn(xc, lap_rn(xc, acc, l.dim, l.fused != 0), bj, omega, n.ends, l.cB, l.inv2d);
-        sts(out + 4u * k, n.dir ? 0.f : v);
-    }
+// The first sweep's result from zero, omega b / diag K.
+__device__ __forceinline__ float first_sweep(const CoarseLevel& l, float omega, unsigned d, float b) {
+    return d & 64u ? 0.f : omega * l.cB * (float)(1 << ends_of(d)) * b;
 }
 
 template <bool SPREAD>
-__device__ __forceinline__ void coarse_residual(const CoarseLevel l) {
+__device__ __forceinline__ void coarse_sweep(const CoarseLevel l, unsigned in, unsigned out, float omega) {
+    const Put<SPREAD> put(l, out);
     for (int k = (int)threadIdx.x; k < l.cnt; k += (int)blockDim.x) {
-        const CoarseNode n = coarse_node(l, k);
-        const float bj = lds(l.b + 4u * k), xc = lds(l.x + 4u * k);
-        const float s = 1.f / (float)(1 << n.ends);
-        const float L = lap_rn(xc, neighbour_sum<SPREAD, false>(l, l.x, n, 0.f), l.dim, l.fused != 0);
-        const float v = __fmaf_rn(-__fmul_rn(l.cK, s), L, bj);
-        sts(l.r + 4u * k, n.dir ? 0.f : v);
+        const unsigned d = node_byte(l, k);
+        const float bj = lds(l.b + 4u * k), xc = lds(in + 4u * k);
+        const float acc = neighbour_sum(l, in, k, d);
+        const float v = relax_rn(xc, lap_rn(xc, acc, l.dim, l.fused != 0), bj, omega, ends_of(d), l.cB, l.inv2d);
+        put(k, d & 64u ? 0.f : v);
     }
 }
 
-// restrict_nested with every read issued before the sum (rows and columns outside the grid are read
-// at a clamped place and left out): the same terms in the same order.
-template <int DIM, typename F>
-__device__ __forceinline__ float restrict_nested_ahead(const CoarseLevel& f, F rf, int jx, int jy, int jz) {
-    constexpr int NZ = DIM == 3 ? 3 : 1;
-    const int cx = 2 * jx, cy = 2 * jy, cz = DIM == 3 ? 2 * jz : 0;
-    const bool xm = cx > 0, xp = cx < f.nx;
-    float a[NZ][3], l[NZ][3], q[NZ][3];
-    bool ok[NZ][3];
-#pragma unroll
-    for (int z = 0; z < NZ; ++z)
-#pragma unroll
-        for (int y = 0; y < 3; ++y) {
-            const int fz = DIM == 3 ? cz + z - 1 : 0, fy = cy + y - 1;
-            ok[z][y] = fy >= 0 && fy <= f.ny && fz >= 0 && fz <= f.nz;
-            const int row = (ok[z][y] ? fy : cy) * f.sx + (ok[z][y] ? fz : cz) * f.sxy;
-            a[z][y] = rf(row + cx);
-            l[z][y] = rf(row + (xm ? cx - 1 : cx));
-            q[z][y] = rf(row + (xp ? cx + 1 : cx));
-        }
-    float acc = 0.f;
-#pragma unroll
-    for (int z = 0; z < NZ; ++z)
-#pragma unroll
-        for (int y = 0; y < 3; ++y) {
-            float r = a[z][y];
-            if (xm) r += 0.5f * l[z][y];
-            if (xp) r += 0.5f * q[z][y];
-            const float w = (y == 1 ? 1.f : 0.5f) * (DIM == 2 || z == 1 ? 1.f : 0.5f);
-            if (ok[z][y]) acc += w * r;
-        }
-    return acc;
+__device__ __forceinline__ void coarse_residual(const CoarseLevel l) {
+    for (int k = (int)threadIdx.x; k < l.cnt; k += (int)blockDim.x) {
+        const unsigned d = node_byte(l, k);
+        const float bj = lds(l.b + 4u * k), xc = lds(l.x + 4u * k);
+        const float s = __int_as_float((127 - ends_of(d)) << 23);  // 2^-ends
+        const float L = lap_rn(xc, neighbour_sum(l, l.x, k, d), l.dim, l.fused != 0);
+        const float v = __fmaf_rn(-__fmul_rn(l.cK, s), L, bj);
+        sts(l.r + 4u * k, d & 64u ? 0.f : v);
+    }
 }
 
-// b of the coarse level = restriction of the fine level's residual.  TO_FIRST: CTA 0 holds the
-// coarse level; every CTA works out a share of it (CTA 0 alone would read all of the residual
-// through its one port) and stores it there.
+// Where a restricted value goes: b of the coarse level, and the first sweep's result from zero in its
+// r.  TO_FIRST: CTA 0 holds the coarse level; every CTA works out a share of it (CTA 0 alone would
+// read all of the residual through its one port) and stores it there.
 template <bool SPREAD, bool TO_FIRST>
-__device__ __forceinline__ void coarse_restrict(const Geom& gf, const Geom& gc, const CoarseLevel f, const CoarseLevel c) {
-    auto rf = [&](long long i) { return at<SPREAD>(f, f.r, (int)i); };
+struct PutRestricted {
+    const CoarseLevel& c;
+    const Put<SPREAD && !TO_FIRST> put;
+    float omega;
+    __device__ __forceinline__ PutRestricted(const CoarseLevel& c_, float omega_) : c(c_), put(c_, c_.r), omega(omega_) {}
+    __device__ __forceinline__ void operator()(int k, float v) const {
+        if (!TO_FIRST) {
+            const unsigned d = node_byte(c, k);
+            v = d & 64u ? 0.f : v;
+            sts(c.b + 4u * (unsigned)k, v);
+            put(k, first_sweep(c, omega, d, v));
+            return;
+        }
+        unsigned p, d;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(c.node + (unsigned)k), "r"(0));
+        asm volatile("ld.shared::cluster.u8 %0, [%1];" : "=r"(d) : "r"(p) : "memory");
+        v = d & 64u ? 0.f : v;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(c.b + 4u * (unsigned)k), "r"(0));
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(p), "f"(v) : "memory");
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(c.r + 4u * (unsigned)k), "r"(0));
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(p), "f"(first_sweep(c, omega, d, v)) : "memory");
+    }
+};
+
+// restrict_nested with a thread per fine row of a coarse node (three in 2D, nine in 3D): a node's
+// thread would wait for 27 reads in a row where few nodes are left for it.  The rows' terms are
+// summed in restrict_nested's order by the node's first thread.
+template <int DIM, bool SPREAD, bool TO_FIRST>
+__device__ __forceinline__ void restrict_rows(const CoarseLevel& f, const CoarseLevel& c, int lo, int end,
+                                              const PutRestricted<SPREAD, TO_FIRST>& put) {
+    constexpr int G = DIM == 3 ? 9 : 3, NPW = 32 / G;  // nodes per warp
+    const int lane = (int)threadIdx.x & 31, g = lane / G, row = lane - g * G;
+    const int fy0 = row % 3 - 1, fz0 = DIM == 3 ? row / 3 - 1 : 0;
+    const float w = (fy0 == 0 ? 1.f : 0.5f) * (fz0 == 0 ? 1.f : 0.5f);
+    for (int k0 = lo + ((int)threadIdx.x >> 5) * NPW; k0 < end; k0 += ((int)blockDim.x >> 5) * NPW) {
+        const int k = k0 + g;
+        const bool here = g < NPW && k < end;
+        const CoarseNode n = coarse_node(c, here ? k : k0);
+        const int cx = 2 * n.ix, fy = 2 * n.iy + fy0, fz = DIM == 3 ? 2 * n.iz + fz0 : 0;
+        const bool ok = here && fy >= 0 && fy <= f.ny && fz >= 0 && fz <= f.nz;
+        float t = 0.f;
+        if (ok) {
+            const int j = fz * f.sxy + fy * f.sx + cx;
+            const bool xm = cx > 0, xp = cx < f.nx;
+            t = at<SPREAD>(f, f.r, j);
+            const float l = at<SPREAD>(f, f.r, xm ? j - 1 : j), q = at<SPREAD>(f, f.r, xp ? j + 1 : j);
+            if (xm) t += 0.5f * l;
+            if (xp) t += 0.5f * q;
+            t *= w;
+        }
+        const unsigned oks = __ballot_sync(0xffffffffu, ok) >> (lane - row);
+        float acc = 0.f;
+#pragma unroll
+        for (int i = 0; i < G; ++i) {
+            const float v = __shfl_down_sync(0xffffffffu, t, i);
+            if (oks >> i & 1u) acc += v;
+        }
+        if (here && row == 0) put(k, acc);
+    }
+}
+
+// b of the coarse level = restriction of the fine level's residual.
+template <bool SPREAD, bool TO_FIRST>
+__device__ __forceinline__ void coarse_restrict(const Geom& gf, const Geom& gc, const CoarseLevel f, const CoarseLevel c,
+                                                float omega) {
     const int share = TO_FIRST ? (c.np + (int)gridDim.x - 1) / (int)gridDim.x : 0;
     const int lo = TO_FIRST ? (int)blockIdx.x * share : 0, end = TO_FIRST ? min(lo + share, c.np) : c.cnt;
-    const bool two = nested(gf, gc);
+    const PutRestricted<SPREAD, TO_FIRST> put(c, omega);
+    if (nested(gf, gc)) {
+        if (f.dim == 3) restrict_rows<3>(f, c, lo, end, put);
+        else restrict_rows<2>(f, c, lo, end, put);
+        return;
+    }
+    auto rf = [&](long long i) { return at<SPREAD>(f, f.r, (int)i); };
     for (int k = lo + (int)threadIdx.x; k < end; k += (int)blockDim.x) {
-        CoarseNode n = coarse_node(c, k, !TO_FIRST);
-        const float v = !two         ? restrict_node(gf, gc, rf, n.ix, n.iy, n.iz)
-                        : f.dim == 3 ? restrict_nested_ahead<3>(f, rf, n.ix, n.iy, n.iz)
-                                     : restrict_nested_ahead<2>(f, rf, n.ix, n.iy, n.iz);
-        if (TO_FIRST) {  // its Dirichlet bytes are in CTA 0 too
-            unsigned p;
-            if (c.mask) {
-                unsigned m;
-                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(c.mask + (unsigned)k), "r"(0));
-                asm volatile("ld.shared::cluster.u8 %0, [%1];" : "=r"(m) : "r"(p) : "memory");
-                n.dir = m != 0u;
-            }
-            asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(p) : "r"(c.b + 4u * (unsigned)k), "r"(0));
-            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(p), "f"(n.dir ? 0.f : v) : "memory");
-        } else {
-            sts(c.b + 4u * k, n.dir ? 0.f : v);
-        }
+        const CoarseNode n = coarse_node(c, k);
+        put(k, restrict_weighted(gf, rf, axis_weights(n.ix, gf.nx, gc.nx), axis_weights(n.iy, gf.ny, gc.ny),
+                                 axis_weights_z(gf, gc, n.iz)));
     }
 }
 
@@ -792,6 +865,7 @@ __device__ __forceinline__ void coarse_prolong(const Geom& gf, const Geom& gc, c
         __syncthreads();
     }
     auto xc = [&](int i) { return at<SPREAD && !FIRST>(c, c.x, i); };
+    const Put<SPREAD> put(f, f.x);
     for (int k = (int)threadIdx.x; k < f.cnt; k += (int)blockDim.x) {
         const CoarseNode n = coarse_node(f, k);
         const Interp1 px = interp1_fast(n.ix, gf.nx, gc.nx), py = interp1_fast(n.iy, gf.ny, gc.ny);
@@ -811,7 +885,7 @@ __device__ __forceinline__ void coarse_prolong(const Geom& gf, const Geom& gc, c
             const float w = blend_rn(ay, blend_rn(ax, b0, px.t, b1), py.t, blend_rn(ax, b2, px.t, b3));
             v = blend_rn(1.f - pz.t, v, pz.t, w);
         }
-        if (!n.dir) sts(f.x + 4u * k, lds(f.x + 4u * k) + v);
+        if (!(node_byte(f, k) & 64u)) put(k, lds(f.x + 4u * k) + v);
     }
 }
 
@@ -820,16 +894,16 @@ __device__ __forceinline__ void coarsest_sweeps(const CoarseLevel l, float omega
     const int threads = (l.np + 31) & ~31;
     if ((int)threadIdx.x >= threads) return;
     const bool here = (int)threadIdx.x < l.np;
-    const CoarseNode n = coarse_node(l, here ? (int)threadIdx.x : 0);
-    const unsigned x = l.x + 4u * (unsigned)n.i, flip = l.r - l.x;
-    const int d3 = l.dim == 3;
-    const unsigned a0 = x + 4u * (unsigned)(n.ix > 0 ? -1 : 1), a1 = x + 4u * (unsigned)(n.ix < l.nx ? 1 : -1);
-    const unsigned a2 = x + 4u * (unsigned)(n.iy > 0 ? -l.sx : l.sx), a3 = x + 4u * (unsigned)(n.iy < l.ny ? l.sx : -l.sx);
-    const unsigned a4 = x + 4u * (unsigned)(d3 ? (n.iz > 0 ? -l.sxy : l.sxy) : 0);
-    const unsigned a5 = x + 4u * (unsigned)(d3 ? (n.iz < l.nz ? l.sxy : -l.sxy) : 0);
-    const float bj = lds(l.b + 4u * (unsigned)n.i);
-    const float w = __fmul_rn(l.cB, (float)(1 << n.ends)), inv2d = l.inv2d, dd = d3 ? 6.f : 4.f;
-    float xj = n.dir ? 0.f : omega * l.cB * (float)(1 << n.ends) * bj;
+    const int i = here ? (int)threadIdx.x : 0;
+    const unsigned d = node_byte(l, i), sy = 4u * (unsigned)l.sx, sz = 4u * (unsigned)l.sxy;
+    const unsigned x = l.x + 4u * (unsigned)i, flip = l.r - l.x;
+    const bool dir = (d & 64u) != 0u, d3 = l.dim == 3;
+    const unsigned a0 = x + (d & 1u ? 4u : -4u), a1 = x + (d & 2u ? -4u : 4u);
+    const unsigned a2 = x + (d & 4u ? sy : -sy), a3 = x + (d & 8u ? -sy : sy);
+    const unsigned a4 = x + (d3 ? (d & 16u ? sz : -sz) : 0u), a5 = x + (d3 ? (d & 32u ? -sz : sz) : 0u);
+    const float bj = lds(l.b + 4u * (unsigned)i);
+    const float w = __fmul_rn(l.cB, (float)(1 << ends_of(d))), inv2d = l.inv2d, dd = d3 ? 6.f : 4.f;
+    float xj = first_sweep(l, omega, d, bj);
     if (here) sts(x, xj);
     if (threads == 32) {  // one warp: the neighbours' values by shuffle
         const unsigned all = 0xffffffffu;
@@ -843,7 +917,7 @@ __device__ __forceinline__ void coarsest_sweeps(const CoarseLevel l, float omega
             if (d3) acc += __shfl_sync(all, xj, n4) + __shfl_sync(all, xj, n5);
             const float L = __fsub_rn(__fmul_rn(dd, xj), acc);
             const float v = __fmaf_rn(omega, __fmaf_rn(w, bj, -__fmul_rn(inv2d, L)), xj);
-            xj = n.dir ? 0.f : v;
+            xj = dir ? 0.f : v;
         }
         if (here) sts(x, xj);
         return;
@@ -856,7 +930,7 @@ __device__ __forceinline__ void coarsest_sweeps(const CoarseLevel l, float omega
         if (d3) acc += lds(a4 + o) + lds(a5 + o);
         const float L = __fsub_rn(__fmul_rn(dd, xj), acc);
         const float v = __fmaf_rn(omega, __fmaf_rn(w, bj, -__fmul_rn(inv2d, L)), xj);
-        xj = n.dir ? 0.f : v;
+        xj = dir ? 0.f : v;
         o = flip - o;
         if (here) sts(x + o, xj);
     }
@@ -877,42 +951,58 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle(const __grid_constant__ 
             l.lo = min(rank * l.chunk, l.np);
             l.cnt = min(l.chunk, l.np - l.lo);
         }
-        l.x += base, l.r += base, l.b += base;
-        if (l.mask) l.mask += base;
+        l.x += base, l.r += base, l.b += base, l.node += base;
         lev[tid] = l;
     }
     __syncthreads();
-    // masks, and the first level's right-hand side
+    // the first level's right-hand side; the nodes' bytes
     for (int q = 0; q < nl; ++q) {
         if (q >= nc && rank != 0) break;
         const CoarseLevel& l = lev[q];
+        const unsigned char* const mask = lv.mask[q];
         for (int k = tid; k < l.cnt; k += nt) {
-            if (l.mask) asm volatile("st.shared.u8 [%0], %1;" ::"r"(l.mask + (unsigned)k), "r"((unsigned)lv.mask[q][l.lo + k]) : "memory");
-            if (q == 0) sts(l.b + 4u * k, bglob[l.lo + k]);
+            float b = 0.f;
+            unsigned dir = 0u;
+            if (q == 0) b = bglob[l.lo + k];
+            if (mask) dir = mask[l.lo + k];
+            const unsigned d = faces_of(l, coarse_node(l, k)) | (dir ? 64u : 0u);
+            asm volatile("st.shared.u8 [%0], %1;" ::"r"(l.node + (unsigned)k), "r"(d) : "memory");
+            if (q == 0) sts(l.b + 4u * k, b);
         }
     }
-    if (nc > 0) cluster_sync();
+    if (nc > 0) cluster_sync();  // (every CTA has started)
     else __syncthreads();
+    {
+        const CoarseLevel& l = lev[0];
+        if (nc > 0) {
+            const Put<true> put(l, l.r);
+            for (int k = tid; k < l.cnt; k += nt) put(k, first_sweep(l, omega, node_byte(l, k), lds(l.b + 4u * k)));
+            cluster_sync();
+        } else {
+            for (int k = tid; k < l.cnt; k += nt) sts(l.r + 4u * k, first_sweep(l, omega, node_byte(l, k), lds(l.b + 4u * k)));
+            __syncthreads();
+        }
+    }
     // down through the spread levels
     for (int q = 0; q < nc; ++q) {
         const CoarseLevel& l = lev[q];
-        coarse_sweep<true, true>(l, 0u, l.x, omega);
+        coarse_sweep<true>(l, l.r, l.x, omega);
         cluster_sync();
-        coarse_residual<true>(l);
+        coarse_residual(l);
         cluster_sync();
-        if (q + 1 < nc) coarse_restrict<true, false>(lv.g[q], lv.g[q + 1], l, lev[q + 1]);
-        else coarse_restrict<true, true>(lv.g[q], lv.g[q + 1], l, lev[q + 1]);
+        if (q + 1 < nc) coarse_restrict<true, false>(lv.g[q], lv.g[q + 1], l, lev[q + 1], omega);
+        else coarse_restrict<true, true>(lv.g[q], lv.g[q + 1], l, lev[q + 1], omega);
         cluster_sync();
     }
     // the small levels, in CTA 0
     if (rank == 0) {
         for (int q = nc; q + 1 < nl; ++q) {
             const CoarseLevel& l = lev[q];
-            coarse_sweep<false, true>(l, 0u, l.x, omega);
+            coarse_sweep<false>(l, l.r, l.x, omega);
             __syncthreads();
-            coarse_residual<false>(l);
+            coarse_residual(l);
             __syncthreads();
-            coarse_restrict<false, false>(lv.g[q], lv.g[q + 1], l, lev[q + 1]);
+            coarse_restrict<false, false>(lv.g[q], lv.g[q + 1], l, lev[q + 1], omega);
             __syncthreads();
         }
         {
@@ -921,11 +1011,11 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle(const __grid_constant__ 
                 coarsest_sweeps(l, omega, coarse_sweeps);
                 __syncthreads();
             } else {
-                coarse_sweep<false, true>(l, 0u, l.x, omega);  // two sweeps
+                coarse_sweep<false>(l, l.r, l.x, omega);  // the second sweep
                 __syncthreads();
                 unsigned in = l.x, out = l.r;
                 for (int s = 2; s < coarse_sweeps; ++s) {
-                    coarse_sweep<false, false>(l, in, out, omega);
+                    coarse_sweep<false>(l, in, out, omega);
                     __syncthreads();
                     const unsigned t = in;
                     in = out;
@@ -941,9 +1031,9 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle(const __grid_constant__ 
             const CoarseLevel& l = lev[q];
             coarse_prolong<false, false>(lv.g[q], lv.g[q + 1], l, lev[q + 1]);
             __syncthreads();
-            coarse_sweep<false, false>(l, l.x, l.r, omega);
+            coarse_sweep<false>(l, l.x, l.r, omega);
             __syncthreads();
-            coarse_sweep<false, false>(l, l.r, l.x, omega);
+            coarse_sweep<false>(l, l.r, l.x, omega);
             __syncthreads();
         }
     }
@@ -954,9 +1044,9 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle(const __grid_constant__ 
         if (q + 1 < nc) coarse_prolong<true, false>(lv.g[q], lv.g[q + 1], l, lev[q + 1]);
         else coarse_prolong<true, true>(lv.g[q], lv.g[q + 1], l, lev[q + 1]);
         cluster_sync();
-        coarse_sweep<true, false>(l, l.x, l.r, omega);
+        coarse_sweep<true>(l, l.x, l.r, omega);
         cluster_sync();
-        coarse_sweep<true, false>(l, l.r, l.x, omega);
+        coarse_sweep<true>(l, l.r, l.x, omega);
         cluster_sync();
     }
     if (nc > 0 || rank == 0) {
@@ -1140,13 +1230,12 @@ void launch_mg_residual(const MGLevel& L, const float* x, const float* b, float*
 
 void launch_mg_restrict(const MGLevel& fine, const float* rf, const MGLevel& coarse, float* bc, cudaStream_t st) {
     note_launch(1);
-    const int zc = coarse.g.dim == 3 ? 4 : 1;
     const Geom& gf = fine.g;
     const Geom& gc = coarse.g;
     if (gf.dim == 3 && gf.nx == 2 * gc.nx && gf.ny == 2 * gc.ny && gf.nz == 2 * gc.nz)
-        k_restrict3_nested<<<mg_grid(gc, zc), kT, 0, st>>>(gf, rf, gc, coarse.mask, bc, zc);
+        k_restrict3_nested<<<mg_grid(gc, 4), kT, 0, st>>>(gf, rf, gc, coarse.mask, bc, 4);
     else
-        k_restrict<<<mg_grid(gc, zc), kT, 0, st>>>(gf, rf, gc, coarse.mask, bc, zc);
+        k_restrict<<<mg_grid(gc, 1), kT, 0, st>>>(gf, rf, gc, coarse.mask, bc, 1);
 }
 
 void launch_mg_prolong_add(const MGLevel& coarse, const float* xc, const MGLevel& fine, float* xf, cudaStream_t st) {
@@ -1165,8 +1254,8 @@ void launch_mg_prolong_add(const MGLevel& coarse, const float* xc, const MGLevel
 size_t mg_coarse_smem(const CoarseLevels& lv) {
     size_t n = 0;
     for (int l = 0; l < lv.n; ++l) {
-        const size_t np = (size_t)lv.g[l].np;
-        n += 13 * (l < lv.nc ? (np + lv.ctas - 1) / lv.ctas : np);
+        const CoarseLevel& c = lv.level[l];
+        n += 13 * (size_t)(l < lv.nc ? c.chunk : c.np) + 16 * (size_t)c.halo;
     }
     return n + 16;
 }
@@ -1189,21 +1278,24 @@ bool mg_coarse_plan(const MGLevel* levels, int nlev, int first, CoarseLevels* lv
         CoarseLevel& l = lv->level[i];
         l.np = l.cnt = (int)g.np;
         l.lo = 0;
-        l.chunk = (int)((g.np + lv->ctas - 1) / lv->ctas);
+        // (runs of at least a row or plane: a node's neighbours are in the runs next to its own)
+        l.halo = i < lv->nc ? (g.dim == 3 ? g.sx * g.sy : g.sx) : 0;
+        l.chunk = std::max((int)((g.np + lv->ctas - 1) / lv->ctas), l.halo);
         l.sx = g.sx, l.sy = g.sy, l.sxy = g.sx * g.sy;
         l.nx = g.nx, l.ny = g.ny, l.nz = g.nz, l.dim = g.dim;
         l.m_chunk = magic(l.chunk), l.m_sx = magic(g.sx), l.m_sy = magic(g.sy);
         const unsigned n = (unsigned)(i < lv->nc ? l.chunk : l.np);
-        l.x = 4 * floats, l.r = l.x + 4 * n, l.b = l.r + 4 * n;
-        floats += 3 * n;
+        const unsigned h = (unsigned)l.halo;
+        l.x = 4 * (floats + h), l.r = l.x + 4 * (n + 2 * h), l.b = l.r + 4 * (n + h);
+        floats += 3 * n + 4 * h;
         l.fused = g.np > kCoarsestMaxNodes;
-        const float h = (float)g.h, hd = g.dim == 3 ? h * h * h : h * h;  // as mg_const
-        l.cK = hd / (h * h);
+        const float gh = (float)g.h, hd = g.dim == 3 ? gh * gh * gh : gh * gh;  // as mg_const
+        l.cK = hd / (gh * gh);
         l.inv2d = 1.f / (float)(2 * g.dim);
-        l.cB = (h * h) / (hd * (float)(2 * g.dim));
+        l.cB = (gh * gh) / (hd * (float)(2 * g.dim));
     }
     for (int i = 0; i < lv->n; ++i) {
-        if (lv->mask[i]) lv->level[i].mask = 4 * floats + bytes;
+        lv->level[i].node = 4 * floats + bytes;
         bytes += (unsigned)(i < lv->nc ? lv->level[i].chunk : lv->level[i].np);
     }
     return mg_coarse_smem(*lv) <= (size_t)220 * 1024;

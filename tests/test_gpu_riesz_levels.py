@@ -18,7 +18,8 @@ from oracle.grid import Discretization  # noqa: E402
 from paper_1903_12522_gb300 import cmcg  # noqa: E402
 
 SIZES = [(2, 2), (4, 4), (7, 9), (32, 32), (43, 45), (64, 64), (101, 86), (200, 170), (257, 300), (260, 5),
-         (2, 2, 2), (4, 4, 4), (12, 9, 10), (16, 16, 16), (33, 30, 29), (34, 33, 32), (50, 47, 44)]
+         (9, 300), (300, 9), (2, 2, 2), (4, 4, 4), (12, 9, 10), (16, 16, 16), (33, 30, 29), (34, 33, 32), (50, 47, 44),
+         (90, 87, 40), (57, 63, 44)]
 
 
 @pytest.mark.parametrize("obstacle", [False, True])
