@@ -302,7 +302,7 @@ void launch_mg_prolong_add(const MGLevel& coarse, const float* xc, const MGLevel
 // Coarse end of the V-cycle in one cluster launch (riesz.cu): levels 0 .. nc-1 spread over ctas
 // CTAs, the rest in the first one.
 constexpr int kCoarseMax = 10;
-constexpr long long kSpreadMaxNodes = 40000;
+constexpr long long kSpreadMaxNodes = 70000;
 constexpr long long kSpreadMinNodes = 2000;
 constexpr long long kCoarsestMaxNodes = 6000;  // larger: the coarsest level gets a few grid-wide sweeps instead
 struct CoarseLevel {

@@ -1248,9 +1248,10 @@ void launch_mg_prolong_add(const MGLevel& coarse, const float* xc, const MGLevel
 }
 
 // Which levels, from the first that fits, run in the cluster: spread ones of up to kSpreadMaxNodes
-// nodes (2.4 per thread: an operation on 33^3 nodes takes 3 us there, as a launch 6; on 49^3 8 us
-// against 5) while they have more than kSpreadMinNodes (below, one CTA is faster than the
-// cluster's barriers).
+// nodes (four per thread: a 257^2 Riesz map takes 919 us with its finest level in the cluster, 1030 as
+// launches; 81^3 with 41^3 nodes there 2176 and 2237; with 49^3 there 97^3 is slower, 2513 against
+// 2389) while they have more than kSpreadMinNodes (below, one CTA is faster than the cluster's
+// barriers).
 size_t mg_coarse_smem(const CoarseLevels& lv) {
     size_t n = 0;
     for (int l = 0; l < lv.n; ++l) {
