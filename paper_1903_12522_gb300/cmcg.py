@@ -343,20 +343,28 @@ class Solver:
     def _after_caller(self):
         # inputs produced on the caller's stream must be complete before this solver's stream
         # reads them (torch's side streams do not synchronise with the default stream)
+        # (a caller's stream with nothing pending needs no event: 2 us of host time instead of 8 per call.
+        # The way back needs none at all: every entry point returns with the solver's stream idle.)
         cur = self.torch.cuda.current_stream(self.device)
-        if cur.cuda_stream != self.stream.cuda_stream:
+        if cur.cuda_stream != self.stream.cuda_stream and not self._idle(cur):
             self.stream.wait_stream(cur)
 
-    def _before_caller(self):
-        cur = self.torch.cuda.current_stream(self.device)
-        if cur.cuda_stream != self.stream.cuda_stream:
-            cur.wait_stream(self.stream)
+    @staticmethod
+    def _idle(stream):
+        try:
+            return stream.query()
+        except RuntimeError:  # a stream that is being captured cannot be asked
+            return False
 
     def _dev(self, a, dtype):
         torch = self.torch
         if a is None:
             return None
         if isinstance(a, torch.Tensor):
+            if a.dtype is dtype and a.is_cuda and a.is_contiguous():
+                index = self.device.index
+                if a.get_device() == (torch.cuda.current_device() if index is None else index):
+                    return a.view(-1)
             return a.to(device=self.device, dtype=dtype).contiguous().reshape(-1)
         # writeable C-contiguous host array (torch does not take read-only numpy buffers)
         return torch.as_tensor(np.require(a, requirements=["C", "W"])).to(device=self.device, dtype=dtype).reshape(-1)
@@ -380,7 +388,6 @@ class Solver:
         uT, vT = torch.empty_like(u0), torch.empty_like(v0)
         self._after_caller()
         cmcg_wave_period(self.handle, u0, v0, f, g, uT, vT)
-        self._before_caller()
         return uT.reshape(self.shape), vT.reshape(self.shape)
 
     def adjoint_period(self, a, b):
@@ -389,7 +396,6 @@ class Solver:
         q0, q1 = torch.empty_like(a), torch.empty_like(b)
         self._after_caller()
         cmcg_adjoint_period(self.handle, a, b, q0, q1)
-        self._before_caller()
         return q0.reshape(self.shape), q1.reshape(self.shape)
 
     def fo_period(self, s0, f=None, g=None):
@@ -401,7 +407,6 @@ class Solver:
         sT = torch.empty_like(s0)
         self._after_caller()
         cmcg_fo_period(self.handle, s0, f, g, sT)
-        self._before_caller()
         return sT
 
     def fo_adjoint_period(self, y):
@@ -410,7 +415,6 @@ class Solver:
         out = torch.empty_like(y)
         self._after_caller()
         cmcg_fo_adjoint_period(self.handle, y, out)
-        self._before_caller()
         return out
 
     def riesz(self, rhs):
@@ -419,7 +423,6 @@ class Solver:
         s = torch.empty_like(rhs)
         self._after_caller()
         code = cmcg_riesz(self.handle, rhs, s)
-        self._before_caller()
         return s.reshape(self.shape), code
 
     def history(self):
@@ -438,7 +441,6 @@ class Solver:
         self._after_caller()
         code = (cmcg_solve(self.handle, f, g, tol, u, st) if u0 is None
                 else cmcg_solve_warm(self.handle, f, g, tol, u, st))
-        self._before_caller()
         out = st.as_dict()
         out["status"] = code
         return u.reshape(self.shape), out
