@@ -613,6 +613,27 @@ void forward_period(cmcg_handle* H, const double* w0, const double* w1, bool src
     fwd_end<T>(H, b, w1, src, mode, out0, out1);
 }
 
+// An FP32 period of FP64 data (mode 1): on 2D 5-point grids the source, the conversions and the start
+// values come from one kernel.  The stencils need u0 with zeros on the Dirichlet nodes (v0's entries
+// there are selected away).
+void source_period(cmcg_handle* H, const double* u0, const double* v0, bool src, const double* f, const double* g,
+                   double* uT, double* vT) {
+    const unsigned char* mask = H->has_dir ? H->mask : nullptr;
+    if (H->g.dim == 3 || H->order != 2) {
+        if (src) set_source(H, f, g);
+        launch_mask_copy<float>(H->g, u0, mask, (float*)H->tmp, H->st);
+        forward_period<float>(H, u0, v0, src, 1, uT, vT, true);
+        return;
+    }
+    Range range("cmcg forward period");
+    if (src) H->src_faces = !f;
+    PeriodBuffers b{H->yb, H->ya, nullptr};
+    launch_source_start(H->g, u0, mask, v0, (float*)b.prev, (float*)b.cur, H->kap32, src, f, g, H->kap64, H->S, H->S32, H->dt,
+                        H->st);
+    fwd_steps<float>(H, b, src);
+    fwd_end<float>(H, b, v0, src, 1, uT, vT);
+}
+
 // Adjoint (transposed) period of the cotangents (a, b).
 template <typename T>
 PeriodBuffers adj_begin(cmcg_handle* H, const double* a, const double* bb, int mode) {
@@ -1724,13 +1745,12 @@ int cmcg_wave_period(cmcg_handle* h, const double* u0, const double* v0, const d
     if (!h || !u0 || !v0 || !uT || !vT) return CMCG_ERR_INVALID_ARG;
     if (h->first_order) return CMCG_ERR_UNSUPPORTED;
     const bool src = f || g;
-    if (src) set_source(h, f, g);
     // the stencils need u0 with zeros on the Dirichlet nodes (v0's entries there are selected away
-    // by the start kernel); FP32 periods read it as the float copy of the temp buffer
+    // by the start kernel)
     if (h->opt.precision == CMCG_FP32) {
-        launch_mask_copy<float>(h->g, u0, h->has_dir ? h->mask : nullptr, (float*)h->tmp, h->st);
-        forward_period<float>(h, u0, v0, src, 1, uT, vT, true);
+        source_period(h, u0, v0, src, f, g, uT, vT);
     } else {
+        if (src) set_source(h, f, g);
         const double* w0 = u0;
         if (h->has_dir) {
             launch_mask_copy<double>(h->g, u0, h->mask, h->z0, h->st);

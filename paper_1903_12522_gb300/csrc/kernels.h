@@ -111,6 +111,11 @@ void launch_scale_complex(long long n, double* u, double s, cudaStream_t st);
 // scol (both nullable; scol must be zeroed before); accumulate: S += instead, without the copies.
 void launch_make_source(const Geom& g, const double* f, const double* gb, const double* kap64, double* S, float* S32,
                         unsigned char* scol, int zc, bool accumulate, cudaStream_t st);
+// A 2D 5-point FP32 period's start from FP64 data (u0, w1): with src the source as launch_make_source,
+// and y0, y1 as launch_start, u0 read as zero where mask (nullable) is set.
+void launch_source_start(const Geom& g, const double* u0, const unsigned char* mask, const double* w1, float* y0, float* y1,
+                         const float* kap, bool src, const double* f, const double* gb, const double* kap64, double* S,
+                         float* S32, double dt, cudaStream_t st);
 long long plane_blocks(const Geom& g, int zc);
 
 // ---- step_soft.cu -----------------------------------------------------------------------

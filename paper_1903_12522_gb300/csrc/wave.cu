@@ -875,6 +875,27 @@ __global__ void __launch_bounds__(kThreads, kEndMinBlocks<T>) k_adj_final(const 
     }
 }
 
+// The source at node j: kappa h^2 (f + (2 nb / h) g); a1..a3 = 2 nb / h for nb = 1..3.
+__device__ __forceinline__ double2 source_value(const Geom& g, const double* __restrict__ f, const double* __restrict__ gb,
+                                                const double* __restrict__ kap64, long long j, int ix, int iy, int iz,
+                                                double a1, double a2, double a3) {
+    const int nb = gb ? num_abc(g, ix, iy, iz) : 0;
+    if (!f && !nb) return make_double2(0.0, 0.0);
+    const double k = kap64[j];
+    const double sc = k * g.h * g.h;
+    double re = 0.0, im = 0.0;
+    if (f) {
+        re += f[2 * j];
+        im += f[2 * j + 1];
+    }
+    if (nb) {
+        const double a = nb == 1 ? a1 : (nb == 2 ? a2 : a3);
+        re += a * gb[2 * j];
+        im += a * gb[2 * j + 1];
+    }
+    return make_double2(sc * re, sc * im);
+}
+
 // S = dt^2 M^-1 (W f + A g) = kappa h^2 (f + (2 nb / h) g), zero on Dirichlet nodes (or added
 // to S when accumulating), its FP32 copy S32 (nullable) and the source columns scol (nullable,
 // zeroed by the caller): scol[x + sx y] = 1 if S != 0 at some node (x, y, z) with 0 < z < nz.
@@ -892,35 +913,64 @@ __global__ void __launch_bounds__(kThreads) k_make_source(const double* __restri
     long long j = node(g, m.ix, m.iy, m.z0);
     bool any = false;
     for (int iz = m.z0; iz < m.z1; ++iz, j += sZ) {
-        const int nb = gb ? num_abc(g, m.ix, m.iy, iz) : 0;
-        double sr = 0.0, si = 0.0;
-        if (f || nb) {
-            const double k = kap64[j];
-            const double sc = k * g.h * g.h;
-            double re = 0.0, im = 0.0;
-            if (f) {
-                re += f[2 * j];
-                im += f[2 * j + 1];
-            }
-            if (nb) {
-                const double a = nb == 1 ? a1 : (nb == 2 ? a2 : a3);
-                re += a * gb[2 * j];
-                im += a * gb[2 * j + 1];
-            }
-            sr = sc * re;
-            si = sc * im;
-            if (ACC) {
-                S[2 * j] += sr;
-                S[2 * j + 1] += si;
-            }
+        const double2 v = source_value(g, f, gb, kap64, j, m.ix, m.iy, iz, a1, a2, a3);
+        if (ACC) {
+            S[2 * j] += v.x;
+            S[2 * j + 1] += v.y;
+            continue;
         }
-        if (ACC) continue;
-        reinterpret_cast<double2*>(S)[j] = make_double2(sr, si);
-        if (S32) reinterpret_cast<float2*>(S32)[j] = make_float2(soft64::to_f32(sr), soft64::to_f32(si));
-        any |= iz > 0 && iz < g.nz && !(soft64::is_zero(sr) && soft64::is_zero(si));
+        reinterpret_cast<double2*>(S)[j] = v;
+        if (S32) reinterpret_cast<float2*>(S32)[j] = make_float2(soft64::to_f32(v.x), soft64::to_f32(v.y));
+        any |= iz > 0 && iz < g.nz && !(soft64::is_zero(v.x) && soft64::is_zero(v.y));
     }
     if (scol && any) scol[m.ix + (long long)g.sx * m.iy] = 1;
 }
+
+// u0 as the start's stencils read it: in the stepping precision, zero on Dirichlet nodes.
+struct LdStart {
+    const double* __restrict__ p;
+    const unsigned char* __restrict__ mask;
+    __device__ __forceinline__ float operator()(long long i) const {
+        const float v = soft64::to_f32(p[i]);
+        return mask && mask[i] ? 0.f : v;
+    }
+};
+
+// One FP32 period's start from FP64 data on a 2D 5-point grid in one pass: k_make_source (SRC), the
+// conversion of u0 and k_start, with the latter's roundings.  Bound: launches; as three of them they
+// were half of what a 129^2 period does beside its steps (92 us, 85 now; 1025^2 187 and 180).  In 3D
+// the neighbours' FP64 values and conversions cost more than the saved passes (257^3: 2471 us against
+// 2430), so it stays with three.
+template <bool SRC>
+__global__ void __launch_bounds__(kThreads) k_source_start(const double* __restrict__ u0, const unsigned char* __restrict__ mask,
+                                                           const double* __restrict__ w1, float* __restrict__ y0,
+                                                           float* __restrict__ y1, const float* __restrict__ kap,
+                                                           const double* __restrict__ f, const double* __restrict__ gb,
+                                                           const double* __restrict__ kap64, double* __restrict__ S,
+                                                           float* __restrict__ S32, Geom g, double dt, double a1, double a2,
+                                                           double a3) {
+    const PlaneMap m = plane_map(g, 1, 1);
+    if (!m.valid) return;
+    const LdStart ld{u0, mask};
+    const float dtT = (float)dt;
+    const long long j = node(g, m.ix, m.iy, 0);
+    const float k = kap[j];
+    const float L = lap_t<2, float>(g, ld, j, m.ix, m.iy, 0);
+    const int nbf = num_abc(g, m.ix, m.iy, 0);
+    const float beta = nbf ? (float)nbf * sqrt(k) : 0.f;
+    const float w0j = ld(j);
+    float v = w0j + dtT * (1.f - beta) * as_step<float>(w1[j]) - 0.5f * k * L;
+    if (SRC) {
+        const double2 s = source_value(g, f, gb, kap64, j, m.ix, m.iy, 0, a1, a2, a3);
+        reinterpret_cast<double2*>(S)[j] = s;
+        reinterpret_cast<float2*>(S32)[j] = make_float2(soft64::to_f32(s.x), soft64::to_f32(s.y));
+        if (nbf || f) v += as_step<float>(0.5 * s.x);
+    }
+    const bool dir = k == 0.f;
+    y0[j] = dir ? 0.f : w0j;
+    y1[j] = dir ? 0.f : v;
+}
+
 
 // ---------------------------------------------------------------------------------------
 // Batched persistent step loop: one cooperative launch advances the step loops of many solves
@@ -1346,6 +1396,17 @@ void launch_make_source(const Geom& g, const double* f, const double* gb, const 
         k_make_source<true><<<plane_grid(g, zc), kThreads, 0, st>>>(f, gb, kap64, S, nullptr, nullptr, g, zc, a1, a2, a3);
     else
         k_make_source<false><<<plane_grid(g, zc), kThreads, 0, st>>>(f, gb, kap64, S, S32, scol, g, zc, a1, a2, a3);
+}
+
+void launch_source_start(const Geom& g, const double* u0, const unsigned char* mask, const double* w1, float* y0, float* y1,
+                         const float* kap, bool src, const double* f, const double* gb, const double* kap64, double* S,
+                         float* S32, double dt, cudaStream_t st) {
+    note_launch(1);
+    auto go = [&](auto kernel) {
+        kernel<<<plane_grid(g, 1), kThreads, 0, st>>>(u0, mask, w1, y0, y1, kap, f, gb, kap64, S, S32, g, dt, 2.0 * 1 / g.h,
+                                                      2.0 * 2 / g.h, 2.0 * 3 / g.h);
+    };
+    src ? go(k_source_start<true>) : go(k_source_start<false>);
 }
 
 long long plane_blocks(const Geom& g, int zc) {
