@@ -123,6 +123,7 @@ size_t layout(cmcg_handle* H, const Geom& g, const cmcg_options& o, char* base) 
     H->mass32 = f32_copies ? c.take<float>(np) : nullptr;
     H->minv32 = f32_copies ? c.take<float>(np) : nullptr;
     H->scol = g.dim == 3 ? c.take<unsigned char>((size_t)g.sx * g.sy) : nullptr;
+    H->sflag = f32_copies && g.dim == 3 ? c.take<unsigned char>(source_flag_bytes(g)) : nullptr;
     if (o.flags & CMCG_FLAG_FIRST_ORDER) {
         // first-order state (p, v): CG vectors and the two stepping buffers; no Riesz map
         const size_t ns = (size_t)(g.dim + 1) * np;
@@ -259,8 +260,9 @@ void set_source(cmcg_handle* H, const double* f, const double* g) {
     const Geom& G = H->g;
     H->src_faces = !f;
     if (H->scol) cudaMemsetAsync(H->scol, 0, (size_t)G.sx * G.sy, H->st);
+    if (H->sflag) cudaMemsetAsync(H->sflag, 0, source_flag_bytes(G), H->st);
     if (f || g) {
-        launch_make_source(G, f, g, H->kap64, H->S, H->S32, H->scol, G.dim == 3 ? kZcEnds : 1, false, H->st);
+        launch_make_source(G, f, g, H->kap64, H->S, H->S32, H->scol, H->sflag, G.dim == 3 ? kZcEnds : 1, false, H->st);
     } else {
         cudaMemsetAsync(H->S, 0, sizeof(double) * 2 * G.np, H->st);
         if (H->S32) cudaMemsetAsync(H->S32, 0, sizeof(float) * 2 * G.np, H->st);
@@ -270,6 +272,7 @@ void set_source(cmcg_handle* H, const double* f, const double* g) {
 void source_updated(cmcg_handle* H) {
     if (H->S32) launch_to_float(2 * H->g.np, H->S, H->S32, H->st);
     if (H->scol) launch_source_columns(H->g, H->S, H->scol, H->st);
+    if (H->sflag) launch_source_flags(H->g, H->S32, H->sflag, H->st);
 }
 
 // Fold completed event pairs into the per-precision step times.
@@ -457,7 +460,7 @@ bool band_steps(cmcg_handle* H, PeriodBuffers& b, long long count, bool src, boo
         for (int s = 0; src && s < m; ++s) factors(n0 + s, &cs[s], &sn[s]);
         const bool a0 = adjoint && n0 == 0, a1 = adjoint && n0 + m == count;
         const cudaError_t e =
-            block ? launch_step_block(H->g, H->block, (float*)b.cur, (float*)b.prev, H->kap32, (const float*)S, H->scol,
+            block ? launch_step_block(H->g, H->block, (float*)b.cur, (float*)b.prev, H->kap32, (const float*)S, H->sflag,
                                       H->src_faces, H->band_words, H->band_count, H->hsc + SC_COUNT, m, cs, sn, a0, a1,
                                       H->st)
                   : launch_step_band<T>(H->g, H->order, band, (T*)b.cur, (T*)b.prev, kap, S, H->src_faces, H->wface,
@@ -489,7 +492,7 @@ bool row_steps(cmcg_handle* H, PeriodBuffers& b, long long count, bool src, bool
     a.kap = H->row_kap;
     a.S = src ? H->S32 : nullptr;
     a.src_faces = H->src_faces;
-    a.scol = H->scol;
+    a.sflag = H->sflag;
     float *cur = H->row_a, *prev = H->row_b;
     const int tp = timing_begin(H, true, (int)std::min<long long>(count, INT32_MAX));
     for (long long n = 0; n < count; ++n) {
@@ -1554,7 +1557,7 @@ int wave_period_in_scratch(const cmcg_grid* grid, const double* c, double omega,
     launch_face_weights(H.g, H.kap64, H.wface, st);
     const bool src = f || g;
     const int zce = H.g.dim == 3 ? kZcEnds : 1;
-    if (src) launch_make_source(H.g, f, g, H.kap64, H.S, nullptr, nullptr, zce, false, st);
+    if (src) launch_make_source(H.g, f, g, H.kap64, H.S, nullptr, nullptr, nullptr, zce, false, st);
     H.src_faces = !f;
     launch_mask_copy<double>(H.g, u0, H.has_dir ? H.mask : nullptr, H.z0, st);
     forward_period<double>(&H, H.z0, v0, src, 1, uT, vT);  // the start kernel selects v0's Dirichlet entries
@@ -1861,11 +1864,11 @@ int cmcg_solve_host(cmcg_handle* h, const double* f_host, const double* g_host, 
     launch_fill(h->S, 2 * n, 0.0, h->st);
     if (f_host) {
         cudaMemcpyAsync(h->stage, f_host, bytes, cudaMemcpyHostToDevice, h->st);
-        launch_make_source(h->g, h->stage, nullptr, h->kap64, h->S, nullptr, nullptr, zce, true, h->st);
+        launch_make_source(h->g, h->stage, nullptr, h->kap64, h->S, nullptr, nullptr, nullptr, zce, true, h->st);
     }
     if (g_host) {
         cudaMemcpyAsync(h->stage, g_host, bytes, cudaMemcpyHostToDevice, h->st);
-        launch_make_source(h->g, nullptr, h->stage, h->kap64, h->S, nullptr, nullptr, zce, true, h->st);
+        launch_make_source(h->g, nullptr, h->stage, h->kap64, h->S, nullptr, nullptr, nullptr, zce, true, h->st);
     }
     h->src_faces = !f_host;
     source_updated(h);

@@ -108,9 +108,13 @@ void launch_step_filter(const Geom& g, int order, const double* cur, double* pre
                         cudaStream_t st);
 void launch_scale_complex(long long n, double* u, double s, cudaStream_t st);
 // The source array S from f and g (either nullable), with its FP32 copy S32 and the source columns
-// scol (both nullable; scol must be zeroed before); accumulate: S += instead, without the copies.
+// scol and flags sflag (all nullable; scol and sflag must be zeroed before, sflag with zc a multiple of
+// 4); accumulate: S += instead, without the copies.
 void launch_make_source(const Geom& g, const double* f, const double* gb, const double* kap64, double* S, float* S32,
-                        unsigned char* scol, int zc, bool accumulate, cudaStream_t st);
+                        unsigned char* scol, unsigned char* sflag, int zc, bool accumulate, cudaStream_t st);
+// sflag of S32 (3D): a byte per four nodes of a row and four planes, z-major
+size_t source_flag_bytes(const Geom& g);
+void launch_source_flags(const Geom& g, const float* S32, unsigned char* sflag, cudaStream_t st);
 // A 2D 5-point FP32 period's start from FP64 data (u0, w1): with src the source as launch_make_source,
 // and y0, y1 as launch_start, u0 read as zero where mask (nullable) is set.
 void launch_source_start(const Geom& g, const double* u0, const unsigned char* mask, const double* w1, float* y0, float* y1,
@@ -192,9 +196,9 @@ struct BlockPlan {
     size_t smem = 0, words = 0;        // shared memory per block; exchange words (8 bytes each)
 };
 bool block_plan(const Geom& g, int sms, BlockPlan* p);
-// As launch_step_band; scol as in launch_step.
+// As launch_step_band; sflag of S.
 cudaError_t launch_step_block(const Geom& g, const BlockPlan& p, float* cur, float* prev, const float* kap, const float* S,
-                              const unsigned char* scol, bool src_faces, unsigned long long* words, unsigned* count,
+                              const unsigned char* sflag, bool src_faces, unsigned long long* words, unsigned* count,
                               double* err, int nsteps, const double* cs, const double* sn, bool adj_first, bool adj_last,
                               cudaStream_t st);
 
@@ -211,7 +215,7 @@ struct RowStep {
     double cs, sn;
     bool src_faces;
     int reverse;
-    const unsigned char* scol;
+    const unsigned char* sflag;  // of S
 };
 int row_pitch(const Geom& g);
 bool row_fits(const Geom& g);

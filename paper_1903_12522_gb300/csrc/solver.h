@@ -52,6 +52,7 @@ struct cmcg_handle {
     int coarse_level = -1;    // first level of the V-cycle's coarse end in one launch (-1: none)
     CoarseLevels coarse{};
     int riesz_guess = 0;      // PCG iterations of the previous Riesz solve
+    unsigned char* sflag = nullptr;  // 3D FP32 steps: where S32 is not zero (launch_source_flags)
     // FP32 3D step loops on padded rows (step_row.cu): the two wave fields and kappa
     float *row_a = nullptr, *row_b = nullptr, *row_kap = nullptr;
     // step loops in one launch, 2D (step_band.cu) and FP32 3D 7-point (step_block.cu): exchange_words

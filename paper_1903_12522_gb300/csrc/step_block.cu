@@ -40,7 +40,7 @@ struct BlockArgs {
     float* buf1;
     const float* kap;
     const float* S;
-    const unsigned char* scol;  // columns of nodes with sources inside the grid (or null)
+    const unsigned char* sflag;  // where there are sources (launch_source_flags)
     unsigned long long* words;
     unsigned* count;  // per block: steps done in all launches so far; [kBandStop]: stop word
     double* err;
@@ -235,10 +235,7 @@ __global__ void __launch_bounds__(kBT, 1) k_block3(const __grid_constant__ Block
                 f |= (unsigned)(slot + 1) << kSlotShift | (unsigned)nby << kFacesShift | (left ? kLeft : 0u) | (right ? kRight : 0u);
             }
             bool source = SRC == 1 && (f >> kSlotShift);
-            if (SRC == 2) {
-                source = !a.scol || z == 0 || z == g.nz;
-                for (int e = 0; e < m && !source; ++e) source = a.scol[x0 + e + sx * y] != 0;
-            }
+            if (SRC == 2) source = a.sflag[((long long)(z >> 2) * g.sy + y) * cx + ic] != 0;
             fl[q] = f | (source ? kSource : 0u);
         }
     }
@@ -483,7 +480,7 @@ bool block_plan(const Geom& g, int sms, BlockPlan* p) {
 }
 
 cudaError_t launch_step_block(const Geom& g, const BlockPlan& p, float* cur, float* prev, const float* kap, const float* S,
-                              const unsigned char* scol, bool src_faces, unsigned long long* words, unsigned* count,
+                              const unsigned char* sflag, bool src_faces, unsigned long long* words, unsigned* count,
                               double* err, int nsteps, const double* cs, const double* sn, bool adj_first, bool adj_last,
                               cudaStream_t st) {
     BlockArgs a;
@@ -491,7 +488,7 @@ cudaError_t launch_step_block(const Geom& g, const BlockPlan& p, float* cur, flo
     a.buf1 = prev;
     a.kap = kap;
     a.S = S;
-    a.scol = scol;
+    a.sflag = sflag;
     a.words = words;
     a.count = count;
     a.err = err;

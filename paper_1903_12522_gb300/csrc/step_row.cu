@@ -72,7 +72,7 @@ template <int ORDER, int FLAGS, bool SRC_FACES, int FLAT>
 __global__ void __launch_bounds__(kRT, ORDER == 2 ? 10 : 7)
     k_step_row(const float* __restrict__ cur, const float* prev, float* pout, float* pcopy,  // pout may be prev
                const float* __restrict__ kap, const float* __restrict__ S, float cs, float sn,
-               Geom g, int px, int zc, int reverse, const unsigned char* __restrict__ scol) {
+               Geom g, int px, int zc, int reverse, const unsigned char* __restrict__ sflag) {
     const int cx = px >> 2, plane4 = cx * g.sy;
     const int bx = reverse ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
     const int by = reverse ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
@@ -96,10 +96,7 @@ __global__ void __launch_bounds__(kRT, ORDER == 2 ? 10 : 7)
     const bool needl = lane == 0 && !first, needr = lane == 31 && xe >= 4;
     const int nby = (iy == 0 ? (int)((g.abc >> 2) & 1u) : 0) + (iy == g.ny ? (int)((g.abc >> 3) & 1u) : 0);
     const int nbl = first ? (int)(g.abc & 1u) : 0, nbr = xe < 4 ? (int)((g.abc >> 1) & 1u) : 0;
-    bool vol = false;  // a source inside the grid in one of the four columns
-    if ((FLAGS & kStepSrc) && !SRC_FACES) {
-        for (int e = 0; e < m; ++e) vol = vol || !scol || scol[x0 + e + g.sx * iy];
-    }
+    bool vol = false;  // a source in one of the four columns in these four planes
     auto get = [&](const float* f, int j) -> V4 {
         if constexpr (FLAT != 1) {
             return load4(f + j);
@@ -129,6 +126,7 @@ __global__ void __launch_bounds__(kRT, ORDER == 2 ? 10 : 7)
         zp = get(cur, ji + (int)off_p1(z0, g.nz, isZ));
     }
     for (int iz = z0; iz < z1; ++iz) {
+        if ((FLAGS & kStepSrc) && !SRC_FACES && (iz == z0 || (iz & 3) == 0)) vol = sflag[(iz >> 2) * plane4 + pp] != 0;
         V4 zp2{};
         if (ORDER == 2) zp = get(cur, ji + (int)off_p1(iz, g.nz, isZ));
         else zp2 = get(cur, ji + (int)off_p2(iz, g.nz, isZ));
@@ -188,7 +186,7 @@ __global__ void __launch_bounds__(kRT, ORDER == 2 ? 10 : 7)
             rb = fma2(k.b, Lb, add2(c.b, c.b));
         }
         const int nbz = (iz == 0 ? (int)((g.abc >> 4) & 1u) : 0) + (iz == g.nz ? (int)((g.abc >> 5) & 1u) : 0);
-        if ((FLAGS & kStepSrc) && !SRC_FACES && (vol || iz == 0 || iz == g.nz)) {
+        if ((FLAGS & kStepSrc) && !SRC_FACES && vol) {
             float t[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -270,7 +268,7 @@ void row_launch(const RowStep& a, cudaStream_t st) {
     const dim3 grid(bxy, (unsigned)((g.sz + zc - 1) / zc));
     const float cs = (float)a.cs, sn = (float)a.sn;
     auto go = [&](auto kernel) {
-        kernel<<<grid, kRT, 0, st>>>(a.cur, a.prev, a.out, a.copy, a.kap, a.S, cs, sn, g, a.px, zc, a.reverse, a.scol);
+        kernel<<<grid, kRT, 0, st>>>(a.cur, a.prev, a.out, a.copy, a.kap, a.S, cs, sn, g, a.px, zc, a.reverse, a.sflag);
     };
     if (a.flat == 0) go(k_step_row<ORDER, FLAGS, SRC_FACES, 0>);
     else if (a.flat == 1) go(k_step_row<ORDER, FLAGS, SRC_FACES, 1>);

@@ -62,3 +62,26 @@ def test_loops_of_one_and_two_steps(steps):
     b = periods((17, 9, 12), 2, (0,) * 6, (0, 0, 0, 0), 1, 1, steps=steps)
     for x, y in zip(a, b):
         assert torch.equal(x, y)
+
+
+@pytest.mark.parametrize("order", [2, 4])
+@pytest.mark.parametrize("n", [(33, 30, 29), (9, 5, 7), (130, 21, 12), (301, 90, 101)])
+def test_sources_at_a_few_nodes(n, order):
+    # corners, the last planes, single nodes inside, and values that are zero in FP32
+    shape = tuple(m + 1 for m in reversed(n))
+    f = torch.zeros(shape, dtype=torch.complex128, device="cuda")
+    for z, y, x in ((0, 0, 0), (-1, -1, -1), (n[2] // 2, 1, n[0] // 2), (n[2] - 1, n[1] // 2, 3), (3, 2, n[0] - 1), (4, n[1], 4)):
+        f[z, y, x] = 3e3 - 2e3j
+    f[f == 0] = 1e-60
+    h = 1.0 / max(n)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(5)
+    y = torch.randn(shape, generator=gen, device="cuda", dtype=torch.float64)
+    out = []
+    for tile in ((16, 0, 0, 3), (0, 0, 0, 0)):
+        s = cmcg.Solver(n, h, torch.ones_like(y), 2 * math.pi / (10 * h), (0,) * 6, precision=cmcg.FP32, order=order, tile=tile,
+                        dt=0.3 * h)
+        out.append([*s.wave_period(y, y, f, f), *s.wave_period(y, y, None, None), *s.wave_period(y, y, f, None)])
+        s.close()
+    for a, b in zip(*out):
+        assert torch.equal(a, b)
