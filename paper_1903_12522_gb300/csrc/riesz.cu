@@ -1192,9 +1192,17 @@ void launch_mg_coarsen_mask(const MGLevel& fine, const MGLevel& coarse, cudaStre
     k_coarsen_mask<<<node_blocks(coarse.g.np), kT, 0, st>>>(fine.g, fine.mask, coarse.g, coarse.mask);
 }
 
-// z-planes per thread of the 3D level kernels: eight, or fewer where eight leave less than one wave
-// of blocks (65^3: a sweep takes 4.3 us with two planes, 6.0 with eight; 129^3: 12.2 and 10.5).
+// z-planes per thread of the 3D level kernels.  Sweeps and residuals: as many as make one wave of
+// blocks, 2 to 16 (129^3: a sweep takes 9.3 us with ten planes, 10.4 with eight, whose second wave is
+// a fifth full, 12.2 with two; 65^3: 4.3 with two, 6.0 with eight).  Prolongation, whose threads
+// reuse the coarse planes between pairs of fine ones: eight, or fewer where eight leave less than
+// one wave (129^3: 13.7 us, with ten 15.2).
 static int mg_zc(const Geom& g) {
+    if (g.dim != 3) return 1;
+    const long long bxy = ((long long)g.sx * g.sy + kT - 1) / kT;
+    return (int)std::min(16ll, std::max(2ll, (bxy * g.sz + 152 * 6 - 1) / (152 * 6)));
+}
+static int mg_zc_prolong(const Geom& g) {
     if (g.dim != 3) return 1;
     const long long bxy = ((long long)g.sx * g.sy + kT - 1) / kT;
     int zc = 8;
@@ -1240,7 +1248,7 @@ void launch_mg_restrict(const MGLevel& fine, const float* rf, const MGLevel& coa
 
 void launch_mg_prolong_add(const MGLevel& coarse, const float* xc, const MGLevel& fine, float* xf, cudaStream_t st) {
     note_launch(1);
-    const int zc = mg_zc(fine.g);
+    const int zc = mg_zc_prolong(fine.g);
     if (fine.g.dim == 3)
         k_prolong_add3<<<mg_grid(fine.g, zc), kT, 0, st>>>(coarse.g, xc, fine.g, fine.mask, xf, zc);
     else
