@@ -882,15 +882,21 @@ int riesz_solve(cmcg_handle* H, const double* rhs, double* x, int* iters_out) {
         launch_pcg_dots_after_precond(n, H->pr, H->lv[0].x, first ? nullptr : H->pAp, H->pzd, red, H->st);
         launch_pcg_p_update(n, H->pp, H->pzd, red, first, H->st);
     };
+    // small grids: an iteration's vector part, from z on, in one launch
+    const bool small = fast && pcg_cluster_fits(g);
     if (!fast) launch_fill(x, n, 0.0, H->st);
-    direction(true);
+    if (small) launch_to_float(n, H->pr, zf, H->st);
+    else direction(true);
     int it = 0;
     bool converged = false;
     double bb = -1.0;
     // the previous solve's iteration count, less a margin, runs without host checks
     const int blind = std::max(0, std::min(H->riesz_guess - 2, H->opt.riesz_max_iter - 1));
     for (it = 1; it <= H->opt.riesz_max_iter; ++it) {
-        if (fast) {
+        if (small) {
+            vcycle(H, 0);
+            launch_pcg_cluster(g, H->order, H->mask, x, H->pr, H->pp, H->pAp, H->lv[0].x, zf, red, it == 1, H->st);
+        } else if (fast) {
             launch_pcg_applyK(g, H->order, H->mask, H->pp, H->pAp, red, zce, H->st);
             launch_pcg_xr(n, x, H->pr, H->pp, H->pAp, zf, red, it == 1, H->st);
         } else {
@@ -898,7 +904,7 @@ int riesz_solve(cmcg_handle* H, const double* rhs, double* x, int* iters_out) {
             launch_pcg_xr_update(n, x, H->pr, H->pp, H->pAp, red, H->st);
         }
         if (it <= blind) {
-            direction(false);
+            if (!small) direction(false);
             continue;
         }
         int rc = sync_read(H);
@@ -910,7 +916,7 @@ int riesz_solve(cmcg_handle* H, const double* rhs, double* x, int* iters_out) {
             converged = true;
             break;
         }
-        direction(false);
+        if (!small) direction(false);
     }
     if (project) launch_mean_remove(g, x, H->volume, red, H->st);
     if (converged) H->riesz_guess = it;

@@ -187,6 +187,12 @@ void launch_pcg_xr(long long n, double* x, double* r, const double* p, const dou
                    cudaStream_t st);  // SC_P_RR; first: x starts at zero
 void launch_pcg_dots(long long n, const double* r, const float* z, const double* Ap, Red red, cudaStream_t st);
 void launch_pcg_p(long long n, double* p, const float* z, Red red, bool first, cudaStream_t st);
+// All four for one iteration in one cluster launch (grids of up to kPcgClusterNodes nodes, three per
+// thread): from z = B r to the next residual and bf.  first: p and x start at zero.
+constexpr long long kPcgClusterNodes = 36864;
+bool pcg_cluster_fits(const Geom& g);
+void launch_pcg_cluster(const Geom& g, int order, const unsigned char* mask, double* x, double* r, double* p, double* Ap,
+                        const float* z, float* bf, Red red, bool first, cudaStream_t st);
 
 // ---- step_block.cu ----------------------------------------------------------------------
 // FP32 3D 7-point step loops in one cooperative launch, the grid held on chip in blocks of x rows.

@@ -561,6 +561,143 @@ __global__ void __launch_bounds__(kST, 4) k_pcg_p(long long n, double* __restric
     });
 }
 
+// One PCG iteration's vector part in one launch of one thread-block cluster, for grids of up to
+// kPcgClusterNodes nodes: beta from r . z and z . Ap, p, Ap, alpha, x and r, with cluster barriers in
+// place of launches.  The sums are those of the passes above in another order.
+//
+// Bound: latency and the FP64 pipe of 16 SMs.  Neighbours' p comes from L2 (__ldcg: another CTA wrote
+// it).  As four launches the part costs 22 us whatever the size, here 14 at 129^2.  Whole Riesz maps:
+// 65^2 680 and 568 us, 129^2 740 and 672, 191^2 1036 and 981, 33^3 1084 and 958; with four to six
+// nodes per thread, past 36864 nodes, no gain (226x241 1103 and 1102).
+constexpr int kClusterThreads = 768;  // 85 registers, which the stencil sum needs
+constexpr int kClusterCtas = 16;
+
+struct Latest {  // values that other CTAs may have written in this launch
+    const double* p;
+    __device__ __forceinline__ double operator()(int i) const { return __ldcg(p + i); }
+};
+
+__device__ __forceinline__ void pcg_cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// The cluster's totals of v in every thread.  slots: room for the CTAs' sums, not used by the call
+// before (another CTA may still read those).
+template <int NV>
+__device__ __forceinline__ void cluster_total(double (&v)[NV], double (*part)[kClusterThreads], double (*slots)[kClusterCtas]) {
+    const int tid = (int)threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < NV; ++k) part[k][tid] = v[k];
+    __syncthreads();
+    if (tid < 32) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            double x = 0.0;
+#pragma unroll
+            for (int q = 0; q < kClusterThreads / 32; ++q) x += part[k][tid + 32 * q];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            if (tid < kClusterCtas) {
+                const unsigned here = (unsigned)__cvta_generic_to_shared(&slots[k][blockIdx.x]);
+                unsigned there;
+                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(here), "r"(tid));
+                asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there), "d"(x) : "memory");
+            }
+        }
+    }
+    pcg_cluster_sync();
+    if (tid < 32) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            double x = slots[k][tid & (kClusterCtas - 1)];
+#pragma unroll
+            for (int o = kClusterCtas / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            if (tid == 0) part[k][0] = x;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < NV; ++k) v[k] = part[k][0];
+}
+
+// NPT nodes per thread at most, whose values stay in registers.
+template <int DIM, int ORDER, int NPT>
+__global__ void __launch_bounds__(kClusterThreads, 1)
+    k_pcg_cluster(double* __restrict__ x, double* __restrict__ r, double* p, double* __restrict__ Ap,
+                  const float* __restrict__ z, float* __restrict__ bf, const unsigned char* __restrict__ mask,
+                  double* __restrict__ sc, Geom g, double ck, int first) {
+    __shared__ double part[2][kClusterThreads];
+    __shared__ double slots[3][2][kClusterCtas];
+    const int n = (int)g.np, chunk = (n + kClusterCtas - 1) / kClusterCtas;
+    const int lo = min((int)blockIdx.x * chunk, n), hi = min(lo + chunk, n), t0 = lo + (int)threadIdx.x;
+    const double rz_old = sc[SC_P_RZ], alpha_old = sc[SC_P_ALPHA];
+    double zv[NPT], rv[NPT], pv[NPT], av[NPT], xv[NPT], rz[2] = {0.0, 0.0};
+#pragma unroll
+    for (int q = 0; q < NPT; ++q) {
+        const int j = t0 + q * kClusterThreads;
+        zv[q] = rv[q] = pv[q] = av[q] = xv[q] = 0.0;
+        if (j < hi) {
+            zv[q] = soft64::to_f64(z[j]);
+            rv[q] = r[j];
+            if (!first) av[q] = Ap[j], pv[q] = p[j], xv[q] = x[j];
+        }
+    }
+    pcg_cluster_sync();  // every CTA has started
+#pragma unroll
+    for (int q = 0; q < NPT; ++q) {
+        rz[0] = fma(rv[q], zv[q], rz[0]);
+        if (!first) rz[1] = fma(av[q], zv[q], rz[1]);
+    }
+    cluster_total<2>(rz, part, slots[0]);
+    const double beta = first || rz_old == 0.0 ? 0.0 : -alpha_old * rz[1] / rz_old;
+#pragma unroll
+    for (int q = 0; q < NPT; ++q) {
+        const int j = t0 + q * kClusterThreads;
+        pv[q] = first ? zv[q] : fma(beta, pv[q], zv[q]);
+        if (j < hi) p[j] = pv[q];
+    }
+    pcg_cluster_sync();
+    double pap[1] = {0.0};
+#pragma unroll
+    for (int q = 0; q < NPT; ++q) {
+        const int j = t0 + q * kClusterThreads;
+        if (j >= hi) continue;
+        const unsigned t = (unsigned)j / (unsigned)g.sx;
+        const int ix = j - (int)t * g.sx, iz = DIM == 3 ? (int)(t / (unsigned)g.sy) : 0, iy = (int)t - iz * g.sy;
+        SoftLap<DIM, ORDER, Latest> lap(Latest{p}, g, ix, iy);
+        double pj;
+        lap.start(j, iz);
+        const double L = lap.next(j, iz, &pj);
+        int ends = (ix == 0 || ix == g.nx) + (iy == 0 || iy == g.ny);
+        if (DIM == 3) ends += (iz == 0 || iz == g.nz);
+        const double c = __hiloint2double(__double2hiint(ck) - (ends << 20), __double2loint(ck));
+        av[q] = mask && mask[j] ? 0.0 : c * L;
+        Ap[j] = av[q];
+        pap[0] = fma(pv[q], av[q], pap[0]);
+    }
+    cluster_total<1>(pap, part, slots[1]);
+    const double alpha = pap[0] != 0.0 ? rz[0] / pap[0] : 0.0;  // p = 0 only for a zero residual
+    double rr[1] = {0.0};
+#pragma unroll
+    for (int q = 0; q < NPT; ++q) {
+        const int j = t0 + q * kClusterThreads;
+        if (j >= hi) continue;
+        x[j] = fma(alpha, pv[q], xv[q]);
+        const double v = fma(-alpha, av[q], rv[q]);
+        r[j] = v;
+        bf[j] = soft64::to_f32(v);
+        rr[0] = fma(v, v, rr[0]);
+    }
+    cluster_total<1>(rr, part, slots[2]);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        sc[SC_P_BETA] = beta;
+        sc[SC_P_RZ] = rz[0];
+        sc[SC_P_PAP] = pap[0];
+        sc[SC_P_ALPHA] = alpha;
+        sc[SC_P_RR] = rr[0];
+    }
+}
+
 // w = 1 / (1 + beta) on the nodes of absorbing faces (other entries are not read).
 __global__ void __launch_bounds__(kST) k_face_weights(Geom g, const double* __restrict__ kap, double* __restrict__ w) {
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -733,6 +870,35 @@ void launch_pcg_xr(long long n, double* x, double* r, const double* p, const dou
     note_launch(1);
     if (((uintptr_t)x & 15u) == 0) k_pcg_xr<true><<<pcg_blocks(n), kST, 0, st>>>(n, x, r, p, Ap, bf, red, first);
     else k_pcg_xr<false><<<pcg_blocks(n), kST, 0, st>>>(n, x, r, p, Ap, bf, red, first);
+}
+
+// Grids of up to kPcgClusterNodes nodes (see there).
+bool pcg_cluster_fits(const Geom& g) { return g.np <= kPcgClusterNodes; }
+
+void launch_pcg_cluster(const Geom& g, int order, const unsigned char* mask, double* x, double* r, double* p, double* Ap,
+                        const float* z, float* bf, Red red, bool first, cudaStream_t st) {
+    const double ck = -h_pow(g);
+    auto go = [&](auto kernel) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(kClusterCtas);
+        cfg.blockDim = dim3(kClusterThreads);
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = kClusterCtas;
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return;
+        cudaLaunchKernelEx(&cfg, kernel, x, r, p, Ap, z, bf, mask, red.sc, g, ck, first ? 1 : 0);
+    };
+    const bool two = g.np <= 2ll * kClusterCtas * kClusterThreads;
+    static_assert(3ll * kClusterCtas * kClusterThreads >= kPcgClusterNodes, "nodes per thread");
+    by_stencil(g, order, [&](auto D, auto O) {
+        if (two) go(k_pcg_cluster<D(), O(), 2>);
+        else go(k_pcg_cluster<D(), O(), 3>);
+    });
 }
 
 void launch_pcg_dots(long long n, const double* r, const float* z, const double* Ap, Red red, cudaStream_t st) {
