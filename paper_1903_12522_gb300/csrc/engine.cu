@@ -44,6 +44,8 @@ struct EngineSlot {
     // batched loops, 0.55 ms with loops of their own; the whole run 7.4 and 4.4 ms.  (The 9-point
     // steps round differently in the batched kernel: they stay there.)
     bool own = false;
+    // 2D 5-point grids past a cluster whose loops the whole chip holds (step_band.cu)
+    bool whole = false;
     int status = CMCG_OK;
     int iters = 0, inner_iters = 0, outer = 0;
     long long periods = 0, riesz = 0;  // counted per tick (graph replays skip the launch-time counters)
@@ -193,6 +195,12 @@ void inner_update(cmcg_handle* h, const PeriodBuffers& b) {
     launch_cg_direction(n, h->r0, h->r1, h->d0, h->d1, h->red(), h->st, nullptr, h->vec32);
 }
 
+// Loops that each fill the chip run one after the other instead of batched, up to this many: an engine
+// run of five iterations takes 3.7 ms with one 901^2 slot (batched 5.4), 4.9 with a 508^2 slot beside
+// two smaller ones (6.4), 9.4 with four of 601^2 to 1001^2 (12.6), 8.0 with five of 461^2 (8.2), but 14.5
+// with eight of 471^2 (13.6).
+constexpr int kWholeSlots = 5;
+
 // Enqueue one tick on the engine's stream (also used while capturing).
 cudaError_t enqueue_tick(cmcg_engine* e, const std::vector<int>& act) {
     cudaMemsetAsync(e->err, 0, sizeof(int), e->st);
@@ -268,7 +276,19 @@ cudaError_t enqueue_tick(cmcg_engine* e, const std::vector<int>& act) {
             fork_sides(e);
         }
         const int m = (int)inner.size();
+        const bool whole = m <= kWholeSlots && std::all_of(inner.begin(), inner.end(), [e](int s) { return e->slots[s].whole; });
         std::vector<PeriodBuffers> fb(m), ab(m);
+        auto whole_loops = [&](std::vector<PeriodBuffers> bufs, bool adjoint) {
+            for (int i = 0; i < m; ++i) {
+                cmcg_handle* h = e->slots[inner[i]].h;  // (its stream is the engine's)
+                const bool timing = h->timing;
+                h->timing = false;
+                if (adjoint) adj_steps<float>(h, bufs[i]);
+                else fwd_steps<float>(h, bufs[i], false);
+                h->timing = timing;
+            }
+            return cudaPeekAtLastError();
+        };
         // forward periods from d: start kernels, one batched step loop, end kernels
         int total = 0, maxs = 0;
         std::vector<BatchItem> items(2 * (size_t)m);
@@ -285,7 +305,8 @@ cudaError_t enqueue_tick(cmcg_engine* e, const std::vector<int>& act) {
             maxs = std::max(maxs, items[i].nsteps);
         }
         join_sides(e);  // the cooperative kernel runs alone: all its blocks are co-resident
-        cudaError_t ce = launch_batch_steps(e->items_dev, m, total, maxs, e->bar, e->err, e->grid, e->st);
+        cudaError_t ce = whole ? whole_loops(fb, false)
+                               : launch_batch_steps(e->items_dev, m, total, maxs, e->bar, e->err, e->grid, e->st);
         if (ce != cudaSuccess) return ce;
         fork_sides(e);
         int total_a = 0, maxa = 0;
@@ -303,7 +324,8 @@ cudaError_t enqueue_tick(cmcg_engine* e, const std::vector<int>& act) {
             maxa = std::max(maxa, items[m + i].nsteps);
         }
         join_sides(e);
-        ce = launch_batch_steps(e->items_dev + e->max_slots, m, total_a, maxa, e->bar, e->err, e->grid, e->st);
+        ce = whole ? whole_loops(ab, true)
+                   : launch_batch_steps(e->items_dev + e->max_slots, m, total_a, maxa, e->bar, e->err, e->grid, e->st);
         if (ce != cudaSuccess) return ce;
         fork_sides(e);
         for (int i = 0; i < m; ++i) {
@@ -493,6 +515,7 @@ int cmcg_engine_submit(cmcg_engine* e, cmcg_handle* h, const double* f, const do
     sl = EngineSlot();
     sl.h = h;
     sl.own = h->side.bands > 0 && h->order == 2;
+    sl.whole = !sl.own && h->band.bands > 0 && h->order == 2 && h->g.dim == 2;
     sl.submission = ++e->submissions;
     sl.u = u;
     sl.tol = tol;
@@ -609,7 +632,7 @@ int cmcg_engine_tick(cmcg_engine* e, int* finished, int max_finished, int* n_fin
         }
         sl.periods += 2;  // every other unit runs one forward and one adjoint period
         sl.riesz += 1;    // and one approximate Riesz map
-        const bool late = band_status(h) != CMCG_OK || (timeout && sl.unit == U_INNER && !sl.own);
+        const bool late = band_status(h) != CMCG_OK || (timeout && sl.unit == U_INNER && !sl.own);  // (the batched kernel's)
         any_late |= late;
         if (late) {
             sl.status = CMCG_ERR_DEVICE_TIMEOUT;
