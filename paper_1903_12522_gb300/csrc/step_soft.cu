@@ -181,10 +181,14 @@ struct SoftLap {
 //
 // Bound: issue slots of the integer pipes and latency (FP64 work left per update: 2 y - y_prev
 // and the fused multiply-add with kappa, against nine operations and, on the faces, a square
-// root and a division).  193^3, with a source on the faces: 246 us a step in FP64 arithmetic, 98 us
-// now (230 MB of algorithmic bytes, 34 us at the copy bandwidth); 257^3: 424 and 182 us.
-template <int DIM, int ORDER, int FLAGS, bool SRC_FACES>
-__global__ void __launch_bounds__(kST, ORDER == 2 ? 4 : 3)
+// root and a division).  193^3, with a source on the faces: 246 us a step in FP64 arithmetic, 87 us
+// now, 73 without one (230 MB of algorithmic bytes, 34 us at the copy bandwidth).
+//
+// B: resident blocks per SM.  Whole backward periods of 57 steps: 7-point 193^3 4.66 ms with four, 4.47
+// with five, 4.19 with six (40 registers, a few spills); 177x171x151 2.98, 2.93, 2.80; 129^3 1.67, 1.62,
+// 1.68.  13-point 151x141x131 2.83 ms with three, 2.70 with four, 2.93 with five.
+template <int DIM, int ORDER, int FLAGS, bool SRC_FACES, int B>
+__global__ void __launch_bounds__(kST, B)
     k_step_soft(const double* __restrict__ cur, double* __restrict__ prev_out, const double* __restrict__ kap,
                 const double* __restrict__ wface, const double* __restrict__ S, double cs, double sn, Geom g, int zc,
                 int reverse) {
@@ -721,15 +725,31 @@ int soft_zc(const Geom& g, int per_sm) {
     return zc;
 }
 
+template <int DIM, int ORDER, int FLAGS, int B>
+void soft_launch_b(const Geom& g, const double* cur, double* prev, const double* kap, const double* wface,
+                   const double* S, double cs, double sn, bool src_faces, bool reverse, cudaStream_t st) {
+    const int zc = soft_zc(g, B);
+    const dim3 grid((unsigned)(((long long)g.sx * g.sy + kST - 1) / kST), (unsigned)((g.sz + zc - 1) / zc));
+    if ((FLAGS & kStepSrc) && src_faces)
+        k_step_soft<DIM, ORDER, FLAGS, true, B><<<grid, kST, 0, st>>>(cur, prev, kap, wface, S, cs, sn, g, zc, reverse);
+    else
+        k_step_soft<DIM, ORDER, FLAGS, false, B><<<grid, kST, 0, st>>>(cur, prev, kap, wface, S, cs, sn, g, zc, reverse);
+}
+
+// Six blocks per SM on 7-point grids of two such waves and more, five on smaller ones; four of the
+// 13-point kernel (see k_step_soft).
 template <int DIM, int ORDER, int FLAGS>
 void soft_launch(const Geom& g, const double* cur, double* prev, const double* kap, const double* wface,
                  const double* S, double cs, double sn, bool src_faces, bool reverse, cudaStream_t st) {
-    const int zc = soft_zc(g, ORDER == 2 ? 4 : 3);
-    const dim3 grid((unsigned)(((long long)g.sx * g.sy + kST - 1) / kST), (unsigned)((g.sz + zc - 1) / zc));
-    if ((FLAGS & kStepSrc) && src_faces)
-        k_step_soft<DIM, ORDER, FLAGS, true><<<grid, kST, 0, st>>>(cur, prev, kap, wface, S, cs, sn, g, zc, reverse);
-    else
-        k_step_soft<DIM, ORDER, FLAGS, false><<<grid, kST, 0, st>>>(cur, prev, kap, wface, S, cs, sn, g, zc, reverse);
+    if constexpr (DIM == 3 && ORDER == 2) {
+        const long long blocks = ((long long)g.sx * g.sy + kST - 1) / kST * ((g.sz + 7) / 8);
+        if (blocks >= 2ll * 152 * 6)
+            soft_launch_b<DIM, ORDER, FLAGS, 6>(g, cur, prev, kap, wface, S, cs, sn, src_faces, reverse, st);
+        else
+            soft_launch_b<DIM, ORDER, FLAGS, 5>(g, cur, prev, kap, wface, S, cs, sn, src_faces, reverse, st);
+    } else {
+        soft_launch_b<DIM, ORDER, FLAGS, 4>(g, cur, prev, kap, wface, S, cs, sn, src_faces, reverse, st);
+    }
 }
 
 template <int DIM, int ORDER>
