@@ -312,6 +312,14 @@ int cmcg_fo_adjoint_period(cmcg_handle* h, const double* y, double* out);
  * context stays usable. */
 int cmcg_bulk_wait_selftest(int spin_limit, void* stream);
 
+/* Self-test of the plan of 2D step loops in one launch (needs no GPU): for this grid, elements of
+ * elem_size bytes (4 or 8) and at most max_bands bands, out[0] = bands (0: the grid is stepped step
+ * by step), out[1] = most rows of a band, out[2] = CTAs of the cluster (0: none), and the kernel
+ * that would run: out[3] = nodes per item (1, or 4 of a row), out[4] = the stencil's reach, out[5] =
+ * items per thread (0: no kernel fits the plan), out[6] = threads per CTA, out[7] = bytes of shared
+ * memory without a source. */
+int cmcg_band_plan_selftest(const cmcg_grid* grid, int elem_size, int max_bands, int* out);
+
 /* Compiled-in bounds checks.  libcmcg_checked.so is the same library built with -DCMCG_CHECKED:
  * its step, period-end, source, two-step, batched-step and multigrid kernels test, per thread,
  * that every node index they will touch lies inside its array; a thread that fails records the

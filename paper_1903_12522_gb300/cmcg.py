@@ -42,7 +42,7 @@ EXPORTED = (
     "cmcg_engine_workspace_size", "cmcg_engine_create", "cmcg_engine_destroy", "cmcg_engine_submit",
     "cmcg_engine_tick", "cmcg_engine_result", "cmcg_engine_active", "cmcg_engine_info", "cmcg_engine_set_shape",
     "cmcg_engine_barrier_selftest", "cmcg_engine_cuda_error", "cmcg_fo_period", "cmcg_fo_adjoint_period",
-    "cmcg_bulk_wait_selftest", "cmcg_check_status",
+    "cmcg_bulk_wait_selftest", "cmcg_check_status", "cmcg_band_plan_selftest",
 )
 
 
@@ -111,6 +111,8 @@ def load(path: str = None):
     lib.cmcg_adjoint_period.restype = I
     lib.cmcg_bulk_wait_selftest.argtypes = [I, P]
     lib.cmcg_bulk_wait_selftest.restype = I
+    lib.cmcg_band_plan_selftest.argtypes = [C.POINTER(Grid), I, I, C.POINTER(I)]
+    lib.cmcg_band_plan_selftest.restype = I
     lib.cmcg_fo_period.argtypes = [P, P, P, P, P]
     lib.cmcg_fo_period.restype = I
     lib.cmcg_fo_adjoint_period.argtypes = [P, P, P]
@@ -237,6 +239,15 @@ def cmcg_bulk_wait_selftest(spin_limit: int, stream=None) -> int:
     """Bounded-wait self-test of the bulk-copy step kernel; returns the status code
     (ERR_DEVICE_TIMEOUT is the expected outcome)."""
     return int(load().cmcg_bulk_wait_selftest(int(spin_limit), stream))
+
+
+def cmcg_band_plan_selftest(grid, elem_size: int, max_bands: int = 152):
+    """The plan of 2D step loops in one launch and its kernel: (bands, rows, cluster, nodes per item,
+    reach, items per thread, threads, shared memory); bands = 0: step by step."""
+    out = (C.c_int * 8)()
+    _check(load().cmcg_band_plan_selftest(C.byref(grid), int(elem_size), int(max_bands), out),
+           "cmcg_band_plan_selftest")
+    return tuple(out)
 
 
 def cmcg_check_status():

@@ -1798,6 +1798,12 @@ int cmcg_bulk_wait_selftest(int spin_limit, void* stream) {
     return bulk_wait_selftest(spin_limit, (cudaStream_t)stream);
 }
 
+int cmcg_band_plan_selftest(const cmcg_grid* grid, int elem_size, int max_bands, int* out) {
+    if (!valid_grid(grid) || (elem_size != 4 && elem_size != 8) || max_bands < 1 || !out) return CMCG_ERR_INVALID_ARG;
+    band_plan_query(make_geom(grid, 0), grid->order, elem_size, max_bands, out);
+    return CMCG_OK;
+}
+
 int cmcg_check_status(long long* count, long long* site, long long* index) {
     if (cudaDeviceSynchronize() != cudaSuccess) return CMCG_ERR_CUDA;
     long long total = 0, first_site = -1, first_index = 0;

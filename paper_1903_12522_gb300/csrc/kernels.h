@@ -167,6 +167,9 @@ struct BandPlan {
 // one cluster.
 bool band_plan(const Geom& g, int order, int elem_size, int sms, BandPlan* p);
 bool band_fits(const BandPlan& p, bool volume_source);
+// For tests: bands (0: no plan), most rows of a band, CTAs of the cluster (0: none), and the kernel: nodes per
+// item, reach, items per thread, threads; bytes of shared memory without a source.
+void band_plan_query(const Geom& g, int order, int elem_size, int sms, int* out);
 // nsteps <= kBandSteps steps from (cur = y^n, prev = y^{n-1}); cur and prev have swapped roles
 // afterwards if nsteps is odd.  S (nullable) with the factors cs, sn of each step; src_faces as
 // for launch_step_soft; adj_first / adj_last: the first / last step is the adjoint's.  words

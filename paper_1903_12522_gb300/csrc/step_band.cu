@@ -771,27 +771,47 @@ cudaError_t band_go(K kernel, const BandArgs<T>& a, const BandPlan& p, size_t sm
     return cudaLaunchKernelEx(&cfg, kernel, a);
 }
 
+// The kernel that runs a plan: k_band4, or k_band with its reach R, made for npt chunks or nodes per
+// thread; npt 0: there is none.
+struct BandKernel {
+    bool four;
+    int reach, npt;
+};
+BandKernel band_kernel_of(int order, int elem_size, const BandPlan& p) {
+    const bool four = elem_size == 4 && order == 2;
+    auto made_for = [&](int most) { return p.npt <= most; };
+    int npt = 0;
+    if (four) npt = made_for(1) ? 1 : (made_for(2) ? 2 : (made_for(3) && p.cluster ? 3 : 0));
+    else if (order == 2) npt = made_for(1) ? 1 : (made_for(2) ? 2 : (made_for(4) ? 4 : (made_for(8) ? 8 : 0)));
+    else npt = made_for(2) ? 2 : (made_for(8) ? 8 : 0);
+    return BandKernel{four, order / 2, npt};
+}
+
 template <int SRC, bool CL, typename T>
 cudaError_t band_kernel(int order, const BandArgs<T>& a, const BandPlan& p, cudaStream_t st) {
     const size_t smem = p.smem[SRC == 2];
+    const BandKernel k = band_kernel_of(order, (int)sizeof(T), p);
     if constexpr (std::is_same<T, float>::value) {
-        if (order == 2) {
-            if (p.npt <= 1) return band_go(k_band4<1, SRC, CL>, a, p, smem, st);
-            if (p.npt <= 2) return band_go(k_band4<2, SRC, CL>, a, p, smem, st);
-            if constexpr (CL) return band_go(k_band4<3, SRC, CL>, a, p, smem, st);
+        if (k.four) {
+            if (k.npt == 1) return band_go(k_band4<1, SRC, CL>, a, p, smem, st);
+            if (k.npt == 2) return band_go(k_band4<2, SRC, CL>, a, p, smem, st);
+            if constexpr (CL) {
+                if (k.npt == 3) return band_go(k_band4<3, SRC, CL>, a, p, smem, st);
+            }
+            return cudaErrorInvalidValue;
         }
-        if (p.npt <= 2) return band_go(k_band<float, 2, 2, SRC, CL>, a, p, smem, st);
-        return band_go(k_band<float, 2, 8, SRC, CL>, a, p, smem, st);
     } else {
-        if (order == 2) {
-            if (p.npt <= 1) return band_go(k_band<double, 1, 1, SRC, CL>, a, p, smem, st);
-            if (p.npt <= 2) return band_go(k_band<double, 1, 2, SRC, CL>, a, p, smem, st);
-            if (p.npt <= 4) return band_go(k_band<double, 1, 4, SRC, CL>, a, p, smem, st);
-            return band_go(k_band<double, 1, 8, SRC, CL>, a, p, smem, st);
+        if (k.reach == 1) {
+            if (k.npt == 1) return band_go(k_band<double, 1, 1, SRC, CL>, a, p, smem, st);
+            if (k.npt == 2) return band_go(k_band<double, 1, 2, SRC, CL>, a, p, smem, st);
+            if (k.npt == 4) return band_go(k_band<double, 1, 4, SRC, CL>, a, p, smem, st);
+            if (k.npt == 8) return band_go(k_band<double, 1, 8, SRC, CL>, a, p, smem, st);
+            return cudaErrorInvalidValue;
         }
-        if (p.npt <= 2) return band_go(k_band<double, 2, 2, SRC, CL>, a, p, smem, st);
-        return band_go(k_band<double, 2, 8, SRC, CL>, a, p, smem, st);
     }
+    if (k.npt == 2) return band_go(k_band<T, 2, 2, SRC, CL>, a, p, smem, st);
+    if (k.npt == 8) return band_go(k_band<T, 2, 8, SRC, CL>, a, p, smem, st);
+    return cudaErrorInvalidValue;
 }
 
 }  // namespace
@@ -813,7 +833,7 @@ bool band_plan(const Geom& g, int order, int elem_size, int sms, BandPlan* p) {
     // costs half of what the exchange through L2 does, so a grid that 16 hold stays there
     bands = std::min(bands, (items + bt / 2 - 1) / (bt / 2));
     long long in_cluster = 16;  // largest cluster of at least R + 1 rows per band, a power of two
-    while (in_cluster > g.sy / (R + 1)) in_cluster >>= 1;
+    while (in_cluster > std::min<long long>(g.sy / (R + 1), sms)) in_cluster >>= 1;
     if (in_cluster > 1 && ((g.sy + in_cluster - 1) / in_cluster) * cx <= bt && bands > in_cluster)
         bands = in_cluster;
     if (bands <= 16) {
@@ -825,9 +845,11 @@ bool band_plan(const Geom& g, int order, int elem_size, int sms, BandPlan* p) {
     const long long rows = (g.sy + bands - 1) / bands;
     const long long per_thread = (rows * cx + bt - 1) / bt;
     const long long buf = (rows + 2 * R) * pitch;
-    if (per_thread > (vec ? (bands <= 16 ? 3 : 2) : 8) || buf > 65535) return false;
+    const int cluster = bands > 1 && bands <= 16 ? (int)bands : 0;
+    // (three chunks per thread in clusters only: one band of more than two runs step by step)
+    if (per_thread > (vec ? (cluster ? 3 : 2) : 8) || buf > 65535) return false;
     const long long side_words = (vec ? 4 * cx : R * g.sx) * (elem_size / 4);
-    p->cluster = bands > 1 && bands <= 16 ? (int)bands : 0;
+    p->cluster = cluster;
     p->face_slots = (int)(2 * rows + (bands == 1 ? 2 : 1) * cx);
     if (!vec && p->face_slots > 8190) return false;  // slot numbers have 13 bits
     const long long slot_bytes = vec ? sizeof(FaceChunk) : (elem_size == 4 ? sizeof(FaceNode<float>) : sizeof(FaceNode<double>));
@@ -841,6 +863,20 @@ bool band_plan(const Geom& g, int order, int elem_size, int sms, BandPlan* p) {
     p->npt = (int)per_thread;
     p->words = p->cluster ? 0 : (size_t)(4 * side_words * bands);
     return true;
+}
+
+void band_plan_query(const Geom& g, int order, int elem_size, int sms, int* out) {
+    BandPlan p;
+    if (!band_plan(g, order, elem_size, sms, &p)) return (void)(out[0] = 0);
+    const BandKernel k = band_kernel_of(order, elem_size, p);
+    out[0] = p.bands;
+    out[1] = p.rows + (p.extra ? 1 : 0);
+    out[2] = p.cluster;
+    out[3] = k.four ? 4 : 1;
+    out[4] = k.reach;
+    out[5] = k.npt;
+    out[6] = elem_size == 4 ? kBandThreads<float> : kBandThreads<double>;
+    out[7] = (int)p.smem[0];
 }
 
 bool band_fits(const BandPlan& p, bool volume_source) {
