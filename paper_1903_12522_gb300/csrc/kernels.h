@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include "coarse_level.h"
 #include "common.cuh"
 
 namespace cmcg {
@@ -323,16 +324,6 @@ constexpr int kCoarseMax = 10;
 constexpr long long kSpreadMaxNodes = 70000;
 constexpr long long kSpreadMinNodes = 2000;
 constexpr long long kCoarsestMaxNodes = 6000;  // larger: the coarsest level gets a few grid-wide sweeps instead
-struct CoarseLevel {
-    int np, lo, cnt;  // nodes, and the CTA's run of them
-    int halo;         // entries of the neighbours' runs that x and r hold copies of, on either side
-    int chunk, sx, sy, sxy, nx, ny, nz, dim;
-    int fused;                 // see lap_rn
-    float cK, cB, inv2d;       // MGConst
-    unsigned x, r, b;          // offsets in shared memory: iterate, residual / second buffer, right-hand side
-    unsigned node;             // a byte per node
-    unsigned long long m_chunk, m_sx, m_sy;  // factors of the divisions by chunk, sx, sy
-};
 struct CoarseLevels {
     int n = 0, nc = 0, ctas = 1;
     Geom g[kCoarseMax] = {};
