@@ -585,44 +585,12 @@ __device__ __forceinline__ void pcg_cluster_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-// The cluster's totals of v in every thread.  slots: room for the CTAs' sums, not used by the call
-// before (another CTA may still read those).
-template <int NV>
-__device__ __forceinline__ void cluster_total(double (&v)[NV], double (*part)[kClusterThreads], double (*slots)[kClusterCtas]) {
-    const int tid = (int)threadIdx.x;
-#pragma unroll
-    for (int k = 0; k < NV; ++k) part[k][tid] = v[k];
-    __syncthreads();
-    if (tid < 32) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            double x = 0.0;
-#pragma unroll
-            for (int q = 0; q < kClusterThreads / 32; ++q) x += part[k][tid + 32 * q];
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            if (tid < kClusterCtas) {
-                const unsigned here = (unsigned)__cvta_generic_to_shared(&slots[k][blockIdx.x]);
-                unsigned there;
-                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"(here), "r"(tid));
-                asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there), "d"(x) : "memory");
-            }
-        }
-    }
-    pcg_cluster_sync();
-    if (tid < 32) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            double x = slots[k][tid & (kClusterCtas - 1)];
-#pragma unroll
-            for (int o = kClusterCtas / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            if (tid == 0) part[k][0] = x;
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] = part[k][0];
+__device__ __forceinline__ void store_to_cta(double* slot, int cta, double v) {
+    unsigned there;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(there) : "r"((unsigned)__cvta_generic_to_shared(slot)), "r"(cta));
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(there), "d"(v) : "memory");
 }
+#include "cluster_total.cuh"
 
 // NPT nodes per thread at most, whose values stay in registers.
 template <int DIM, int ORDER, int NPT>
@@ -631,7 +599,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
                   const float* __restrict__ z, float* __restrict__ bf, const unsigned char* __restrict__ mask,
                   double* __restrict__ sc, Geom g, double ck, int first) {
     __shared__ double part[2][kClusterThreads];
-    __shared__ double slots[3][2][kClusterCtas];
+    __shared__ double slots[3][2][kClusterCtas + 1];
     const int n = (int)g.np, chunk = (n + kClusterCtas - 1) / kClusterCtas;
     const int lo = min((int)blockIdx.x * chunk, n), hi = min(lo + chunk, n), t0 = lo + (int)threadIdx.x;
     const double rz_old = sc[SC_P_RZ], alpha_old = sc[SC_P_ALPHA];

@@ -9,7 +9,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(os.path.dirname(HERE), "paper_1903_12522_gb300", "csrc")
 
 
-@pytest.mark.parametrize("name", ["coarsest"])
+@pytest.mark.parametrize("name", ["coarsest", "cluster_total"])
 def test_every_order_of_the_threads_gives_the_same(name, tmp_path):
     exe = tmp_path / name
     src = os.path.join(HERE, "simt", name + ".cpp")
