@@ -1213,6 +1213,7 @@ void launch_mg_prolong_add(const MGLevel& coarse, const float* xc, const MGLevel
 // launches; 81^3 with 41^3 nodes there 2176 and 2237; with 49^3 there 97^3 is slower, 2513 against
 // 2389) while they have more than kSpreadMinNodes (below, one CTA is faster than the cluster's
 // barriers).
+constexpr size_t kCoarseSmemMax = 220 * 1024;  // shared memory of a CTA
 size_t mg_coarse_smem(const CoarseLevels& lv) {
     size_t n = 0;
     for (int l = 0; l < lv.n; ++l) {
@@ -1260,13 +1261,14 @@ bool mg_coarse_plan(const MGLevel* levels, int nlev, int first, CoarseLevels* lv
         lv->level[i].node = 4 * floats + bytes;
         bytes += (unsigned)(i < lv->nc ? lv->level[i].chunk : lv->level[i].np);
     }
-    return mg_coarse_smem(*lv) <= (size_t)220 * 1024;
+    return mg_coarse_smem(*lv) <= kCoarseSmemMax;
 }
 
 cudaError_t launch_mg_coarse(const CoarseLevels& lv, const float* b, float* x, float omega, int coarse_sweeps,
                              cudaStream_t st) {
     const size_t smem = mg_coarse_smem(lv);
-    cudaError_t e = cudaFuncSetAttribute(k_coarse_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (always the same value: threads with other plans set it too, between this call and the launch)
+    cudaError_t e = cudaFuncSetAttribute(k_coarse_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemMax);
     if (e == cudaSuccess && lv.ctas > 8)
         e = cudaFuncSetAttribute(k_coarse_vcycle, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;

@@ -747,7 +747,8 @@ __global__ void __launch_bounds__(kBandThreads<float>, 1) k_band4(const __grid_c
 
 template <typename T, typename K>
 cudaError_t band_go(K kernel, const BandArgs<T>& a, const BandPlan& p, size_t smem, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (always the same value: threads with other plans set it too, between this call and the launch)
+    cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
     if (e == cudaSuccess && p.cluster > 8)
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     if (e != cudaSuccess) return e;

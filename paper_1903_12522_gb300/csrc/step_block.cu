@@ -421,7 +421,8 @@ __global__ void __launch_bounds__(kBT, 1) k_block3(const __grid_constant__ Block
 template <int NPC, int SRC>
 cudaError_t block_go(const BlockArgs& a, const BlockPlan& p, cudaStream_t st) {
     auto kernel = k_block3<NPC, SRC>;
-    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    // (always the same value: threads with other plans set it too, between this call and the launch)
+    const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax3);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(p.ny_blocks * p.nz_blocks));
