@@ -702,7 +702,7 @@ void row_launch(const Geom& g, const float* a, float* b, const float* kap, const
     const unsigned bxy = (unsigned)((plane4 + kFR - 1) / kFR);
     // planes per thread: one while that makes one wave of blocks at most (65^3, backward period: 338
     // us with one, 424 with four), else two (129^3: 771, 811 with one; 201^3: 2438, 2516 with four)
-    const int zc = (long long)bxy * g.sz <= 152ll * 8 ? 1 : 2;
+    const int zc = planes_per_thread((long long)bxy * g.sz <= 152ll * 8 ? 1 : 2, g.sz);
     const dim3 grid(bxy, (unsigned)((g.sz + zc - 1) / zc));
     auto go = [&](auto kernel) {
         kernel<<<grid, kFR, 0, st>>>(a, b, kap, S, scol, cs, sn, (float)tau, (float)sig, g, px, zc, reverse);

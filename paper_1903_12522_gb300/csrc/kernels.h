@@ -35,6 +35,13 @@ void check_read_band(long long* out);
 void check_read_block(long long* out);
 long long launch_count();
 
+// Planes per thread, zc or as many more as bring a launch of sz planes to the 65535 blocks that a grid has
+// along y.
+inline int planes_per_thread(int zc, int sz) {
+    const int least = (sz + 65534) / 65535;
+    return zc > least ? zc : least;
+}
+
 // ---- wave.cu --------------------------------------------------------------------------
 template <typename T>
 // S: the source dt^2 M^-1 F^ (complex interleaved) in the stepping precision T; scol (3D,

@@ -1192,11 +1192,11 @@ void launch_mg_restrict(const MGLevel& fine, const float* rf, const MGLevel& coa
     // four, fewer where that leaves less than a wave of blocks (to 33^3: 4.3 us with one, 7.7 with
     // four; to 65^3: 7.3 and 8.7)
     const long long bxy = ((long long)gc.sx * gc.sy + kT - 1) / kT;
-    const int zc = (int)std::min(4ll, std::max(1ll, bxy * gc.sz / (152 * 6)));
+    const int zc = (int)std::min(4ll, std::max(1ll, bxy * gc.sz / (152 * 6))), one = planes_per_thread(1, gc.sz);
     if (gf.dim == 3 && gf.nx == 2 * gc.nx && gf.ny == 2 * gc.ny && gf.nz == 2 * gc.nz)
         k_restrict3_nested<<<mg_grid(gc, zc), kT, 0, st>>>(gf, rf, gc, coarse.mask, bc, zc);
     else
-        k_restrict<<<mg_grid(gc, 1), kT, 0, st>>>(gf, rf, gc, coarse.mask, bc, 1);
+        k_restrict<<<mg_grid(gc, one), kT, 0, st>>>(gf, rf, gc, coarse.mask, bc, one);
 }
 
 void launch_mg_prolong_add(const MGLevel& coarse, const float* xc, const MGLevel& fine, float* xf, cudaStream_t st) {

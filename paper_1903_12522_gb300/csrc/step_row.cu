@@ -264,7 +264,7 @@ void row_launch(const RowStep& a, cudaStream_t st) {
     const unsigned bxy = (unsigned)((plane4 + kRT - 1) / kRT);
     // planes per thread: four where that makes at least four waves of blocks, else two
     const int per_sm = ORDER == 2 ? 10 : 7;
-    const int zc = (long long)bxy * ((g.sz + 3) / 4) >= 4ll * 152 * per_sm ? 4 : 2;
+    const int zc = planes_per_thread((long long)bxy * ((g.sz + 3) / 4) >= 4ll * 152 * per_sm ? 4 : 2, g.sz);
     const dim3 grid(bxy, (unsigned)((g.sz + zc - 1) / zc));
     const float cs = (float)a.cs, sn = (float)a.sn;
     auto go = [&](auto kernel) {
