@@ -8,8 +8,8 @@ Single solves: for a grid class (dimension, size bucket = the power of two neare
 interval count, precision) it times the homogeneous adjoint period for every candidate step
 scheme and launch shape in cmcg_options.tile and records the fastest in autotune_cache.json
 next to this file; Solver() looks the class up when no tile is given.  The 3D candidates
-include the temporal-blocking depth (one or two leapfrog steps per sweep: schemes 1/3/4/5/6
-against scheme 2) and the number of planes in flight of the staged kernel (scheme 6).
+include the library's default (padded rows, loops on chip), the temporal-blocking depth (one or two leapfrog
+steps per sweep: schemes 1/3/4/5/6 against scheme 2) and the number of planes in flight of the staged kernel (scheme 6).
 
 Engine: for a batch class ("batch2d": uneven 2D instances; "mix": 2D and 3D requests) it
 times engine ticks of a fixed set of solves in their inner iterations for every launch shape
@@ -48,6 +48,23 @@ def candidates_3d():
 def candidates_2d():
     """2D 5-point grids: the generic one-step kernel and the vector form."""
     return [(0, 0, 0, 1), (0, 0, 0, 5)]
+
+
+# The library's own choice: in 3D the padded rows and the on-chip loops, which no other tile gives.
+DEFAULT = (0, 0, 0, 0)
+
+
+def candidates(dim):
+    """What tune() times: the default first, then the other tiles."""
+    return [DEFAULT] + (candidates_3d() if dim == 3 else candidates_2d())
+
+
+def choose(best):
+    """The tile to record from {tile: ms}: the fastest, but the default unless another one is faster by more
+    than 5 %.  (2D grids that fit on chip run the same kernels whatever the tile, and the times of one kernel
+    differ by up to 7 % there, most of them host time; scheme 5 is what the default is on larger 2D grids.)"""
+    ms, tile = min((ms, tile) for tile, ms in best.items())
+    return tile if ms < 0.95 * best[DEFAULT] else DEFAULT
 
 
 def engine_candidates():
@@ -111,17 +128,18 @@ def tune(dim, n, precision, reps=5, rounds=2):
     w = wl.sphere_3d(n=n) if dim == 3 else wl.gaussian_2d(n=n)
     act = 1.0 if w.mask is None else 1.0 - w.mask.astype("float64")
     a, b = [torch.as_tensor(x * act, device="cuda").reshape(-1) for x in wl.random_fields(w.shape, 2, 17)]
-    cands = candidates_3d() if dim == 3 else candidates_2d()
+    cands = candidates(dim)
     best = {}
-    for _ in range(rounds):  # the best of several rounds, the candidates interleaved
-        for tile in cands:
+    for r in range(rounds):  # the best of several rounds, the candidates interleaved, each round in the other order
+        for tile in cands if r % 2 == 0 else cands[::-1]:
             s = cmcg.Solver(w.n, w.h, w.c, w.omega, w.faces, mask=w.mask, precision=precision, dt=w.dt_target,
                             tile=tile)
             ms = _time_adjoint(s, a, b, reps)
             best[tile] = min(best.get(tile, float("inf")), ms)
             s.close()
     results = sorted((ms, tile) for tile, ms in best.items())
-    best_ms, best_tile = results[0]
+    best_tile = choose(best)
+    best_ms = best[best_tile]
     _store(size_class(dim, n, precision), {"tile": list(best_tile), "ms_per_adjoint_period": best_ms,
                                            "candidates": len(results), "worst_ms": results[-1][0]})
     return best_tile, best_ms, results
