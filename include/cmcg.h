@@ -52,7 +52,7 @@ extern "C" {
 #define CMCG_ERR_UNSUPPORTED (-4)
 #define CMCG_ERR_CUDA (-5)
 #define CMCG_ERR_DIVERGED (-6)
-#define CMCG_ERR_DEVICE_TIMEOUT (-7) /* a bounded device-side wait ran out (batched kernel barrier) */
+#define CMCG_ERR_DEVICE_TIMEOUT (-7) /* a bounded device-side wait ran out (batched kernel barrier, step loop in one launch) */
 
 /* ---- boundary codes (face order -x, +x, -y, +y, -z, +z) --------------------------- */
 #define CMCG_BC_ABC 0       /* first-order absorbing (impedance) face, Eq. HE_ABC      */
@@ -319,6 +319,13 @@ int cmcg_bulk_wait_selftest(int spin_limit, void* stream);
  * items per thread (0: no kernel fits the plan), out[6] = threads per CTA, out[7] = bytes of shared
  * memory without a source. */
 int cmcg_band_plan_selftest(const cmcg_grid* grid, int elem_size, int max_bands, int* out);
+
+/* Self-test of the bounded waits of step loops in one launch: this handle's loops wait at most `polls`
+ * polls for a neighbour's rows from now on (0: as long as by default).  With a few polls a period on a
+ * grid of more than one band or block runs out of its wait: the call returns CMCG_ERR_DEVICE_TIMEOUT, the
+ * context stays usable and so does the handle, with the default wait again.  CMCG_ERR_UNSUPPORTED: the
+ * handle has no such loop. */
+int cmcg_loop_wait_selftest(cmcg_handle* h, int polls);
 
 /* Compiled-in bounds checks.  libcmcg_checked.so is the same library built with -DCMCG_CHECKED:
  * its step, period-end, source, two-step, batched-step and multigrid kernels test, per thread,

@@ -43,6 +43,7 @@ EXPORTED = (
     "cmcg_engine_tick", "cmcg_engine_result", "cmcg_engine_active", "cmcg_engine_info", "cmcg_engine_set_shape",
     "cmcg_engine_barrier_selftest", "cmcg_engine_cuda_error", "cmcg_fo_period", "cmcg_fo_adjoint_period",
     "cmcg_bulk_wait_selftest", "cmcg_check_status", "cmcg_band_plan_selftest",
+    "cmcg_loop_wait_selftest",
 )
 
 
@@ -113,6 +114,8 @@ def load(path: str = None):
     lib.cmcg_bulk_wait_selftest.restype = I
     lib.cmcg_band_plan_selftest.argtypes = [C.POINTER(Grid), I, I, C.POINTER(I)]
     lib.cmcg_band_plan_selftest.restype = I
+    lib.cmcg_loop_wait_selftest.argtypes = [P, I]
+    lib.cmcg_loop_wait_selftest.restype = I
     lib.cmcg_fo_period.argtypes = [P, P, P, P, P]
     lib.cmcg_fo_period.restype = I
     lib.cmcg_fo_adjoint_period.argtypes = [P, P, P]
@@ -248,6 +251,11 @@ def cmcg_band_plan_selftest(grid, elem_size: int, max_bands: int = 152):
     _check(load().cmcg_band_plan_selftest(C.byref(grid), int(elem_size), int(max_bands), out),
            "cmcg_band_plan_selftest")
     return tuple(out)
+
+
+def cmcg_loop_wait_selftest(h, polls: int) -> None:
+    """Sets the longest wait of this handle's step loops in one launch (0: the default)."""
+    _check(load().cmcg_loop_wait_selftest(h, int(polls)), "cmcg_loop_wait_selftest")
 
 
 def cmcg_check_status():

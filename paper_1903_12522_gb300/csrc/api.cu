@@ -461,10 +461,11 @@ bool band_steps(cmcg_handle* H, PeriodBuffers& b, long long count, bool src, boo
         const bool a0 = adjoint && n0 == 0, a1 = adjoint && n0 + m == count;
         const cudaError_t e =
             block ? launch_step_block(H->g, H->block, (float*)b.cur, (float*)b.prev, H->kap32, (const float*)S, H->sflag,
-                                      H->src_faces, H->band_words, H->band_count, H->hsc + SC_COUNT, m, cs, sn, a0, a1,
-                                      H->st)
+                                      H->src_faces, H->band_words, H->band_count, H->hsc + SC_COUNT, H->loop_polls, m, cs,
+                                      sn, a0, a1, H->st)
                   : launch_step_band<T>(H->g, H->order, band, (T*)b.cur, (T*)b.prev, kap, S, H->src_faces, H->wface,
-                                        H->band_words, H->band_count, H->hsc + SC_COUNT, m, cs, sn, a0, a1, H->st);
+                                        H->band_words, H->band_count, H->hsc + SC_COUNT, H->loop_polls, m, cs, sn, a0, a1,
+                                        H->st);
         if (e != cudaSuccess) {
             if (n0 == 0) {  // no cooperative launch to be had (shared device limits): step by step
                 cudaGetLastError();
@@ -1331,7 +1332,7 @@ void compat_shift(cmcg_handle* h, double* u, double* lre, double* lim) {
 
 int recover(cmcg_handle* h, double* u, cmcg_stats* st) {
     launch_recover(h->g, h->w0, h->w1, h->wh, h->S, h->kap64, h->mass, u, h->red(), h->st);
-    if (sync_read(h) != CMCG_OK) return CMCG_ERR_CUDA;
+    if (const int rc = sync_read(h)) return rc;
     double lre = 0.0, lim = 0.0;
     if (!h->has_dir) compat_shift(h, u, &lre, &lim);
     if (cudaStreamSynchronize(h->st) != cudaSuccess) return CMCG_ERR_CUDA;
@@ -1365,7 +1366,7 @@ int filter_recover(cmcg_handle* h, double* u, cmcg_stats* st) {
     st->lambda_re = st->lambda_im = 0.0;
     if (!h->has_dir && g.abc == 0u) {
         launch_compat_sums(g, u, h->S, h->kap64, h->mass, h->red(), h->st);
-        if (sync_read(h) != CMCG_OK) return CMCG_ERR_CUDA;
+        if (const int rc = sync_read(h)) return rc;
         compat_shift(h, u, &st->lambda_re, &st->lambda_im);
     }
     if (cudaStreamSynchronize(h->st) != cudaSuccess) return CMCG_ERR_CUDA;
@@ -1420,7 +1421,7 @@ int solve_prepared(cmcg_handle* h, double tol, double* u, cmcg_stats* st, bool w
             runup<double>(h, ell, h->w0, h->w1);
         else
             runup<float>(h, ell, h->w0, h->w1);
-        rc = cuda_status();
+        rc = sync_read(h);
     } else if (h->opt.precision == CMCG_FP64)
         rc = solve_plain<double>(h, tol, st);
     else if (h->opt.precision == CMCG_FP32)
@@ -1440,15 +1441,12 @@ int solve_prepared(cmcg_handle* h, double tol, double* u, cmcg_stats* st, bool w
         }
         forward_period<double>(h, h->w0, h->w1, true, 0, h->z0, h->z1);
         h->wface = own;
-        if (sync_read(h) != CMCG_OK) return CMCG_ERR_CUDA;
+        if (const int rj = sync_read(h)) return rj;
         st->J_final = h->hsc[SC_J];
     }
     // (6) recovery: the compatibility-condition shift, or the filter of Sec. 2.2
-    if (h->opt.flags & CMCG_FLAG_FILTER) {
-        if (filter_recover(h, u, st) != CMCG_OK) return CMCG_ERR_CUDA;
-    } else if (recover(h, u, st) != CMCG_OK) {
-        return CMCG_ERR_CUDA;
-    }
+    const int r6 = (h->opt.flags & CMCG_FLAG_FILTER) ? filter_recover(h, u, st) : recover(h, u, st);
+    if (r6 != CMCG_OK) return r6;
     st->steps_per_period = h->N;
     st->dt = h->dt;
     st->omega_tilde = h->wt;
@@ -1801,6 +1799,13 @@ int cmcg_bulk_wait_selftest(int spin_limit, void* stream) {
 int cmcg_band_plan_selftest(const cmcg_grid* grid, int elem_size, int max_bands, int* out) {
     if (!valid_grid(grid) || (elem_size != 4 && elem_size != 8) || max_bands < 1 || !out) return CMCG_ERR_INVALID_ARG;
     band_plan_query(make_geom(grid, 0), grid->order, elem_size, max_bands, out);
+    return CMCG_OK;
+}
+
+int cmcg_loop_wait_selftest(cmcg_handle* h, int polls) {
+    if (!h || polls < 0) return CMCG_ERR_INVALID_ARG;
+    if (h->band.bands == 0 && h->block.ny_blocks == 0) return CMCG_ERR_UNSUPPORTED;
+    h->loop_polls = polls ? std::min(polls, kLoopPolls) : kLoopPolls;
     return CMCG_OK;
 }
 

@@ -398,7 +398,7 @@ int finish_slot(cmcg_engine* e, int s) {
         cudaMemcpyAsync(h->w0, h->wo0, sizeof(double) * n, cudaMemcpyDeviceToDevice, h->st);
         cudaMemcpyAsync(h->w1, h->wo1, sizeof(double) * n, cudaMemcpyDeviceToDevice, h->st);
     }
-    if (recover(h, sl.u, &sl.st) != CMCG_OK) return CMCG_ERR_CUDA;
+    if (const int rc = recover(h, sl.u, &sl.st)) return rc;
     sl.st.iterations = sl.iters;
     sl.st.outer_iterations = sl.outer;
     sl.st.rel_residual = sl.rel;
@@ -688,7 +688,10 @@ int cmcg_engine_tick(cmcg_engine* e, int* finished, int max_finished, int* n_fin
             }
         }
         if (done) {
-            if (sl.status >= 0 && finish_slot(e, s) != CMCG_OK) sl.status = CMCG_ERR_CUDA;
+            if (sl.status >= 0) {
+                const int rc = finish_slot(e, s);
+                if (rc != CMCG_OK) sl.status = rc;
+            }
             sl.unit = U_DONE;
             if (*n_finished < max_finished) finished[*n_finished] = s;
             *n_finished += 1;

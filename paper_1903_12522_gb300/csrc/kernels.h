@@ -163,6 +163,7 @@ void launch_adj_final_soft(const Geom& g, int order, int mode, const double* s, 
 // 2D step loops in one cooperative launch, the grid held on chip in bands of rows, one per SM.
 constexpr int kBandSteps = 200;  // most steps of one launch (their source factors are arguments)
 constexpr int kBandStop = 152;   // index of the stop word behind the per-band step counts
+constexpr int kLoopPolls = 1 << 21;  // a loop's longest wait, in polls: about a second and a half
 struct BandPlan {
     int bands = 0, rows = 0, extra = 0;  // bands (0: the grid does not suit the kernel) and their rows
     int npt = 0;                         // nodes, or float4 chunks, per thread
@@ -182,11 +183,11 @@ void band_plan_query(const Geom& g, int order, int elem_size, int sms, int* out)
 // afterwards if nsteps is odd.  S (nullable) with the factors cs, sn of each step; src_faces as
 // for launch_step_soft; adj_first / adj_last: the first / last step is the adjoint's.  words
 // (p.words of them, zero at first), count (kBandStop + 1, zero at first) and err (host memory)
-// as described in step_band.cu.
+// as described in step_band.cu; polls: the longest wait.
 template <typename T>
 cudaError_t launch_step_band(const Geom& g, int order, const BandPlan& p, T* cur, T* prev, const T* kap, const T* S,
                              bool src_faces, const double* wface, unsigned long long* words, unsigned* count,
-                             double* err, int nsteps, const double* cs, const double* sn, bool adj_first,
+                             double* err, int polls, int nsteps, const double* cs, const double* sn, bool adj_first,
                              bool adj_last, cudaStream_t st);
 
 // The FP64 vector passes of the Riesz PCG for FP64 handles: as launch_applyK and launch_pcg_*, with
@@ -216,8 +217,8 @@ bool block_plan(const Geom& g, int sms, BlockPlan* p);
 // As launch_step_band; sflag of S.
 cudaError_t launch_step_block(const Geom& g, const BlockPlan& p, float* cur, float* prev, const float* kap, const float* S,
                               const unsigned char* sflag, bool src_faces, unsigned long long* words, unsigned* count,
-                              double* err, int nsteps, const double* cs, const double* sn, bool adj_first, bool adj_last,
-                              cudaStream_t st);
+                              double* err, int polls, int nsteps, const double* cs, const double* sn, bool adj_first,
+                              bool adj_last, cudaStream_t st);
 
 // ---- step_row.cu ------------------------------------------------------------------------
 // FP32 3D steps on rows padded to whole float4s (pitch row_pitch).  flat: 0 cur, prev, out padded

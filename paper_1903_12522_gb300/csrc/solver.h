@@ -65,6 +65,7 @@ struct cmcg_handle {
     unsigned long long* band_words = nullptr;
     size_t exchange_words = 0;
     unsigned* band_count = nullptr;
+    int loop_polls = kLoopPolls;  // their longest wait
     bool side_by_side = false;
     // first-order formulation (CMCG_FLAG_FIRST_ORDER): CG vectors on the state (p, v) of
     // (dim + 1) N_p doubles, and the two stepping buffers (sized for double)

@@ -42,7 +42,6 @@ namespace {
 
 constexpr int kMaxBands = kBandStop;   // one CTA per SM of a GB300
 constexpr int kSmemMax = 227 * 1024;   // shared memory a CTA can have
-constexpr int kWaitPolls = 1 << 21;    // about a second and a half
 
 template <typename T>
 constexpr int kBandThreads = std::is_same<T, float>::value ? 1024 : 512;  // FP64 needs the registers
@@ -62,6 +61,7 @@ struct BandArgs {
     int nsteps;
     int face_slots;       // shared-memory slots of face factors
     int adj_first, adj_last;  // step 0 is the adjoint's first, step nsteps - 1 its last
+    int polls;            // the longest wait
     T cs[kBandSteps], sn[kBandSteps];
 };
 
@@ -77,6 +77,7 @@ struct Exchange {
     int band, n;
     unsigned* stop;
     double* err;
+    int limit;  // polls of the longest wait
     __device__ __forceinline__ long long at(unsigned tag, int from) const { return (long long)((tag & 1u) * 2 + from) * n; }
     // where band `to` looks for words of this step that come from side `from`
     __device__ __forceinline__ unsigned long long* global_of(int to, unsigned tag, int from) const {
@@ -144,8 +145,8 @@ struct Exchange {
     }
     // after an unsuccessful poll: true to give up
     __device__ __forceinline__ bool give_up(int& polls) const {
-        if (++polls & 1023) return false;
-        if (polls > kWaitPolls) {
+        if ((++polls & 1023) && polls < limit) return false;
+        if (polls >= limit) {
             *(volatile unsigned*)stop = 1u;
             *(volatile double*)err = (double)CMCG_ERR_DEVICE_TIMEOUT;
         }
@@ -334,7 +335,7 @@ __global__ void __launch_bounds__(kBandThreads<T>, 1) k_band(const __grid_consta
     T* const ssrc = reinterpret_cast<T*>(faces + a.face_slots);
     const bool up = band > 0, down = band + 1 < nbands;  // is there a band before / after?
     const unsigned base = CL ? 0u : a.count[band];
-    const Exchange<CL> ex{a.words, smem_addr(sm_words), band, side_words, a.count + kBandStop, a.err};
+    const Exchange<CL> ex{a.words, smem_addr(sm_words), band, side_words, a.count + kBandStop, a.err, a.polls};
 
     // the band and its halo rows of y^n; rows outside the grid hold their mirror rows
     for (int i = tid; i < (rows + 2 * R) * P; i += BT) {
@@ -583,7 +584,7 @@ __global__ void __launch_bounds__(kBandThreads<float>, 1) k_band4(const __grid_c
     float2* const ssrc = reinterpret_cast<float2*>(faces + a.face_slots);
     const bool up = band > 0, down = band + 1 < nbands;
     const unsigned base = CL ? 0u : a.count[band];
-    const Exchange<CL> ex{a.words, smem_addr(sm_words), band, side_words, a.count + kBandStop, a.err};
+    const Exchange<CL> ex{a.words, smem_addr(sm_words), band, side_words, a.count + kBandStop, a.err, a.polls};
 
     for (int i = tid; i < (rows + 2) * P; i += BT) {
         const int lr = i / P, x = i - lr * P - 4;
@@ -887,9 +888,10 @@ bool band_fits(const BandPlan& p, bool volume_source) {
 template <typename T>
 cudaError_t launch_step_band(const Geom& g, int order, const BandPlan& p, T* cur, T* prev, const T* kap, const T* S,
                              bool src_faces, const double* wface, unsigned long long* words, unsigned* count,
-                             double* err, int nsteps, const double* cs, const double* sn, bool adj_first,
+                             double* err, int polls, int nsteps, const double* cs, const double* sn, bool adj_first,
                              bool adj_last, cudaStream_t st) {
     BandArgs<T> a;
+    a.polls = polls;
     a.face_slots = p.face_slots;
     a.buf0 = cur;
     a.buf1 = prev;
@@ -924,10 +926,12 @@ cudaError_t launch_step_band(const Geom& g, int order, const BandPlan& p, T* cur
 }
 template cudaError_t launch_step_band<float>(const Geom&, int, const BandPlan&, float*, float*, const float*,
                                              const float*, bool, const double*, unsigned long long*, unsigned*,
-                                             double*, int, const double*, const double*, bool, bool, cudaStream_t);
+                                             double*, int, int, const double*, const double*, bool, bool,
+                                             cudaStream_t);
 template cudaError_t launch_step_band<double>(const Geom&, int, const BandPlan&, double*, double*, const double*,
                                               const double*, bool, const double*, unsigned long long*, unsigned*,
-                                              double*, int, const double*, const double*, bool, bool, cudaStream_t);
+                                              double*, int, int, const double*, const double*, bool, bool,
+                                             cudaStream_t);
 
 CMCG_CHECK_TU(band)
 

@@ -32,7 +32,6 @@ namespace {
 constexpr int kBT = 512;                 // 128 registers: 64 of them hold y^{n-1} and kappa
 constexpr int kMaxBlocks3 = kBandStop;   // one per SM of a GB300
 constexpr int kSmemMax3 = 226 * 1024;
-constexpr int kPolls = 1 << 21;          // about a second and a half
 constexpr int kHalo = 4;                 // halo chunks per thread
 
 struct BlockArgs {
@@ -49,6 +48,7 @@ struct BlockArgs {
     int ty, ey, tz, ez;         // rows of a block: ty + 1 for the first ey along y, ty for the others; same for z
     int side;                   // words of one side (4 per chunk, rows in the buffer's pitch)
     int nsteps, adj_first, adj_last;
+    int polls;                  // the longest wait
     float cs[kBandSteps], sn[kBandSteps];
 };
 
@@ -380,8 +380,8 @@ __global__ void __launch_bounds__(kBT, 1) k_block3(const __grid_constant__ Block
                         place(w1, hoff[h + 1]);
                         m1 = false;
                     }
-                    if ((m0 || m1) && !(++polls & 1023)) {
-                        if (polls > kPolls) {
+                    if ((m0 || m1) && (!(++polls & 1023) || polls >= a.polls)) {
+                        if (polls >= a.polls) {
                             *(volatile unsigned*)(a.count + kBandStop) = 1u;
                             *(volatile double*)a.err = (double)CMCG_ERR_DEVICE_TIMEOUT;
                         }
@@ -482,9 +482,10 @@ bool block_plan(const Geom& g, int sms, BlockPlan* p) {
 
 cudaError_t launch_step_block(const Geom& g, const BlockPlan& p, float* cur, float* prev, const float* kap, const float* S,
                               const unsigned char* sflag, bool src_faces, unsigned long long* words, unsigned* count,
-                              double* err, int nsteps, const double* cs, const double* sn, bool adj_first, bool adj_last,
-                              cudaStream_t st) {
+                              double* err, int polls, int nsteps, const double* cs, const double* sn, bool adj_first,
+                              bool adj_last, cudaStream_t st) {
     BlockArgs a;
+    a.polls = polls;
     a.buf0 = cur;
     a.buf1 = prev;
     a.kap = kap;
