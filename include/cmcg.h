@@ -327,6 +327,10 @@ int cmcg_band_plan_selftest(const cmcg_grid* grid, int elem_size, int max_bands,
  * handle has no such loop. */
 int cmcg_loop_wait_selftest(cmcg_handle* h, int polls);
 
+/* Self-test of the Riesz map on a device (or a part of one) that cannot hold a cluster of 16 CTAs: this
+ * handle's V-cycle and PCG use none from now on, as they do where cmcg_create finds that none fits. */
+int cmcg_no_cluster_selftest(cmcg_handle* h);
+
 /* Compiled-in bounds checks.  libcmcg_checked.so is the same library built with -DCMCG_CHECKED:
  * its step, period-end, source, two-step, batched-step and multigrid kernels test, per thread,
  * that every node index they will touch lies inside its array; a thread that fails records the

@@ -43,7 +43,7 @@ EXPORTED = (
     "cmcg_engine_tick", "cmcg_engine_result", "cmcg_engine_active", "cmcg_engine_info", "cmcg_engine_set_shape",
     "cmcg_engine_barrier_selftest", "cmcg_engine_cuda_error", "cmcg_fo_period", "cmcg_fo_adjoint_period",
     "cmcg_bulk_wait_selftest", "cmcg_check_status", "cmcg_band_plan_selftest",
-    "cmcg_loop_wait_selftest",
+    "cmcg_loop_wait_selftest", "cmcg_no_cluster_selftest",
 )
 
 
@@ -114,6 +114,8 @@ def load(path: str = None):
     lib.cmcg_bulk_wait_selftest.restype = I
     lib.cmcg_band_plan_selftest.argtypes = [C.POINTER(Grid), I, I, C.POINTER(I)]
     lib.cmcg_band_plan_selftest.restype = I
+    lib.cmcg_no_cluster_selftest.argtypes = [P]
+    lib.cmcg_no_cluster_selftest.restype = I
     lib.cmcg_loop_wait_selftest.argtypes = [P, I]
     lib.cmcg_loop_wait_selftest.restype = I
     lib.cmcg_fo_period.argtypes = [P, P, P, P, P]
@@ -256,6 +258,11 @@ def cmcg_band_plan_selftest(grid, elem_size: int, max_bands: int = 152):
 def cmcg_loop_wait_selftest(h, polls: int) -> None:
     """Sets the longest wait of this handle's step loops in one launch (0: the default)."""
     _check(load().cmcg_loop_wait_selftest(h, int(polls)), "cmcg_loop_wait_selftest")
+
+
+def cmcg_no_cluster_selftest(h) -> None:
+    """This handle's Riesz map without thread-block clusters from now on."""
+    _check(load().cmcg_no_cluster_selftest(h), "cmcg_no_cluster_selftest")
 
 
 def cmcg_check_status():

@@ -826,6 +826,17 @@ int coarse_sweeps(const Geom& g) {
     return std::min(512, std::max(32, 8 * nmax * nmax));
 }
 
+void plan_riesz(cmcg_handle* H, bool clusters) {
+    H->pcg_cluster = clusters && H->nlev > 0 && H->opt.precision == CMCG_FP64 && pcg_cluster_fits(H->g, H->order);
+    H->coarse_level = -1;
+    for (int l = 0; l < H->nlev; ++l) {
+        if (!mg_coarse_plan(H->lv, H->nlev, l, clusters, &H->coarse)) continue;
+        if (H->coarse.nc > 0 && !mg_coarse_resident(H->coarse)) return plan_riesz(H, false);
+        H->coarse_level = l;
+        return;
+    }
+}
+
 void vcycle(cmcg_handle* H, int l) {
     MGLevel& L = H->lv[l];
     const float om = jacobi_omega(L.g);
@@ -884,7 +895,7 @@ int riesz_solve(cmcg_handle* H, const double* rhs, double* x, int* iters_out) {
         launch_pcg_p_update(n, H->pp, H->pzd, red, first, H->st);
     };
     // small grids: an iteration's vector part, from z on, in one launch
-    const bool small = fast && pcg_cluster_fits(g);
+    const bool small = fast && H->pcg_cluster;
     if (!fast) launch_fill(x, n, 0.0, H->st);
     if (small) launch_to_float(n, H->pr, zf, H->st);
     else direction(true);
@@ -1709,8 +1720,7 @@ int cmcg_create(const cmcg_grid* grid, const double* c, double omega, const cmcg
         launch_to_float(H->g.np, H->mass, H->mass32, H->st);
         launch_to_float(H->g.np, H->minv, H->minv32, H->st);
     }
-    for (int l = 0; l < H->nlev && H->coarse_level < 0; ++l)
-        if (mg_coarse_plan(H->lv, H->nlev, l, &H->coarse)) H->coarse_level = l;
+    plan_riesz(H, true);
     if (sync_read(H) != CMCG_OK) return fail(CMCG_ERR_CUDA);
     if (o.flags & CMCG_FLAG_L2_KAPPA) l2_kappa_begin(H);
     *out = H;
@@ -1806,6 +1816,13 @@ int cmcg_loop_wait_selftest(cmcg_handle* h, int polls) {
     if (!h || polls < 0) return CMCG_ERR_INVALID_ARG;
     if (h->band.bands == 0 && h->block.ny_blocks == 0) return CMCG_ERR_UNSUPPORTED;
     h->loop_polls = polls ? std::min(polls, kLoopPolls) : kLoopPolls;
+    return CMCG_OK;
+}
+
+int cmcg_no_cluster_selftest(cmcg_handle* h) {
+    if (!h) return CMCG_ERR_INVALID_ARG;
+    if (h->first_order) return CMCG_ERR_UNSUPPORTED;
+    plan_riesz(h, false);
     return CMCG_OK;
 }
 

@@ -202,7 +202,7 @@ void launch_pcg_p(long long n, double* p, const float* z, Red red, bool first, c
 // All four for one iteration in one cluster launch (grids of up to kPcgClusterNodes nodes, three per
 // thread): from z = B r to the next residual and bf.  first: p and x start at zero.
 constexpr long long kPcgClusterNodes = 36864;
-bool pcg_cluster_fits(const Geom& g);
+bool pcg_cluster_fits(const Geom& g, int order);  // and the device can hold the cluster
 void launch_pcg_cluster(const Geom& g, int order, const unsigned char* mask, double* x, double* r, double* p, double* Ap,
                         const float* z, float* bf, Red red, bool first, cudaStream_t st);
 
@@ -338,8 +338,11 @@ struct CoarseLevels {
     const unsigned char* mask[kCoarseMax] = {};
     CoarseLevel level[kCoarseMax] = {};
 };
-// The levels first .. nlev-1; false if they do not fit.
-bool mg_coarse_plan(const MGLevel* levels, int nlev, int first, CoarseLevels* lv);
+// The levels first .. nlev-1; false if they do not fit.  clusters: larger levels spread over a cluster of
+// 16 CTAs; else one CTA for levels of up to kCoarsestMaxNodes nodes.
+bool mg_coarse_plan(const MGLevel* levels, int nlev, int first, bool clusters, CoarseLevels* lv);
+// Can the device hold the plan's cluster?
+bool mg_coarse_resident(const CoarseLevels& lv);
 cudaError_t launch_mg_coarse(const CoarseLevels& lv, const float* b, float* x, float omega, int coarse_sweeps,
                              cudaStream_t st);
 // FP64 PCG pieces on the fine level

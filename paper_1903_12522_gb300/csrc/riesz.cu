@@ -1223,15 +1223,16 @@ size_t mg_coarse_smem(const CoarseLevels& lv) {
     return n + 16;
 }
 
-bool mg_coarse_plan(const MGLevel* levels, int nlev, int first, CoarseLevels* lv) {
+bool mg_coarse_plan(const MGLevel* levels, int nlev, int first, bool clusters, CoarseLevels* lv) {
     *lv = CoarseLevels();
     lv->n = nlev - first;
-    if (lv->n > kCoarseMax || levels[first].g.np > kSpreadMaxNodes || levels[nlev - 1].g.np > kCoarsestMaxNodes)
+    if (lv->n > kCoarseMax || levels[first].g.np > (clusters ? kSpreadMaxNodes : kCoarsestMaxNodes) ||
+        levels[nlev - 1].g.np > kCoarsestMaxNodes)
         return false;
     for (int i = 0; i < lv->n; ++i) {
         lv->g[i] = levels[first + i].g;
         lv->mask[i] = levels[first + i].mask;
-        if (lv->g[i].np > kSpreadMinNodes && i + 1 < lv->n) lv->nc = i + 1;
+        if (clusters && lv->g[i].np > kSpreadMinNodes && i + 1 < lv->n) lv->nc = i + 1;
     }
     lv->ctas = lv->nc > 0 ? 16 : 1;
     auto magic = [](long long d) { return (1ull << 40) / (unsigned long long)d + 1ull; };
@@ -1264,26 +1265,42 @@ bool mg_coarse_plan(const MGLevel* levels, int nlev, int first, CoarseLevels* lv
     return mg_coarse_smem(*lv) <= kCoarseSmemMax;
 }
 
-cudaError_t launch_mg_coarse(const CoarseLevels& lv, const float* b, float* x, float omega, int coarse_sweeps,
-                             cudaStream_t st) {
-    const size_t smem = mg_coarse_smem(lv);
+static cudaError_t coarse_config(const CoarseLevels& lv, cudaStream_t st, cudaLaunchAttribute* attr,
+                                 cudaLaunchConfig_t* cfg) {
     // (always the same value: threads with other plans set it too, between this call and the launch)
     cudaError_t e = cudaFuncSetAttribute(k_coarse_vcycle, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCoarseSmemMax);
     if (e == cudaSuccess && lv.ctas > 8)
         e = cudaFuncSetAttribute(k_coarse_vcycle, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    *cfg = {};
+    cfg->gridDim = dim3((unsigned)lv.ctas);
+    cfg->blockDim = dim3(1024);
+    cfg->dynamicSmemBytes = mg_coarse_smem(lv);
+    cfg->stream = st;
+    attr->id = cudaLaunchAttributeClusterDimension;
+    attr->val.clusterDim.x = (unsigned)lv.ctas;
+    attr->val.clusterDim.y = 1;
+    attr->val.clusterDim.z = 1;
+    cfg->attrs = attr;
+    cfg->numAttrs = 1;
+    return e;
+}
+
+bool mg_coarse_resident(const CoarseLevels& lv) {
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t cfg;
+    int clusters = 0;
+    const bool ok = coarse_config(lv, nullptr, &attr, &cfg) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&clusters, k_coarse_vcycle, &cfg) == cudaSuccess && clusters > 0;
+    if (!ok) cudaGetLastError();
+    return ok;
+}
+
+cudaError_t launch_mg_coarse(const CoarseLevels& lv, const float* b, float* x, float omega, int coarse_sweeps,
+                             cudaStream_t st) {
+    cudaLaunchAttribute attr;
+    cudaLaunchConfig_t cfg;
+    const cudaError_t e = coarse_config(lv, st, &attr, &cfg);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)lv.ctas);
-    cfg.blockDim = dim3(1024);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)lv.ctas;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
     note_launch(1);
     return cudaLaunchKernelEx(&cfg, k_coarse_vcycle, lv, b, x, omega, coarse_sweeps);
 }

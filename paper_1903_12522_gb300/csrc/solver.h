@@ -51,6 +51,7 @@ struct cmcg_handle {
     int nlev = 0;
     int coarse_level = -1;    // first level of the V-cycle's coarse end in one launch (-1: none)
     CoarseLevels coarse{};
+    bool pcg_cluster = false;  // FP64, small grids: a Riesz PCG iteration's vector part in one cluster launch
     int riesz_guess = 0;      // PCG iterations of the previous Riesz solve
     unsigned char* sflag = nullptr;  // 3D FP32 steps: where S32 is not zero (launch_source_flags)
     // FP32 3D step loops on padded rows (step_row.cu): the two wave fields and kappa
@@ -133,6 +134,9 @@ const T* step_source(const cmcg_handle* H) {
     else return H->S;
 }
 int sync_read(cmcg_handle* H);
+// The V-cycle's coarse end and the small-grid PCG: in clusters of 16 CTAs where allowed and the device can
+// hold them, else in one CTA and in launches.
+void plan_riesz(cmcg_handle* H, bool clusters);
 int band_status(cmcg_handle* H);  // after a synchronisation: CMCG_ERR_DEVICE_TIMEOUT if a one-launch loop gave up
 bool inexact(const cmcg_handle* H);
 // b_ready: the finest level's right-hand side already holds float(rhat0) (written by the

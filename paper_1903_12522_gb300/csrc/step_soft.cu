@@ -860,12 +860,9 @@ void launch_pcg_xr(long long n, double* x, double* r, const double* p, const dou
     else k_pcg_xr<false><<<pcg_blocks(n), kST, 0, st>>>(n, x, r, p, Ap, bf, red, first);
 }
 
-// Grids of up to kPcgClusterNodes nodes (see there).
-bool pcg_cluster_fits(const Geom& g) { return g.np <= kPcgClusterNodes; }
-
-void launch_pcg_cluster(const Geom& g, int order, const unsigned char* mask, double* x, double* r, double* p, double* Ap,
-                        const float* z, float* bf, Red red, bool first, cudaStream_t st) {
-    const double ck = -h_pow(g);
+// f(kernel, its launch configuration) for the k_pcg_cluster of this grid.
+template <typename F>
+static void with_pcg_cluster(const Geom& g, int order, cudaStream_t st, F f) {
     auto go = [&](auto kernel) {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(kClusterCtas);
@@ -878,14 +875,34 @@ void launch_pcg_cluster(const Geom& g, int order, const unsigned char* mask, dou
         attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) return;
-        cudaLaunchKernelEx(&cfg, kernel, x, r, p, Ap, z, bf, mask, red.sc, g, ck, first ? 1 : 0);
+        // (a refusal stays pending, for cuda_status or pcg_cluster_fits)
+        if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) f(kernel, cfg);
     };
     const bool two = g.np <= 2ll * kClusterCtas * kClusterThreads;
     static_assert(3ll * kClusterCtas * kClusterThreads >= kPcgClusterNodes, "nodes per thread");
     by_stencil(g, order, [&](auto D, auto O) {
         if (two) go(k_pcg_cluster<D(), O(), 2>);
         else go(k_pcg_cluster<D(), O(), 3>);
+    });
+}
+
+// Grids of up to kPcgClusterNodes nodes (see there).
+bool pcg_cluster_fits(const Geom& g, int order) {
+    if (g.np > kPcgClusterNodes) return false;
+    int clusters = 0;
+    with_pcg_cluster(g, order, nullptr, [&](auto kernel, cudaLaunchConfig_t& cfg) {
+        if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) != cudaSuccess) clusters = 0;
+    });
+    note_launch(-1);  // (by_stencil counts a launch)
+    if (clusters < 1) cudaGetLastError();
+    return clusters > 0;
+}
+
+void launch_pcg_cluster(const Geom& g, int order, const unsigned char* mask, double* x, double* r, double* p, double* Ap,
+                        const float* z, float* bf, Red red, bool first, cudaStream_t st) {
+    const double ck = -h_pow(g);
+    with_pcg_cluster(g, order, st, [&](auto kernel, cudaLaunchConfig_t& cfg) {
+        cudaLaunchKernelEx(&cfg, kernel, x, r, p, Ap, z, bf, mask, red.sc, g, ck, first ? 1 : 0);
     });
 }
 
