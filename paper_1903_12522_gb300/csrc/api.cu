@@ -1829,7 +1829,8 @@ int cmcg_no_cluster_selftest(cmcg_handle* h) {
 int cmcg_check_status(long long* count, long long* site, long long* index) {
     if (cudaDeviceSynchronize() != cudaSuccess) return CMCG_ERR_CUDA;
     long long total = 0, first_site = -1, first_index = 0;
-    for (auto read : {check_read_wave, check_read_riesz, check_read_pair, check_read_soft, check_read_band, check_read_block}) {
+    for (auto read : {check_read_wave, check_read_riesz, check_read_pair, check_read_soft, check_read_band, check_read_block,
+                      check_read_row, check_read_first_order}) {
         long long w[3];
         read(w);
         if (w[0] > 0 && first_site < 0) {

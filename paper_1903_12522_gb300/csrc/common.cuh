@@ -119,6 +119,9 @@ enum CheckSite {
     kSitePairGlobal = 4, // two-step kernel: a column's node or plane
     kSitePairShared = 5, // two-step kernel: a shared-memory neighbour
     kSiteMultigrid = 6,  // column-marching multigrid kernels of riesz.cu
+    kSiteRow = 7,        // kernels on padded rows (step_row.cu, first_order.cu)
+    kSiteCoarse = 8,     // the V-cycle's coarse end in a cluster (riesz.cu)
+    kSitePcgCluster = 9, // k_pcg_cluster
 };
 
 // Does the index range of a column-marching thread lie inside the grid: node (ix, iy, iz) for
@@ -162,6 +165,17 @@ __device__ __forceinline__ bool column_in_range(const Geom& g, int ix, int iy, i
     return check_range(lo, hi, g.np, site);
 #else
     (void)g, (void)ix, (void)iy, (void)z0, (void)z1, (void)radius, (void)site;
+    return true;
+#endif
+}
+
+// The same for the nodes x0 .. x0 + 3 of a row, as far as there are.
+__device__ __forceinline__ bool chunk_in_range(const Geom& g, int x0, int iy, int z0, int z1, int radius, int site) {
+#ifdef CMCG_CHECKED
+    const int x1 = x0 + 3 < g.nx ? x0 + 3 : g.nx;
+    return column_in_range(g, x0, iy, z0, z1, radius, site) && column_in_range(g, x1, iy, z0, z1, radius, site);
+#else
+    (void)g, (void)x0, (void)iy, (void)z0, (void)z1, (void)radius, (void)site;
     return true;
 #endif
 }

@@ -246,10 +246,16 @@ __global__ void __launch_bounds__(kFR, 8) k_fo_row(const float* __restrict__ in,
     const int bx = reverse ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
     const int by = reverse ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
     const int p = bx * kFR + (int)threadIdx.x;
-    const bool valid = p < plane4;
-    const int pc = valid ? p : plane4 - 1;  // (idle lanes take part in the shuffles)
-    const int iy = (int)((unsigned)pc / (unsigned)cx), ic = pc - iy * cx, x0 = 4 * ic;
     const int z0 = by * zc, z1 = min(z0 + zc, g.sz);
+    if (!CMCG_RANGE_OK(z0, z1 - 1, g.sz, kSiteRow)) return;  // uniform over the block
+    bool valid = p < plane4;
+    int pc = valid ? p : plane4 - 1;  // (idle lanes take part in the shuffles)
+    int iy = (int)((unsigned)pc / (unsigned)cx), ic = pc - iy * cx;
+    if (!chunk_in_range(g, 4 * ic, iy, z0, z1, 1, kSiteRow)) {
+        valid = false;
+        pc = iy = ic = 0;
+    }
+    const int x0 = 4 * ic;
     const int lane = (int)threadIdx.x & 31;
     const bool first = ic == 0;
     const int xe = g.nx - x0;  // element of the node x = nx (0 .. 3 in a row's last chunk)
@@ -509,6 +515,7 @@ __global__ void __launch_bounds__(kFT) k_fo_row_load(const double* __restrict__ 
     }
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < field; i += stride) {
         const RowNode r = row_node(g, px, i);
+        if (r.in && !CMCG_RANGE_OK(r.j, r.j, g.np, kSiteRow)) continue;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             float x = 0.f;
@@ -548,7 +555,7 @@ __global__ void __launch_bounds__(kFT) k_fo_row_end(const float* __restrict__ s,
     const double h3 = g.h * g.h * g.h;
     for (unsigned i = blockIdx.x * blockDim.x + threadIdx.x; i < field; i += stride) {
         const RowNode r = row_node(g, px, i);
-        if (!r.in) continue;
+        if (!r.in || !CMCG_RANGE_OK(r.j, r.j, g.np, kSiteRow)) continue;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
             double x = soft64::to_f64(s[i + (size_t)a * field]);
@@ -1054,4 +1061,7 @@ int fo_adjoint(cmcg_handle* H, const double* y, double* out) {
 }
 
 }  // namespace detail
+
+CMCG_CHECK_TU(first_order)
+
 }  // namespace cmcg

@@ -33,6 +33,8 @@ void check_read_pair(long long* out);
 void check_read_soft(long long* out);
 void check_read_band(long long* out);
 void check_read_block(long long* out);
+void check_read_row(long long* out);
+void check_read_first_order(long long* out);
 long long launch_count();
 
 // Planes per thread, zc or as many more as bring a launch of sz planes to the 65535 blocks that a grid has

@@ -636,6 +636,7 @@ __device__ __forceinline__ void sts(unsigned a, float v) { asm volatile("st.shar
 // that the reads of a node's neighbours overlap); else in this CTA.
 template <bool SPREAD>
 __device__ __forceinline__ float at(const CoarseLevel& l, unsigned a, int i) {
+    if (!CMCG_RANGE_OK(i, i, l.np, kSiteCoarse)) return 0.f;
     if (!SPREAD) return lds(a + 4u * (unsigned)i);
     const unsigned k = (unsigned)(i - l.lo);
     const unsigned owner = (unsigned)(((unsigned)i * l.m_chunk) >> 40);
@@ -729,6 +730,19 @@ __device__ __forceinline__ float blend_rn(float wa, float a, float wb, float b) 
 
 // The neighbour sum at node k (byte d) of the array at `a`.
 __device__ __forceinline__ float neighbour_sum(const CoarseLevel& l, unsigned a, int k, unsigned d) {
+#ifdef CMCG_CHECKED  // the sum's reach in the CTA's run and its copies of the neighbours'
+    {
+        int lo = d & 1u && !(d & 2u) ? 0 : -1, hi = d & 2u && !(d & 1u) ? 0 : 1;
+        auto axis = [&](bool first, bool last, int stride) {
+            if (!first || last) lo = min(lo, -stride);
+            if (!last || first) hi = max(hi, stride);
+        };
+        axis((d & 4u) != 0u, (d & 8u) != 0u, l.sx);
+        if (l.dim == 3) axis((d & 16u) != 0u, (d & 32u) != 0u, l.sxy);
+        const int n = l.halo ? l.chunk : l.np;
+        if (!CMCG_RANGE_OK(k + l.halo + lo, k + l.halo + hi, n + 2 * l.halo, kSiteCoarse)) return 0.f;
+    }
+#endif
     const unsigned p = a + 4u * (unsigned)k, sy = 4u * (unsigned)l.sx, sz = 4u * (unsigned)l.sxy;
     const float v0 = lds(p + (d & 1u ? 4u : -4u)), v1 = lds(p + (d & 2u ? -4u : 4u));
     const float v2 = lds(p + (d & 4u ? sy : -sy)), v3 = lds(p + (d & 8u ? -sy : sy));
@@ -909,6 +923,7 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle(const __grid_constant__ 
         const CoarseLevel& l = lev[q];
         const unsigned char* const mask = lv.mask[q];
         for (int k = tid; k < l.cnt; k += nt) {
+            if (!CMCG_RANGE_OK(l.lo + k, l.lo + k, lv.g[q].np, kSiteCoarse)) continue;
             float b = 0.f;
             unsigned dir = 0u;
             if (q == 0) b = bglob[l.lo + k];
@@ -1000,7 +1015,8 @@ __global__ void __launch_bounds__(1024) k_coarse_vcycle(const __grid_constant__ 
     if (nc > 0 || rank == 0) {
         const CoarseLevel& l = lev[0];
         if (nc == 0) __syncthreads();
-        for (int k = tid; k < l.cnt; k += nt) xglob[l.lo + k] = lds(l.x + 4u * k);
+        for (int k = tid; k < l.cnt; k += nt)
+            if (CMCG_RANGE_OK(l.lo + k, l.lo + k, lv.g[0].np, kSiteCoarse)) xglob[l.lo + k] = lds(l.x + 4u * k);
     }
 }
 

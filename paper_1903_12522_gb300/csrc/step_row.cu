@@ -77,10 +77,16 @@ __global__ void __launch_bounds__(kRT, ORDER == 2 ? 10 : 7)
     const int bx = reverse ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
     const int by = reverse ? (int)(gridDim.y - 1 - blockIdx.y) : (int)blockIdx.y;
     const int p = bx * kRT + (int)threadIdx.x;
-    const bool valid = p < plane4;
-    const int pp = valid ? p : plane4 - 1;  // (idle lanes take part in the shuffles)
-    const int iy = (int)((unsigned)pp / (unsigned)cx), ic = pp - iy * cx, x0 = 4 * ic;
     const int z0 = by * zc, z1 = min(z0 + zc, g.sz);
+    if (!CMCG_RANGE_OK(z0, z1 - 1, g.sz, kSiteRow)) return;  // uniform over the block
+    bool valid = p < plane4;
+    int pp = valid ? p : plane4 - 1;  // (idle lanes take part in the shuffles)
+    int iy = (int)((unsigned)pp / (unsigned)cx), ic = pp - iy * cx;
+    if (!chunk_in_range(g, 4 * ic, iy, z0, z1, ORDER / 2, kSiteRow)) {
+        valid = false;
+        pp = iy = ic = 0;
+    }
+    const int x0 = 4 * ic;
     const int lane = (int)threadIdx.x & 31;
     const bool first = ic == 0;
     const int xe = g.nx - x0;  // element of the node x = nx (0 .. 3 in a row's last chunk)
@@ -304,5 +310,7 @@ void launch_step_row(const RowStep& a, int order, cudaStream_t st) {
     if (order == 2) row_flags<2>(a, st);
     else row_flags<4>(a, st);
 }
+
+CMCG_CHECK_TU(row)
 
 }  // namespace cmcg

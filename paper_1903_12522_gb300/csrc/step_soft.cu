@@ -636,6 +636,7 @@ __global__ void __launch_bounds__(kClusterThreads, 1)
         if (j >= hi) continue;
         const unsigned t = (unsigned)j / (unsigned)g.sx;
         const int ix = j - (int)t * g.sx, iz = DIM == 3 ? (int)(t / (unsigned)g.sy) : 0, iy = (int)t - iz * g.sy;
+        if (!column_in_range(g, ix, iy, iz, iz + 1, ORDER / 2, kSitePcgCluster)) continue;
         SoftLap<DIM, ORDER, Latest> lap(Latest{p}, g, ix, iy);
         double pj;
         lap.start(j, iz);
