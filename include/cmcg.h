@@ -110,7 +110,8 @@ extern "C" {
                                to its size (restored when the last such handle is destroyed).
                                Applies to CMCG_FP32 / CMCG_MIXED handles on a created stream
                                whose kappa fits the device's largest set-aside (84.7 MB on a
-                               GB300: grids up to 21 M nodes); otherwise ignored.  Side effects
+                               GB300: grids up to 21 M nodes) and whose step loops do not hold
+                               the grid, and with it kappa, on chip; otherwise ignored.  Side effects
                                beyond the handle: the stream attribute (cleared at destroy) and
                                the set-aside, which other work in the process shares. */
 

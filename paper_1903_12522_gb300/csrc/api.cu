@@ -205,6 +205,8 @@ static size_t g_l2_prev_limit = 0;
 void l2_kappa_begin(cmcg_handle* H) {
     const cudaStream_t st = H->st;
     if (!H->kap32 || st == nullptr || st == cudaStreamLegacy || st == cudaStreamPerThread) return;
+    // loops that hold the grid on chip read kappa once: the set-aside would only take cache from the rest
+    if (H->band.bands > 0 || (H->block.ny_blocks > 0 && H->opt.tile[3] == 0)) return;
     int dev = 0, max_persist = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&max_persist, cudaDevAttrMaxPersistingL2CacheSize, dev) != cudaSuccess) {
