@@ -153,12 +153,6 @@ size_t layout(cmcg_handle* H, const Geom& g, const cmcg_options& o, char* base) 
         H->wo0 = c.take<double>(np);
         H->wo1 = c.take<double>(np);
     }
-    if (o.precision != CMCG_FP64 && row_fits(g)) {
-        const size_t pp = (size_t)row_pitch(g) * g.sy * g.sz;
-        H->row_a = c.take<float>(pp);
-        H->row_b = c.take<float>(pp);
-        H->row_kap = c.take<float>(pp);
-    }
     // at most as many bands or blocks as a GB300 has SMs (fewer SMs: a plan of fewer words, at create)
     if (band_plan(g, H->order, o.precision == CMCG_FP64 ? 8 : 4, kBandStop, &H->band) ||
         (o.precision != CMCG_FP64 && H->order == 2 && block_plan(g, kBandStop, &H->block))) {
@@ -172,7 +166,14 @@ size_t layout(cmcg_handle* H, const Geom& g, const cmcg_options& o, char* base) 
     H->pr = c.take<double>(np);
     H->pp = c.take<double>(np);
     H->pAp = c.take<double>(np);
-    H->pzd = c.take<double>(np);
+    H->pzd = o.precision != CMCG_FP64 ? c.take<double>(np) : nullptr;  // (FP64: z is read as the V-cycle's floats)
+    if (o.precision != CMCG_FP64 && row_fits(g)) {
+        // no Riesz PCG is under way while a period's steps run: the padded fields use its vectors, whose
+        // 2 N_p floats are enough for rows of nine nodes and more
+        H->row_a = (float*)H->pr;
+        H->row_b = (float*)H->pp;
+        H->row_kap = c.take<float>((size_t)row_pitch(g) * g.sy * g.sz);
+    }
     Geom lg[kMaxLevels];
     H->nlev = mg_geometries(g, lg);
     for (int l = 0; l < H->nlev; ++l) {

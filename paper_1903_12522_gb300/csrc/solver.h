@@ -54,7 +54,7 @@ struct cmcg_handle {
     bool pcg_cluster = false;  // FP64, small grids: a Riesz PCG iteration's vector part in one cluster launch
     int riesz_guess = 0;      // PCG iterations of the previous Riesz solve
     unsigned char* sflag = nullptr;  // 3D FP32 steps: where S32 is not zero (launch_source_flags)
-    // FP32 3D step loops on padded rows (step_row.cu): the two wave fields and kappa
+    // FP32 3D step loops on padded rows (step_row.cu): the two wave fields (in pr and pp) and kappa
     float *row_a = nullptr, *row_b = nullptr, *row_kap = nullptr;
     // step loops in one launch, 2D (step_band.cu) and FP32 3D 7-point (step_block.cu): exchange_words
     // exchange words, and the steps done per band or block; side_by_side: in the engine, whose
