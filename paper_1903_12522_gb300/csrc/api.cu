@@ -163,16 +163,19 @@ size_t layout(cmcg_handle* H, const Geom& g, const cmcg_options& o, char* base) 
     }
     H->side.bands = 0;
     if (o.precision != CMCG_FP64 && H->band.bands > 0) band_plan(g, H->order, 4, 16, &H->side);
+    const bool rows = o.precision != CMCG_FP64 && row_fits(g);
+    // (here, not behind the PCG's vectors: a 257^3 solve takes 3.378 s, there 3.410; 241^3 2.443 and 2.447,
+    // 249^3 2.798 and 2.796)
+    if (rows) H->row_kap = c.take<float>((size_t)row_pitch(g) * g.sy * g.sz);
     H->pr = c.take<double>(np);
     H->pp = c.take<double>(np);
     H->pAp = c.take<double>(np);
     H->pzd = o.precision != CMCG_FP64 ? c.take<double>(np) : nullptr;  // (FP64: z is read as the V-cycle's floats)
-    if (o.precision != CMCG_FP64 && row_fits(g)) {
+    if (rows) {
         // no Riesz PCG is under way while a period's steps run: the padded fields use its vectors, whose
         // 2 N_p floats are enough for rows of nine nodes and more
         H->row_a = (float*)H->pr;
         H->row_b = (float*)H->pp;
-        H->row_kap = c.take<float>((size_t)row_pitch(g) * g.sy * g.sz);
     }
     Geom lg[kMaxLevels];
     H->nlev = mg_geometries(g, lg);
@@ -390,9 +393,8 @@ PeriodBuffers fwd_begin(cmcg_handle* H, const double* w0, const double* w1, bool
 
 // z-planes per thread of the one-step kernels; negative selects the variant that processes two
 // planes per loop iteration (tile[3] == 3), kZcFlat the FP32 vector form (tile[3] == 5)
-// tile[3] == 0 takes the scheme the autotuner found fastest on every measured class: the
-// z-pair kernel on 3D 7- and 13-point grids, the vector form on 2D 5-point grids (FP64 steps
-// fall back to their one-step kernels).
+// tile[3] == 0, where neither the loops on chip nor the padded rows (row_steps) take the grid: the
+// z-pair kernel on 3D 7- and 13-point grids, the vector form on 2D 5-point grids.
 int step_zc(const cmcg_handle* H) {
     const int scheme = H->opt.tile[3];
     if (H->order == 2 && (scheme == 5 || (scheme == 0 && H->g.dim == 2))) return kZcFlat;
@@ -412,8 +414,10 @@ bool use_pairs(const cmcg_handle* H, bool src) {
 
 // One leapfrog step cur -> prev (in place).  FP64 handles step with the integer stencil sum.  The
 // FP64 periods of a mixed-precision handle (its outer gradients) keep the plain FP64 step: a
-// change of their last bits would send the FP32 inner solve along other roundings.  FP32 3D 7-point steps without a source go through
-// the bulk-copy kernel when tile[3] == 4 (tile[1] = band rows, tile[0] = planes per CTA).
+// change of their last bits would send the FP32 inner solve along other roundings.  FP32 steps come here in
+// 3D with another scheme than the default and where neither the on-chip loops nor the padded rows take the
+// grid; 7-point ones without a source go through the bulk-copy kernel when tile[3] == 4 (tile[1] = band
+// rows, tile[0] = planes per CTA).
 template <typename T>
 void step_one(cmcg_handle* H, const T* cur, T* prev, const T* kap, const T* S, double cs, double sn, int flags,
               int zc) {
