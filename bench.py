@@ -228,7 +228,8 @@ def kernel_traffic(profile, kernel_src_hash):
 
 def kernel_src_hash(name="k_step3d7("):
     """Hash of a kernel's source text (the kernel that ncu counters describe)."""
-    fname = "step_bulk.cu" if "bulk" in name else ("step_pair.cu" if "pair" in name else "wave.cu")
+    fname = ("step_bulk.cu" if "bulk" in name else "step_pair.cu" if "pair" in name else
+             "step_row.cu" if "row" in name else "wave.cu")
     src = open(os.path.join(ROOT, "paper_1903_12522_gb300", "csrc", fname)).read()
     start = src.index(name)
     end = src.index("\n}\n", start) + 2  # the kernel's closing brace
@@ -566,9 +567,15 @@ def run_ours(args):
         per_launch, bpl, upl = s32 / n32, STEP_BYTES_FP32, 1
         name, prof, src = ("k_step3d7_z2<float>: FP32 leapfrog step, 3D 7-point, two z-planes per thread",
                            "step3d7z2_fp32_sphere.json", "k_step3d7_z2(")
+    elif n32 > 0 and s.opts.tile[3] == 0 and n32 <= 2 * sum(st.periods for st in stats):
+        # grids that fit on chip: one launch per period's step loop, which reads y^n, y^{n-1} and kappa
+        # and writes the two fields once
+        per_launch, bpl, upl = s32 / n32, 20, stats[0].steps_per_period - 1
+        name, prof, src = "k_block3: FP32 leapfrog step loop, 3D 7-point, the grid held on chip", None, None
     elif n32 > 0 and s.opts.tile[3] == 0:
         per_launch, bpl, upl = s32 / n32, STEP_BYTES_FP32, 1
-        name, prof, src = "k_step_row<2>: FP32 leapfrog step, 3D 7-point, rows padded to float4s", None, None
+        name, prof, src = ("k_step_row<2>: FP32 leapfrog step, 3D 7-point, rows padded to float4s",
+                           "step_row_fp32_sphere.json", "k_step_row(")
     elif n32 > 0:
         per_launch, bpl, upl = s32 / n32, STEP_BYTES_FP32, 1
         name, prof, src = "k_step3d7<float>: FP32 leapfrog step, 3D 7-point", "step3d7_fp32_sphere.json", "k_step3d7("
