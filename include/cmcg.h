@@ -158,7 +158,8 @@ typedef struct {
                                at a given tol does not depend on the run-up.                  */
     int tile[4];            /* launch shape of the leapfrog kernels, 0 = default.  [3] selects
                                the step scheme of 3D 7-point steps (the others keep one step per
-                               launch): 0 = the default (the fastest measured): FP32 3D steps on
+                               launch): 0 = the default (the fastest measured): FP32 3D 7-point
+                               loops of grids that fit on chip in one launch, other FP32 3D steps on
                                rows padded to whole float4s (scheme 3 where the grid is too narrow
                                or too large for it), scheme 5 on 2D 5-point grids; 1 = one
                                step per launch, [0] z-planes per thread

@@ -268,7 +268,9 @@ void row_launch(const RowStep& a, cudaStream_t st) {
     const Geom& g = a.g;
     const int plane4 = (a.px >> 2) * g.sy;
     const unsigned bxy = (unsigned)((plane4 + kRT - 1) / kRT);
-    // planes per thread: four where that makes at least four waves of blocks, else two
+    // planes per thread: four where that makes at least four waves of blocks, else two (us a step of a
+    // backward period with two and with four: 151^3 12.2 and 14.3, 193^3 21.7 and 21.6, 225^3 35.3 and 33.6,
+    // 257^3 51.3 and 49.4; 13-point 129^3 12.0 and 14.0, 193^3 28.3 and 28.3, 257^3 66.4 and 62.5)
     const int per_sm = ORDER == 2 ? 10 : 7;
     const int zc = planes_per_thread((long long)bxy * ((g.sz + 3) / 4) >= 4ll * 152 * per_sm ? 4 : 2, g.sz);
     const dim3 grid(bxy, (unsigned)((g.sz + zc - 1) / zc));

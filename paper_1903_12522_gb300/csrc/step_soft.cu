@@ -179,9 +179,9 @@ struct SoftLap {
 
 // One leapfrog step, one thread per (x, y) column of zc planes (2D: one node).
 //
-// Bound: issue slots of the integer pipes and latency (FP64 work left per update: 2 y - y_prev
-// and the fused multiply-add with kappa, against nine operations and, on the faces, a square
-// root and a division).  193^3, with a source on the faces: 246 us a step in FP64 arithmetic, 87 us
+// Bound: latency; the FP64 and ALU pipes and the issue slots are each busy 43 to 44 % of the time at
+// half of the warp slots (FP64 work left per update: 2 y - y_prev and the fused multiply-add with kappa,
+// against nine operations and, on the faces, a square root and a division).  193^3, with a source on the faces: 246 us a step in FP64 arithmetic, 87 us
 // now, 73 without one (230 MB of algorithmic bytes, 34 us at the copy bandwidth).
 //
 // B: resident blocks per SM.  Whole backward periods of 57 steps: 7-point 193^3 4.66 ms with four, 4.47
