@@ -61,6 +61,10 @@ __device__ __noinline__ double add_source(double d, const double* __restrict__ S
     return d + fma(s.x, cs, s.y * sn);
 }
 
+// The period's start takes the real part only: an imaginary part that is not finite acts from the first
+// step on, not here through a product with zero.
+__device__ __noinline__ double add_half_re(double d, const double* __restrict__ S, int j) { return fma(0.5, S[2 * j], d); }
+
 // One thread's column of a launch: its (x, y), its planes, its faces.
 template <int DIM>
 struct Column {
@@ -235,7 +239,7 @@ __global__ void __launch_bounds__(kST, 3)
         const bool face = m.face(iz);
         if (face) vj = face_minus(vj, wface[j]);
         double v = fma(0.5 * k, L, fma(dt, vj, yc));
-        if (SRC && (face || !src_faces)) v = add_source(v, S, j, 0.5, 0.0);
+        if (SRC && (face || !src_faces)) v = add_half_re(v, S, j);
         const bool dir = soft64::is_zero(k);  // Dirichlet
         y0[j] = dir ? 0.0 : yc;
         y1[j] = dir ? 0.0 : v;
