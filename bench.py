@@ -119,7 +119,7 @@ def method_config(args):
 
 def tile_config(solver):
     t = list(solver.opts.tile)
-    scheme = {0: "one step per launch, rows padded to float4s", 2: "two steps per launch", 3: "one step per launch, two z-planes per thread",
+    scheme = {0: "step loops on chip where the grid fits, else one step per launch on rows padded to float4s", 2: "two steps per launch", 3: "one step per launch, two z-planes per thread",
               4: "one step per launch, operands staged by TMA bulk copies into a shared-memory ring"}
     return {"tile": t, "step_scheme": scheme.get(t[3], "one step per launch")}
 
